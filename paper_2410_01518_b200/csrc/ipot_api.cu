@@ -434,10 +434,11 @@ int launch_novelty(ipot *p, const void *logits, size_t row_stride, const int32_t
 {
     const size_t rows = (size_t)p->cfg.batch * n_tokens;
     const int segs = (vocab + kNovSegElems - 1) / kNovSegElems;
+    const int seg_elems = ((vocab + segs - 1) / segs + 63) / 64 * 64;   // at most kNovSegElems, itself a multiple of 64
     int *counters = reinterpret_cast<int *>(p->nov_scratch);
     float2 *partial = reinterpret_cast<float2 *>(p->nov_scratch + kNovCounterBytes);
     dim3 grid(segs, (unsigned)rows);
-    novelty_kernel<T><<<grid, kNovThreads, 0, p->stream>>>((const T *)logits, row_stride, vocab, segs, partial, counters, labels,
+    novelty_kernel<T><<<grid, kNovThreads, 0, p->stream>>>((const T *)logits, row_stride, vocab, segs, seg_elems, partial, counters, labels,
                                                            n_tokens, out, out_stride, slot0, p->status);
     p->launches += 1;
     IPOT_CUDA(cudaGetLastError());
