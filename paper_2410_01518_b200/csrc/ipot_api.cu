@@ -60,6 +60,7 @@ struct ipot {
     float *dec_partial;  // [units][dec_splits][G][d + 2]: ipot_decode_attention's split results
     int *dec_counters;   // [units], zero between calls
     int dec_splits;
+    bool dec_ready[2];   // the fp32-FMA and the tensor-core kernel's shared memory limit is set (once per pot)
     char *nov_scratch;   // scratch of ipot_nuc_scores, grown on demand: 65536 row counters (always zero between
                          // calls), then [tokens][segments] float2
     size_t nov_capacity;  // float2 entries behind the counters
@@ -474,7 +475,8 @@ int launch_decode_g(ipot *p, const void *q, float *out, float *lse)
     if (splits > (N + tile_keys - 1) / tile_keys) splits = (N + tile_keys - 1) / tile_keys;  // at least one stage of rows per block
     const size_t smem = decode_smem_bytes(G, d);
     auto kern = decode_attn_kernel<T, G>;
-    if (smem > 48 * 1024) IPOT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024 && !p->dec_ready[0]) IPOT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    p->dec_ready[0] = true;
     dim3 grid(splits, p->units);
     kern<<<grid, kDecThreads, smem, p->stream>>>((const T *)score_keys(p), (const T *)p->V, (const T *)q, out, lse, p->dec_partial,
                                                  p->dec_counters, N, d, p->row_bytes / 16, (size_t)p->cfg.pot_size * d,
@@ -493,7 +495,8 @@ int launch_decode_mma(ipot *p, const void *q, float *out, float *lse)
     if (splits > (N + 63) / 64) splits = (N + 63) / 64;  // at least one 16-key tile per warp
     const size_t smem = decode_mma_smem_bytes(p->G, D);
     auto kern = decode_attn_mma_kernel<D>;
-    IPOT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (!p->dec_ready[1]) IPOT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    p->dec_ready[1] = true;
     dim3 grid(splits, p->units);
     kern<<<grid, kMmaWarps * 32, smem, p->stream>>>((const __nv_bfloat16 *)score_keys(p), (const __nv_bfloat16 *)p->V,
                                                     (const __nv_bfloat16 *)q, out, lse, p->dec_partial, p->dec_counters, N, p->G,

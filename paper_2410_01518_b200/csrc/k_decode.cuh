@@ -31,12 +31,32 @@ __device__ __forceinline__ float dec_scale(float m, float ref) { return m == -IN
 
 // The end of a block's work: dec_sm holds, per warp and head, the unnormalised output (d floats), the reference
 // exponent and the sum.  The warps are merged into the block's entry of `partial`; the block that finishes a unit
-// last merges the unit's splits and writes the normalised output and the log-sum-exp.
-__device__ __forceinline__ void dec_finish(const float *dec_sm, int warps, int G, int d, int unit, int split, int splits,
+// last merges the unit's splits (at most 32) and writes the normalised output and the log-sum-exp.  That tail is what a
+// small call consists of (8 units x 2048 rows: 64 keys per block), so it is a chain of as few round trips as possible: one
+// atomic that releases and acquires, the splits' references and sums read by a warp per head, one lane each, and then
+// their rows eight loads at a time.  (With a thread walking over the splits element by element it took 15 of 24 us.)
+__device__ __forceinline__ void dec_finish(float *dec_sm, int warps, int G, int d, int unit, int split, int splits,
                                            float *partial, int *counters, float *__restrict__ out, float *__restrict__ lse, int *is_last)
 {
     const int ds = d + 2;
     __syncthreads();
+    if (splits == 1) {   // nothing to exchange: the warps' results are normalised where they are
+        for (int e = threadIdx.x; e < G * d; e += blockDim.x) {
+            const int h = e / d, c = e - h * d;
+            float ref = -INFINITY;
+            for (int w = 0; w < warps; ++w) ref = fmaxf(ref, dec_sm[((size_t)w * G + h) * ds + d]);
+            float o = 0.f, den = 0.f;
+            for (int w = 0; w < warps; ++w) {
+                const float *row = dec_sm + ((size_t)w * G + h) * ds;
+                const float f = dec_scale(row[d], ref);
+                o = fmaf(row[c], f, o);
+                den = fmaf(row[d + 1], f, den);
+            }
+            out[((size_t)unit * G + h) * d + c] = o / den;
+            if (c == 0 && lse) lse[(size_t)unit * G + h] = 0.6931471805599453f * (ref + log2f(den));
+        }
+        return;
+    }
     float *dst = partial + ((size_t)unit * splits + split) * G * ds;
     for (int e = threadIdx.x; e < G * ds; e += blockDim.x) {
         const int h = e / ds, c = e - h * ds;
@@ -55,30 +75,50 @@ __device__ __forceinline__ void dec_finish(const float *dec_sm, int warps, int G
         __stcg(dst + e, v);
     }
     // ---- the splits of the unit: the block that arrives last merges them
-    __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        const int done = splits > 1 ? atomicAdd(&counters[unit], 1) : 0;
+        int done;   // releases the block's entry (the barrier orders the other threads' stores before it), acquires the others'
+        asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(done) : "l"(counters + unit) : "memory");
         *is_last = done == splits - 1;
-        if (*is_last && splits > 1) counters[unit] = 0;  // ready for the next call
+        if (*is_last) counters[unit] = 0;  // ready for the next call
     }
     __syncthreads();
     if (!*is_last) return;
-    __threadfence();
     const float *src = partial + (size_t)unit * splits * G * ds;
+    // a warp takes a head, a lane a split: weights 2^(ref - largest ref) / denominator into shared memory
+    float *wsm = dec_sm;   // [G][splits]: the warps' results are merged, their memory is free
+    const int lane = threadIdx.x & 31;
+    for (int h = threadIdx.x >> 5; h < G; h += blockDim.x >> 5) {
+        float r = -INFINITY, l = 0.f;
+        if (lane < splits) {
+            r = __ldcg(src + ((size_t)lane * G + h) * ds + d);
+            l = __ldcg(src + ((size_t)lane * G + h) * ds + d + 1);
+        }
+        float ref = r;
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) ref = fmaxf(ref, __shfl_xor_sync(0xffffffffu, ref, off));
+        const float w = dec_scale(r, ref);
+        float den = l * w;
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
+        if (lane < splits) wsm[h * splits + lane] = w / den;
+        if (lane == 0 && lse) lse[(size_t)unit * G + h] = 0.6931471805599453f * (ref + log2f(den));
+    }
+    __syncthreads();
     for (int e = threadIdx.x; e < G * d; e += blockDim.x) {
         const int h = e / d, c = e - h * d;
-        float ref = -INFINITY;
-        for (int sp = 0; sp < splits; ++sp) ref = fmaxf(ref, __ldcg(src + ((size_t)sp * G + h) * ds + d));
-        float o = 0.f, den = 0.f;
-        for (int sp = 0; sp < splits; ++sp) {
-            const float *row = src + ((size_t)sp * G + h) * ds;
-            const float w = dec_scale(__ldcg(row + d), ref);
-            o = fmaf(__ldcg(row + c), w, o);
-            den = fmaf(__ldcg(row + d + 1), w, den);
+        const float *row = src + (size_t)h * ds + c, *w = wsm + h * splits;
+        float o[4] = {0.f, 0.f, 0.f, 0.f};
+        int sp = 0;
+        for (; sp + 8 <= splits; sp += 8) {
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = __ldcg(row + (size_t)(sp + i) * G * ds);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o[i & 3] = fmaf(v[i], w[sp + i], o[i & 3]);
         }
-        out[((size_t)unit * G + h) * d + c] = o / den;
-        if (c == 0 && lse) lse[(size_t)unit * G + h] = 0.6931471805599453f * (ref + log2f(den));
+        for (; sp < splits; ++sp) o[0] = fmaf(__ldcg(row + (size_t)sp * G * ds), w[sp], o[0]);
+        out[((size_t)unit * G + h) * d + c] = (o[0] + o[1]) + (o[2] + o[3]);
     }
 }
 
