@@ -160,7 +160,7 @@ int ipot_append_chunk(ipot_t *pot, const void *K, const void *V, int n_tokens);
  *     chunk, so rows that the cycle drops are never copied and survivors move once instead of twice;
  *   - every other call that reads or exposes the pot's rows (ipot_view, ipot_decode_attention, a further append,
  *     ipot_append_chunk_host, ipot_set_stream, ipot_sync_status, turning the mode off) first queues the plain copy.
- * In rotary mode only the values are deferred (the scorers read the rotated copy, which is written at append).
+ * In rotary mode the scorers read the rotated copy, which is written at append; values and unrotated keys are deferred.
  * The pot's contents after any of these calls are the same as without the mode.  What changes is the lifetime of
  * the chunk buffers: they must stay alive and unchanged until the next ipot_score_and_compress*() has run on the
  * stream or ipot_sync_status() has returned - synchronising the stream right after the append is not enough.

@@ -15,6 +15,13 @@ __device__ __forceinline__ void set_status(int *status, int code)
     if (status) atomicCAS(status, 0, code);
 }
 
+__device__ __forceinline__ unsigned long long global_timer_ns()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 // Monotone map float -> uint32: a < b  <=>  key(a) < key(b) (for non-NaN values).
 __device__ __forceinline__ uint32_t order_key(float f)
 {

@@ -30,11 +30,11 @@ struct ipot {
     int sm_count;
     int scorer;
     int G, units, elem_bytes, row_bytes;
-    int compact_slices, rope_slices;
     cudaStream_t stream;
     // Deferred append (ipot_set_deferred_append): the newest chunk's rows (slots pend_first .. len - 1) still lie in
     // the caller's buffers; the tensor-core scorer reads its keys there and the compaction fetches the survivors
-    // from there, so rows that the cycle drops are never copied.  NULL = those rows are in the pot.
+    // from there, so rows that the cycle drops are never copied.  NULL = those rows are in the pot.  In rotary mode
+    // pend_K are the unrotated keys; their rotated copy is complete.
     int deferred;
     const void *pend_K, *pend_V;
     int pend_n, pend_first;
@@ -54,6 +54,7 @@ struct ipot {
     float2 *cap_stats;   // [units][max M]: (max, sum) over the CaP's own keys, CaP-inclusive scoring only
     uint8_t *nuc_mask;   // [batch][pot_size]
     int32_t *idx;        // [units][keep]
+    GatherPlan gather;   // what the selection leaves for the gather
     int *status;         // sticky device status word
     void *stage_q;       // device staging for the *_host calls
     void *stage_kc;
@@ -119,7 +120,7 @@ void free_all(ipot *p)
 {
     tc_plan_destroy(p->tc);
     cudaFree(p->K); cudaFree(p->V); cudaFree(p->Krot); cudaFree(p->scores); cudaFree(p->summed);
-    cudaFree(p->row_stats); cudaFree(p->mma_part); cudaFree(p->cap_stats); cudaFree(p->nuc_mask); cudaFree(p->idx); cudaFree(p->status);
+    cudaFree(p->row_stats); cudaFree(p->mma_part); cudaFree(p->cap_stats); cudaFree(p->nuc_mask); cudaFree(p->idx); cudaFree(p->gather.ints); cudaFree(p->status);
     cudaFree(p->stage_q); cudaFree(p->stage_kc); cudaFree(p->stage_aux); cudaFree(p->nov_scratch); cudaFree(p->dec_partial); cudaFree(p->dec_counters);
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
     if (p->ev_join) cudaEventDestroy(p->ev_join);
@@ -256,8 +257,8 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
     // keys of a deferred append: the tensor-core scorers read whole slabs of them where they are, anything else
     // wants them in the pot
     const int slab_keys = scorer == IPOT_SCORER_TENSOR ? kTcSlab : scorer == IPOT_SCORER_TENSOR_SWEEPS ? kTsSlab : 0;
-    const bool keys_in_chunk = p->pend_K && slab_keys && p->pend_first % slab_keys == 0;
-    if (p->pend_K && !keys_in_chunk) {
+    const bool keys_in_chunk = p->pend_K && !p->rope && slab_keys && p->pend_first % slab_keys == 0;
+    if (p->pend_K && !p->rope && !keys_in_chunk) {
         int mrc = materialise(p, true, false);
         if (mrc != IPOT_OK) return mrc;
     }
@@ -320,28 +321,37 @@ int check_cycle_args(ipot *p, const void *Q, int cap_rows, const float *aux, boo
     return IPOT_OK;
 }
 
-// One launch: z = 0 gathers the unrotated keys and writes the rotated copy, z = 1 gathers the values.
-template <typename T>
-void launch_compact_rope_t(ipot *p, int keep, int N, int row_vecs, size_t unit_vecs)
+// The gather of the survivors (and, in rotary mode, the rotated copy of the keys).  Programmatic dependent launch: the grid
+// is set up while the selection still runs and waits inside the kernel.
+template <typename Kernel, typename... Rot>
+cudaError_t launch_gather(ipot *p, Kernel kern, const GatherParams &g, const Rot &...rot)
 {
-    const int ks = p->rope_slices, vs = p->compact_slices;
-    dim3 grid(ks > vs ? ks : vs, p->units, 2);
-    auto kern = p->rope == IPOT_ROPE_INTERLEAVED ? compact_rope_kernel<T, true> : compact_rope_kernel<T, false>;
-    kern<<<grid, kMoveThreads, 0, p->stream>>>((uint4 *)p->K, (uint4 *)p->Krot, (const T *)p->rope_cos, (const T *)p->rope_sin, p->idx,
-                                               keep, N, row_vecs, ks, row_vecs / 2 / ks, unit_vecs, p->status, (uint4 *)p->V, vs,
-                                               row_vecs / vs, pending_rows(p));
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(p->gather.chunks, 2, p->units);
+    lc.blockDim = dim3(kGatherThreads, 1, 1);
+    lc.stream = p->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kern, g, rot...);
 }
 
-void launch_compact_rope(ipot *p, int keep, int N, int row_vecs, size_t unit_vecs)
+template <typename T>
+cudaError_t launch_gather_rope(ipot *p, const GatherParams &g)
 {
-    if (p->cfg.dtype == IPOT_F32) launch_compact_rope_t<float>(p, keep, N, row_vecs, unit_vecs);
-    else launch_compact_rope_t<__nv_bfloat16>(p, keep, N, row_vecs, unit_vecs);
+    if (p->rope == IPOT_ROPE_INTERLEAVED)
+        return launch_gather(p, compact_rope_kernel<T, true>, g,
+                             GatherRotate<T, true>{(uint4 *)p->Krot, (const T *)p->rope_cos, (const T *)p->rope_sin, g.unit_vecs});
+    return launch_gather(p, compact_rope_kernel<T, false>, g,
+                         GatherRotate<T, false>{(uint4 *)p->Krot, (const T *)p->rope_cos, (const T *)p->rope_sin, g.unit_vecs});
 }
 
-// New key rows (src, unit stride src_unit_vecs) -> pot rows [len, len + n) unrotated and rotated; if srcV is not
-// NULL the same launch copies the value rows ([units][n rows]) into the pot.
+// New key rows (src, unit stride src_unit_vecs) -> pot rows [len, len + n) rotated and, with keys_too, unrotated; if srcV
+// is not NULL the same launch copies the value rows ([units][n rows]) into the pot.
 template <typename T>
-void launch_append_rope_t(ipot *p, const void *src, size_t src_unit_vecs, const void *srcV, int n)
+void launch_append_rope_t(ipot *p, const void *src, size_t src_unit_vecs, const void *srcV, int n, bool keys_too)
 {
     const int row_vecs = p->row_bytes / 16;
     const size_t items = (size_t)n * (row_vecs / 2), unit_vecs = (size_t)p->cfg.pot_size * row_vecs;
@@ -349,74 +359,35 @@ void launch_append_rope_t(ipot *p, const void *src, size_t src_unit_vecs, const 
     if (pieces < 1) pieces = 1;
     dim3 grid(pieces, p->units, srcV ? 2 : 1);
     auto kern = p->rope == IPOT_ROPE_INTERLEAVED ? append_rope_kernel<T, true> : append_rope_kernel<T, false>;
-    kern<<<grid, kMoveThreads, 0, p->stream>>>((const uint4 *)src, src_unit_vecs, (uint4 *)p->K, (uint4 *)p->Krot, (const T *)p->rope_cos,
+    kern<<<grid, kMoveThreads, 0, p->stream>>>((const uint4 *)src, src_unit_vecs, (uint4 *)(keys_too ? p->K : nullptr), (uint4 *)p->Krot, (const T *)p->rope_cos,
                                                (const T *)p->rope_sin, n, row_vecs, unit_vecs, p->len, (const uint4 *)srcV, (uint4 *)p->V);
 }
 
-void launch_append_rope(ipot *p, const void *src, size_t src_unit_vecs, const void *srcV, int n)
+void launch_append_rope(ipot *p, const void *src, size_t src_unit_vecs, const void *srcV, int n, bool keys_too = true)
 {
-    if (p->cfg.dtype == IPOT_F32) launch_append_rope_t<float>(p, src, src_unit_vecs, srcV, n);
-    else launch_append_rope_t<__nv_bfloat16>(p, src, src_unit_vecs, srcV, n);
-}
-
-// Byte-column slices per row for the compaction grid: enough blocks to fill the device, slices of >= 64 bytes.
-int compact_slices(const ipot *p)
-{
-    const int row_vecs = p->row_bytes / 16;
-    int slices = 1;
-    while (row_vecs % (slices * 2) == 0 && row_vecs / (slices * 2) >= 4 &&
-           (long long)p->units * 2 * slices < 8LL * p->sm_count)
-        slices *= 2;
-    return slices;
-}
-
-// The same for the vector pairs (g, g + row_vecs / 2) of compact_rope_kernel: slices of >= 2 pairs.
-int rope_slices(const ipot *p)
-{
-    const int half_vecs = p->row_bytes / 32;
-    int slices = 1;
-    while (half_vecs % (slices * 2) == 0 && half_vecs / (slices * 2) >= 2 &&
-           (long long)p->units * slices < 8LL * p->sm_count)
-        slices *= 2;
-    return slices;
+    if (p->cfg.dtype == IPOT_F32) launch_append_rope_t<float>(p, src, src_unit_vecs, srcV, n, keys_too);
+    else launch_append_rope_t<__nv_bfloat16>(p, src, src_unit_vecs, srcV, n, keys_too);
 }
 
 int run_cycle(ipot *p, const void *Q, const void *Kc, int cap_rows, const float *aux)
 {
-    const int N = p->len, keep = p->cfg.keep, T = p->cfg.nuc_slots;
+    const int N = p->len, keep = p->cfg.keep, T = p->cfg.nuc_slots, row_vecs = p->row_bytes / 16;
     int parts = 1;
     cudaEvent_t *ev = (p->profiling && p->ev_used < kProfSlots) ? p->ev[p->ev_used] : nullptr;
     int rc = run_scoring(p, Q, Kc, cap_rows, aux, &parts);
     if (rc != IPOT_OK) return rc;
     const size_t part_stride = (size_t)p->units * p->cfg.pot_size;
     launch_select(p->units, p->stream, p->scores, parts, part_stride, T > 0 ? p->nuc_mask : nullptr, p->idx,
-                  parts > 1 ? p->summed : nullptr, N, keep, p->cfg.Hkv, p->cfg.batch, p->status);
+                  parts > 1 ? p->summed : nullptr, N, keep, p->cfg.Hkv, p->cfg.batch, p->status, p->gather);
     p->launches += 1;
     IPOT_CUDA(cudaGetLastError());
     if (ev) IPOT_CUDA(cudaEventRecord(ev[3], p->stream));
 
-    const int row_vecs = p->row_bytes / 16;
-    const int slices = p->compact_slices;
-    const size_t unit_vecs = (size_t)p->cfg.pot_size * row_vecs;
-    if (!p->rope) {
-        // programmatic dependent launch: the grid is set up while the selection still runs and waits inside the kernel
-        cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3(slices, 2, p->units);
-        lc.blockDim = dim3(kMoveThreads, 1, 1);
-        lc.stream = p->stream;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[0].val.programmaticStreamSerializationAllowed = 1;
-        lc.attrs = at;
-        lc.numAttrs = 1;
-        IPOT_CUDA(cudaLaunchKernelEx(&lc, compact_kernel, (uint4 *)p->K, (uint4 *)p->V, (const int32_t *)p->idx, keep, N, row_vecs,
-                                     row_vecs / slices, unit_vecs, p->status, pending_rows(p)));
-        p->launches += 1;
-    } else {
-        launch_compact_rope(p, keep, N, row_vecs, unit_vecs);
-        p->launches += 1;
-    }
-    IPOT_CUDA(cudaGetLastError());
+    const GatherParams g{(uint4 *)p->K, (uint4 *)p->V, p->idx, p->gather, p->status, keep, N, row_vecs,
+                         (size_t)p->cfg.pot_size * row_vecs, pending_rows(p), p->ts.wait_ns};
+    if (!p->rope) IPOT_CUDA(launch_gather(p, compact_kernel, g));
+    else IPOT_CUDA(p->cfg.dtype == IPOT_F32 ? launch_gather_rope<float>(p, g) : launch_gather_rope<__nv_bfloat16>(p, g));
+    p->launches += 1;
     p->pend_K = p->pend_V = nullptr;  // the survivors are in the pot, the rest of the chunk is dropped
     if (ev) {
         IPOT_CUDA(cudaEventRecord(ev[4], p->stream));
@@ -567,6 +538,9 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
     alloc((void **)&p->mma_part, (size_t)kMmaSplits * p->units * maxM * sizeof(float2));
     alloc((void **)&p->nuc_mask, (size_t)cfg->batch * cfg->pot_size);
     alloc((void **)&p->idx, (size_t)p->units * cfg->keep * 4);
+    p->gather.rows = gather_rows(p->row_bytes / 16);
+    p->gather.chunks = gather_chunks(cfg->keep, p->row_bytes / 16);
+    alloc((void **)&p->gather.ints, (size_t)p->units * p->gather.per_unit() * 4);
     alloc((void **)&p->status, 16);
     p->dec_splits = decode_splits(p->units, 2 * p->sm_count);  // both decode kernels keep two blocks per SM
     alloc((void **)&p->dec_partial, (size_t)p->units * p->dec_splits * p->G * (cfg->d + 2) * sizeof(float));
@@ -603,8 +577,6 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
         delete p;
         return IPOT_E_CUDA;
     }
-    p->compact_slices = compact_slices(p);
-    p->rope_slices = rope_slices(p);
     tc_plan_init(p->tc, p->cfg, p->K, p->sm_count);
     *out = p;
     return IPOT_OK;
@@ -701,10 +673,9 @@ int ipot_append_chunk(ipot_t *p, const void *K, const void *V, int n)
         p->pend_first = p->len;
         p->pend_n = n;
         p->pend_V = V;
-        if (!p->rope) {
-            p->pend_K = K;
-        } else {  // the rotated copy is what the scorers read: the keys go into the pot now, the values wait
-            launch_append_rope(p, K, n_vecs, nullptr, n);
+        p->pend_K = K;
+        if (p->rope) {  // the rotated copy is what the scorers read: it is made now
+            launch_append_rope(p, K, n_vecs, nullptr, n, false);
             p->launches += 1;
             IPOT_CUDA(cudaGetLastError());
         }

@@ -2,7 +2,6 @@
 //   append_kernel  : Sec. 3.2 - new rows go into the free slots behind the survivors, in order;
 //   compact_kernel : Appendix B "KV-cache compression" - K'[r] = K[idx[r]],
 //                    V'[r] = V[idx[r]] - done in place.
-// Both move 16-byte vectors.
 #pragma once
 #include "common.cuh"
 
@@ -37,53 +36,6 @@ append_kernel(const uint4 *__restrict__ srcK, const uint4 *__restrict__ srcV, ui
     append_body(src, dst, n_vecs, blockIdx.x, gridDim.x);
 }
 
-// In-place gather.  grid (slices, 2, units).  A block owns byte columns
-// [slice * slice_vecs, (slice + 1) * slice_vecs) (in 16-byte vectors) of every
-// row of one tensor of one unit, so blocks never touch the same bytes.  idx is
-// ascending, hence idx[r] >= r: the block walks the rows in ascending chunks,
-// reads a whole chunk into registers, synchronises, then writes it.  A chunk's
-// writes land in rows below the next chunk's first row, and every later source
-// row lies at or above it, so nothing that is still needed is overwritten.
-// Rows with idx[r] == r are left alone.
-// base: the block's first vector of row 0 (its byte-column slice of one tensor of one unit).
-// Rows from alt_first on may still lie outside the pot, in the caller's chunk of a deferred append: alt is then the
-// block's first vector of the chunk's row 0 (same byte columns; slot alt_first), else alt_first = INT_MAX.  Such
-// rows are fetched from there, also when they keep their slot number, so after the gather the pot holds every
-// survivor and nothing else of the chunk was ever copied.
-__device__ __forceinline__ void compact_body(uint4 *__restrict__ base, const int32_t *__restrict__ ix, int keep, int N,
-                                             int row_vecs, int slice_vecs, int *status, const uint4 *__restrict__ alt = nullptr,
-                                             int alt_first = 0x7fffffff)
-{
-    const int rows_per_pass = kMoveThreads / slice_vecs;  // rows covered by one vector per thread
-    const int chunk_rows = rows_per_pass * kMoveVecs;
-    const int my_row = threadIdx.x / slice_vecs, my_vec = threadIdx.x - my_row * slice_vecs;
-    for (int r0 = 0; r0 < keep; r0 += chunk_rows) {
-        uint4 t[kMoveVecs];
-        int src[kMoveVecs];
-#pragma unroll
-        for (int i = 0; i < kMoveVecs; ++i) {
-            const int r = r0 + i * rows_per_pass + my_row;
-            src[i] = -1;
-            if (r < keep && my_row < rows_per_pass) {
-                const int s = ix[r];
-                if (s < r || s >= N) set_status(status, kStatusBounds);
-                else if (s != r || s >= alt_first) src[i] = s;
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < kMoveVecs; ++i)
-            if (src[i] >= 0)
-                t[i] = src[i] >= alt_first ? __ldg(alt + (size_t)(src[i] - alt_first) * row_vecs + my_vec)
-                                           : base[(size_t)src[i] * row_vecs + my_vec];
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < kMoveVecs; ++i) {
-            const int r = r0 + i * rows_per_pass + my_row;
-            if (src[i] >= 0) base[(size_t)r * row_vecs + my_vec] = t[i];
-        }
-    }
-}
-
 // A deferred append's chunk: rows of slot numbers first, first + 1, ... of every unit, still in the caller's buffers
 // ([units][rows][row_vecs]); K or V is NULL where the pot already holds those rows.
 struct PendingRows {
@@ -92,21 +44,146 @@ struct PendingRows {
     int first;
 };
 
-__global__ void __launch_bounds__(kMoveThreads)
-compact_kernel(uint4 *__restrict__ potK, uint4 *__restrict__ potV, const int32_t *__restrict__ idx,
-               int keep, int N, int row_vecs, int slice_vecs, size_t unit_vecs, int *status, PendingRows pend)
+// ------------------------------------------------------------------ the in-place gather
+// row r <- row idx[r] for every tensor (K, V) of every unit.  A tensor's kept rows are cut into chunks of about 16 KiB of
+// whole rows; a block takes one chunk, gathers it into shared memory (16-byte cp.async, everything in flight at once), and
+// then writes it back as one bulk copy.  idx is ascending, so idx[r] >= r, and a slot of the chunk's own destination
+// range can only be the source of a row r' <= r: before a block overwrites slots [r0, r1) it waits until the chunks
+// holding those r' (at most two, as at most r1 - r0 survivors come from r1 - r0 slots) have been read.  Chunks are handed out
+// by a ticket per tensor in ascending order and a block reads its chunk before it waits for anything, so every wait
+// is for a block that is already running and does not itself wait first.  The flags are relaxed accesses: when one is
+// raised the chunk's bytes ARE in shared memory (the copies have been waited for), so there is no access left that a
+// fence would have to order, and a release / acquire pair per block costs more than the copy of a chunk
+// (256 units x 4096 -> 2048 rows of 256 bytes, all in the pot: 138 us with the pair, 91 without any flag).
+//
+// Bound: HBM, 2 * keep rows per tensor.  Whole rows per block because a row's 64-byte pieces fetched by different blocks
+// at different times cost a DRAM access each (256 units x 4096 -> 2048 rows of 256 bytes: 80 us = 6.7 TB/s instead of 116),
+// and because a unit is then not walked by one block (8 units: 11 us instead of 26).
+constexpr int kGatherThreads = 128;
+constexpr int kGatherBytes = 16384;
+
+inline int gather_rows(int row_vecs) { return kGatherBytes / 16 / row_vecs; }
+inline int gather_chunks(int keep, int row_vecs) { return (keep + gather_rows(row_vecs) - 1) / gather_rows(row_vecs); }
+
+// What the selection leaves for the gather, ints of one unit: [0, chunks] the number of survivors in slots below c * rows
+// (which survivors come from a chunk's own slots), then per tensor a ticket and a flag for every chunk, zero, raised when
+// the chunk has been read.
+struct GatherPlan {
+    int *ints;
+    int rows, chunks;
+    __host__ __device__ int per_unit() const { return 3 * (chunks + 1); }
+};
+
+struct GatherParams {
+    uint4 *K, *V;
+    const int32_t *idx;      // [units][keep]
+    GatherPlan plan;
+    int *status;
+    int keep, N, row_vecs;
+    size_t unit_vecs;
+    PendingRows pend;
+    unsigned long long wait_ns;
+};
+
+__device__ __forceinline__ void gather_cp_async16(uint32_t dst, const void *src)
 {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// What a rotary pot does with a gathered key chunk in shared memory besides moving it (k_rope.cuh); nothing here.
+struct GatherNoRotate {
+    __device__ __forceinline__ void operator()(const uint4 *, int, int, int, int) const {}
+};
+
+// grid (chunks, 2, units), block kGatherThreads.  rotate(chunk, unit, r0, rows, row_vecs) is called for key chunks.
+template <typename Rotate>
+__device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate &rotate)
+{
+    __shared__ __align__(128) uint4 buf[kGatherBytes / 16];
+    __shared__ int src_sm[kGatherBytes / 64];   // (rows have at least 64 bytes)
+    __shared__ int chunk_sm, gave_up;
     // Block order: the units from the last one down, K then V of a unit next to each other.  The scorer of the next
-    // cycle starts at unit 0 and finds the rows written last still in L2, and the two tensors of a unit share their
-    // index list while it is hot (measured against units ascending, all K before all V: step 183.2 -> 181.3 us).
+    // cycle starts at unit 0 and finds the rows written last still in L2.
     const unsigned unit = gridDim.z - 1 - blockIdx.z, tensor = blockIdx.y;
-    uint4 *base = (tensor ? potV : potK) + (size_t)unit * unit_vecs + (size_t)blockIdx.x * slice_vecs;
+    uint4 *base = (tensor ? p.V : p.K) + (size_t)unit * p.unit_vecs;
+    const int32_t *ix = p.idx + (size_t)unit * p.keep;
+    const int rows = p.plan.rows, chunks = p.plan.chunks;
+    const int *below = p.plan.ints + (size_t)unit * p.plan.per_unit();
+    int *sync = p.plan.ints + (size_t)unit * p.plan.per_unit() + (1 + tensor) * (chunks + 1);
+    const uint4 *alt = tensor ? p.pend.V : p.pend.K;
+    const int alt_first = alt ? p.pend.first : 0x7fffffff;
+    if (alt) alt += (size_t)unit * p.pend.unit_vecs;
     // launched as a programmatic dependent of the selection: the blocks may be resident before it has ended and
     // wait here for its index lists (returns at once after an ordinary launch)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const uint4 *alt = tensor ? pend.V : pend.K;
-    if (alt) alt += (size_t)unit * pend.unit_vecs + (size_t)blockIdx.x * slice_vecs;
-    compact_body(base, idx + (size_t)unit * keep, keep, N, row_vecs, slice_vecs, status, alt, alt ? pend.first : 0x7fffffff);
+    if (threadIdx.x == 0) {
+        gave_up = 0;
+        chunk_sm = atomicAdd(sync, 1);
+    }
+    __syncthreads();
+    const int chunk = chunk_sm, r0 = chunk * rows, n = min(rows, p.keep - r0);
+    const uint32_t sbuf = (uint32_t)__cvta_generic_to_shared(buf);
+    const int nvec = n * p.row_vecs;
+    for (int i = threadIdx.x; i < n; i += kGatherThreads) {
+        int src = __ldg(ix + r0 + i);
+        if (src < r0 + i || src >= p.N) {
+            set_status(p.status, kStatusBounds);
+            src = r0 + i;
+        }
+        src_sm[i] = src;
+    }
+    __syncthreads();
+    {
+        int r = (int)threadIdx.x / p.row_vecs, c = (int)threadIdx.x - r * p.row_vecs;
+        const int dr = kGatherThreads / p.row_vecs, dc = kGatherThreads - dr * p.row_vecs;
+        for (int v = threadIdx.x; v < nvec; v += kGatherThreads) {
+            const int src = src_sm[r];
+            gather_cp_async16(sbuf + 16 * v, src >= alt_first ? alt + (size_t)(src - alt_first) * p.row_vecs + c : base + (size_t)src * p.row_vecs + c);
+            r += dr;
+            c += dc;
+            if (c >= p.row_vecs) {
+                c -= p.row_vecs;
+                r += 1;
+            }
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (threadIdx.x == kGatherThreads - 32 && r0 < alt_first && chunk > 0) {
+        // while the rows are on their way: the chunks whose sources lie in this chunk's slots (no source in slots whose rows
+        // are outside the pot) have been read
+        const int q0 = __ldg(below + chunk), q1 = __ldg(below + chunk + 1);
+        const int c1 = q1 > q0 ? min(chunk - 1, (q1 - 1) / rows) : -1;
+        const unsigned long long t0 = global_timer_ns();
+        for (int c = max(0, q0 / rows); c <= c1; ++c) {
+            int up = 0;
+            for (uint32_t tries = 1; !up; ++tries) {
+                asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(up) : "l"(sync + 1 + c) : "memory");
+                if (!up && (tries & 255u) == 0 && global_timer_ns() - t0 > p.wait_ns) {
+                    set_status(p.status, kStatusTimeout);
+                    gave_up = 1;
+                    up = 1;
+                }
+            }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk copy below reads what the threads have brought in
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(sync + 1 + chunk), "r"(1) : "memory");
+        if (!gave_up) {   // (a wait that ran out: the rows stay as they are)
+            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                         ::"l"(base + (size_t)r0 * p.row_vecs), "r"(sbuf), "r"((uint32_t)nvec * 16u) : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        }
+    }
+    if (tensor == 0) rotate(buf, (int)unit, r0, n, p.row_vecs);
+    if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the block's memory is free again
+}
+
+__global__ void __launch_bounds__(kGatherThreads) compact_kernel(const __grid_constant__ GatherParams p)
+{
+    gather_block(p, GatherNoRotate{});
 }
 
 }  // namespace ipotk

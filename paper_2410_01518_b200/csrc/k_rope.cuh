@@ -2,11 +2,10 @@
 // embedding; beside it lives a rotated copy in which slot j carries position j, the copy the CaP queries (and the
 // model's attention) read.  Positions only change when rows move, so the two kernels that move rows also write
 // the rotated copy:
-//   append_rope_kernel  : new key rows -> pot rows [first_row, first_row + n) unrotated, and rotated at those
-//                         positions into the copy;
-//   compact_rope_kernel : the in-place gather of compact_kernel on the unrotated keys; every moved row is also
-//                         rotated at its new slot number into the copy.  Rows that stay where they are keep
-//                         their rotated row.
+//   append_rope_kernel  : new key rows -> rotated at the slots they land in into the copy, and (unless the chunk of a
+//                         deferred append still holds them) unrotated into the pot;
+//   compact_rope_kernel : the in-place gather of compact_kernel; every gathered key row is also rotated at its new
+//                         slot number into the copy, out of the shared memory it passes through.
 // Both are HBM-bound copies with idle ALUs, so the rotation costs its extra store traffic only, and no separate
 // pass over the pot follows a cycle.
 //
@@ -20,8 +19,6 @@
 #include "k_move.cuh"
 
 namespace ipotk {
-
-constexpr int kRopeVecs = 4;  // row pairs of vectors in flight per thread in compact_rope_kernel
 
 template <typename T> struct RopeVec;
 template <> struct RopeVec<float> {
@@ -132,7 +129,7 @@ __device__ __forceinline__ void rope_two_vectors(const uint4 &a, const uint4 &b,
 }
 
 // grid (pieces, units, 2 or 1).  z = 0: src: key rows of unit y at src + y * src_unit_vecs, n rows of row_vecs vectors;
-// the rows go to pot rows first_row ... of potK (unchanged) and potKrot (rotated at their slot numbers).  src may be
+// the rows go to pot rows first_row ... of potK (unchanged; NULL: not written) and potKrot (rotated at their slot numbers).  src may be
 // the pot rows themselves (rows that a host copy already put in place): the plain copy then rewrites them as they
 // are.  z = 1: the value rows, a plain copy as in append_kernel (srcV is [units][n * row_vecs]).
 template <typename T, bool kInterleaved>
@@ -171,8 +168,10 @@ append_rope_kernel(const uint4 *__restrict__ src, size_t src_unit_vecs, uint4 *p
         for (int u = 0; u < 2; ++u) {
             uint4 ra, rb;
             rope_two_vectors<T, kInterleaved>(a[u], b[u], g[u], half_vecs, first_row + r[u], cos_t, sin_t, ra, rb);
-            dk[ia[u]] = a[u];
-            dk[ib[u]] = b[u];
+            if (potK) {
+                dk[ia[u]] = a[u];
+                dk[ib[u]] = b[u];
+            }
             dr[ia[u]] = ra;
             dr[ib[u]] = rb;
         }
@@ -183,78 +182,41 @@ append_rope_kernel(const uint4 *__restrict__ src, size_t src_unit_vecs, uint4 *p
         const uint4 a = s[ia], b = s[ib];
         uint4 ra, rb;
         rope_two_vectors<T, kInterleaved>(a, b, g, half_vecs, first_row + r, cos_t, sin_t, ra, rb);
-        dk[ia] = a;
-        dk[ib] = b;
+        if (potK) {
+            dk[ia] = a;
+            dk[ib] = b;
+        }
         dr[ia] = ra;
         dr[ib] = rb;
     }
 }
 
-// In-place gather of the unrotated keys with the rotated copy written beside it.
-// grid (max(k_slices, v_slices), units, 2).  For z = 0 a block
-// owns the vector pairs (g, g + row_vecs / 2) with g in [slice * slice_vecs, (slice + 1) * slice_vecs) of every row
-// of one unit; the walk over the rows is compact_kernel's (ascending chunks, read - barrier - write), which is
-// safe in place because idx[r] >= r.  The rotated copy is only written, never read.
-// z = 1 (if launched): the value rows, compact_kernel's walk with its own slicing (v_slices slices of v_slice_vecs);
-// pend.V names the value rows of a deferred append, if any (pend.K is not used: the keys are in the pot).
+// The gather of k_move.cuh with the rotated copy written beside it.  The copy is only written, so its rows wait for
+// nothing; keys and values share the launch.  Bound: HBM, 5 * keep rows per unit.  (A walk over the rows with the
+// row pair's halves in registers across a barrier took 170 us for 256 units x 4096 -> 2048 rows, this one 106.)
+template <typename T, bool kInterleaved> struct GatherRotate {
+    uint4 *Krot;
+    const T *cos_t, *sin_t;
+    size_t unit_vecs;
+    __device__ __forceinline__ void operator()(const uint4 *chunk, int unit, int r0, int n, int row_vecs) const
+    {
+        const int half_vecs = row_vecs / 2;
+        uint4 *dst = Krot + (size_t)unit * unit_vecs + (size_t)r0 * row_vecs;
+        for (int it = threadIdx.x; it < n * half_vecs; it += kGatherThreads) {
+            const int r = it / half_vecs, g = it - r * half_vecs, v = r * row_vecs + g;
+            uint4 ra, rb;
+            rope_two_vectors<T, kInterleaved>(chunk[v], chunk[v + half_vecs], g, half_vecs, r0 + r, cos_t, sin_t, ra, rb);
+            dst[v] = ra;
+            dst[v + half_vecs] = rb;
+        }
+    }
+};
+
 template <typename T, bool kInterleaved>
-__global__ void __launch_bounds__(kMoveThreads)
-compact_rope_kernel(uint4 *potK, uint4 *__restrict__ potKrot, const T *__restrict__ cos_t, const T *__restrict__ sin_t,
-                    const int32_t *__restrict__ idx, int keep, int N, int row_vecs, int k_slices, int slice_vecs, size_t unit_vecs,
-                    int *status, uint4 *potV, int v_slices, int v_slice_vecs, PendingRows pend)
+__global__ void __launch_bounds__(kGatherThreads)
+compact_rope_kernel(const __grid_constant__ GatherParams p, const __grid_constant__ GatherRotate<T, kInterleaved> rot)
 {
-    if (blockIdx.z == 1) {
-        if ((int)blockIdx.x < v_slices) {
-            const uint4 *alt = pend.V ? pend.V + (size_t)blockIdx.y * pend.unit_vecs + (size_t)blockIdx.x * v_slice_vecs : nullptr;
-            compact_body(potV + (size_t)blockIdx.y * unit_vecs + (size_t)blockIdx.x * v_slice_vecs, idx + (size_t)blockIdx.y * keep,
-                         keep, N, row_vecs, v_slice_vecs, status, alt, alt ? pend.first : 0x7fffffff);
-        }
-        return;
-    }
-    if ((int)blockIdx.x >= k_slices) return;
-    const int half_vecs = row_vecs / 2;
-    uint4 *base = potK + (size_t)blockIdx.y * unit_vecs;
-    uint4 *rbase = potKrot + (size_t)blockIdx.y * unit_vecs;
-    const int32_t *ix = idx + (size_t)blockIdx.y * keep;
-    const int rows_per_pass = kMoveThreads / slice_vecs;
-    const int chunk_rows = rows_per_pass * kRopeVecs;
-    const int my_row = threadIdx.x / slice_vecs, g = blockIdx.x * slice_vecs + (threadIdx.x - my_row * slice_vecs);
-    for (int r0 = 0; r0 < keep; r0 += chunk_rows) {
-        uint4 ta[kRopeVecs], tb[kRopeVecs];
-        int src[kRopeVecs];
-#pragma unroll
-        for (int i = 0; i < kRopeVecs; ++i) {
-            const int r = r0 + i * rows_per_pass + my_row;
-            src[i] = -1;
-            if (r < keep && my_row < rows_per_pass) {
-                const int s = ix[r];
-                if (s < r || s >= N) set_status(status, kStatusBounds);
-                else if (s != r) src[i] = s;
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < kRopeVecs; ++i) {
-            if (src[i] >= 0) {
-                ta[i] = base[(size_t)src[i] * row_vecs + g];
-                tb[i] = base[(size_t)src[i] * row_vecs + g + half_vecs];
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < kRopeVecs; ++i) {
-            const int r = r0 + i * rows_per_pass + my_row;
-            if (src[i] >= 0) {
-                uint4 ra, rb;
-                // the table vectors are fetched here, not with the rows: holding them across the barrier costs a
-                // third of the resident blocks (measured: 164 us against 142 us on the 32-layer workload)
-                rope_two_vectors<T, kInterleaved>(ta[i], tb[i], g, half_vecs, r, cos_t, sin_t, ra, rb);
-                base[(size_t)r * row_vecs + g] = ta[i];
-                base[(size_t)r * row_vecs + g + half_vecs] = tb[i];
-                rbase[(size_t)r * row_vecs + g] = ra;
-                rbase[(size_t)r * row_vecs + g + half_vecs] = rb;
-            }
-        }
-    }
+    gather_block(p, rot);
 }
 
 }  // namespace ipotk

@@ -129,12 +129,6 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)   
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ unsigned long long global_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
 // Bounded wait.  Every block notes a deadline (its start + the launch's wait limit) next to its give-up flag; a
 // wait that is still unsatisfied then records IPOT_E_TIMEOUT and raises the flag.  Once the flag is up, later waits
 // of the block return at once (false) - unless heed_flag is off, which is how a role waits for work it has itself
@@ -146,7 +140,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         if (mbar_try_wait(bar, parity)) return true;
         if ((i & 1023u) == 1023u) {
             if (heed_flag && *abort_flag) return false;
-            if (global_ns() > *reinterpret_cast<volatile unsigned long long *>(abort_flag + 1)) {
+            if (global_timer_ns() > *reinterpret_cast<volatile unsigned long long *>(abort_flag + 1)) {
                 *abort_flag = 1;
                 set_status(status, kStatusTimeout);
                 return false;
@@ -439,7 +433,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        *reinterpret_cast<unsigned long long *>(gbase + kTcOffAbort + 4) = global_ns() + prm.wait_ns;
+        *reinterpret_cast<unsigned long long *>(gbase + kTcOffAbort + 4) = global_timer_ns() + prm.wait_ns;
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar(kBarFull + b), 1);
             mbar_init(bar(kBarEmpty + b), 1);
@@ -697,7 +691,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                         if (!(sv[s].y * sgn > 0.f)) sv[s] = ld_gpu_f32x2(&st[(size_t)(s0 + s) * kTcRows]);
                         fresh = fresh && (sv[s].y * sgn > 0.f);
                     }
-                    if (!fresh && (*ab || ((++tries & 1023u) == 0 && global_ns() > *reinterpret_cast<volatile unsigned long long *>(ab + 1)))) {
+                    if (!fresh && (*ab || ((++tries & 1023u) == 0 && global_timer_ns() > *reinterpret_cast<volatile unsigned long long *>(ab + 1)))) {
                         if (!*ab) {
                             *ab = 1;
                             set_status(prm.status, kStatusTimeout);

@@ -322,7 +322,7 @@ struct TsWait {
     template <bool kCluster>
     __device__ __noinline__ bool slow(uint32_t bar, uint32_t parity) const
     {
-        const unsigned long long t0 = global_ns();
+        const unsigned long long t0 = global_timer_ns();
         for (;;) {
 #pragma unroll 1
             for (int i = 0; i < 64; ++i) {
@@ -330,7 +330,7 @@ struct TsWait {
                 if (sleep_ns) __nanosleep(sleep_ns);
             }
             if (*abort_flag) return false;
-            if (global_ns() - t0 > limit_ns) {
+            if (global_timer_ns() - t0 > limit_ns) {
                 *abort_flag = 1;
                 set_status(status, kStatusTimeout);
                 return false;

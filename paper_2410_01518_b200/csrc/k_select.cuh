@@ -17,6 +17,7 @@
 // 0, which no score maps to, and are never taken.
 #pragma once
 #include "common.cuh"
+#include "k_move.cuh"  // GatherPlan
 
 namespace ipotk {
 
@@ -225,7 +226,7 @@ template <int kThreads, int kKpt>
 __global__ void __launch_bounds__(kThreads)
 select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
               const uint8_t *__restrict__ mask, int32_t *__restrict__ idx, float *__restrict__ summed,
-              int N, int keep, int Hkv, int batch, int *status)
+              int N, int keep, int Hkv, int batch, int *status, GatherPlan plan)
 {
     __shared__ SelShared sh;
     __shared__ __align__(16) int32_t stage[kSelStage];
@@ -237,6 +238,8 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
     // the compaction may be made resident now; it waits for this grid's end before it reads an index
     asm volatile("griddepcontrol.launch_dependents;");
     if (threadIdx.x < 256) sh.hist[threadIdx.x] = 0;
+    int *below = plan.ints + (size_t)unit * plan.per_unit();   // for the gather that follows
+    for (int i = plan.chunks + 1 + threadIdx.x; i < plan.per_unit(); i += kThreads) below[i] = 0;
     uint32_t key[kKpt];
     // a reserved slot outranks every score: finite scores map below 0xFF800000
     if ((N & 15) == 0 && (part_stride & 3) == 0 && slot0 + kKpt <= N) {
@@ -292,6 +295,18 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
     const uint32_t before = block_count_before<kThreads, kKpt>(key, tau, sh, total);
     const int taken = (int)(total & 0xFFFFu) + min((int)(total >> 16), need_eq);
     if (taken != keep && threadIdx.x == 0) set_status(status, kStatusBounds);
+    // for the gather: survivors below the first slot of every chunk of slots (at most one or two such slots per thread)
+    for (int c = (slot0 + plan.rows - 1) / plan.rows; c <= plan.chunks && c * plan.rows < slot0 + kKpt; ++c) {
+        int gt = (int)(before & 0xFFFFu), eq = (int)(before >> 16);
+#pragma unroll
+        for (int i = 0; i < kKpt; ++i) {
+            const bool in = slot0 + i < c * plan.rows;
+            gt += in && key[i] > tau;
+            eq += in && key[i] == tau;
+        }
+        below[c] = gt + min(eq, need_eq);
+    }
+    if (threadIdx.x == 0 && plan.chunks * plan.rows >= kThreads * kKpt) below[plan.chunks] = keep;
     int32_t *out = idx + (size_t)unit * keep;
     for (int base = 0; base < keep; base += kSelStage) {
         block_ordered_sweep<kThreads, kKpt>(key, slot0, tau, need_eq, before, SelStageIndex{stage, base}, SelNoEvery{});
@@ -324,9 +339,9 @@ inline void launch_nuc_mask(int blocks, cudaStream_t st, const float *aux, uint8
     IPOT_SEL_DISPATCH(nuc_mask_kernel, blocks, st, N, aux, mask, N, T);
 }
 inline void launch_select(int blocks, cudaStream_t st, const float *scores, int parts, size_t part_stride, const uint8_t *mask,
-                          int32_t *idx, float *summed, int N, int keep, int Hkv, int batch, int *status)
+                          int32_t *idx, float *summed, int N, int keep, int Hkv, int batch, int *status, const GatherPlan &plan)
 {
-    IPOT_SEL_DISPATCH(select_kernel, blocks, st, N, scores, parts, part_stride, mask, idx, summed, N, keep, Hkv, batch, status);
+    IPOT_SEL_DISPATCH(select_kernel, blocks, st, N, scores, parts, part_stride, mask, idx, summed, N, keep, Hkv, batch, status, plan);
 }
 
 // summed[i] = parts[0][i] + parts[1][i] + ... in index order (the order select_kernel uses).
