@@ -113,10 +113,10 @@ __device__ __forceinline__ void nov_group(NovStat &st, const uint4 &v, const __n
     for (int i = 0; i < 4; ++i) st.add_pair(make_float2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u)));
 }
 
-// grid (segs, rows), block 128.  counters: [rows] ints, zero on entry and zero again on exit; partial: [rows][segs].
+// grid (segs, rows), block 128.  kAligned: every row starts on a 16-byte boundary.  counters: [rows] ints, zero on entry and zero again on exit; partial: [rows][segs].
 // Token `row` = (stream b, position t) = (row / n_tokens, row % n_tokens) writes out[b * out_stride + slot0 + t].
 // A negative label marks an ignored position (novelty 0); a label >= V also gives 0 and raises kStatusBounds.
-template <typename T>
+template <typename T, bool kAligned>
 __global__ void __launch_bounds__(kNovThreads)
 novelty_kernel(const T *__restrict__ logits, size_t row_stride, int V, int segs, int seg_elems, float2 *partial, int *counters,
                const int32_t *__restrict__ labels, int n_tokens, float *__restrict__ out, size_t out_stride, int slot0,
@@ -131,8 +131,8 @@ novelty_kernel(const T *__restrict__ logits, size_t row_stride, int V, int segs,
     // The row may start anywhere (an odd vocabulary): the elements before its first 16-byte boundary and behind its last
     // one, fewer than VE each, are read one by one by different warps, everything between them in 16-byte loads.
     const T *p = z + v0;
-    const int n = max(0, v1 - v0);
-    const int head = min(n, (int)((0u - (uint32_t)reinterpret_cast<uintptr_t>(p)) & 15u) / (int)sizeof(T));
+    const int n = kAligned ? v1 - v0 : max(0, v1 - v0);
+    const int head = kAligned ? 0 : min(n, (int)((0u - (uint32_t)reinterpret_cast<uintptr_t>(p)) & 15u) / (int)sizeof(T));
     const int nvec = (n - head) / VE;
     const uint4 *zv = reinterpret_cast<const uint4 *>(p + head);
     constexpr uint32_t kNegInf = sizeof(T) == 2 ? 0xFF80FF80u : 0xFF800000u;  // -inf: no term, never the maximum
@@ -148,9 +148,9 @@ novelty_kernel(const T *__restrict__ logits, size_t row_stride, int V, int segs,
 #pragma unroll
         for (int u = 0; u < kNovBatch; ++u) nov_group(st, v[u], z);
     }
-    if ((int)threadIdx.x < head) st.add_one(nov_load1(p + threadIdx.x));
-    const int behind = head + nvec * VE + (int)threadIdx.x - 32;
-    if (threadIdx.x >= 32 && behind < n) st.add_one(nov_load1(p + behind));
+    if (!kAligned && (int)threadIdx.x < head) st.add_one(nov_load1(p + threadIdx.x));
+    for (int i = head + nvec * VE + (int)threadIdx.x - (kAligned ? 0 : 32); i < n; i += kNovThreads)
+        if (kAligned || threadIdx.x >= 32) st.add_one(nov_load1(p + i));
     // block reduction in two steps (largest reference, then the sums rescaled once): one exponential per thread
     __shared__ float wred[2][kNovThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

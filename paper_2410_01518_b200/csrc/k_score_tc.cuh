@@ -20,7 +20,7 @@
 //            exponentials of the first chunk's second half;
 //   combine  (4 warps, one thread per query row) merges the eight (max, sum) pairs of
 //            its row into the slab's statistics and publishes them with one 8-byte
-//            store whose sum carries the launch's sign as a "fresh" mark; then reads
+//            store whose reference carries the launch's number as a "fresh" mark; then reads
 //            the row's statistics of all slabs of the item, re-reading until every
 //            one is fresh, and turns them into the row's global maximum m, its
 //            denominator l (plus, when given, the share of the CaP's own keys) and the
@@ -60,6 +60,11 @@ constexpr int kTcThreads = 704;      // warp 0: TMA, 1: MMA + TMEM owner, 2-17: 
 constexpr int kTcRows = 128;         // query rows per item (TMEM lanes)
 constexpr int kTcSlab = 256;         // keys per task (TMEM columns per buffer)
 constexpr int kTcFmaEighths = 2;     // share of pass 1's exponentials evaluated on the FMA pipe
+// The published reference is the slab's maximum with its lowest mantissa bits replaced by the launch's mark: any number
+// near the maximum serves as a reference (the sum is taken relative to the one that is published), so the mark costs no
+// precision.  Marks count up, so whatever an earlier launch left in the array - of another layout, or of one that gave
+// up half way - never looks fresh, and the array is only cleared when they start over.
+constexpr uint32_t kTcMarkBits = 6, kTcMarks = (1u << kTcMarkBits) - 1;
 constexpr int kTcD = 128;            // largest head dimension; 64 uses the first 64-channel half of every tile
 constexpr uint32_t kTcQBytes = kTcRows * kTcD * 2;           // 32 KiB: two halves of 128 rows x 64 channels
 constexpr uint32_t kTcKBytes = kTcSlab * kTcD * 2;           // 64 KiB: two halves of 256 rows x 64 channels
@@ -81,9 +86,9 @@ enum { kBarFull = 0, kBarEmpty = 2, kBarEReady = 4, kBarFReady = 6, kBarSFull = 
 struct TcParams {
     float *scores;        // partial array p (query rows 128p ...) at scores + p * part_stride, unit stride N
     size_t part_stride;
-    float2 *stats;        // [items][slabs][128] (max in log2 units, sum * sign); all of the other sign or 0 at launch
+    float2 *stats;        // [items][slabs][128] (reference in log2 units, sum relative to it); see kTcMarkBits
     const float2 *cap_stats;  // NULL, or [units][M] (max, sum) over the CaP's own keys that join every row's denominator
-    float sign;           // +1 or -1: this launch's "fresh" mark
+    uint32_t mark;        // this launch's "fresh" mark, 1 .. kTcMarks
     unsigned long long wait_ns;  // limit of every wait
     int withhold_cta;     // -1; test hook: this CTA never publishes its slab statistics
     int *status;
@@ -642,7 +647,9 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         const int row = threadIdx.x - 576;
         const float2 *tstat = reinterpret_cast<const float2 *>(gbase + kTcOffTstat);
         float *fbuf = reinterpret_cast<float *>(gbase + kTcOffFbuf);
-        const float sgn = prm.sign;
+        const uint32_t mark = prm.mark;
+        auto marked = [&](float x) { return __uint_as_float((__float_as_uint(x) & ~kTcMarks) | mark); };
+        auto is_fresh = [&](float2 v) { return (__float_as_uint(v.x) & kTcMarks) == mark; };
         uint32_t k = 0;
         for (int task = blockIdx.x; task < prm.tasks; task += gridDim.x, ++k) {
             const int item = task / tasks_per_item, slab = task - item * tasks_per_item;
@@ -662,13 +669,13 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 for (int i = 0; i < 8; ++i) t[i] = tstat[(b * 8 + i) * kTcRows + row];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) cm[i] = t[i].x;
-                const float ms0 = max3(max3(cm[0], cm[1], cm[2]), max3(cm[3], cm[4], cm[5]), fmaxf(cm[6], cm[7]));  // chunk 0 always holds a valid key
+                const float ms0 = marked(max3(max3(cm[0], cm[1], cm[2]), max3(cm[3], cm[4], cm[5]), fmaxf(cm[6], cm[7])));  // chunk 0 always holds a valid key
 #pragma unroll
                 for (int i = 0; i < 8; ++i) ce[i] = (cm[i] == -INFINITY) ? 0.f : t[i].y * ex2(cm[i] - ms0);
             }
-            const float ms = max3(max3(cm[0], cm[1], cm[2]), max3(cm[3], cm[4], cm[5]), fmaxf(cm[6], cm[7]));
+            const float ms = marked(max3(max3(cm[0], cm[1], cm[2]), max3(cm[3], cm[4], cm[5]), fmaxf(cm[6], cm[7])));
             const float ls = ((ce[0] + ce[1]) + (ce[2] + ce[3])) + ((ce[4] + ce[5]) + (ce[6] + ce[7]));
-            if (tasks_per_item > 1 && (int)blockIdx.x != prm.withhold_cta) st_gpu_f32x2(&prm.stats[((size_t)item * tasks_per_item + slab) * kTcRows + row], ms, ls * sgn);
+            if (tasks_per_item > 1 && (int)blockIdx.x != prm.withhold_cta) st_gpu_f32x2(&prm.stats[((size_t)item * tasks_per_item + slab) * kTcRows + row], ms, ls);
 
             // ---- this row's statistics of every slab of the item; re-read until all carry this launch's mark
             const float2 *st = prm.stats + (size_t)item * tasks_per_item * kTcRows + row;
@@ -683,13 +690,13 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 bool fresh;
 #pragma unroll
                 for (int s = 0; s < 16; ++s)  // beyond the item: neutral and fresh; this CTA's own slab: known; others: stale
-                    sv[s] = (s0 + s >= tasks_per_item) ? make_float2(-INFINITY, sgn) : (s0 + s == slab) ? make_float2(ms, ls * sgn) : make_float2(0.f, 0.f);
+                    sv[s] = (s0 + s >= tasks_per_item) ? make_float2(marked(-3e38f), 0.f) : (s0 + s == slab) ? make_float2(ms, ls) : make_float2(0.f, 0.f);
                 do {  // only the entries that are still stale are read again
                     fresh = true;
 #pragma unroll
                     for (int s = 0; s < 16; ++s) {
-                        if (!(sv[s].y * sgn > 0.f)) sv[s] = ld_gpu_f32x2(&st[(size_t)(s0 + s) * kTcRows]);
-                        fresh = fresh && (sv[s].y * sgn > 0.f);
+                        if (!is_fresh(sv[s])) sv[s] = ld_gpu_f32x2(&st[(size_t)(s0 + s) * kTcRows]);
+                        fresh = fresh && is_fresh(sv[s]);
                     }
                     if (!fresh && (*ab || ((++tries & 1023u) == 0 && global_timer_ns() > *reinterpret_cast<volatile unsigned long long *>(ab + 1)))) {
                         if (!*ab) {
@@ -703,7 +710,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                                       max3(max3(sv[9].x, sv[10].x, sv[11].x), max3(sv[12].x, sv[13].x, sv[14].x), fmaxf(sv[15].x, m)), -INFINITY);
                 float w[16];
 #pragma unroll
-                for (int s = 0; s < 16; ++s) w[s] = fabsf(sv[s].y) * ex2(sv[s].x - mb);
+                for (int s = 0; s < 16; ++s) w[s] = sv[s].y * ex2(sv[s].x - mb);
 #pragma unroll
                 for (int step = 1; step < 16; step <<= 1) {
 #pragma unroll
@@ -747,10 +754,7 @@ struct TcPlan {
     int sm_count = 0;
     int max_items = 0, max_slabs = 0;
     float2 *stats = nullptr;          // [max_items][max_slabs][128]
-    // "fresh" marking of the statistics: every launch writes all entries of its (items x slabs) layout
-    // with the sign opposite to the previous launch's; a layout change clears the array first
-    float sign = 1.f;
-    int last_items = 0, last_slabs = 0;
+    uint32_t mark = 0;                // of the last launch
 };
 
 inline void tc_plan_destroy(TcPlan &plan)
@@ -786,7 +790,8 @@ inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, const void *, i
     const int units = cfg.layers * cfg.batch * cfg.Hkv;
     plan.max_items = units * ((G * cfg.max_cap_rows + kTcRows - 1) / kTcRows);
     plan.max_slabs = (cfg.pot_size + kTcSlab - 1) / kTcSlab;
-    if (cudaMalloc(&plan.stats, (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float2)) != cudaSuccess) {
+    const size_t stats_bytes = (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float2);
+    if (cudaMalloc(&plan.stats, stats_bytes) != cudaSuccess || cudaMemset(plan.stats, 0, stats_bytes) != cudaSuccess) {
         cudaGetLastError();
         tc_plan_destroy(plan);
         return;
@@ -845,16 +850,14 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
     prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d));
     prm.wait_ns = wait_ns;
     prm.withhold_cta = withhold_cta;
-    if (items != plan.last_items || prm.slabs != plan.last_slabs) {
-        if (cudaMemsetAsync(plan.stats, 0, (size_t)items * prm.slabs * kTcRows * sizeof(float2), stream) != cudaSuccess) {
+    if (plan.mark == kTcMarks) {
+        if (cudaMemsetAsync(plan.stats, 0, (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float2), stream) != cudaSuccess) {
             cudaGetLastError();
             return IPOT_E_CUDA;
         }
-        plan.last_items = items;
-        plan.last_slabs = prm.slabs;
+        plan.mark = 0;
     }
-    plan.sign = -plan.sign;
-    prm.sign = plan.sign;
+    prm.mark = ++plan.mark;
     cudaLaunchConfig_t lc = {};
     // spare_sms: SMs left to a small kernel of the same cycle that runs beside this one on another stream
     const int ctas = plan.sm_count - spare_sms > 0 ? plan.sm_count - spare_sms : 1;

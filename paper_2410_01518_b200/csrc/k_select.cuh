@@ -173,49 +173,78 @@ struct SelPackMask {  // byte i of the thread's mask bytes, four to a word
     __device__ void operator()(int i, bool s) const { packed[i >> 2] |= (s ? 1u : 0u) << (8 * (i & 3)); }
 };
 
-// grid (batch).  mask[b][j] = 1 iff slot j is one of the T most novel slots of stream b.
-template <int kThreads, int kKpt>
-__global__ void __launch_bounds__(kThreads)
-nuc_mask_kernel(const float *__restrict__ aux, uint8_t *__restrict__ mask, int N, int T)
+// Slots [slot0, slot0 + kKpt) of a row of N floats that may start on any 4-byte boundary (rows of an odd length): whole
+// 16-byte vectors from the boundary below the first slot on, shifted into place (the shift is the same for every
+// thread of a block), one by one at the row's ends; slots at or beyond N are left alone.
+// (With one 4-byte load per slot, 64 bytes apart across a warp, such a row took 3 us more.)
+template <int kKpt, int kShift>
+__device__ __forceinline__ void shift_row(const float4 (&q)[kKpt / 4 + 1], float (&s)[kKpt])
 {
-    __shared__ SelShared sh;
-    const float *a = aux + (size_t)blockIdx.x * N;
-    uint8_t *m = mask + (size_t)blockIdx.x * N;
-    const int slot0 = threadIdx.x * kKpt;
-    if (threadIdx.x < 256) sh.hist[threadIdx.x] = 0;
-    uint32_t key[kKpt];
-    const bool vec = (N & 15) == 0 && slot0 + kKpt <= N;   // rows of N floats (and of N bytes) stay 16-byte aligned
-    if (vec) {
 #pragma unroll
-        for (int i = 0; i < kKpt; i += 4) {
-            const float4 v = *reinterpret_cast<const float4 *>(a + slot0 + i);
-            key[i] = order_key(v.x);
-            key[i + 1] = order_key(v.y);
-            key[i + 2] = order_key(v.z);
-            key[i + 3] = order_key(v.w);
+    for (int i = 0; i < kKpt; ++i) {
+        const float4 v = q[(i + kShift) / 4];
+        s[i] = (i + kShift) % 4 == 0 ? v.x : (i + kShift) % 4 == 1 ? v.y : (i + kShift) % 4 == 2 ? v.z : v.w;
+    }
+}
+template <int kKpt>
+__device__ __forceinline__ void load_row(const float *__restrict__ row, int slot0, int N, float (&s)[kKpt])
+{
+    const int shift = (int)(reinterpret_cast<uintptr_t>(row) >> 2) & 3;
+    if (shift == 0 ? slot0 + kKpt <= N : (slot0 > 0 && slot0 + kKpt + 4 <= N)) {
+        const float4 *v = reinterpret_cast<const float4 *>(row + slot0 - shift);
+        float4 q[kKpt / 4 + 1];
+#pragma unroll
+        for (int i = 0; i < kKpt / 4; ++i) q[i] = __ldg(v + i);
+        q[kKpt / 4] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (shift) q[kKpt / 4] = __ldg(v + kKpt / 4);
+        switch (shift) {
+        case 0: shift_row<kKpt, 0>(q, s); break;
+        case 1: shift_row<kKpt, 1>(q, s); break;
+        case 2: shift_row<kKpt, 2>(q, s); break;
+        default: shift_row<kKpt, 3>(q, s); break;
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < kKpt; ++i) key[i] = slot0 + i < N ? order_key(a[slot0 + i]) : 0u;
-    }
-    __syncthreads();
-    uint32_t tau;
-    int need_eq;
-    block_radix_select<kThreads, kKpt>(key, T, sh, tau, need_eq);
-    uint32_t packed[kKpt / 4];
-#pragma unroll
-    for (int i = 0; i < kKpt / 4; ++i) packed[i] = 0;
-    uint32_t total;
-    const uint32_t before = block_count_before<kThreads, kKpt>(key, tau, sh, total);
-    block_ordered_sweep<kThreads, kKpt>(key, slot0, tau, need_eq, before, SelNoTaken{}, SelPackMask{packed});
-    if (vec) {
-#pragma unroll
-        for (int i = 0; i < kKpt / 4; i += 4)
-            *reinterpret_cast<uint4 *>(m + slot0 + 4 * i) = make_uint4(packed[i], packed[i + 1], packed[i + 2], packed[i + 3]);
-    } else {
-#pragma unroll
         for (int i = 0; i < kKpt; ++i)
-            if (slot0 + i < N) m[slot0 + i] = (uint8_t)((packed[i >> 2] >> (8 * (i & 3))) & 1u);
+            if (slot0 + i < N) s[i] = row[slot0 + i];
+    }
+}
+__host__ __device__ inline int mask_stride(int N) { return (N + 31) & ~31; }   // bytes of a stream's mask row
+
+// mask[b][j] = 1 iff slot j is one of the T most novel slots of stream b.  A block takes streams blockIdx.x,
+// blockIdx.x + gridDim.x, ...
+template <int kThreads, int kKpt>
+__global__ void __launch_bounds__(kThreads)
+nuc_mask_kernel(const float *__restrict__ aux, uint8_t *__restrict__ mask, int N, int T, int batch)
+{
+    __shared__ SelShared sh;
+    const int slot0 = threadIdx.x * kKpt;
+    if (threadIdx.x < 256) sh.hist[threadIdx.x] = 0;
+    for (int b = blockIdx.x; b < batch; b += gridDim.x) {
+        uint8_t *m = mask + (size_t)b * mask_stride(N);
+        uint32_t key[kKpt];
+        {
+            float s[kKpt];
+            load_row<kKpt>(aux + (size_t)b * N, slot0, N, s);
+#pragma unroll
+            for (int i = 0; i < kKpt; ++i) key[i] = slot0 + i < N ? order_key(s[i]) : 0u;
+        }
+        __syncthreads();
+        uint32_t tau;
+        int need_eq;
+        block_radix_select<kThreads, kKpt>(key, T, sh, tau, need_eq);
+        uint32_t packed[kKpt / 4];
+#pragma unroll
+        for (int i = 0; i < kKpt / 4; ++i) packed[i] = 0;
+        uint32_t total;
+        const uint32_t before = block_count_before<kThreads, kKpt>(key, tau, sh, total);
+        block_ordered_sweep<kThreads, kKpt>(key, slot0, tau, need_eq, before, SelNoTaken{}, SelPackMask{packed});
+        if (slot0 < N) {   // (a row has room for whole vectors)
+#pragma unroll
+            for (int i = 0; i < kKpt / 4; i += 4)
+                *reinterpret_cast<uint4 *>(m + slot0 + 4 * i) = make_uint4(packed[i], packed[i + 1], packed[i + 2], packed[i + 3]);
+        }
+        __syncthreads();
     }
 }
 
@@ -233,7 +262,7 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
     const int unit = blockIdx.x;
     const int b = (unit / Hkv) % batch;
     const float *u = scores + (size_t)unit * N;
-    const uint8_t *m = mask ? mask + (size_t)b * N : nullptr;
+    const uint8_t *m = mask ? mask + (size_t)b * mask_stride(N) : nullptr;
     const int slot0 = threadIdx.x * kKpt;
     // the compaction may be made resident now; it waits for this grid's end before it reads an index
     asm volatile("griddepcontrol.launch_dependents;");
@@ -242,50 +271,38 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
     for (int i = plan.chunks + 1 + threadIdx.x; i < plan.per_unit(); i += kThreads) below[i] = 0;
     uint32_t key[kKpt];
     // a reserved slot outranks every score: finite scores map below 0xFF800000
-    if ((N & 15) == 0 && (part_stride & 3) == 0 && slot0 + kKpt <= N) {
-        float4 s[kKpt / 4];
-        uint32_t r[kKpt / 4];
+    constexpr int kPiece = kKpt > 16 ? 8 : 16;   // slots loaded at a time (what 64 registers a thread allow)
 #pragma unroll
-        for (int i = 0; i < kKpt / 4; ++i) s[i] = *reinterpret_cast<const float4 *>(u + slot0 + 4 * i);   // all loads in flight together
+    for (int h = 0; h < kKpt; h += kPiece) {
+        const int first = slot0 + h;
+        float s[kPiece];
+        uint32_t r[kPiece / 4];
+        load_row<kPiece>(u, first, N, s);
 #pragma unroll
-        for (int i = 0; i < kKpt / 4; ++i) r[i] = m ? *reinterpret_cast<const uint32_t *>(m + slot0 + 4 * i) : 0u;
+        for (int i = 0; i < kPiece / 4; ++i) r[i] = (m && first < N) ? *reinterpret_cast<const uint32_t *>(m + first + 4 * i) : 0u;
         if (parts > 1) {
 #pragma unroll 1
             for (int p = 1; p < parts; ++p) {
+                float t[kPiece];
+                load_row<kPiece>(u + (size_t)p * part_stride, first, N, t);
 #pragma unroll
-                for (int i = 0; i < kKpt / 4; ++i) {
-                    const float4 t = *reinterpret_cast<const float4 *>(u + (size_t)p * part_stride + slot0 + 4 * i);
-                    s[i].x += t.x;
-                    s[i].y += t.y;
-                    s[i].z += t.z;
-                    s[i].w += t.w;
+                for (int i = 0; i < kPiece; ++i) s[i] += t[i];
+            }
+            float *to = summed + (size_t)unit * N + first;
+            if (summed) {
+                if ((reinterpret_cast<uintptr_t>(to) & 15u) == 0 && first + kPiece <= N) {
+#pragma unroll
+                    for (int i = 0; i < kPiece; i += 4) *reinterpret_cast<float4 *>(to + i) = make_float4(s[i], s[i + 1], s[i + 2], s[i + 3]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < kPiece; ++i)
+                        if (first + i < N) to[i] = s[i];
                 }
             }
-            if (summed) {
-#pragma unroll
-                for (int i = 0; i < kKpt / 4; ++i) *reinterpret_cast<float4 *>(summed + (size_t)unit * N + slot0 + 4 * i) = s[i];
-            }
         }
 #pragma unroll
-        for (int i = 0; i < kKpt / 4; ++i) {
-            key[4 * i] = (r[i] & 0xFFu) ? 0xFFFFFFFFu : order_key(s[i].x);
-            key[4 * i + 1] = (r[i] & 0xFF00u) ? 0xFFFFFFFFu : order_key(s[i].y);
-            key[4 * i + 2] = (r[i] & 0xFF0000u) ? 0xFFFFFFFFu : order_key(s[i].z);
-            key[4 * i + 3] = (r[i] & 0xFF000000u) ? 0xFFFFFFFFu : order_key(s[i].w);
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < kKpt; ++i) {
-            const int j = slot0 + i;
-            key[i] = 0u;
-            if (j < N) {
-                float s = u[j];
-#pragma unroll 1
-                for (int p = 1; p < parts; ++p) s += u[(size_t)p * part_stride + j];
-                if (summed && parts > 1) summed[(size_t)unit * N + j] = s;
-                key[i] = (m && m[j]) ? 0xFFFFFFFFu : order_key(s);
-            }
-        }
+        for (int i = 0; i < kPiece; ++i)
+            key[h + i] = first + i >= N ? 0u : (r[i >> 2] >> (8 * (i & 3))) & 0xFFu ? 0xFFFFFFFFu : order_key(s[i]);
     }
     __syncthreads();
     uint32_t tau;
@@ -334,9 +351,9 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
         else kernel<1024, 32><<<(blocks), 1024, 0, (stream)>>>(__VA_ARGS__);                     \
     } while (0)
 
-inline void launch_nuc_mask(int blocks, cudaStream_t st, const float *aux, uint8_t *mask, int N, int T)
+inline void launch_nuc_mask(int blocks, cudaStream_t st, const float *aux, uint8_t *mask, int N, int T, int batch)
 {
-    IPOT_SEL_DISPATCH(nuc_mask_kernel, blocks, st, N, aux, mask, N, T);
+    IPOT_SEL_DISPATCH(nuc_mask_kernel, blocks, st, N, aux, mask, N, T, batch);
 }
 inline void launch_select(int blocks, cudaStream_t st, const float *scores, int parts, size_t part_stride, const uint8_t *mask,
                           int32_t *idx, float *summed, int N, int keep, int Hkv, int batch, int *status, const GatherPlan &plan)
