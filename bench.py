@@ -35,7 +35,7 @@ REFERENCE_BUDGET_S = 150.0   # wall-clock budget of a whole --impl reference run
 NOVELTY_WORKLOADS = {"nuc32k": (32000, 2048), "nuc128k": (128256, 2048)}
 # generation over a full pot alone: one new token's attention over all layers' units, configs[cfg - 1] shape
 DECODE_WORKLOADS = {"decode3": 3, "decode4": 4, "decode5": 5}
-SCORERS = {"auto": 0, "simt": 1, "tensor": 2, "warp_mma": 3, "sweeps": 4}
+SCORERS = {"auto": 0, "simt": 1, "tensor": 2, "warp_mma": 3, "sweeps": 4, "items": 5}
 SCORER_KERNELS = {1: "cap_row_stats + cap_column_sums (fp32 FMA)", 2: "cap_score_tc_kernel (tcgen05, one sweep)",
                   3: "cap_row_stats_mma + cap_column_sums_mma (mma.sync)", 4: "cap_score_ts_kernel (tcgen05, two sweeps)"}
 MIN_SAMPLED_S = 1.0   # the clock sampler should see at least this much of timed running

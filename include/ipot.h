@@ -72,11 +72,15 @@ enum {
     IPOT_SCORER_SIMT = 1,   /* fp32 FMA kernel: any supported shape, f32 or bf16 */
     IPOT_SCORER_TENSOR = 2, /* tcgen05 kernel (bf16, d = 64 or 128): IPOT_E_INVALID if the shape does not allow it */
     IPOT_SCORER_WARP_MMA = 3, /* warp-level tensor-core kernels (bf16, d a multiple of 16): what AUTO takes for bf16
-                                pots the tcgen05 kernel does not; IPOT_E_INVALID if the shape does not allow it */
-    IPOT_SCORER_TENSOR_SWEEPS = 4 /* tcgen05 kernel that goes over the keys twice (row log-sum-exps, then probabilities
+                                pots the tcgen05 kernels do not; IPOT_E_INVALID if the shape does not allow it */
+    IPOT_SCORER_TENSOR_SWEEPS = 4, /* tcgen05 kernel that goes over the keys twice (row log-sum-exps, then probabilities
                                 and their column sums) inside thread-block clusters, so that no block waits for a block
                                 it is not co-scheduled with (bf16, d = 64 or 128, at most 512 folded query rows):
                                 IPOT_E_INVALID if the shape does not allow it */
+    IPOT_SCORER_TENSOR_ITEMS = 5 /* tcgen05 kernel in two sweeps whose pieces are dealt to the SMs one by one (bf16, any
+                                d, at most 1024 folded query rows): what AUTO takes for head dimensions other than
+                                64 and 128, and for many query rows over many long units; IPOT_E_INVALID if the shape
+                                does not allow it */
 };
 
 typedef struct {
@@ -122,11 +126,12 @@ int ipot_set_scorer(ipot_t *pot, int scorer);
  *                                 FMA pipe instead of the special-function unit: 2, 3, or -1 = default
  *   IPOT_TUNE_WAIT_LIMIT_NS       time after which a device-side wait of a tensor-core scorer gives up and the launch
  *                                 ends with IPOT_E_TIMEOUT in the status word (default 200 ms; at least 1000).
- *                                 IPOT_SCORER_TENSOR_SWEEPS counts it from the start of each wait, IPOT_SCORER_TENSOR
+ *                                 The two-sweep scorers count it from the start of each wait, IPOT_SCORER_TENSOR
  *                                 from the start of each thread block (a launch of either takes well under 1 ms)
  *   IPOT_TUNE_TEST_WITHHOLD_RANK  for tests of the give-up path only: CTA `value` (0-7) of every cluster
- *                                 (IPOT_SCORER_TENSOR_SWEEPS) or of the grid (IPOT_SCORER_TENSOR) never reports its
- *                                 statistics, so every wait for them runs into the limit; -1 = off (default)
+ *                                 (IPOT_SCORER_TENSOR_SWEEPS) or of the grid (IPOT_SCORER_TENSOR), or job `value` of
+ *                                 IPOT_SCORER_TENSOR_ITEMS, never reports its statistics, so every wait for them runs into
+ *                                 the limit; -1 = off (default)
  * Errors: INVALID (unknown `what`, value out of range).  Takes effect at the next launch.
  */
 enum {
@@ -315,7 +320,7 @@ int ipot_sync_status(ipot_t *pot);
  * over the recorded cycles in milliseconds - ms[0] NuC ranking, ms[1] CaP
  * scoring, ms[2] per-head selection, ms[3] K/V compaction - and starts a new
  * series.  *cycles (may be NULL) = cycles averaged; *scorer_used (may be NULL)
- * = IPOT_SCORER_SIMT, IPOT_SCORER_TENSOR or IPOT_SCORER_WARP_MMA.  STATE if nothing was recorded.
+ * = the IPOT_SCORER_* that ran.  STATE if nothing was recorded.
  */
 int ipot_set_profiling(ipot_t *pot, int on);
 int ipot_kernel_ms(ipot_t *pot, float ms[4], int *cycles, int *scorer_used);

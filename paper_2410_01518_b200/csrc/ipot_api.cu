@@ -20,6 +20,7 @@
 #include "k_score_simt.cuh"
 #include "k_score_tc.cuh"
 #include "k_score_ts.cuh"
+#include "k_score_tw.cuh"
 #include "k_select.cuh"
 
 using namespace ipotk;
@@ -77,6 +78,7 @@ struct ipot {
     int ev_used;
     long long launches;
     TcPlan tc;           // tensor-core scorer state
+    TwPlan tw;
     TsTuning ts;         // launch parameters of the two-sweep tensor-core scorer
     TsOccupancy ts_occ;
     // the novelty ranking does not depend on the scores: it runs beside the scorer on a stream of its own
@@ -120,6 +122,7 @@ int check_config(const ipot_config_t &c)
 void free_all(ipot *p)
 {
     tc_plan_destroy(p->tc);
+    tw_plan_destroy(p->tw);
     cudaFree(p->K); cudaFree(p->V); cudaFree(p->Krot); cudaFree(p->scores); cudaFree(p->summed);
     cudaFree(p->row_stats); cudaFree(p->mma_part); cudaFree(p->cap_stats); cudaFree(p->nuc_mask); cudaFree(p->idx); cudaFree(p->gather.ints); cudaFree(p->status);
     cudaFree(p->stage_q); cudaFree(p->stage_kc); cudaFree(p->stage_aux); cudaFree(p->nov_scratch); cudaFree(p->dec_partial); cudaFree(p->dec_counters);
@@ -229,15 +232,21 @@ int launch_warp_mma(ipot *p, const void *Q, const float2 *cap_stats, int M, int 
     return IPOT_OK;
 }
 
-// The fastest scorer the shape allows.
-int auto_scorer(const ipot *p, int N, int M, bool tc_ok, bool ts_ok, bool mma_ok)
+// The fastest scorer the shape allows.  d = 64 and 128, measured on 8 to 128 units of 2048 to 32768 keys, M = 128 to 512 (us:
+// one sweep / clusters / items): the one-sweep kernel wins up to about 48 slabs of 256 keys (64 x 8192, M = 256:
+// 100 / 104 / 108; 8 x 16384, M = 512: 75 / 109 / 99), unless there are several row blocks for every one of many units,
+// which the two-sweep kernels fetch the keys for once (128 x 8192, M = 512: 396 / 388 / 336).  Longer items wait for too
+// many other blocks' statistics (128 x 16384, M = 128: 320 / 221 / 214; 16 x 32768: 117 / 104 / 65); then the item kernel for
+// one row block and for many units of several, else the cluster kernel, whose last units are waited for less
+// (32 x 16384, M = 384: 206 / 152 / 188; 64 x 16384, M = 512: 547 / 377 / 348).
+// Other head dimensions have the item kernel or warp-level tensor cores, and the former wins everywhere
+// (d = 256, 64 x 4096, M = 64: 59 us against 221; d = 96, 8 x 640, M = 16: 12.5 against 18.5).
+int auto_scorer(int units, int N, int M, bool tc_ok, bool ts_ok, bool items_ok, bool mma_ok)
 {
-    (void)p;
-    (void)N;
-    // measured on the three-to-four-row-block shapes (M = 384, 512): the two-sweep kernel holds every query tile of a
-    // unit against a key slab that is fetched once per sweep and is 1.4 x faster there; up to two row blocks the
-    // one-sweep kernel with its statistics exchange is as fast or faster
-    if (ts_ok && (!tc_ok || M > 2 * kTcRows)) return IPOT_SCORER_TENSOR_SWEEPS;
+    const bool long_items = N > 12288 && (long long)units * N >= 32 * 8192;
+    const bool many = M > 2 * kTcRows && N >= 8192 && (long long)units * N >= 128 * 8192;
+    if (items_ok && ((!tc_ok && !ts_ok) || many || (long_items && (M <= kTcRows || !ts_ok)))) return IPOT_SCORER_TENSOR_ITEMS;
+    if (ts_ok && (!tc_ok || (long_items && M > kTcRows))) return IPOT_SCORER_TENSOR_SWEEPS;
     if (tc_ok) return IPOT_SCORER_TENSOR;
     return mma_ok ? IPOT_SCORER_WARP_MMA : IPOT_SCORER_SIMT;
 }
@@ -254,10 +263,15 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
     if (scorer == IPOT_SCORER_TENSOR && !tc_ok) return IPOT_E_INVALID;
     if (scorer == IPOT_SCORER_TENSOR_SWEEPS && !ts_ok) return IPOT_E_INVALID;
     if (scorer == IPOT_SCORER_WARP_MMA && !mma_ok) return IPOT_E_INVALID;
-    if (scorer == IPOT_SCORER_AUTO) scorer = auto_scorer(p, N, M, tc_ok, ts_ok, mma_ok);
+    const bool items_ok = tw_applicable(p->tw, N, M);
+    if (scorer == IPOT_SCORER_TENSOR_ITEMS && !items_ok) return IPOT_E_INVALID;
+    if (scorer == IPOT_SCORER_AUTO) scorer = auto_scorer(p->units, N, M, tc_ok, ts_ok, items_ok, mma_ok);
     // keys of a deferred append: the tensor-core scorers read whole slabs of them where they are, anything else
     // wants them in the pot
-    const int slab_keys = scorer == IPOT_SCORER_TENSOR ? kTcSlab : scorer == IPOT_SCORER_TENSOR_SWEEPS ? kTsSlab : 0;
+    const int slab_keys = scorer == IPOT_SCORER_TENSOR         ? kTcSlab
+                          : scorer == IPOT_SCORER_TENSOR_SWEEPS ? kTsSlab
+                          : scorer == IPOT_SCORER_TENSOR_ITEMS  ? kTwTile
+                                                                : 0;
     const bool keys_in_chunk = p->pend_K && !p->rope && slab_keys && p->pend_first % slab_keys == 0;
     if (p->pend_K && !p->rope && !keys_in_chunk) {
         int mrc = materialise(p, true, false);
@@ -271,7 +285,7 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
     // holds an SM's registers); the selection waits for both.  Other scorers fill the device in waves and need no
     // such care.  A block ranks several streams, one after the other, when that ends before the scorer does: about 8 us
     // a stream against 3 us per round of (128 rows x 256 keys).
-    const bool side_nuc = T > 0 && aux && p->side && (scorer == IPOT_SCORER_TENSOR || scorer == IPOT_SCORER_TENSOR_SWEEPS);
+    const bool side_nuc = T > 0 && aux && p->side && slab_keys;
     const long long rounds = ((long long)p->units * ((M + kTcRows - 1) / kTcRows) * ((N + kTcSlab - 1) / kTcSlab) + p->sm_count - 1) / p->sm_count;
     const int nuc_blocks = (int)std::min<long long>(p->cfg.batch, 1 + (8LL * p->cfg.batch - 1) / (3 * rounds));
     if (T > 0 && aux) {
@@ -299,6 +313,10 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
                        p->stream, parts, &n_launch, keys_in_chunk ? p->pend_K : nullptr, keys_in_chunk ? p->pend_first : 0, p->ts.wait_ns,
                        p->ts.withhold_rank, side_nuc ? nuc_blocks : 0);
         p->launches += n_launch;
+    } else if (scorer == IPOT_SCORER_TENSOR_ITEMS) {
+        rc = tw_launch(p->tw, p->tc, p->cfg, Q, score_keys(p), cap_stats, p->scores, N, M, p->units, p->status, p->stream, p->ts.wait_ns,
+                       p->ts.withhold_rank, keys_in_chunk ? p->pend_K : nullptr, keys_in_chunk ? p->pend_first : 0, side_nuc ? nuc_blocks : 0);
+        p->launches += 1;
     } else if (scorer == IPOT_SCORER_TENSOR_SWEEPS) {
         rc = ts_launch(p->tc, p->ts_occ, p->ts, p->cfg, Q, score_keys(p), cap_stats, p->scores, N, M, p->units, p->status, p->stream,
                        keys_in_chunk ? p->pend_K : nullptr, keys_in_chunk ? p->pend_first : 0, side_nuc ? nuc_blocks : 0);
@@ -586,6 +604,7 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
         return IPOT_E_CUDA;
     }
     tc_plan_init(p->tc, p->cfg, p->K, p->sm_count);
+    tw_plan_init(p->tw, p->tc, p->cfg, p->sm_count);
     *out = p;
     return IPOT_OK;
 }
@@ -617,7 +636,7 @@ int ipot_set_nuc_slots(ipot_t *p, int T)
 
 int ipot_set_scorer(ipot_t *p, int scorer)
 {
-    if (!p || scorer < IPOT_SCORER_AUTO || scorer > IPOT_SCORER_TENSOR_SWEEPS) return IPOT_E_INVALID;
+    if (!p || scorer < IPOT_SCORER_AUTO || scorer > IPOT_SCORER_TENSOR_ITEMS) return IPOT_E_INVALID;
     p->scorer = scorer;
     return IPOT_OK;
 }

@@ -768,12 +768,7 @@ inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, const void *, i
 {
     plan.usable = false;
     plan.sm_count = sm_count;
-    if (cfg.dtype != IPOT_BF16 || (cfg.d != 128 && cfg.d != 64)) return;
-    int coop = 0, dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) {
-        cudaGetLastError();
-        return;
-    }
+    if (cfg.dtype != IPOT_BF16) return;
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess ||
@@ -781,7 +776,13 @@ inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, const void *, i
         cudaGetLastError();
         return;
     }
-    plan.encode = reinterpret_cast<TcEncodeFn>(fn);
+    plan.encode = reinterpret_cast<TcEncodeFn>(fn);   // (the two-sweep scorers need it too)
+    if (cfg.d != 128 && cfg.d != 64) return;
+    int coop = 0, dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) {
+        cudaGetLastError();
+        return;
+    }
     if (cudaFuncSetAttribute(cap_score_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes) != cudaSuccess) {
         cudaGetLastError();
         return;
