@@ -19,6 +19,7 @@
 #include "k_score_mma.cuh"
 #include "k_score_simt.cuh"
 #include "k_score_tc.cuh"
+#include "k_score_f32.cuh"
 #include "k_score_ts.cuh"
 #include "k_score_tw.cuh"
 #include "k_select.cuh"
@@ -40,7 +41,8 @@ struct ipot {
     int deferred;
     const void *pend_K, *pend_V;
     int pend_n, pend_first;
-    // device memory (library-owned)
+    // device memory (library-owned; all but Krot and nov_scratch in one allocation)
+    void *arena;
     void *K, *V;
     // CR-RoPE (ipot_enable_rope): K then holds the keys without rotary embedding, Krot the copy rotated at the slot
     // numbers, which is what the scorers read; the tables are the caller's
@@ -79,6 +81,7 @@ struct ipot {
     long long launches;
     TcPlan tc;           // tensor-core scorer state
     TwPlan tw;
+    F32Plan f32;         // scorer of f32 pots
     TsTuning ts;         // launch parameters of the two-sweep tensor-core scorer
     TsOccupancy ts_occ;
     // the novelty ranking does not depend on the scores: it runs beside the scorer on a stream of its own
@@ -121,11 +124,7 @@ int check_config(const ipot_config_t &c)
 
 void free_all(ipot *p)
 {
-    tc_plan_destroy(p->tc);
-    tw_plan_destroy(p->tw);
-    cudaFree(p->K); cudaFree(p->V); cudaFree(p->Krot); cudaFree(p->scores); cudaFree(p->summed);
-    cudaFree(p->row_stats); cudaFree(p->mma_part); cudaFree(p->cap_stats); cudaFree(p->nuc_mask); cudaFree(p->idx); cudaFree(p->gather.ints); cudaFree(p->status);
-    cudaFree(p->stage_q); cudaFree(p->stage_kc); cudaFree(p->stage_aux); cudaFree(p->nov_scratch); cudaFree(p->dec_partial); cudaFree(p->dec_counters);
+    cudaFree(p->arena); cudaFree(p->Krot); cudaFree(p->nov_scratch);
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
     if (p->ev_join) cudaEventDestroy(p->ev_join);
     if (p->side) cudaStreamDestroy(p->side);
@@ -207,6 +206,18 @@ int launch_simt(ipot *p, const void *Q, const float2 *cap_stats, int M, int N)
     return IPOT_OK;
 }
 
+// f32 pots: every logit computed once, unless one unit's logits exceed the scratch (M * N above 16 million)
+int launch_f32(ipot *p, const void *Q, const float2 *cap_stats, int M, int N)
+{
+    if (!f32_applicable(p->f32, M, N)) return launch_simt<float>(p, Q, cap_stats, M, N);
+    const int d = p->cfg.d;
+    int n = 0;
+    IPOT_CUDA(f32_launch(p->f32, (const float *)Q, (const float *)score_keys(p), cap_stats, p->row_stats, p->scores, p->units, M, N, d,
+                         (size_t)p->cfg.pot_size * d, (float)(1.4426950408889634 / std::sqrt((double)d)), p->sm_count, p->stream, &n));
+    p->launches += n;
+    return IPOT_OK;
+}
+
 // bf16 pots with d a multiple of 16 that the tcgen05 kernel does not take: the same two launches on warp-level tensor cores
 int launch_warp_mma(ipot *p, const void *Q, const float2 *cap_stats, int M, int N)
 {
@@ -282,12 +293,12 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
     if (ev) IPOT_CUDA(cudaEventRecord(ev[0], p->stream));
     // Sec. 3.3.3: the T most novel slots per stream.  Independent of the scores, so it is queued on the side stream (after
     // everything the caller has queued so far) and the tensor-core scorers leave it SMs of their own (a scorer block
-    // holds an SM's registers); the selection waits for both.  Other scorers fill the device in waves and need no
-    // such care.  A block ranks several streams, one after the other, when that ends before the scorer does: about 8 us
+    // holds an SM's registers); the selection waits for both.  Other scorers' blocks are small and need no such
+    // care.  A block ranks several streams, one after the other, when that ends before the scorer does: about 8 us
     // a stream against 3 us per round of (128 rows x 256 keys).
-    const bool side_nuc = T > 0 && aux && p->side && slab_keys;
+    const bool side_nuc = T > 0 && aux && p->side;
     const long long rounds = ((long long)p->units * ((M + kTcRows - 1) / kTcRows) * ((N + kTcSlab - 1) / kTcSlab) + p->sm_count - 1) / p->sm_count;
-    const int nuc_blocks = (int)std::min<long long>(p->cfg.batch, 1 + (8LL * p->cfg.batch - 1) / (3 * rounds));
+    const int nuc_blocks = slab_keys ? (int)std::min<long long>(p->cfg.batch, 1 + (8LL * p->cfg.batch - 1) / (3 * rounds)) : p->cfg.batch;
     if (T > 0 && aux) {
         cudaStream_t ns = side_nuc ? p->side : p->stream;
         if (side_nuc) {
@@ -324,7 +335,7 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
     } else if (scorer == IPOT_SCORER_WARP_MMA) {
         rc = launch_warp_mma(p, Q, cap_stats, M, N);
     } else {
-        rc = p->cfg.dtype == IPOT_F32 ? launch_simt<float>(p, Q, cap_stats, M, N) : launch_simt<__nv_bfloat16>(p, Q, cap_stats, M, N);
+        rc = p->cfg.dtype == IPOT_F32 ? launch_f32(p, Q, cap_stats, M, N) : launch_simt<__nv_bfloat16>(p, Q, cap_stats, M, N);
     }
     if (ev && rc == IPOT_OK) IPOT_CUDA(cudaEventRecord(ev[2], p->stream));   // the scorer's end, before the join below
     if (side_nuc) IPOT_CUDA(cudaStreamWaitEvent(p->stream, p->ev_join, 0));   // (also when the scorer refused: nothing is left behind on the side stream)
@@ -551,10 +562,8 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
     const int maxM = p->G * cfg->max_cap_rows;
     p->max_parts = (maxM + 127) / 128;
     const size_t score_elems = (size_t)p->units * cfg->pot_size;
-    bool ok = true;
-    auto alloc = [&](void **ptr, size_t bytes) {
-        if (ok && cudaMalloc(ptr, bytes ? bytes : 16) != cudaSuccess) ok = false;
-    };
+    DeviceArena mem;
+    auto alloc = [&](void **ptr, size_t bytes, bool zero = false) { mem.add(ptr, bytes, zero); };
     alloc(&p->K, pot_bytes);
     alloc(&p->V, pot_bytes);
     alloc((void **)&p->scores, score_elems * 4 * p->max_parts);
@@ -567,14 +576,17 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
     p->gather.rows = gather_rows(p->row_bytes / 16);
     p->gather.chunks = gather_chunks(cfg->keep, p->row_bytes / 16);
     alloc((void **)&p->gather.ints, (size_t)p->units * p->gather.per_unit() * 4);
-    alloc((void **)&p->status, 16);
+    alloc((void **)&p->status, 16, true);
     p->dec_splits = decode_splits(p->units, 2 * p->sm_count);  // both decode kernels keep two blocks per SM
     alloc((void **)&p->dec_partial, (size_t)p->units * p->dec_splits * p->G * (cfg->d + 2) * sizeof(float));
-    alloc((void **)&p->dec_counters, (size_t)p->units * sizeof(int));
+    alloc((void **)&p->dec_counters, (size_t)p->units * sizeof(int), true);
     alloc(&p->stage_q, (size_t)p->units * maxM * p->row_bytes);
     alloc(&p->stage_kc, (size_t)p->units * cfg->max_cap_rows * p->row_bytes);
     alloc((void **)&p->stage_aux, (size_t)cfg->batch * cfg->pot_size * 4);
-    if (ok) ok = cudaMemset(p->status, 0, 16) == cudaSuccess && cudaMemset(p->dec_counters, 0, (size_t)p->units * sizeof(int)) == cudaSuccess;
+    tc_plan_init(p->tc, p->cfg, p->sm_count, mem);
+    tw_plan_init(p->tw, p->tc, p->cfg, p->sm_count, mem);
+    if (cfg->dtype == IPOT_F32) f32_plan_init(p->f32, p->units, maxM, cfg->pot_size, mem);
+    bool ok = mem.allocate(&p->arena);
     if (!ok) {
         cudaGetLastError();
         free_all(p);
@@ -603,8 +615,6 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
         delete p;
         return IPOT_E_CUDA;
     }
-    tc_plan_init(p->tc, p->cfg, p->K, p->sm_count);
-    tw_plan_init(p->tw, p->tc, p->cfg, p->sm_count);
     *out = p;
     return IPOT_OK;
 }

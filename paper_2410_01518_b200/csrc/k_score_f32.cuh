@@ -1,0 +1,254 @@
+// CaP scoring of f32 pots (Sec. 3.3.1, Eq. 2) with fp32 FMAs, every product computed once.
+//
+//   f32_tile_kernel    : a block computes the logits of a tile (rows x keys) of one unit in registers, takes each row's
+//                        maximum m over the tile's keys, and leaves e = 2^(x - m) in a scratch array and (m, sum e) per
+//                        row beside it.  The block that completes a row tile last (a counter, no waiting) folds the
+//                        row's pairs over all key tiles into (maximum, 1 / denominator).
+//   f32_columns_kernel : u_j = sum_i e_ij 2^(m_tile,i - m_i) / l_i: one weight per row and key tile, no exponential per
+//                        element, coalesced reads of the scratch.
+//
+// Bound: the FMA pipe, 2 M N d flops (recomputing the logits for the column sums, as the generic kernels do, doubles
+// that; the scratch, written and read once, costs 8 bytes per logit against 2 d flops, and units are taken in groups whose
+// scratch stays in L2).  A thread holds 8 rows x 4 keys as packed pairs over even and odd channels: per four
+// channels 12 shared-memory vectors feed 64 packed FMAs.  Where such tiles would leave SMs idle the tiles are smaller
+// (32 x 32, 16 x 16).  Measured (64 units x 4096 keys x 128 channels, M = 128): TODO.
+#pragma once
+#include "common.cuh"
+#include "k_score_simt.cuh"  // merge_stats
+
+namespace ipotk {
+
+constexpr int kF32Threads = 128;   // 16 key columns x 8 row groups
+constexpr int kF32Chan = 32;       // channels per stage
+constexpr int kF32Stride = kF32Chan + 4;
+
+struct F32Params {
+    const float *Q, *K;       // [units][M][d], [units][k_unit rows][d]
+    float *e;                 // [group units][M][e_stride]
+    float2 *part;             // [group units][key tiles][M]
+    float2 *row;              // [units][M]: (maximum, 1 / denominator)
+    int *counters;            // [group units][row tiles], zero between launches
+    const float2 *extra;      // NULL, or [units][M] (max, sum) that join every row's denominator
+    float *scores;            // [units][N]
+    int unit0, M, N, d, e_stride, key_tiles;
+    size_t k_unit_stride;
+    float scale_log2e;
+};
+
+// RT x KT tile; thread (tx, ty) = (t % 16, t / 16) owns rows ty + 8 a and keys tx + 16 b.
+template <int RT, int KT>
+__global__ void __launch_bounds__(kF32Threads, 3)
+f32_tile_kernel(const __grid_constant__ F32Params p)
+{
+    constexpr int RA = RT / 8, KB = KT / 16;
+    __shared__ __align__(16) float qs[2][RT * kF32Stride];
+    __shared__ __align__(16) float ks[2][KT * kF32Stride];
+    __shared__ int is_last;
+    const int g = blockIdx.z, unit = p.unit0 + g, i0 = blockIdx.y * RT, j0 = blockIdx.x * KT;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const float *Qu = p.Q + (size_t)unit * p.M * p.d, *Ku = p.K + (size_t)unit * p.k_unit_stride;
+    const int stages = (p.d + kF32Chan - 1) / kF32Chan;
+    auto fetch = [&](int s) {   // rows beyond M or N and channels beyond d become zeros
+        const int b = s & 1, c0 = s * kF32Chan;
+        for (int v = threadIdx.x; v < (RT + KT) * (kF32Chan / 4); v += kF32Threads) {
+            const int r = v / (kF32Chan / 4), c = (v % (kF32Chan / 4)) * 4;
+            const bool is_q = r < RT;
+            const int row = is_q ? i0 + r : j0 + r - RT;
+            const bool ok = row < (is_q ? p.M : p.N) && c0 + c < p.d;
+            const float *src = (is_q ? Qu : Ku) + (ok ? (size_t)row * p.d + c0 + c : 0);
+            float *dst = is_q ? &qs[b][r * kF32Stride + c] : &ks[b][(r - RT) * kF32Stride + c];
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    asm volatile("griddepcontrol.launch_dependents;");   // the column kernel may be made resident; it waits for this grid's end
+    float2 acc[RA][KB];
+#pragma unroll
+    for (int a = 0; a < RA; ++a)
+#pragma unroll
+        for (int b = 0; b < KB; ++b) acc[a][b] = make_float2(0.f, 0.f);
+    fetch(0);
+    for (int s = 0; s < stages; ++s) {
+        if (s + 1 < stages) {
+            fetch(s + 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const float *q = qs[s & 1] + ty * kF32Stride, *k = ks[s & 1] + tx * kF32Stride;
+#pragma unroll 2
+        for (int c = 0; c < kF32Chan; c += 4) {
+            float4 qv[RA], kv[KB];
+#pragma unroll
+            for (int a = 0; a < RA; ++a) qv[a] = *reinterpret_cast<const float4 *>(q + 8 * a * kF32Stride + c);
+#pragma unroll
+            for (int b = 0; b < KB; ++b) kv[b] = *reinterpret_cast<const float4 *>(k + 16 * b * kF32Stride + c);
+#pragma unroll
+            for (int a = 0; a < RA; ++a)
+#pragma unroll
+                for (int b = 0; b < KB; ++b) {
+                    acc[a][b] = __ffma2_rn(make_float2(qv[a].x, qv[a].y), make_float2(kv[b].x, kv[b].y), acc[a][b]);
+                    acc[a][b] = __ffma2_rn(make_float2(qv[a].z, qv[a].w), make_float2(kv[b].z, kv[b].w), acc[a][b]);
+                }
+        }
+        __syncthreads();   // the stage may be overwritten
+    }
+#pragma unroll
+    for (int a = 0; a < RA; ++a) {
+        const int row = i0 + ty + 8 * a;
+        float x[KB], m = -INFINITY, l = 0.f;
+#pragma unroll
+        for (int b = 0; b < KB; ++b) {
+            x[b] = (acc[a][b].x + acc[a][b].y) * p.scale_log2e;
+            if (j0 + tx + 16 * b < p.N) m = fmaxf(m, x[b]);
+        }
+#pragma unroll
+        for (int off = 8; off >= 1; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+#pragma unroll
+        for (int b = 0; b < KB; ++b) {
+            const int key = j0 + tx + 16 * b;
+            const float e = exp2f(x[b] - m);
+            if (key < p.N) {
+                l += e;
+                if (row < p.M) p.e[((size_t)g * p.M + row) * p.e_stride + key] = e;
+            }
+        }
+#pragma unroll
+        for (int off = 8; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+        if (tx == 0 && row < p.M) __stcg(&p.part[((size_t)g * p.key_tiles + blockIdx.x) * p.M + row], make_float2(m, l));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int *counter = p.counters + (size_t)g * gridDim.y + blockIdx.y, done;
+        asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(done) : "l"(counter) : "memory");
+        is_last = done == p.key_tiles - 1;
+        if (is_last) *counter = 0;   // ready for the next launch
+    }
+    __syncthreads();
+    if (!is_last) return;
+    // sixteen lanes per row, each over every sixteenth key tile
+    for (int r = ty; r < RT && i0 + r < p.M; r += kF32Threads / 16) {
+        const int row = i0 + r;
+        float m = -INFINITY, l = 0.f;
+        for (int t = tx; t < p.key_tiles; t += 16) {
+            const float2 s = __ldcg(&p.part[((size_t)g * p.key_tiles + t) * p.M + row]);
+            merge_stats(m, l, s.x, s.y);
+        }
+        const unsigned half = 0xffffu << (threadIdx.x & 16);   // (the two rows of a warp may end apart)
+#pragma unroll
+        for (int off = 8; off >= 1; off >>= 1) {
+            const float m2 = __shfl_xor_sync(half, m, off), l2 = __shfl_xor_sync(half, l, off);
+            merge_stats(m, l, m2, l2);
+        }
+        if (tx == 0) {
+            if (p.extra) {
+                const float2 s = p.extra[(size_t)unit * p.M + row];
+                merge_stats(m, l, s.x, s.y);
+            }
+            p.row[(size_t)unit * p.M + row] = make_float2(m, 1.f / l);
+        }
+    }
+}
+
+// grid (ceil(N / 64), group units), block 256: 64 keys x 4 row quarters.  kt: keys of a tile of the first kernel (16, 32, 64).
+constexpr int kF32ColThreads = 256;
+__global__ void __launch_bounds__(kF32ColThreads)
+f32_columns_kernel(const __grid_constant__ F32Params p, int kt)
+{
+    __shared__ float w[64 / 16][256];   // weights of up to 256 rows for the block's key tiles
+    __shared__ float red[4][64];
+    const int g = blockIdx.y, unit = p.unit0 + g, j = threadIdx.x & 63, part = threadIdx.x >> 6, key = blockIdx.x * 64 + j;
+    const int tiles = 64 / kt, tile0 = blockIdx.x * tiles;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    float u[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int i0 = 0; i0 < p.M; i0 += 256) {
+        const int n = min(256, p.M - i0);
+        __syncthreads();
+        for (int v = threadIdx.x; v < tiles * n; v += kF32ColThreads) {
+            const int t = v / n, i = v - t * n;
+            float f = 0.f;
+            if (tile0 + t < p.key_tiles) {
+                const float2 s = __ldcg(&p.part[((size_t)g * p.key_tiles + tile0 + t) * p.M + i0 + i]), r = __ldcg(&p.row[(size_t)unit * p.M + i0 + i]);
+                f = exp2f(s.x - r.x) * r.y;
+            }
+            w[t][i] = f;
+        }
+        __syncthreads();
+        if (key < p.N) {
+            const float *e = p.e + ((size_t)g * p.M + i0) * p.e_stride + key, *wj = w[j / kt];
+            int i = part;
+            for (; i + 28 < n; i += 32) {   // eight rows in flight
+                float v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = __ldcg(e + (size_t)(i + 4 * k) * p.e_stride);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) u[k & 3] = fmaf(v[k], wj[i + 4 * k], u[k & 3]);
+            }
+            for (; i < n; i += 4) u[0] = fmaf(__ldcg(e + (size_t)i * p.e_stride), wj[i], u[0]);
+        }
+    }
+    red[part][j] = (u[0] + u[1]) + (u[2] + u[3]);
+    __syncthreads();
+    if (threadIdx.x < 64 && key < p.N) p.scores[(size_t)unit * p.N + key] = (red[0][j] + red[1][j]) + (red[2][j] + red[3][j]);
+}
+
+// ------------------------------------------------------------------ host side
+constexpr size_t kF32Scratch = (size_t)64 << 20;   // half of L2
+
+// Bytes a unit needs: its e values and the row pairs of its key tiles (the smallest tile has 16 keys)
+inline size_t f32_unit_bytes(int M, int N) { return (size_t)M * ((N + 3) & ~3) * 4 + (size_t)((N + 15) / 16) * M * 8; }
+
+struct F32Plan {
+    char *scratch = nullptr;
+    int *counters = nullptr;      // [units][row tiles of 16]
+    size_t bytes = 0;
+};
+
+inline void f32_plan_init(F32Plan &plan, int units, int max_M, int pot_size, DeviceArena &mem)
+{
+    const size_t all = (size_t)units * f32_unit_bytes(max_M, pot_size);
+    plan.bytes = all < kF32Scratch ? all : kF32Scratch;
+    mem.add((void **)&plan.scratch, plan.bytes);
+    mem.add((void **)&plan.counters, (size_t)units * ((max_M + 15) / 16) * sizeof(int), true);
+}
+
+inline bool f32_applicable(const F32Plan &plan, int M, int N) { return plan.scratch && f32_unit_bytes(M, N) <= plan.bytes; }
+
+inline cudaError_t f32_launch(const F32Plan &plan, const float *Q, const float *K, const float2 *extra, float2 *row_stats, float *scores, int units,
+                              int M, int N, int d, size_t k_unit_stride, float scale_log2e, int sm_count, cudaStream_t stream, int *launches)
+{
+    // the largest tile that still gives every SM a block
+    int t = 64;
+    while (t > 16 && (long long)units * ((M + t - 1) / t) * ((N + t - 1) / t) < sm_count) t /= 2;
+    F32Params p;
+    p.Q = Q; p.K = K; p.extra = extra; p.row = row_stats; p.scores = scores; p.counters = plan.counters;
+    p.M = M; p.N = N; p.d = d; p.k_unit_stride = k_unit_stride; p.scale_log2e = scale_log2e;
+    p.e_stride = (N + 3) & ~3;
+    p.key_tiles = (N + t - 1) / t;
+    int per = (int)(plan.bytes / f32_unit_bytes(M, N));
+    if (per > 65535) per = 65535;
+    p.e = (float *)plan.scratch;
+    for (int u0 = 0; u0 < units; u0 += per) {
+        const int n = units - u0 < per ? units - u0 : per;
+        p.unit0 = u0;
+        p.part = (float2 *)(plan.scratch + (size_t)n * M * p.e_stride * 4);
+        const dim3 grid(p.key_tiles, (M + t - 1) / t, n);
+        (t == 64 ? f32_tile_kernel<64, 64> : t == 32 ? f32_tile_kernel<32, 32> : f32_tile_kernel<16, 16>)<<<grid, kF32Threads, 0, stream>>>(p);
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3((N + 63) / 64, n);
+        lc.blockDim = dim3(kF32ColThreads);
+        lc.stream = stream;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        lc.attrs = at;
+        lc.numAttrs = 1;
+        const cudaError_t err = cudaLaunchKernelEx(&lc, f32_columns_kernel, p, t);
+        if (err != cudaSuccess) return err;
+        *launches += 2;
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace ipotk

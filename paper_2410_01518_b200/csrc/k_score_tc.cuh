@@ -748,6 +748,39 @@ typedef CUresult (*TcEncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, v
                                const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// Device memory of a pot: every buffer is registered first and all of them come out of one allocation (a cudaMalloc
+// each cost a pot of 20 buffers several milliseconds).  Those that have to start as zeros lie together at the front.
+struct DeviceArena {
+    struct Want { void **ptr; size_t bytes; bool zero; };
+    static constexpr int kMost = 32;
+    Want wants[kMost];
+    int n = 0;
+    void add(void **ptr, size_t bytes, bool zero = false)
+    {
+        if (n < kMost) wants[n] = {ptr, (bytes + 255) / 256 * 256 + (bytes ? 0 : 256), zero};
+        ++n;
+    }
+    // false: out of memory, nothing allocated
+    bool allocate(void **base)
+    {
+        if (n > kMost) return false;
+        size_t total = 0, zeros = 0;
+        for (int i = 0; i < n; ++i) {
+            total += wants[i].bytes;
+            if (wants[i].zero) zeros += wants[i].bytes;
+        }
+        if (cudaMalloc(base, total) != cudaSuccess || cudaMemset(*base, 0, zeros) != cudaSuccess) return false;
+        char *at = (char *)*base, *at_zero = at;
+        at += zeros;
+        for (int i = 0; i < n; ++i) {
+            char *&from = wants[i].zero ? at_zero : at;
+            *wants[i].ptr = from;
+            from += wants[i].bytes;
+        }
+        return true;
+    }
+};
+
 struct TcPlan {
     bool usable = false;
     TcEncodeFn encode = nullptr;
@@ -757,14 +790,7 @@ struct TcPlan {
     uint32_t mark = 0;                // of the last launch
 };
 
-inline void tc_plan_destroy(TcPlan &plan)
-{
-    cudaFree(plan.stats);
-    plan.stats = nullptr;
-    plan.usable = false;
-}
-
-inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, const void *, int sm_count)
+inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, int sm_count, DeviceArena &mem)
 {
     plan.usable = false;
     plan.sm_count = sm_count;
@@ -791,12 +817,7 @@ inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, const void *, i
     const int units = cfg.layers * cfg.batch * cfg.Hkv;
     plan.max_items = units * ((G * cfg.max_cap_rows + kTcRows - 1) / kTcRows);
     plan.max_slabs = (cfg.pot_size + kTcSlab - 1) / kTcSlab;
-    const size_t stats_bytes = (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float2);
-    if (cudaMalloc(&plan.stats, stats_bytes) != cudaSuccess || cudaMemset(plan.stats, 0, stats_bytes) != cudaSuccess) {
-        cudaGetLastError();
-        tc_plan_destroy(plan);
-        return;
-    }
+    mem.add((void **)&plan.stats, (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float2), true);
     plan.usable = true;
 }
 

@@ -682,15 +682,7 @@ struct TwPlan {
     int *sync = nullptr;
 };
 
-inline void tw_plan_destroy(TwPlan &plan)
-{
-    cudaFree(plan.part);
-    cudaFree(plan.nl);
-    cudaFree(plan.sync);
-    plan = TwPlan{};
-}
-
-inline void tw_plan_init(TwPlan &plan, const TcPlan &enc, const ipot_config_t &cfg, int sm_count)
+inline void tw_plan_init(TwPlan &plan, const TcPlan &enc, const ipot_config_t &cfg, int sm_count, DeviceArena &mem)
 {
     plan.sm_count = sm_count;
     if (cfg.dtype != IPOT_BF16 || !enc.encode) return;
@@ -704,12 +696,9 @@ inline void tw_plan_init(TwPlan &plan, const TcPlan &enc, const ipot_config_t &c
     const int tiles = (cfg.pot_size + kTwTile - 1) / kTwTile;
     plan.max_jobs = tiles < kTwMaxJobs ? tiles : kTwMaxJobs;
     const size_t rows = (size_t)units * plan.max_mt * kTwTile, sync_ints = kTwSyncHead + (size_t)units * (1 + plan.max_mt);
-    if (cudaMalloc(&plan.part, rows * plan.max_jobs * sizeof(float2)) != cudaSuccess || cudaMalloc(&plan.nl, rows * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&plan.sync, sync_ints * sizeof(int)) != cudaSuccess || cudaMemset(plan.sync, 0, sync_ints * sizeof(int)) != cudaSuccess) {
-        cudaGetLastError();
-        tw_plan_destroy(plan);
-        return;
-    }
+    mem.add((void **)&plan.part, rows * plan.max_jobs * sizeof(float2));
+    mem.add((void **)&plan.nl, rows * sizeof(float));
+    mem.add((void **)&plan.sync, sync_ints * sizeof(int), true);
     plan.usable = true;
 }
 
