@@ -575,7 +575,7 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
     alloc((void **)&p->idx, (size_t)p->units * cfg->keep * 4);
     p->gather.rows = gather_rows(p->row_bytes / 16);
     p->gather.chunks = gather_chunks(cfg->keep, p->row_bytes / 16);
-    alloc((void **)&p->gather.ints, (size_t)p->units * p->gather.per_unit() * 4);
+    alloc((void **)&p->gather.ints, (size_t)p->units * p->gather.per_unit() * 4, true);
     alloc((void **)&p->status, 16, true);
     p->dec_splits = decode_splits(p->units, 2 * p->sm_count);  // both decode kernels keep two blocks per SM
     alloc((void **)&p->dec_partial, (size_t)p->units * p->dec_splits * p->G * (cfg->d + 2) * sizeof(float));

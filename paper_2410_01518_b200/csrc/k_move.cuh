@@ -66,12 +66,13 @@ inline int gather_rows(int row_vecs) { return kGatherBytes / 16 / row_vecs; }
 inline int gather_chunks(int keep, int row_vecs) { return (keep + gather_rows(row_vecs) - 1) / gather_rows(row_vecs); }
 
 // What the selection leaves for the gather, ints of one unit: [0, chunks] the number of survivors in slots below c * rows
-// (which survivors come from a chunk's own slots), then per tensor a ticket and a flag for every chunk, zero, raised when
-// the chunk has been read.
+// (which survivors come from a chunk's own slots).  Then per tensor the gather's own a ticket, a count of finished blocks and a
+// flag for every chunk, raised when it has been read; zero between launches.
 struct GatherPlan {
     int *ints;
     int rows, chunks;
-    __host__ __device__ int per_unit() const { return 3 * (chunks + 1); }
+    __host__ __device__ int per_tensor() const { return chunks + 2; }
+    __host__ __device__ int per_unit() const { return chunks + 1 + 2 * per_tensor(); }
 };
 
 struct GatherParams {
@@ -109,21 +110,26 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
     const int32_t *ix = p.idx + (size_t)unit * p.keep;
     const int rows = p.plan.rows, chunks = p.plan.chunks;
     const int *below = p.plan.ints + (size_t)unit * p.plan.per_unit();
-    int *sync = p.plan.ints + (size_t)unit * p.plan.per_unit() + (1 + tensor) * (chunks + 1);
+    int *sync = p.plan.ints + (size_t)unit * p.plan.per_unit() + chunks + 1 + tensor * p.plan.per_tensor();
     const uint4 *alt = tensor ? p.pend.V : p.pend.K;
     const int alt_first = alt ? p.pend.first : 0x7fffffff;
     if (alt) alt += (size_t)unit * p.pend.unit_vecs;
-    // launched as a programmatic dependent of the selection: the blocks may be resident before it has ended and
-    // wait here for its index lists (returns at once after an ordinary launch)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (threadIdx.x == 0) {
         gave_up = 0;
         chunk_sm = atomicAdd(sync, 1);
     }
     __syncthreads();
+    // launched as a programmatic dependent of the selection: the blocks may be resident before it has ended and
+    // wait here for its index lists (returns at once after an ordinary launch)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int chunk = chunk_sm, r0 = chunk * rows, n = min(rows, p.keep - r0);
     const uint32_t sbuf = (uint32_t)__cvta_generic_to_shared(buf);
     const int nvec = n * p.row_vecs;
+    int q0 = 0, q1 = 0;   // the survivors whose sources lie in this chunk's slots
+    if (threadIdx.x == kGatherThreads - 32) {
+        q0 = __ldg(below + chunk);
+        q1 = __ldg(below + chunk + 1);
+    }
     for (int i = threadIdx.x; i < n; i += kGatherThreads) {
         int src = __ldg(ix + r0 + i);
         if (src < r0 + i || src >= p.N) {
@@ -151,13 +157,12 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
     if (threadIdx.x == kGatherThreads - 32 && r0 < alt_first && chunk > 0) {
         // while the rows are on their way: the chunks whose sources lie in this chunk's slots (no source in slots whose rows
         // are outside the pot) have been read
-        const int q0 = __ldg(below + chunk), q1 = __ldg(below + chunk + 1);
         const int c1 = q1 > q0 ? min(chunk - 1, (q1 - 1) / rows) : -1;
         const unsigned long long t0 = global_timer_ns();
         for (int c = max(0, q0 / rows); c <= c1; ++c) {
             int up = 0;
             for (uint32_t tries = 1; !up; ++tries) {
-                asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(up) : "l"(sync + 1 + c) : "memory");
+                asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(up) : "l"(sync + 2 + c) : "memory");
                 if (!up && (tries & 255u) == 0 && global_timer_ns() - t0 > p.wait_ns) {
                     set_status(p.status, kStatusTimeout);
                     gave_up = 1;
@@ -170,7 +175,7 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk copy below reads what the threads have brought in
     __syncthreads();
     if (threadIdx.x == 0) {
-        asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(sync + 1 + chunk), "r"(1) : "memory");
+        asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(sync + 2 + chunk), "r"(1) : "memory");
         if (!gave_up) {   // (a wait that ran out: the rows stay as they are)
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
                          ::"l"(base + (size_t)r0 * p.row_vecs), "r"(sbuf), "r"((uint32_t)nvec * 16u) : "memory");
@@ -178,7 +183,11 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
         }
     }
     if (tensor == 0) rotate(buf, (int)unit, r0, n, p.row_vecs);
-    if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the block's memory is free again
+    if (threadIdx.x == 0) {
+        if (atomicAdd(sync + 1, 1) == chunks - 1)   // every block has passed its waits: ready for the next launch
+            for (int i = 0; i < chunks + 2; ++i) sync[i] = 0;
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the block's memory is free again
+    }
 }
 
 __global__ void __launch_bounds__(kGatherThreads) compact_kernel(const __grid_constant__ GatherParams p)

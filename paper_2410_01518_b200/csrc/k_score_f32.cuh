@@ -31,6 +31,7 @@ struct F32Params {
     const float2 *extra;      // NULL, or [units][M] (max, sum) that join every row's denominator
     float *scores;            // [units][N]
     int unit0, M, N, d, e_stride, key_tiles;
+    int fold_here;            // the tile kernel folds the row pairs; else f32_fold_kernel does
     size_t k_unit_stride;
     float scale_log2e;
 };
@@ -61,7 +62,7 @@ f32_tile_kernel(const __grid_constant__ F32Params p)
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    asm volatile("griddepcontrol.launch_dependents;");   // the column kernel may be made resident; it waits for this grid's end
+    asm volatile("griddepcontrol.launch_dependents;");   // the next kernel may be made resident; it waits for this grid's end
     float2 acc[RA][KB];
 #pragma unroll
     for (int a = 0; a < RA; ++a)
@@ -87,10 +88,11 @@ f32_tile_kernel(const __grid_constant__ F32Params p)
 #pragma unroll
             for (int a = 0; a < RA; ++a)
 #pragma unroll
-                for (int b = 0; b < KB; ++b) {
-                    acc[a][b] = __ffma2_rn(make_float2(qv[a].x, qv[a].y), make_float2(kv[b].x, kv[b].y), acc[a][b]);
-                    acc[a][b] = __ffma2_rn(make_float2(qv[a].z, qv[a].w), make_float2(kv[b].z, kv[b].w), acc[a][b]);
-                }
+                for (int b = 0; b < KB; ++b) acc[a][b] = __ffma2_rn(make_float2(qv[a].x, qv[a].y), make_float2(kv[b].x, kv[b].y), acc[a][b]);
+#pragma unroll
+            for (int a = 0; a < RA; ++a)
+#pragma unroll
+                for (int b = 0; b < KB; ++b) acc[a][b] = __ffma2_rn(make_float2(qv[a].z, qv[a].w), make_float2(kv[b].z, kv[b].w), acc[a][b]);
         }
         __syncthreads();   // the stage may be overwritten
     }
@@ -118,6 +120,7 @@ f32_tile_kernel(const __grid_constant__ F32Params p)
         for (int off = 8; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
         if (tx == 0 && row < p.M) __stcg(&p.part[((size_t)g * p.key_tiles + blockIdx.x) * p.M + row], make_float2(m, l));
     }
+    if (!p.fold_here) return;
     __syncthreads();
     if (threadIdx.x == 0) {
         int *counter = p.counters + (size_t)g * gridDim.y + blockIdx.y, done;
@@ -148,6 +151,40 @@ f32_tile_kernel(const __grid_constant__ F32Params p)
             }
             p.row[(size_t)unit * p.M + row] = make_float2(m, 1.f / l);
         }
+    }
+}
+
+// The fold as a launch of its own, grid (ceil(M / 4), group units): a warp per row.  For rows of many key tiles (more than
+// 16 per thread of the block above: its one block's loads would be the longest chain of the cycle).
+__global__ void __launch_bounds__(kF32Threads)
+f32_fold_kernel(const __grid_constant__ F32Params p)
+{
+    const int g = blockIdx.y, unit = p.unit0 + g, row = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (row >= p.M) return;
+    float m = -INFINITY, l = 0.f;
+    for (int t0 = 0; t0 < p.key_tiles; t0 += 256) {
+        float2 s[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int t = t0 + 32 * i + lane;
+            s[i] = t < p.key_tiles ? __ldcg(&p.part[((size_t)g * p.key_tiles + t) * p.M + row]) : make_float2(-INFINITY, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) merge_stats(m, l, s[i].x, s[i].y);
+    }
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+        const float m2 = __shfl_xor_sync(0xffffffffu, m, off), l2 = __shfl_xor_sync(0xffffffffu, l, off);
+        merge_stats(m, l, m2, l2);
+    }
+    if (lane == 0) {
+        if (p.extra) {
+            const float2 s = p.extra[(size_t)unit * p.M + row];
+            merge_stats(m, l, s.x, s.y);
+        }
+        p.row[(size_t)unit * p.M + row] = make_float2(m, 1.f / l);
     }
 }
 
@@ -226,6 +263,7 @@ inline cudaError_t f32_launch(const F32Plan &plan, const float *Q, const float *
     p.M = M; p.N = N; p.d = d; p.k_unit_stride = k_unit_stride; p.scale_log2e = scale_log2e;
     p.e_stride = (N + 3) & ~3;
     p.key_tiles = (N + t - 1) / t;
+    p.fold_here = t * p.key_tiles <= 16 * kF32Threads;
     int per = (int)(plan.bytes / f32_unit_bytes(M, N));
     if (per > 65535) per = 65535;
     p.e = (float *)plan.scratch;
@@ -236,15 +274,22 @@ inline cudaError_t f32_launch(const F32Plan &plan, const float *Q, const float *
         const dim3 grid(p.key_tiles, (M + t - 1) / t, n);
         (t == 64 ? f32_tile_kernel<64, 64> : t == 32 ? f32_tile_kernel<32, 32> : f32_tile_kernel<16, 16>)<<<grid, kF32Threads, 0, stream>>>(p);
         cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3((N + 63) / 64, n);
-        lc.blockDim = dim3(kF32ColThreads);
         lc.stream = stream;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[0].val.programmaticStreamSerializationAllowed = 1;
         lc.attrs = at;
         lc.numAttrs = 1;
-        const cudaError_t err = cudaLaunchKernelEx(&lc, f32_columns_kernel, p, t);
+        cudaError_t err = cudaGetLastError();
+        if (!p.fold_here && err == cudaSuccess) {
+            lc.gridDim = dim3((M + 3) / 4, n);
+            lc.blockDim = dim3(kF32Threads);
+            err = cudaLaunchKernelEx(&lc, f32_fold_kernel, p);
+            *launches += 1;
+        }
+        lc.gridDim = dim3((N + 63) / 64, n);
+        lc.blockDim = dim3(kF32ColThreads);
+        if (err == cudaSuccess) err = cudaLaunchKernelEx(&lc, f32_columns_kernel, p, t);
         if (err != cudaSuccess) return err;
         *launches += 2;
     }

@@ -781,7 +781,19 @@ struct DeviceArena {
     }
 };
 
+// A tensor map and what it was made from.  A pot's buffers and the caller's few query and chunk buffers come back every
+// cycle; making a map is about a microsecond of host work, three times a cycle.
+struct TcMapSlot {
+    CUtensorMap map;
+    const void *ptr = nullptr;
+    int d = 0, rows = 0, units = 0, box_rows = 0;
+    size_t unit_rows = 0;
+};
+constexpr int kTcMapSlots = 16;
+
 struct TcPlan {
+    TcMapSlot maps[kTcMapSlots];
+    int next_map = 0;                 // the slot that is overwritten next
     bool usable = false;
     TcEncodeFn encode = nullptr;
     int sm_count = 0;
@@ -831,6 +843,11 @@ inline bool tc_applicable(TcPlan &plan, const ipot_config_t &cfg, int N, int M)
 // [units][unit_rows][d] bf16, of which `rows` per unit are addressable; box = 64 x box_rows x 1, 128-byte swizzle.
 inline int tc_encode_rows(TcPlan &plan, CUtensorMap *map, const void *ptr, int d, int rows, int units, size_t unit_rows, int box_rows)
 {
+    for (const TcMapSlot &s : plan.maps)
+        if (s.ptr == ptr && s.d == d && s.rows == rows && s.units == units && s.box_rows == box_rows && s.unit_rows == unit_rows) {
+            *map = s.map;
+            return IPOT_OK;
+        }
     cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)rows, (cuuint64_t)units};
     cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)unit_rows * d * 2};
     cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
@@ -838,7 +855,12 @@ inline int tc_encode_rows(TcPlan &plan, CUtensorMap *map, const void *ptr, int d
     CUresult r = plan.encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(ptr), dims, strides, box, estr,
                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? IPOT_OK : IPOT_E_CUDA;
+    if (r != CUDA_SUCCESS) return IPOT_E_CUDA;
+    TcMapSlot &s = plan.maps[plan.next_map];
+    plan.next_map = (plan.next_map + 1) % kTcMapSlots;
+    s.map = *map;
+    s.ptr = ptr; s.d = d; s.rows = rows; s.units = units; s.box_rows = box_rows; s.unit_rows = unit_rows;
+    return IPOT_OK;
 }
 
 // scores: partial array p (query rows 128 p ...) is written at scores + p * part_stride, unit stride N.

@@ -268,7 +268,6 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
     asm volatile("griddepcontrol.launch_dependents;");
     if (threadIdx.x < 256) sh.hist[threadIdx.x] = 0;
     int *below = plan.ints + (size_t)unit * plan.per_unit();   // for the gather that follows
-    for (int i = plan.chunks + 1 + threadIdx.x; i < plan.per_unit(); i += kThreads) below[i] = 0;
     uint32_t key[kKpt];
     // a reserved slot outranks every score: finite scores map below 0xFF800000
     constexpr int kPiece = kKpt > 16 ? 8 : 16;   // slots loaded at a time (what 64 registers a thread allow)
