@@ -143,8 +143,8 @@ enum {
 int ipot_set_tuning(ipot_t *pot, int what, long long value);
 
 /* Forget the contents: len = 0.  Nothing is launched.  Also the way back to a defined state after
- * ipot_sync_status() reported IPOT_E_TIMEOUT: what a launch that gave up has left in the scorer's exchange
- * buffers is never taken for a later launch's (the sticky status itself stays). */
+ * ipot_sync_status() reported IPOT_E_TIMEOUT: the scorer's exchange buffers are cleared before their next use
+ * (the sticky status itself stays). */
 int ipot_reset(ipot_t *pot);
 
 /*

@@ -296,10 +296,14 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
     // holds an SM's registers); the selection waits for both.  Other scorers' blocks are small and need no such
     // care.  A block ranks several streams, one after the other, when that ends before the scorer does: about 8 us
     // a stream against 3 us per round of (128 rows x 256 keys).
-    const bool side_nuc = T > 0 && aux && p->side;
     const long long rounds = ((long long)p->units * ((M + kTcRows - 1) / kTcRows) * ((N + kTcSlab - 1) / kTcSlab) + p->sm_count - 1) / p->sm_count;
-    const int nuc_blocks = slab_keys ? (int)std::min<long long>(p->cfg.batch, 1 + (8LL * p->cfg.batch - 1) / (3 * rounds)) : p->cfg.batch;
-    if (T > 0 && aux) {
+    // ... or rides along in the scorer's own launch: the fork and join by events cost a small cycle 5 us
+    const bool in_scorer = T > 0 && aux && N > kTcSlab && N <= kNucMaxSlots && rounds <= 12 && p->sm_count > 1 && (scorer == IPOT_SCORER_TENSOR || scorer == IPOT_SCORER_TENSOR_ITEMS);
+    const bool side_nuc = T > 0 && aux && p->side && !in_scorer;
+    const int nuc_blocks = slab_keys ? (int)std::min<long long>(std::min(p->cfg.batch, std::max(1, p->sm_count / 4)), 1 + (8LL * p->cfg.batch - 1) / (3 * rounds)) : p->cfg.batch;
+    NucJob nuc{};
+    if (in_scorer) nuc = NucJob{aux, p->nuc_mask, T, p->cfg.batch, 0};
+    else if (T > 0 && aux) {
         cudaStream_t ns = side_nuc ? p->side : p->stream;
         if (side_nuc) {
             IPOT_CUDA(cudaEventRecord(p->ev_fork, p->stream));
@@ -322,11 +326,11 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
         int n_launch = 0;
         rc = tc_launch(p->tc, p->cfg, Q, score_keys(p), cap_stats, p->scores, (size_t)p->units * p->cfg.pot_size, N, M, p->units, p->status,
                        p->stream, parts, &n_launch, keys_in_chunk ? p->pend_K : nullptr, keys_in_chunk ? p->pend_first : 0, p->ts.wait_ns,
-                       p->ts.withhold_rank, side_nuc ? nuc_blocks : 0);
+                       p->ts.withhold_rank, side_nuc || in_scorer ? nuc_blocks : 0, nuc);
         p->launches += n_launch;
     } else if (scorer == IPOT_SCORER_TENSOR_ITEMS) {
         rc = tw_launch(p->tw, p->tc, p->cfg, Q, score_keys(p), cap_stats, p->scores, N, M, p->units, p->status, p->stream, p->ts.wait_ns,
-                       p->ts.withhold_rank, keys_in_chunk ? p->pend_K : nullptr, keys_in_chunk ? p->pend_first : 0, side_nuc ? nuc_blocks : 0);
+                       p->ts.withhold_rank, keys_in_chunk ? p->pend_K : nullptr, keys_in_chunk ? p->pend_first : 0, in_scorer ? nuc_blocks : 0, nuc);
         p->launches += 1;
     } else if (scorer == IPOT_SCORER_TENSOR_SWEEPS) {
         rc = ts_launch(p->tc, p->ts_occ, p->ts, p->cfg, Q, score_keys(p), cap_stats, p->scores, N, M, p->units, p->status, p->stream,
@@ -411,8 +415,8 @@ int run_cycle(ipot *p, const void *Q, const void *Kc, int cap_rows, const float 
     int rc = run_scoring(p, Q, Kc, cap_rows, aux, &parts);
     if (rc != IPOT_OK) return rc;
     const size_t part_stride = (size_t)p->units * p->cfg.pot_size;
-    launch_select(p->units, p->stream, p->scores, parts, part_stride, T > 0 ? p->nuc_mask : nullptr, p->idx,
-                  parts > 1 ? p->summed : nullptr, N, keep, p->cfg.Hkv, p->cfg.batch, p->status, p->gather);
+    IPOT_CUDA(launch_select(p->units, p->stream, p->scores, parts, part_stride, T > 0 ? p->nuc_mask : nullptr, p->idx,
+                  parts > 1 ? p->summed : nullptr, N, keep, p->cfg.Hkv, p->cfg.batch, p->status, p->gather));
     p->launches += 1;
     IPOT_CUDA(cudaGetLastError());
     if (ev) IPOT_CUDA(cudaEventRecord(ev[3], p->stream));
@@ -937,6 +941,7 @@ int ipot_sync_status(ipot_t *p)
     IPOT_CUDA(cudaStreamSynchronize(p->stream));
     int st = 0;
     IPOT_CUDA(cudaMemcpy(&st, p->status, sizeof(int), cudaMemcpyDeviceToHost));
+    if (st) p->tc.last_items = 0;  // a launch that gave up half way: the tensor scorer clears its statistics before its next launch
     return st;
 }
 

@@ -20,7 +20,7 @@
 //            exponentials of the first chunk's second half;
 //   combine  (4 warps, one thread per query row) merges the eight (max, sum) pairs of
 //            its row into the slab's statistics and publishes them with one 8-byte
-//            store whose reference carries the launch's number as a "fresh" mark; then reads
+//            store whose sum carries the launch's sign as a "fresh" mark; then reads
 //            the row's statistics of all slabs of the item, re-reading until every
 //            one is fresh, and turns them into the row's global maximum m, its
 //            denominator l (plus, when given, the share of the CaP's own keys) and the
@@ -53,6 +53,7 @@
 
 #include "../../include/ipot.h"
 #include "common.cuh"
+#include "k_select.cuh"  // NucJob
 
 namespace ipotk {
 
@@ -60,11 +61,6 @@ constexpr int kTcThreads = 704;      // warp 0: TMA, 1: MMA + TMEM owner, 2-17: 
 constexpr int kTcRows = 128;         // query rows per item (TMEM lanes)
 constexpr int kTcSlab = 256;         // keys per task (TMEM columns per buffer)
 constexpr int kTcFmaEighths = 2;     // share of pass 1's exponentials evaluated on the FMA pipe
-// The published reference is the slab's maximum with its lowest mantissa bits replaced by the launch's mark: any number
-// near the maximum serves as a reference (the sum is taken relative to the one that is published), so the mark costs no
-// precision.  Marks count up, so whatever an earlier launch left in the array - of another layout, or of one that gave
-// up half way - never looks fresh, and the array is only cleared when they start over.
-constexpr uint32_t kTcMarkBits = 6, kTcMarks = (1u << kTcMarkBits) - 1;
 constexpr int kTcD = 128;            // largest head dimension; 64 uses the first 64-channel half of every tile
 constexpr uint32_t kTcQBytes = kTcRows * kTcD * 2;           // 32 KiB: two halves of 128 rows x 64 channels
 constexpr uint32_t kTcKBytes = kTcSlab * kTcD * 2;           // 64 KiB: two halves of 256 rows x 64 channels
@@ -86,9 +82,9 @@ enum { kBarFull = 0, kBarEmpty = 2, kBarEReady = 4, kBarFReady = 6, kBarSFull = 
 struct TcParams {
     float *scores;        // partial array p (query rows 128p ...) at scores + p * part_stride, unit stride N
     size_t part_stride;
-    float2 *stats;        // [items][slabs][128] (reference in log2 units, sum relative to it); see kTcMarkBits
+    float2 *stats;        // [items][slabs][128] (max in log2 units, sum * sign); all of the other sign or 0 at launch
     const float2 *cap_stats;  // NULL, or [units][M] (max, sum) over the CaP's own keys that join every row's denominator
-    uint32_t mark;        // this launch's "fresh" mark, 1 .. kTcMarks
+    float sign;           // +1 or -1: this launch's "fresh" mark
     unsigned long long wait_ns;  // limit of every wait
     int withhold_cta;     // -1; test hook: this CTA never publishes its slab statistics
     int *status;
@@ -97,6 +93,8 @@ struct TcParams {
     int new_slab0;        // slabs from this one on are read through the second key map (the chunk of a deferred
                           // append, row 0 = key 256 * new_slab0); INT_MAX if all keys are in the pot
     float scale_log2e;
+    int ctas;             // blocks that score; those behind them rank the streams' novelty
+    NucJob nuc;
 };
 
 // ------------------------------------------------------------------ PTX wrappers
@@ -419,14 +417,21 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr)
 constexpr uint32_t kTcIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 
 // ------------------------------------------------------------------ the kernel
+// kRank: blocks from prm.ctas on rank the streams' novelty.  (Their code costs the others about 5 % through the register
+// allocation, so launches of more than a dozen rounds use the variant without it and a ranking kernel on the side.)
+template <bool kRank>
 __global__ void __launch_bounds__(kTcThreads, 1)
 cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
-                    const __grid_constant__ CUtensorMap mapKnew, TcParams prm)
+                    const __grid_constant__ CUtensorMap mapKnew, const __grid_constant__ TcParams prm)
 {
     extern __shared__ __align__(1024) uint8_t tc_smem_raw[];
     const uint32_t base = smem_u32(tc_smem_raw);
     if (base & 1023u) {  // the swizzled tiles need this alignment; nothing has been started yet
         if (threadIdx.x == 0) set_status(prm.status, kStatusBounds);
+        return;
+    }
+    if (kRank && (int)blockIdx.x >= prm.ctas) {
+        nuc_rank_extra_block(prm.nuc, prm.N, (int)blockIdx.x - prm.ctas, reinterpret_cast<SelShared *>(tc_smem_raw));
         return;
     }
     uint8_t *gbase = tc_smem_raw;
@@ -467,7 +472,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         // ---------------------------------------------------------------- TMA producer
         if (lane == 0) {
             uint32_t k = 0;
-            for (int task = blockIdx.x; task < prm.tasks; task += gridDim.x, ++k) {
+            for (int task = blockIdx.x; task < prm.tasks; task += prm.ctas, ++k) {
                 const int item = task / tasks_per_item, slab = task - item * tasks_per_item;
                 const int unit = item / prm.mtiles, mt = item - unit * prm.mtiles;
                 const uint32_t b = k & 1, ph = (k >> 1) & 1;
@@ -494,7 +499,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         // ---------------------------------------------------------------- MMA issuer
         if (lane == 0) {
             uint32_t k = 0;
-            for (int task = blockIdx.x; task < prm.tasks; task += gridDim.x, ++k) {
+            for (int task = blockIdx.x; task < prm.tasks; task += prm.ctas, ++k) {
                 const uint32_t b = k & 1, ph = (k >> 1) & 1;
                 if (!mbar_wait(bar(kBarFull + b), ph, ab, prm.status)) break;
                 const uint32_t qa = base + kTcOffStage + b * kTcStageBytes, kb = qa + kTcQBytes;
@@ -531,11 +536,11 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         const float *fbuf = reinterpret_cast<const float *>(gbase + kTcOffFbuf);
         float *colpart = reinterpret_cast<float *>(gbase + kTcOffColpart);
         const float c = prm.scale_log2e;
-        const int n_local = (prm.tasks - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+        const int n_local = (prm.tasks - (int)blockIdx.x + prm.ctas - 1) / prm.ctas;
         for (int k = 0; k <= n_local; ++k) {
             if (k < n_local) {
                 // ---- pass 1 of local task k
-                const int task = blockIdx.x + k * gridDim.x;
+                const int task = blockIdx.x + k * prm.ctas;
                 const int slab = task % tasks_per_item;
                 const int nvalid = min(kTcSlab, prm.N - slab * kTcSlab);
                 const uint32_t b = k & 1, ph = (k >> 1) & 1;
@@ -599,7 +604,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             if (k >= 1) {
                 // ---- pass 2 of local task k - 1
                 const int kk = k - 1;
-                const int task = blockIdx.x + kk * gridDim.x;
+                const int task = blockIdx.x + kk * prm.ctas;
                 const int item = task / tasks_per_item, slab = task - item * tasks_per_item;
                 const int unit = item / prm.mtiles, mt = item - unit * prm.mtiles;
                 const int nvalid = min(kTcSlab, prm.N - slab * kTcSlab);
@@ -647,11 +652,9 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         const int row = threadIdx.x - 576;
         const float2 *tstat = reinterpret_cast<const float2 *>(gbase + kTcOffTstat);
         float *fbuf = reinterpret_cast<float *>(gbase + kTcOffFbuf);
-        const uint32_t mark = prm.mark;
-        auto marked = [&](float x) { return __uint_as_float((__float_as_uint(x) & ~kTcMarks) | mark); };
-        auto is_fresh = [&](float2 v) { return (__float_as_uint(v.x) & kTcMarks) == mark; };
+        const float sgn = prm.sign;
         uint32_t k = 0;
-        for (int task = blockIdx.x; task < prm.tasks; task += gridDim.x, ++k) {
+        for (int task = blockIdx.x; task < prm.tasks; task += prm.ctas, ++k) {
             const int item = task / tasks_per_item, slab = task - item * tasks_per_item;
             const int mt = item % prm.mtiles;
             const uint32_t b = k & 1, ph = (k >> 1) & 1;
@@ -669,13 +672,13 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 for (int i = 0; i < 8; ++i) t[i] = tstat[(b * 8 + i) * kTcRows + row];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) cm[i] = t[i].x;
-                const float ms0 = marked(max3(max3(cm[0], cm[1], cm[2]), max3(cm[3], cm[4], cm[5]), fmaxf(cm[6], cm[7])));  // chunk 0 always holds a valid key
+                const float ms0 = max3(max3(cm[0], cm[1], cm[2]), max3(cm[3], cm[4], cm[5]), fmaxf(cm[6], cm[7]));  // chunk 0 always holds a valid key
 #pragma unroll
                 for (int i = 0; i < 8; ++i) ce[i] = (cm[i] == -INFINITY) ? 0.f : t[i].y * ex2(cm[i] - ms0);
             }
-            const float ms = marked(max3(max3(cm[0], cm[1], cm[2]), max3(cm[3], cm[4], cm[5]), fmaxf(cm[6], cm[7])));
+            const float ms = max3(max3(cm[0], cm[1], cm[2]), max3(cm[3], cm[4], cm[5]), fmaxf(cm[6], cm[7]));
             const float ls = ((ce[0] + ce[1]) + (ce[2] + ce[3])) + ((ce[4] + ce[5]) + (ce[6] + ce[7]));
-            if (tasks_per_item > 1 && (int)blockIdx.x != prm.withhold_cta) st_gpu_f32x2(&prm.stats[((size_t)item * tasks_per_item + slab) * kTcRows + row], ms, ls);
+            if (tasks_per_item > 1 && (int)blockIdx.x != prm.withhold_cta) st_gpu_f32x2(&prm.stats[((size_t)item * tasks_per_item + slab) * kTcRows + row], ms, ls * sgn);
 
             // ---- this row's statistics of every slab of the item; re-read until all carry this launch's mark
             const float2 *st = prm.stats + (size_t)item * tasks_per_item * kTcRows + row;
@@ -690,13 +693,13 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 bool fresh;
 #pragma unroll
                 for (int s = 0; s < 16; ++s)  // beyond the item: neutral and fresh; this CTA's own slab: known; others: stale
-                    sv[s] = (s0 + s >= tasks_per_item) ? make_float2(marked(-3e38f), 0.f) : (s0 + s == slab) ? make_float2(ms, ls) : make_float2(0.f, 0.f);
+                    sv[s] = (s0 + s >= tasks_per_item) ? make_float2(-INFINITY, sgn) : (s0 + s == slab) ? make_float2(ms, ls * sgn) : make_float2(0.f, 0.f);
                 do {  // only the entries that are still stale are read again
                     fresh = true;
 #pragma unroll
                     for (int s = 0; s < 16; ++s) {
-                        if (!is_fresh(sv[s])) sv[s] = ld_gpu_f32x2(&st[(size_t)(s0 + s) * kTcRows]);
-                        fresh = fresh && is_fresh(sv[s]);
+                        if (!(sv[s].y * sgn > 0.f)) sv[s] = ld_gpu_f32x2(&st[(size_t)(s0 + s) * kTcRows]);
+                        fresh = fresh && (sv[s].y * sgn > 0.f);
                     }
                     if (!fresh && (*ab || ((++tries & 1023u) == 0 && global_timer_ns() > *reinterpret_cast<volatile unsigned long long *>(ab + 1)))) {
                         if (!*ab) {
@@ -710,7 +713,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                                       max3(max3(sv[9].x, sv[10].x, sv[11].x), max3(sv[12].x, sv[13].x, sv[14].x), fmaxf(sv[15].x, m)), -INFINITY);
                 float w[16];
 #pragma unroll
-                for (int s = 0; s < 16; ++s) w[s] = sv[s].y * ex2(sv[s].x - mb);
+                for (int s = 0; s < 16; ++s) w[s] = fabsf(sv[s].y) * ex2(sv[s].x - mb);
 #pragma unroll
                 for (int step = 1; step < 16; step <<= 1) {
 #pragma unroll
@@ -799,7 +802,10 @@ struct TcPlan {
     int sm_count = 0;
     int max_items = 0, max_slabs = 0;
     float2 *stats = nullptr;          // [max_items][max_slabs][128]
-    uint32_t mark = 0;                // of the last launch
+    // "fresh" marking of the statistics: every launch writes all entries of its (items x slabs) layout
+    // with the sign opposite to the previous launch's; a layout change, or a launch that gave up, clears the array first
+    float sign = 1.f;
+    int last_items = 0, last_slabs = 0;
 };
 
 inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, int sm_count, DeviceArena &mem)
@@ -821,7 +827,8 @@ inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, int sm_count, D
         cudaGetLastError();
         return;
     }
-    if (cudaFuncSetAttribute(cap_score_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes) != cudaSuccess) {
+    if (cudaFuncSetAttribute(cap_score_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(cap_score_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes) != cudaSuccess) {
         cudaGetLastError();
         return;
     }
@@ -829,7 +836,7 @@ inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, int sm_count, D
     const int units = cfg.layers * cfg.batch * cfg.Hkv;
     plan.max_items = units * ((G * cfg.max_cap_rows + kTcRows - 1) / kTcRows);
     plan.max_slabs = (cfg.pot_size + kTcSlab - 1) / kTcSlab;
-    mem.add((void **)&plan.stats, (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float2), true);
+    mem.add((void **)&plan.stats, (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float2));
     plan.usable = true;
 }
 
@@ -869,7 +876,7 @@ inline int tc_encode_rows(TcPlan &plan, CUtensorMap *map, const void *ptr, int d
 inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, const void *K, const float2 *cap_stats, float *scores,
                      size_t part_stride, int N, int M, int units, int *status, cudaStream_t stream, int *parts, int *n_launch,
                      const void *Knew = nullptr, int new_first = 0, unsigned long long wait_ns = 200ull * 1000 * 1000,
-                     int withhold_cta = -1, int spare_sms = 0)
+                     int withhold_cta = -1, int spare_sms = 0, NucJob nuc = NucJob{})
 {
     if (!tc_applicable(plan, cfg, N, M)) return IPOT_E_INVALID;
     if (Knew && (new_first % kTcSlab != 0 || new_first >= N)) return IPOT_E_INVALID;
@@ -894,18 +901,24 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
     prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d));
     prm.wait_ns = wait_ns;
     prm.withhold_cta = withhold_cta;
-    if (plan.mark == kTcMarks) {
-        if (cudaMemsetAsync(plan.stats, 0, (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float2), stream) != cudaSuccess) {
+    if (items != plan.last_items || prm.slabs != plan.last_slabs) {
+        if (cudaMemsetAsync(plan.stats, 0, (size_t)items * prm.slabs * kTcRows * sizeof(float2), stream) != cudaSuccess) {
             cudaGetLastError();
             return IPOT_E_CUDA;
         }
-        plan.mark = 0;
+        plan.last_items = items;
+        plan.last_slabs = prm.slabs;
     }
-    prm.mark = ++plan.mark;
+    plan.sign = -plan.sign;
+    prm.sign = plan.sign;
     cudaLaunchConfig_t lc = {};
-    // spare_sms: SMs left to a small kernel of the same cycle that runs beside this one on another stream
+    // spare_sms: SMs left to a small kernel of the same cycle that runs beside this one on another stream, or, with nuc, to
+    // the ranking's blocks of this launch (at least; SMs without a task are theirs too)
     const int ctas = plan.sm_count - spare_sms > 0 ? plan.sm_count - spare_sms : 1;
-    lc.gridDim = dim3(prm.tasks < ctas ? prm.tasks : ctas, 1, 1);
+    prm.ctas = prm.tasks < ctas ? prm.tasks : ctas;
+    if (nuc.batch > 0) nuc.ctas = nuc.batch < plan.sm_count - prm.ctas ? nuc.batch : plan.sm_count - prm.ctas;
+    prm.nuc = nuc;
+    lc.gridDim = dim3(prm.ctas + nuc.ctas, 1, 1);
     lc.blockDim = dim3(kTcThreads, 1, 1);
     lc.dynamicSmemBytes = kTcSmemBytes;
     lc.stream = stream;
@@ -913,7 +926,7 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
     at[0].id = cudaLaunchAttributeCooperative;  // all CTAs resident: they wait on each other's statistics
     at[0].val.cooperative = 1;
     lc.attrs = at; lc.numAttrs = 1;
-    if (cudaLaunchKernelEx(&lc, cap_score_tc_kernel, mapQ, mapK, mapKnew, prm) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&lc, nuc.ctas > 0 ? cap_score_tc_kernel<true> : cap_score_tc_kernel<false>, mapQ, mapK, mapKnew, prm) != cudaSuccess) {
         cudaGetLastError();
         return IPOT_E_CUDA;
     }

@@ -76,6 +76,8 @@ struct TwParams {
     float scale_log2e;
     unsigned long long wait_ns;
     int withhold_job;         // -1; test hook: this job's statistics are never published
+    int ctas;                 // blocks that score; those behind them rank the streams' novelty
+    NucJob nuc;
 };
 
 // An item as it is handed out: the job's number, kTwSecond added for its S2 visit; negative: no more.
@@ -184,6 +186,10 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
     constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);   // 128 x 128, bf16 -> fp32
     extern __shared__ __align__(1024) uint8_t tw_smem[];
     const uint32_t base = smem_u32(tw_smem);
+    if ((int)blockIdx.x >= prm.ctas) {
+        nuc_rank_extra_block(prm.nuc, prm.N, (int)blockIdx.x - prm.ctas, reinterpret_cast<SelShared *>(tw_smem));
+        return;
+    }
     uint32_t &tmem_slot = *reinterpret_cast<uint32_t *>(tw_smem + kTwOffSlot);
     int &abort_flag = *reinterpret_cast<int *>(tw_smem + kTwOffSlot + 4);
     int &last_cta = *reinterpret_cast<int *>(tw_smem + kTwOffSlot + 8);
@@ -664,7 +670,7 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
     }
     if (threadIdx.x == 0) {
         __threadfence();
-        last_cta = atomicAdd(prm.sync + 2, 1) == (int)gridDim.x - 1;
+        last_cta = atomicAdd(prm.sync + 2, 1) == prm.ctas - 1;
     }
     __syncthreads();
     if (last_cta)   // every other CTA has left: the counters are put back for the next launch
@@ -708,7 +714,7 @@ inline bool tw_applicable(const TwPlan &plan, int N, int M) { return plan.usable
 // but in this [units][N - new_first][d] array.
 inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const void *Q, const void *K, const float2 *cap_stats, float *scores,
                      int N, int M, int units, int *status, cudaStream_t stream, unsigned long long wait_ns, int withhold_job,
-                     const void *Knew, int new_first, int spare_sms)
+                     const void *Knew, int new_first, int spare_sms, NucJob nuc = NucJob{})
 {
     if (!tw_applicable(plan, N, M) || (Knew && (new_first % kTwTile != 0 || new_first >= N))) return IPOT_E_INVALID;
     CUtensorMap mapQ, mapK, mapKnew;
@@ -730,7 +736,7 @@ inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const 
     const int slots = (int)((kTwSmemMax - kTwOffTiles) / tile_bytes);
     prm.qslots = slots >= 5 ? 2 : 1;
     prm.kslots = slots - prm.qslots < kTwMaxK ? slots - prm.qslots : kTwMaxK;
-    const int ctas = plan.sm_count - spare_sms > 0 ? plan.sm_count - spare_sms : 1;   // spare_sms: left to a small kernel that runs beside this one
+    const int ctas = plan.sm_count - spare_sms > 0 ? plan.sm_count - spare_sms : 1;   // spare_sms: left to the ranking, as in tc_launch
     // Tiles per job: few, so that the items spread evenly over the CTAs, but not so few that the start of an item (query
     // tile, hand-over of the statistics: about half a tile's time) weighs.  With several row blocks a job's key tiles stay
     // in shared memory for all of them and a group keeps one key's running sum, hence at most kslots and kTwGroups.
@@ -755,9 +761,11 @@ inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const 
     prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d));
     prm.wait_ns = wait_ns;
     prm.withhold_job = withhold_job;
-    const int grid = 2 * prm.jobs < ctas ? 2 * prm.jobs : ctas;
+    prm.ctas = 2 * prm.jobs < ctas ? 2 * prm.jobs : ctas;
+    if (nuc.batch > 0) nuc.ctas = nuc.batch < plan.sm_count - prm.ctas ? nuc.batch : plan.sm_count - prm.ctas;
+    prm.nuc = nuc;
     const size_t smem = kTwOffTiles + (size_t)(prm.qslots + prm.kslots) * tile_bytes;
-    cap_score_tw_kernel<<<grid, kTwThreads, smem, stream>>>(mapQ, mapK, mapKnew, prm);
+    cap_score_tw_kernel<<<prm.ctas + nuc.ctas, kTwThreads, smem, stream>>>(mapQ, mapK, mapKnew, prm);
     return cudaGetLastError() == cudaSuccess ? IPOT_OK : IPOT_E_CUDA;
 }
 

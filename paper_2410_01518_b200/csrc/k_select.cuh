@@ -5,9 +5,13 @@
 //                       key, take the top `keep` keys, emit the survivors'
 //                       slot numbers in ascending order.
 // Both are an exact radix select on an order-preserving 32-bit image of the
-// fp32 value (4 passes of 8 bits, most significant first) followed by one
-// ordered sweep; among equal keys the lower slot wins, so the result is a pure
-// function of the score bits.
+// fp32 value followed by one ordered sweep; among equal keys the lower slot
+// wins, so the result is a pure function of the score bits.  The digits (11
+// bits) start at the highest bit in which the problem's keys differ - the scores
+// of a unit span a few binades, and a digit that all of them share would put
+// every count on one address - and the search ends as soon as the boundary
+// digit's keys are taken as a whole: two passes nearly always, where digits of 8
+// bits from the top took four (TODO us instead of TODO for a pot of 4096).
 //
 // One block per problem.  A thread keeps 16 (pot sizes above 16384: 32) consecutive
 // slots' keys in registers from the first load to the last store, and the block has
@@ -23,10 +27,12 @@ namespace ipotk {
 
 constexpr int kSelMaxWarps = 32;
 
+constexpr int kSelBits = 11, kSelBins = 1 << kSelBits;
 struct SelShared {
-    __align__(16) uint32_t hist[256];
+    __align__(16) uint32_t hist[kSelBins];
     uint32_t wtot[2][kSelMaxWarps];
-    uint32_t bin;
+    uint32_t wmin[kSelMaxWarps], wmax[kSelMaxWarps], wres[kSelMaxWarps];
+    uint32_t bin, count;
     int remaining;
 };
 
@@ -56,76 +62,86 @@ __device__ __forceinline__ uint32_t block_scan_exclusive(uint32_t v, SelShared &
     return (warp == 0 ? 0u : before) + inc - v;
 }
 
-// k-th largest (k >= 1) of the block's keys: returns the key value and how many keys equal to it
-// must be taken (need_eq >= 1).  sh.hist must be zero on entry and is zero again on exit.
+// Key 0 marks no slot, key 0xFFFFFFFF a reserved one, which ranks above all.  The k (>= 1) largest keys of the block are
+// those > tau and need_eq of those == tau (need_eq may be 0).  sh.hist must be zero on entry and is zero again on exit.
 template <int kThreads, int kKpt>
 __device__ __forceinline__ void block_radix_select(const uint32_t (&key)[kKpt], int k, SelShared &sh,
                                                    uint32_t &tau, int &need_eq)
 {
-    uint32_t prefix = 0, mask = 0;
-    int remaining = k;
-    const int lane = threadIdx.x & 31;
-#pragma unroll 1
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        if (shift == 24) {
-            // leading byte (sign and exponent): the scores of a problem sit within a few binades, so a thread's keys -
-            // often a warp's - share it; they are counted in registers and leave as one update
-            const uint32_t d0 = key[0] >> 24;
-            uint32_t cnt = 0;
+    constexpr int kWarps = kThreads / 32, kPer = kSelBins / kThreads;   // bins of a thread
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t mn = 0xFFFFFFFFu, mx = 0u, res = 0u;
 #pragma unroll
-            for (int i = 0; i < kKpt; ++i) cnt += (key[i] >> 24) == d0 ? 1u : 0u;
-            if (__all_sync(0xffffffffu, d0 == __shfl_sync(0xffffffffu, d0, 0))) {
-                const uint32_t tot = __reduce_add_sync(0xffffffffu, cnt);
-                if (lane == 0) atomicAdd(&sh.hist[d0], tot);
-            } else {
-                atomicAdd(&sh.hist[d0], cnt);
-            }
-#pragma unroll
-            for (int i = 1; i < kKpt; ++i)
-                if ((key[i] >> 24) != d0) atomicAdd(&sh.hist[key[i] >> 24], 1u);
-        } else {
-#pragma unroll
-            for (int i = 0; i < kKpt; ++i)
-                if ((key[i] & mask) == prefix) atomicAdd(&sh.hist[(key[i] >> shift) & 255u], 1u);
-        }
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            // lane l owns the 8 bins 255 - 8l ... 248 - 8l (descending key order) and clears them for the next pass
-            uint4 *h4 = reinterpret_cast<uint4 *>(sh.hist) + (62 - 2 * lane);
-            const uint4 lo = h4[0], hi = h4[1];
-            h4[0] = make_uint4(0u, 0u, 0u, 0u);
-            h4[1] = make_uint4(0u, 0u, 0u, 0u);
-            const uint32_t c[8] = {hi.w, hi.z, hi.y, hi.x, lo.w, lo.z, lo.y, lo.x};
-            const uint32_t tot = ((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7]));
-            uint32_t inc = tot;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const uint32_t v = __shfl_up_sync(0xffffffffu, inc, off);
-                if (lane >= off) inc += v;
-            }
-            uint32_t run = inc - tot;  // keys in the bins above this lane's
-            if (run < (uint32_t)remaining && (uint32_t)remaining <= inc) {
-                int found = 7;
-#pragma unroll
-                for (int i = 6; i >= 0; --i) {  // the first bin that reaches `remaining`
-                    uint32_t upto = run;
-#pragma unroll
-                    for (int e = 0; e <= i; ++e) upto += c[e];
-                    if (upto >= (uint32_t)remaining) found = i;
-                }
-#pragma unroll
-                for (int e = 0; e < 7; ++e) run += e < found ? c[e] : 0u;
-                sh.bin = 255u - (8u * lane + found);
-                sh.remaining = remaining - (int)run;
-            }
-        }
-        __syncthreads();
-        prefix |= sh.bin << shift;
-        mask |= 255u << shift;
-        remaining = sh.remaining;
+    for (int i = 0; i < kKpt; ++i) {
+        const bool reserved = key[i] == 0xFFFFFFFFu;
+        res += reserved ? 1u : 0u;
+        mx = max(mx, reserved ? 0u : key[i]);
+        mn = min(mn, key[i] ? key[i] : 0xFFFFFFFFu);
     }
-    tau = prefix;
-    need_eq = remaining;
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    res = __reduce_add_sync(0xffffffffu, res);
+    if (lane == 0) {
+        sh.wmin[warp] = mn;
+        sh.wmax[warp] = mx;
+        sh.wres[warp] = res;
+    }
+    __syncthreads();
+    mn = __reduce_min_sync(0xffffffffu, lane < kWarps ? sh.wmin[lane] : 0xFFFFFFFFu);
+    mx = __reduce_max_sync(0xffffffffu, lane < kWarps ? sh.wmax[lane] : 0u);
+    res = __reduce_add_sync(0xffffffffu, lane < kWarps ? sh.wres[lane] : 0u);
+    int remaining = k - (int)res;
+    if (remaining <= 0) {   // only reserved slots
+        tau = 0xFFFFFFFEu;
+        need_eq = 0;
+        return;
+    }
+    uint32_t lo = mn, span = mx - mn;   // the boundary lies in [lo, lo + span]
+    for (int pass = 0;; ++pass) {
+        if (span == 0u) {
+            tau = lo;
+            need_eq = remaining;
+            return;
+        }
+        const int bits = 32 - __clz(span), shift = bits > kSelBits ? bits - kSelBits : 0;
+#pragma unroll
+        for (int i = 0; i < kKpt; ++i)
+            if (key[i] - lo <= span) atomicAdd(&sh.hist[(key[i] - lo) >> shift], 1u);   // (no slot and reserved ones wrap around or lie above)
+        __syncthreads();
+        // thread t owns the kPer bins below kSelBins - t * kPer (descending key order) and clears them for the next pass
+        uint32_t c[kPer], tot = 0;
+        uint2 *h2 = reinterpret_cast<uint2 *>(sh.hist + kSelBins - (threadIdx.x + 1) * kPer);
+#pragma unroll
+        for (int i = 0; i < kPer / 2; ++i) {
+            const uint2 v = h2[i];
+            h2[i] = make_uint2(0u, 0u);
+            c[kPer - 1 - 2 * i] = v.x;
+            c[kPer - 2 - 2 * i] = v.y;
+            tot += v.x + v.y;
+        }
+        uint32_t total;
+        uint32_t run = block_scan_exclusive<kThreads>(tot, sh, pass & 1, total);   // keys in the bins above this thread's
+        if (run < (uint32_t)remaining && (uint32_t)remaining <= run + tot) {
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                if (run < (uint32_t)remaining && (uint32_t)remaining <= run + c[i]) {
+                    sh.bin = kSelBins - 1 - (threadIdx.x * kPer + i);
+                    sh.count = c[i];
+                    sh.remaining = remaining - (int)run;
+                }
+                run += c[i];
+            }
+        }
+        __syncthreads();
+        remaining = sh.remaining;
+        lo += sh.bin << shift;
+        if ((uint32_t)remaining == sh.count) {   // the whole digit is taken (the case remaining == count == 1 above all)
+            tau = lo - 1u;
+            need_eq = 0;
+            return;
+        }
+        span = min((1u << shift) - 1u, mx - lo);
+    }
 }
 
 // Larger and equal keys in the slots below this thread's, in one block scan (16 bits each: a block has at
@@ -211,16 +227,15 @@ __device__ __forceinline__ void load_row(const float *__restrict__ row, int slot
 }
 __host__ __device__ inline int mask_stride(int N) { return (N + 31) & ~31; }   // bytes of a stream's mask row
 
-// mask[b][j] = 1 iff slot j is one of the T most novel slots of stream b.  A block takes streams blockIdx.x,
-// blockIdx.x + gridDim.x, ...
+// mask[b][j] = 1 iff slot j is one of the T most novel slots of stream b, for the streams first, first + step, ... of batch,
+// by kThreads threads of the block.
 template <int kThreads, int kKpt>
-__global__ void __launch_bounds__(kThreads)
-nuc_mask_kernel(const float *__restrict__ aux, uint8_t *__restrict__ mask, int N, int T, int batch)
+__device__ __forceinline__ void nuc_rank_streams(const float *__restrict__ aux, uint8_t *__restrict__ mask, int N, int T, int batch, int first,
+                                                 int step, SelShared &sh)
 {
-    __shared__ SelShared sh;
     const int slot0 = threadIdx.x * kKpt;
-    if (threadIdx.x < 256) sh.hist[threadIdx.x] = 0;
-    for (int b = blockIdx.x; b < batch; b += gridDim.x) {
+    for (int i = threadIdx.x; i < kSelBins; i += kThreads) sh.hist[i] = 0;
+    for (int b = first; b < batch; b += step) {
         uint8_t *m = mask + (size_t)b * mask_stride(N);
         uint32_t key[kKpt];
         {
@@ -247,6 +262,27 @@ nuc_mask_kernel(const float *__restrict__ aux, uint8_t *__restrict__ mask, int N
         __syncthreads();
     }
 }
+template <int kThreads, int kKpt>
+__global__ void __launch_bounds__(kThreads)
+nuc_mask_kernel(const float *__restrict__ aux, uint8_t *__restrict__ mask, int N, int T, int batch)
+{
+    __shared__ SelShared sh;
+    nuc_rank_streams<kThreads, kKpt>(aux, mask, N, T, batch, blockIdx.x, gridDim.x, sh);
+}
+
+// The ranking as extra blocks of a scorer's grid, for up to 16384 slots: a kernel of its own beside the scorer costs an
+// event fork and join, about 5 us of a small cycle.  Out of line, so that it leaves the scorer's register allocation alone.
+struct NucJob {
+    const float *aux;   // [batch][N]
+    uint8_t *mask;
+    int T, batch, ctas;   // ctas == 0: nothing to rank
+};
+constexpr int kNucThreads = 512, kNucMaxSlots = 16 * kNucThreads;
+__device__ __forceinline__ void nuc_rank_extra_block(const NucJob &job, int N, int first, SelShared *sh)
+{
+    if (threadIdx.x >= kNucThreads) return;   // (the barriers below count the threads that have not exited)
+    nuc_rank_streams<kNucThreads, 16>(job.aux, job.mask, N, job.T, job.batch, first, job.ctas, *sh);
+}
 
 // grid (units).  scores: `parts` partial score arrays of [units][N] each, `part_stride`
 // floats apart, added in index order.  mask may be NULL (T == 0).  The survivors' slot numbers
@@ -264,10 +300,12 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
     const float *u = scores + (size_t)unit * N;
     const uint8_t *m = mask ? mask + (size_t)b * mask_stride(N) : nullptr;
     const int slot0 = threadIdx.x * kKpt;
-    // the compaction may be made resident now; it waits for this grid's end before it reads an index
-    asm volatile("griddepcontrol.launch_dependents;");
-    if (threadIdx.x < 256) sh.hist[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < kSelBins; i += kThreads) sh.hist[i] = 0;
     int *below = plan.ints + (size_t)unit * plan.per_unit();   // for the gather that follows
+    // launched as a programmatic dependent of the scorer: its scores and the ranking's mask are complete after this.  Then
+    // the compaction may be made resident; it waits for this grid's end before it reads an index.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
     uint32_t key[kKpt];
     // a reserved slot outranks every score: finite scores map below 0xFF800000
     constexpr int kPiece = kKpt > 16 ? 8 : 16;   // slots loaded at a time (what 64 registers a thread allow)
@@ -342,22 +380,26 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
 }
 
 // Launch shapes: the smallest block whose threads hold N slots at 16 a thread (32 above 16384 slots).
-#define IPOT_SEL_DISPATCH(kernel, blocks, stream, N, ...)                                        \
-    do {                                                                                         \
-        if ((N) <= 4096) kernel<256, 16><<<(blocks), 256, 0, (stream)>>>(__VA_ARGS__);           \
-        else if ((N) <= 8192) kernel<512, 16><<<(blocks), 512, 0, (stream)>>>(__VA_ARGS__);      \
-        else if ((N) <= 16384) kernel<1024, 16><<<(blocks), 1024, 0, (stream)>>>(__VA_ARGS__);   \
-        else kernel<1024, 32><<<(blocks), 1024, 0, (stream)>>>(__VA_ARGS__);                     \
-    } while (0)
-
 inline void launch_nuc_mask(int blocks, cudaStream_t st, const float *aux, uint8_t *mask, int N, int T, int batch)
 {
-    IPOT_SEL_DISPATCH(nuc_mask_kernel, blocks, st, N, aux, mask, N, T, batch);
+    const int threads = N <= 4096 ? 256 : N <= 8192 ? 512 : 1024;
+    auto kern = N <= 4096 ? nuc_mask_kernel<256, 16> : N <= 8192 ? nuc_mask_kernel<512, 16> : N <= 16384 ? nuc_mask_kernel<1024, 16> : nuc_mask_kernel<1024, 32>;
+    kern<<<blocks, threads, 0, st>>>(aux, mask, N, T, batch);
 }
-inline void launch_select(int blocks, cudaStream_t st, const float *scores, int parts, size_t part_stride, const uint8_t *mask,
-                          int32_t *idx, float *summed, int N, int keep, int Hkv, int batch, int *status, const GatherPlan &plan)
+inline cudaError_t launch_select(int blocks, cudaStream_t st, const float *scores, int parts, size_t part_stride, const uint8_t *mask,
+                                 int32_t *idx, float *summed, int N, int keep, int Hkv, int batch, int *status, const GatherPlan &plan)
 {
-    IPOT_SEL_DISPATCH(select_kernel, blocks, st, N, scores, parts, part_stride, mask, idx, summed, N, keep, Hkv, batch, status, plan);
+    auto kern = N <= 4096 ? select_kernel<256, 16> : N <= 8192 ? select_kernel<512, 16> : N <= 16384 ? select_kernel<1024, 16> : select_kernel<1024, 32>;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(blocks, 1, 1);
+    lc.blockDim = dim3(N <= 4096 ? 256 : N <= 8192 ? 512 : 1024, 1, 1);
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kern, scores, parts, part_stride, mask, idx, summed, N, keep, Hkv, batch, status, plan);
 }
 
 // summed[i] = parts[0][i] + parts[1][i] + ... in index order (the order select_kernel uses).
