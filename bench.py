@@ -37,7 +37,8 @@ NOVELTY_WORKLOADS = {"nuc32k": (32000, 2048), "nuc128k": (128256, 2048)}
 DECODE_WORKLOADS = {"decode3": 3, "decode4": 4, "decode5": 5}
 SCORERS = {"auto": 0, "simt": 1, "tensor": 2, "warp_mma": 3, "sweeps": 4, "items": 5}
 SCORER_KERNELS = {1: "cap_row_stats + cap_column_sums (fp32 FMA)", 2: "cap_score_tc_kernel (tcgen05, one sweep)",
-                  3: "cap_row_stats_mma + cap_column_sums_mma (mma.sync)", 4: "cap_score_ts_kernel (tcgen05, two sweeps)"}
+                  3: "cap_row_stats_mma + cap_column_sums_mma (mma.sync)", 4: "cap_score_ts_kernel (tcgen05, two sweeps)",
+                  5: "cap_score_tw_kernel (tcgen05, two sweeps, items)"}
 MIN_SAMPLED_S = 1.0   # the clock sampler should see at least this much of timed running
 RING = 4  # distinct chunks / query sets cycled through
 PREHEAT_S = 0.5  # untimed running before the warm-up steps, see main()
@@ -684,7 +685,7 @@ def main():
     # DRAM bytes of one launch of the dominant kernel, from the committed ncu captures (profiles/dram_traffic.txt: measured
     # on a few layers of the same shape and scaled by the units, which is how the traffic grows); null if no capture
     # of this kernel and shape is on record
-    tkey = {1: "simt", 2: "cap_score_tc", 3: "warp_mma", 4: "cap_score_ts"}.get(scorer_used, "?") if dom == 1 else "compact"
+    tkey = {1: "simt", 2: "cap_score_tc", 3: "warp_mma", 4: "cap_score_ts", 5: "cap_score_tw"}.get(scorer_used, "?") if dom == 1 else "compact"
     roof["traffic"] = None if (args.cap_keys or args.rope) else recorded_traffic(tkey, f"N{N}_M{M}_d{d}_{cfg.dtype}", units)
     roof["kernel_ms"] = dict(zip(names, [round(x, 5) for x in kms]))
     roof["cycles_averaged"] = kcycles

@@ -85,4 +85,25 @@ __device__ __forceinline__ constexpr bool pair_on_fma(int i)
     return order[i & 7] < kPoly;
 }
 
+// Launch as a programmatic dependent of whatever the stream holds before: the grid may be set up while that still runs.  The
+// kernel starts with pdl_wait(), after which everything the stream has done before is visible (it returns at once after an
+// ordinary predecessor), and pdl_release() lets the next such launch be set up; neither changes the order of the work.
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args)
+{
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = grid;
+    lc.blockDim = block;
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kern, P(args)...);
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 }  // namespace ipotk

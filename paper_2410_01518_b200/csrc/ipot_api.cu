@@ -135,6 +135,18 @@ void free_all(ipot *p)
     }
 }
 
+// Blocks that fit the device at once (the row movers keep eight per SM).
+bool one_wave(const ipot *p, dim3 grid) { return (long long)grid.x * grid.y * grid.z <= 8LL * p->sm_count; }
+
+cudaError_t launch_append(ipot *p, dim3 grid, const uint4 *srcK, const uint4 *srcV, uint4 *potK, uint4 *potV, size_t n_vecs, size_t unit_vecs,
+                          size_t first_vec)
+{
+    if (one_wave(p, grid))
+        return launch_pdl(append_kernel<true>, grid, dim3(kMoveThreads), 0, p->stream, srcK, srcV, potK, potV, n_vecs, unit_vecs, first_vec);
+    append_kernel<false><<<grid, kMoveThreads, 0, p->stream>>>(srcK, srcV, potK, potV, n_vecs, unit_vecs, first_vec);
+    return cudaGetLastError();
+}
+
 // Copies the rows of a deferred append that are still in the caller's buffers into the pot (keys, values or both).
 int materialise(ipot *p, bool keys, bool values)
 {
@@ -145,11 +157,11 @@ int materialise(ipot *p, bool keys, bool values)
     if (pieces < 1) pieces = 1;
     dim3 grid(pieces, p->units, (k && v) ? 2 : 1);
     if (k && v)
-        append_kernel<<<grid, kMoveThreads, 0, p->stream>>>((const uint4 *)k, (const uint4 *)v, (uint4 *)p->K, (uint4 *)p->V, n_vecs,
-                                                           (size_t)p->cfg.pot_size * row_vecs, (size_t)p->pend_first * row_vecs);
+        IPOT_CUDA(launch_append(p, grid, (const uint4 *)k, (const uint4 *)v, (uint4 *)p->K, (uint4 *)p->V, n_vecs,
+                                                           (size_t)p->cfg.pot_size * row_vecs, (size_t)p->pend_first * row_vecs));
     else
-        append_kernel<<<grid, kMoveThreads, 0, p->stream>>>((const uint4 *)(k ? k : v), nullptr, (uint4 *)(k ? p->K : p->V), nullptr, n_vecs,
-                                                           (size_t)p->cfg.pot_size * row_vecs, (size_t)p->pend_first * row_vecs);
+        IPOT_CUDA(launch_append(p, grid, (const uint4 *)(k ? k : v), nullptr, (uint4 *)(k ? p->K : p->V), nullptr, n_vecs,
+                                                           (size_t)p->cfg.pot_size * row_vecs, (size_t)p->pend_first * row_vecs));
     p->launches += 1;
     IPOT_CUDA(cudaGetLastError());
     if (k) p->pend_K = nullptr;
@@ -359,21 +371,11 @@ int check_cycle_args(ipot *p, const void *Q, int cap_rows, const float *aux, boo
     return IPOT_OK;
 }
 
-// The gather of the survivors (and, in rotary mode, the rotated copy of the keys).  Programmatic dependent launch: the grid
-// is set up while the selection still runs and waits inside the kernel.
+// The gather of the survivors (and, in rotary mode, the rotated copy of the keys).
 template <typename Kernel, typename... Rot>
 cudaError_t launch_gather(ipot *p, Kernel kern, const GatherParams &g, const Rot &...rot)
 {
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(p->gather.chunks, 2, p->units);
-    lc.blockDim = dim3(kGatherThreads, 1, 1);
-    lc.stream = p->stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, kern, g, rot...);
+    return launch_pdl(kern, dim3(p->gather.chunks, 2, p->units), dim3(kGatherThreads), 0, p->stream, g, rot...);
 }
 
 template <typename T>
@@ -389,7 +391,7 @@ cudaError_t launch_gather_rope(ipot *p, const GatherParams &g)
 // New key rows (src, unit stride src_unit_vecs) -> pot rows [len, len + n) rotated and, with keys_too, unrotated; if srcV
 // is not NULL the same launch copies the value rows ([units][n rows]) into the pot.
 template <typename T>
-void launch_append_rope_t(ipot *p, const void *src, size_t src_unit_vecs, const void *srcV, int n, bool keys_too)
+cudaError_t launch_append_rope_t(ipot *p, const void *src, size_t src_unit_vecs, const void *srcV, int n, bool keys_too)
 {
     const int row_vecs = p->row_bytes / 16;
     const size_t items = (size_t)n * (row_vecs / 2), unit_vecs = (size_t)p->cfg.pot_size * row_vecs;
@@ -399,12 +401,13 @@ void launch_append_rope_t(ipot *p, const void *src, size_t src_unit_vecs, const 
     auto kern = p->rope == IPOT_ROPE_INTERLEAVED ? append_rope_kernel<T, true> : append_rope_kernel<T, false>;
     kern<<<grid, kMoveThreads, 0, p->stream>>>((const uint4 *)src, src_unit_vecs, (uint4 *)(keys_too ? p->K : nullptr), (uint4 *)p->Krot, (const T *)p->rope_cos,
                                                (const T *)p->rope_sin, n, row_vecs, unit_vecs, p->len, (const uint4 *)srcV, (uint4 *)p->V);
+    return cudaGetLastError();
 }
 
-void launch_append_rope(ipot *p, const void *src, size_t src_unit_vecs, const void *srcV, int n, bool keys_too = true)
+cudaError_t launch_append_rope(ipot *p, const void *src, size_t src_unit_vecs, const void *srcV, int n, bool keys_too = true)
 {
-    if (p->cfg.dtype == IPOT_F32) launch_append_rope_t<float>(p, src, src_unit_vecs, srcV, n, keys_too);
-    else launch_append_rope_t<__nv_bfloat16>(p, src, src_unit_vecs, srcV, n, keys_too);
+    if (p->cfg.dtype == IPOT_F32) return launch_append_rope_t<float>(p, src, src_unit_vecs, srcV, n, keys_too);
+    return launch_append_rope_t<__nv_bfloat16>(p, src, src_unit_vecs, srcV, n, keys_too);
 }
 
 int run_cycle(ipot *p, const void *Q, const void *Kc, int cap_rows, const float *aux)
@@ -422,7 +425,7 @@ int run_cycle(ipot *p, const void *Q, const void *Kc, int cap_rows, const float 
     if (ev) IPOT_CUDA(cudaEventRecord(ev[3], p->stream));
 
     const GatherParams g{(uint4 *)p->K, (uint4 *)p->V, p->idx, p->gather, p->status, keep, N, row_vecs,
-                         (size_t)p->cfg.pot_size * row_vecs, pending_rows(p), p->ts.wait_ns};
+                         (size_t)p->cfg.pot_size * row_vecs, pending_rows(p), p->ts.wait_ns, one_wave(p, dim3(p->gather.chunks, 2, p->units))};
     if (!p->rope) IPOT_CUDA(launch_gather(p, compact_kernel, g));
     else IPOT_CUDA(p->cfg.dtype == IPOT_F32 ? launch_gather_rope<float>(p, g) : launch_gather_rope<__nv_bfloat16>(p, g));
     p->launches += 1;
@@ -451,8 +454,8 @@ int launch_novelty(ipot *p, const void *logits, size_t row_stride, const int32_t
     int *counters = reinterpret_cast<int *>(p->nov_scratch);
     float2 *partial = reinterpret_cast<float2 *>(p->nov_scratch + kNovCounterBytes);
     dim3 grid(segs, (unsigned)rows);
-    (aligned ? novelty_kernel<T, true> : novelty_kernel<T, false>)<<<grid, kNovThreads, 0, p->stream>>>(
-        (const T *)logits, row_stride, vocab, segs, seg_elems, partial, counters, labels, n_tokens, out, out_stride, slot0, p->status);
+    IPOT_CUDA(launch_pdl(aligned ? novelty_kernel<T, true> : novelty_kernel<T, false>, grid, dim3(kNovThreads), 0, p->stream, 
+        (const T *)logits, row_stride, vocab, segs, seg_elems, partial, counters, labels, n_tokens, out, out_stride, slot0, p->status));
     p->launches += 1;
     IPOT_CUDA(cudaGetLastError());
     return IPOT_OK;
@@ -490,9 +493,9 @@ int launch_decode_g(ipot *p, const void *q, float *out, float *lse)
     if (smem > 48 * 1024 && !p->dec_ready[0]) IPOT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     p->dec_ready[0] = true;
     dim3 grid(splits, p->units);
-    kern<<<grid, kDecThreads, smem, p->stream>>>((const T *)score_keys(p), (const T *)p->V, (const T *)q, out, lse, p->dec_partial,
+    IPOT_CUDA(launch_pdl(kern, grid, dim3(kDecThreads), smem, p->stream, (const T *)score_keys(p), (const T *)p->V, (const T *)q, out, lse, p->dec_partial,
                                                  p->dec_counters, N, d, p->row_bytes / 16, (size_t)p->cfg.pot_size * d,
-                                                 (float)(1.4426950408889634 / std::sqrt((double)d)));
+                                                 (float)(1.4426950408889634 / std::sqrt((double)d))));
     p->launches += 1;
     IPOT_CUDA(cudaGetLastError());
     return IPOT_OK;
@@ -510,9 +513,9 @@ int launch_decode_mma(ipot *p, const void *q, float *out, float *lse)
     if (!p->dec_ready[1]) IPOT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     p->dec_ready[1] = true;
     dim3 grid(splits, p->units);
-    kern<<<grid, kMmaWarps * 32, smem, p->stream>>>((const __nv_bfloat16 *)score_keys(p), (const __nv_bfloat16 *)p->V,
+    IPOT_CUDA(launch_pdl(kern, grid, dim3(kMmaWarps * 32), smem, p->stream, (const __nv_bfloat16 *)score_keys(p), (const __nv_bfloat16 *)p->V,
                                                     (const __nv_bfloat16 *)q, out, lse, p->dec_partial, p->dec_counters, N, p->G,
-                                                    (size_t)p->cfg.pot_size * D, (float)(1.4426950408889634 / std::sqrt((double)D)));
+                                                    (size_t)p->cfg.pot_size * D, (float)(1.4426950408889634 / std::sqrt((double)D))));
     p->launches += 1;
     IPOT_CUDA(cudaGetLastError());
     return IPOT_OK;
@@ -715,7 +718,7 @@ int ipot_append_chunk(ipot_t *p, const void *K, const void *V, int n)
         p->pend_V = V;
         p->pend_K = K;
         if (p->rope) {  // the rotated copy is what the scorers read: it is made now
-            launch_append_rope(p, K, n_vecs, nullptr, n, false);
+            IPOT_CUDA(launch_append_rope(p, K, n_vecs, nullptr, n, false));
             p->launches += 1;
             IPOT_CUDA(cudaGetLastError());
         }
@@ -724,10 +727,10 @@ int ipot_append_chunk(ipot_t *p, const void *K, const void *V, int n)
     }
     if (!p->rope) {
         dim3 grid(pieces, p->units, 2);
-        append_kernel<<<grid, kMoveThreads, 0, p->stream>>>((const uint4 *)K, (const uint4 *)V, (uint4 *)p->K, (uint4 *)p->V,
-                                                           n_vecs, (size_t)p->cfg.pot_size * row_vecs, (size_t)p->len * row_vecs);
+        IPOT_CUDA(launch_append(p, grid, (const uint4 *)K, (const uint4 *)V, (uint4 *)p->K, (uint4 *)p->V,
+                                                           n_vecs, (size_t)p->cfg.pot_size * row_vecs, (size_t)p->len * row_vecs));
     } else {
-        launch_append_rope(p, K, n_vecs, V, n);
+        IPOT_CUDA(launch_append_rope(p, K, n_vecs, V, n));
     }
     p->launches += 1;
     IPOT_CUDA(cudaGetLastError());
@@ -746,7 +749,7 @@ int ipot_append_chunk_host(ipot_t *p, const void *K, const void *V, int n)
     IPOT_CUDA(cudaMemcpy2DAsync(dK, dpitch, K, width, width, p->units, cudaMemcpyHostToDevice, p->stream));
     IPOT_CUDA(cudaMemcpy2DAsync(dV, dpitch, V, width, width, p->units, cudaMemcpyHostToDevice, p->stream));
     if (p->rope) {  // the key rows are in place: rotate them into the copy
-        launch_append_rope(p, dK, (size_t)p->cfg.pot_size * (p->row_bytes / 16), nullptr, n);
+        IPOT_CUDA(launch_append_rope(p, dK, (size_t)p->cfg.pot_size * (p->row_bytes / 16), nullptr, n));
         p->launches += 1;
         IPOT_CUDA(cudaGetLastError());
     }

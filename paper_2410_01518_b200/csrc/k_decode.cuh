@@ -146,6 +146,8 @@ __global__ void __launch_bounds__(kDecThreads, G <= 4 ? 2 : 1)  // two blocks pe
 decode_attn_kernel(const T *__restrict__ Kp, const T *__restrict__ Vp, const T *__restrict__ q, float *__restrict__ out,
                    float *__restrict__ lse, float *partial, int *counters, int N, int d, int lpk, size_t unit_elems, float scale_log2e)
 {
+    pdl_wait();
+    pdl_release();
     constexpr int VE = RopeVec<T>::kElems;
     constexpr int KT = kDecKT;
     extern __shared__ __align__(16) uint8_t dec_raw[];
@@ -344,6 +346,8 @@ decode_attn_mma_kernel(const __nv_bfloat16 *__restrict__ Kp, const __nv_bfloat16
                        float *__restrict__ out, float *__restrict__ lse, float *partial, int *counters, int N, int G,
                        size_t unit_elems, float scale_log2e)
 {
+    pdl_wait();
+    pdl_release();
     constexpr int VPR = D / 8;          // 16-byte vectors per row
     constexpr int NT = D / 8;           // output column tiles of 8
     constexpr int STAGE_VECS = 16 * VPR;  // vectors of keys (and of values) per stage

@@ -27,10 +27,17 @@ __device__ __forceinline__ void append_body(const uint4 *__restrict__ src, uint4
 
 // grid (pieces, units, 1 or 2): tensor z of unit y (z = 0 alone: the first pair of pointers); src is [units][n_vecs],
 // dst is the pot.
+// kEarly: set up beside the kernel before it and lets the next one be.  For copies of at most one wave of blocks: there it
+// saves most of two launch gaps, while on large ones the wait in every block costs 5 % of the copy.
+template <bool kEarly>
 __global__ void __launch_bounds__(kMoveThreads)
 append_kernel(const uint4 *__restrict__ srcK, const uint4 *__restrict__ srcV, uint4 *__restrict__ potK,
               uint4 *__restrict__ potV, size_t n_vecs, size_t unit_vecs, size_t first_vec)
 {
+    if (kEarly) {
+        pdl_wait();
+        pdl_release();
+    }
     const uint4 *src = (blockIdx.z ? srcV : srcK) + (size_t)blockIdx.y * n_vecs;
     uint4 *dst = (blockIdx.z ? potV : potK) + (size_t)blockIdx.y * unit_vecs + first_vec;
     append_body(src, dst, n_vecs, blockIdx.x, gridDim.x);
@@ -84,6 +91,7 @@ struct GatherParams {
     size_t unit_vecs;
     PendingRows pend;
     unsigned long long wait_ns;
+    bool release;            // one wave of blocks: the next kernel may be set up
 };
 
 __device__ __forceinline__ void gather_cp_async16(uint32_t dst, const void *src)
@@ -121,7 +129,8 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
     __syncthreads();
     // launched as a programmatic dependent of the selection: the blocks may be resident before it has ended and
     // wait here for its index lists (returns at once after an ordinary launch)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
+    if (p.release) pdl_release();
     const int chunk = chunk_sm, r0 = chunk * rows, n = min(rows, p.keep - r0);
     const uint32_t sbuf = (uint32_t)__cvta_generic_to_shared(buf);
     const int nvec = n * p.row_vecs;

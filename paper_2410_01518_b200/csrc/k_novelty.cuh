@@ -122,6 +122,8 @@ novelty_kernel(const T *__restrict__ logits, size_t row_stride, int V, int segs,
                const int32_t *__restrict__ labels, int n_tokens, float *__restrict__ out, size_t out_stride, int slot0,
                int *status)
 {
+    pdl_wait();
+    pdl_release();
     constexpr int VE = 16 / (int)sizeof(T);
     const int seg = blockIdx.x;
     const size_t row = blockIdx.y;

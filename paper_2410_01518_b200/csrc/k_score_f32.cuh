@@ -45,6 +45,8 @@ f32_tile_kernel(const __grid_constant__ F32Params p)
     __shared__ __align__(16) float qs[2][RT * kF32Stride];
     __shared__ __align__(16) float ks[2][KT * kF32Stride];
     __shared__ int is_last;
+    pdl_wait();
+    pdl_release();
     const int g = blockIdx.z, unit = p.unit0 + g, i0 = blockIdx.y * RT, j0 = blockIdx.x * KT;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const float *Qu = p.Q + (size_t)unit * p.M * p.d, *Ku = p.K + (size_t)unit * p.k_unit_stride;
@@ -62,7 +64,6 @@ f32_tile_kernel(const __grid_constant__ F32Params p)
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    asm volatile("griddepcontrol.launch_dependents;");   // the next kernel may be made resident; it waits for this grid's end
     float2 acc[RA][KB];
 #pragma unroll
     for (int a = 0; a < RA; ++a)
@@ -160,8 +161,8 @@ __global__ void __launch_bounds__(kF32Threads)
 f32_fold_kernel(const __grid_constant__ F32Params p)
 {
     const int g = blockIdx.y, unit = p.unit0 + g, row = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
+    pdl_wait();
+    pdl_release();
     if (row >= p.M) return;
     float m = -INFINITY, l = 0.f;
     for (int t0 = 0; t0 < p.key_tiles; t0 += 256) {
@@ -197,7 +198,8 @@ f32_columns_kernel(const __grid_constant__ F32Params p, int kt)
     __shared__ float red[4][64];
     const int g = blockIdx.y, unit = p.unit0 + g, j = threadIdx.x & 63, part = threadIdx.x >> 6, key = blockIdx.x * 64 + j;
     const int tiles = 64 / kt, tile0 = blockIdx.x * tiles;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
+    pdl_release();
     float u[4] = {0.f, 0.f, 0.f, 0.f};
     for (int i0 = 0; i0 < p.M; i0 += 256) {
         const int n = min(256, p.M - i0);
@@ -272,24 +274,13 @@ inline cudaError_t f32_launch(const F32Plan &plan, const float *Q, const float *
         p.unit0 = u0;
         p.part = (float2 *)(plan.scratch + (size_t)n * M * p.e_stride * 4);
         const dim3 grid(p.key_tiles, (M + t - 1) / t, n);
-        (t == 64 ? f32_tile_kernel<64, 64> : t == 32 ? f32_tile_kernel<32, 32> : f32_tile_kernel<16, 16>)<<<grid, kF32Threads, 0, stream>>>(p);
-        cudaLaunchConfig_t lc = {};
-        lc.stream = stream;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[0].val.programmaticStreamSerializationAllowed = 1;
-        lc.attrs = at;
-        lc.numAttrs = 1;
-        cudaError_t err = cudaGetLastError();
+        auto tile = t == 64 ? f32_tile_kernel<64, 64> : t == 32 ? f32_tile_kernel<32, 32> : f32_tile_kernel<16, 16>;
+        cudaError_t err = launch_pdl(tile, grid, dim3(kF32Threads), 0, stream, p);
         if (!p.fold_here && err == cudaSuccess) {
-            lc.gridDim = dim3((M + 3) / 4, n);
-            lc.blockDim = dim3(kF32Threads);
-            err = cudaLaunchKernelEx(&lc, f32_fold_kernel, p);
+            err = launch_pdl(f32_fold_kernel, dim3((M + 3) / 4, n), dim3(kF32Threads), 0, stream, p);
             *launches += 1;
         }
-        lc.gridDim = dim3((N + 63) / 64, n);
-        lc.blockDim = dim3(kF32ColThreads);
-        if (err == cudaSuccess) err = cudaLaunchKernelEx(&lc, f32_columns_kernel, p, t);
+        if (err == cudaSuccess) err = launch_pdl(f32_columns_kernel, dim3((N + 63) / 64, n), dim3(kF32ColThreads), 0, stream, p, t);
         if (err != cudaSuccess) return err;
         *launches += 2;
     }

@@ -187,6 +187,7 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
     extern __shared__ __align__(1024) uint8_t tw_smem[];
     const uint32_t base = smem_u32(tw_smem);
     if ((int)blockIdx.x >= prm.ctas) {
+        pdl_wait();
         nuc_rank_extra_block(prm.nuc, prm.N, (int)blockIdx.x - prm.ctas, reinterpret_cast<SelShared *>(tw_smem));
         return;
     }
@@ -234,6 +235,8 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    pdl_wait();   // the keys and queries are complete; everything above ran beside the kernel that brings them
+    pdl_release();
     const TsWait wait{&abort_flag, prm.status, prm.wait_ns, warp == 0 || warp == 3 ? 20u : 0u};
     const uint32_t tile_bytes = (uint32_t)prm.dblk * kTwBlkBytes;
     const uint32_t q_base = base + kTwOffTiles, k_base = q_base + (uint32_t)prm.qslots * tile_bytes;
@@ -765,8 +768,7 @@ inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const 
     if (nuc.batch > 0) nuc.ctas = nuc.batch < plan.sm_count - prm.ctas ? nuc.batch : plan.sm_count - prm.ctas;
     prm.nuc = nuc;
     const size_t smem = kTwOffTiles + (size_t)(prm.qslots + prm.kslots) * tile_bytes;
-    cap_score_tw_kernel<<<prm.ctas + nuc.ctas, kTwThreads, smem, stream>>>(mapQ, mapK, mapKnew, prm);
-    return cudaGetLastError() == cudaSuccess ? IPOT_OK : IPOT_E_CUDA;
+    return launch_pdl(cap_score_tw_kernel, dim3(prm.ctas + nuc.ctas), dim3(kTwThreads), smem, stream, mapQ, mapK, mapKnew, prm) == cudaSuccess ? IPOT_OK : IPOT_E_CUDA;
 }
 
 }  // namespace ipotk

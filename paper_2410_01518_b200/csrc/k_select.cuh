@@ -304,8 +304,8 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
     int *below = plan.ints + (size_t)unit * plan.per_unit();   // for the gather that follows
     // launched as a programmatic dependent of the scorer: its scores and the ranking's mask are complete after this.  Then
     // the compaction may be made resident; it waits for this grid's end before it reads an index.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
+    pdl_wait();
+    pdl_release();
     uint32_t key[kKpt];
     // a reserved slot outranks every score: finite scores map below 0xFF800000
     constexpr int kPiece = kKpt > 16 ? 8 : 16;   // slots loaded at a time (what 64 registers a thread allow)
@@ -390,16 +390,8 @@ inline cudaError_t launch_select(int blocks, cudaStream_t st, const float *score
                                  int32_t *idx, float *summed, int N, int keep, int Hkv, int batch, int *status, const GatherPlan &plan)
 {
     auto kern = N <= 4096 ? select_kernel<256, 16> : N <= 8192 ? select_kernel<512, 16> : N <= 16384 ? select_kernel<1024, 16> : select_kernel<1024, 32>;
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(blocks, 1, 1);
-    lc.blockDim = dim3(N <= 4096 ? 256 : N <= 8192 ? 512 : 1024, 1, 1);
-    lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, kern, scores, parts, part_stride, mask, idx, summed, N, keep, Hkv, batch, status, plan);
+    return launch_pdl(kern, dim3(blocks), dim3(N <= 4096 ? 256 : N <= 8192 ? 512 : 1024), 0, st, scores, parts, part_stride, mask, idx, summed, N, keep, Hkv, batch,
+                      status, plan);
 }
 
 // summed[i] = parts[0][i] + parts[1][i] + ... in index order (the order select_kernel uses).
