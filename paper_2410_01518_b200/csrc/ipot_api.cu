@@ -342,7 +342,7 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
         p->launches += n_launch;
     } else if (scorer == IPOT_SCORER_TENSOR_ITEMS) {
         rc = tw_launch(p->tw, p->tc, p->cfg, Q, score_keys(p), cap_stats, p->scores, N, M, p->units, p->status, p->stream, p->ts.wait_ns,
-                       p->ts.withhold_rank, keys_in_chunk ? p->pend_K : nullptr, keys_in_chunk ? p->pend_first : 0, in_scorer ? nuc_blocks : 0, nuc);
+                       p->ts.withhold_rank, keys_in_chunk ? p->pend_K : nullptr, keys_in_chunk ? p->pend_first : 0, side_nuc || in_scorer ? nuc_blocks : 0, nuc);
         p->launches += 1;
     } else if (scorer == IPOT_SCORER_TENSOR_SWEEPS) {
         rc = ts_launch(p->tc, p->ts_occ, p->ts, p->cfg, Q, score_keys(p), cap_stats, p->scores, N, M, p->units, p->status, p->stream,

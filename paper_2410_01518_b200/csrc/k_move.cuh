@@ -73,13 +73,15 @@ inline int gather_rows(int row_vecs) { return kGatherBytes / 16 / row_vecs; }
 inline int gather_chunks(int keep, int row_vecs) { return (keep + gather_rows(row_vecs) - 1) / gather_rows(row_vecs); }
 
 // What the selection leaves for the gather, ints of one unit: [0, chunks] the number of survivors in slots below c * rows
-// (which survivors come from a chunk's own slots).  Then per tensor the gather's own a ticket, a count of finished blocks and a
-// flag for every chunk, raised when it has been read; zero between launches.
+// (which survivors come from a chunk's own slots).  Then per tensor the gather's own: a 64-bit ticket that counts on from launch
+// to launch (a launch takes exactly `chunks` of them, so ticket / chunks numbers the launches) and, for every chunk, the
+// number of the last launch in which it has been read.  Nothing is put back.
 struct GatherPlan {
     int *ints;
     int rows, chunks;
-    __host__ __device__ int per_tensor() const { return chunks + 2; }
-    __host__ __device__ int per_unit() const { return chunks + 1 + 2 * per_tensor(); }
+    __host__ __device__ int below_ints() const { return (chunks + 2) & ~1; }
+    __host__ __device__ int per_tensor() const { return 2 + ((chunks + 1) & ~1); }
+    __host__ __device__ int per_unit() const { return below_ints() + 2 * per_tensor(); }
 };
 
 struct GatherParams {
@@ -110,7 +112,7 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
 {
     __shared__ __align__(128) uint4 buf[kGatherBytes / 16];
     __shared__ int src_sm[kGatherBytes / 64];   // (rows have at least 64 bytes)
-    __shared__ int chunk_sm, gave_up;
+    __shared__ int chunk_sm, launch_sm, gave_up;
     // Block order: the units from the last one down, K then V of a unit next to each other.  The scorer of the next
     // cycle starts at unit 0 and finds the rows written last still in L2.
     const unsigned unit = gridDim.z - 1 - blockIdx.z, tensor = blockIdx.y;
@@ -118,20 +120,22 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
     const int32_t *ix = p.idx + (size_t)unit * p.keep;
     const int rows = p.plan.rows, chunks = p.plan.chunks;
     const int *below = p.plan.ints + (size_t)unit * p.plan.per_unit();
-    int *sync = p.plan.ints + (size_t)unit * p.plan.per_unit() + chunks + 1 + tensor * p.plan.per_tensor();
+    int *sync = p.plan.ints + (size_t)unit * p.plan.per_unit() + p.plan.below_ints() + tensor * p.plan.per_tensor();
     const uint4 *alt = tensor ? p.pend.V : p.pend.K;
     const int alt_first = alt ? p.pend.first : 0x7fffffff;
     if (alt) alt += (size_t)unit * p.pend.unit_vecs;
     if (threadIdx.x == 0) {
         gave_up = 0;
-        chunk_sm = atomicAdd(sync, 1);
+        const unsigned long long ticket = atomicAdd(reinterpret_cast<unsigned long long *>(sync), 1ull), launch = ticket / (unsigned)chunks;
+        chunk_sm = (int)(ticket - launch * (unsigned)chunks);
+        launch_sm = (int)(uint32_t)(launch + 1);
     }
     __syncthreads();
     // launched as a programmatic dependent of the selection: the blocks may be resident before it has ended and
     // wait here for its index lists (returns at once after an ordinary launch)
     pdl_wait();
     if (p.release) pdl_release();
-    const int chunk = chunk_sm, r0 = chunk * rows, n = min(rows, p.keep - r0);
+    const int launch = launch_sm, chunk = chunk_sm, r0 = chunk * rows, n = min(rows, p.keep - r0);
     const uint32_t sbuf = (uint32_t)__cvta_generic_to_shared(buf);
     const int nvec = n * p.row_vecs;
     int q0 = 0, q1 = 0;   // the survivors whose sources lie in this chunk's slots
@@ -169,13 +173,15 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
         const int c1 = q1 > q0 ? min(chunk - 1, (q1 - 1) / rows) : -1;
         const unsigned long long t0 = global_timer_ns();
         for (int c = max(0, q0 / rows); c <= c1; ++c) {
-            int up = 0;
+            bool up = false;
             for (uint32_t tries = 1; !up; ++tries) {
-                asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(up) : "l"(sync + 2 + c) : "memory");
+                int seen;
+                asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(sync + 2 + c) : "memory");
+                up = seen == launch;
                 if (!up && (tries & 255u) == 0 && global_timer_ns() - t0 > p.wait_ns) {
                     set_status(p.status, kStatusTimeout);
                     gave_up = 1;
-                    up = 1;
+                    up = true;
                 }
             }
         }
@@ -184,7 +190,7 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk copy below reads what the threads have brought in
     __syncthreads();
     if (threadIdx.x == 0) {
-        asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(sync + 2 + chunk), "r"(1) : "memory");
+        asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(sync + 2 + chunk), "r"(launch) : "memory");
         if (!gave_up) {   // (a wait that ran out: the rows stay as they are)
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
                          ::"l"(base + (size_t)r0 * p.row_vecs), "r"(sbuf), "r"((uint32_t)nvec * 16u) : "memory");
@@ -192,11 +198,7 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
         }
     }
     if (tensor == 0) rotate(buf, (int)unit, r0, n, p.row_vecs);
-    if (threadIdx.x == 0) {
-        if (atomicAdd(sync + 1, 1) == chunks - 1)   // every block has passed its waits: ready for the next launch
-            for (int i = 0; i < chunks + 2; ++i) sync[i] = 0;
-        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the block's memory is free again
-    }
+    if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the block's memory is free again
 }
 
 __global__ void __launch_bounds__(kGatherThreads) compact_kernel(const __grid_constant__ GatherParams p)
