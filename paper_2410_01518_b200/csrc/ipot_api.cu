@@ -375,7 +375,7 @@ int check_cycle_args(ipot *p, const void *Q, int cap_rows, const float *aux, boo
 template <typename Kernel, typename... Rot>
 cudaError_t launch_gather(ipot *p, Kernel kern, const GatherParams &g, const Rot &...rot)
 {
-    return launch_pdl(kern, dim3(p->gather.chunks, 2, p->units), dim3(kGatherThreads), 0, p->stream, g, rot...);
+    return launch_pdl(kern, dim3(p->gather.chunks * 2 * g.group, (g.units + g.group - 1) / g.group), dim3(kGatherThreads), 0, p->stream, g, rot...);
 }
 
 template <typename T>
@@ -424,8 +424,15 @@ int run_cycle(ipot *p, const void *Q, const void *Kc, int cap_rows, const float 
     IPOT_CUDA(cudaGetLastError());
     if (ev) IPOT_CUDA(cudaEventRecord(ev[3], p->stream));
 
-    const GatherParams g{(uint4 *)p->K, (uint4 *)p->V, p->idx, p->gather, p->status, keep, N, row_vecs,
-                         (size_t)p->cfg.pot_size * row_vecs, pending_rows(p), p->ts.wait_ns, one_wave(p, dim3(p->gather.chunks, 2, p->units))};
+    // Where nothing is read from the pot no block waits for another, and unit after unit finds the last units' keys still in
+    // L2 from the scorer (256 units, 4096 -> 2048 rows: cycle 186 us, chunk after chunk over all units 188).  Otherwise
+    // chunk after chunk: the chunks a block waits for have then been read long ago (all rows in the pot: 92 us instead of
+    // 104; groups of 64 units 94, of 16 units 100).
+    const PendingRows pend = pending_rows(p);
+    const bool outside = pend.K && pend.V && pend.first == 0;
+    const int group = outside ? 1 : (int)std::min<long long>(p->units, (1LL << 30) / p->gather.chunks);
+    const GatherParams g{(uint4 *)p->K, (uint4 *)p->V, p->idx, p->gather, p->status, keep, N, row_vecs, p->units, group,
+                         (size_t)p->cfg.pot_size * row_vecs, pend, p->ts.wait_ns, one_wave(p, dim3(p->gather.chunks, 2, p->units))};
     if (!p->rope) IPOT_CUDA(launch_gather(p, compact_kernel, g));
     else IPOT_CUDA(p->cfg.dtype == IPOT_F32 ? launch_gather_rope<float>(p, g) : launch_gather_rope<__nv_bfloat16>(p, g));
     p->launches += 1;

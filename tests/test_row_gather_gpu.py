@@ -31,3 +31,20 @@ def test_gather_chunk_edges(case, rope):
     gpu = gpu_cycle(cfg, t, ipot.IPOT_SCORER_AUTO, n=n, deferred_from=first)
     same, cnt = compare_cycle(cfg, t, gpu, n=n)
     assert cnt == cfg.units and same >= cnt - 1
+
+
+@pytest.mark.parametrize("rope", [False, True])
+@pytest.mark.parametrize("in_place,first", [(0, None), (63, None), (64, None), (65, None), (192, 192), (192, 191), (192, 100), (192, 0), (256, None)])
+def test_gather_rows_in_place(in_place, first, rope):
+    """The most novel rows are the first ones, so they keep their slots: chunks of 64 rows that stay, that end in a row that
+    moves, that reach into a deferred chunk (whose rows have to be copied all the same), and a gather that moves nothing."""
+    n, keep = 600, 256
+    cfg = inputs.small_config(cfg_id=880, pot_size=n, keep=keep, nuc_slots=keep, cap_rows=4, Hq=6, Hkv=3, d=128, dtype="bf16", batch=2)
+    t = inputs.make_cycle(cfg)
+    t["aux"][:, :in_place] += 2   # (the others are in [0, 1))
+    t["aux"][:, in_place:in_place + 1] = -1
+    if rope:
+        t["rope"] = (*inputs.make_rope_table(cfg.pot_size, 128, "bf16"), False)
+    gpu = gpu_cycle(cfg, t, ipot.IPOT_SCORER_AUTO, n=n, deferred_from=first)
+    same, cnt = compare_cycle(cfg, t, gpu, n=n)
+    assert same == cnt == cfg.units
