@@ -22,7 +22,7 @@
 // Four warps per scheduler work on four different buffers, each at its own place of the load - exponential - sum
 // sequence, so that the two pipes stay busy (16 warps that share a buffer idle together at its ends).  A unit's keys
 // are fetched once per sweep for all of its row blocks.  Measured alone: 64 units x 4096 keys x 256 channels, M = 64:
-// 59 us (warp-level tensor cores: 221); 64 x 16384 x 128, M = 512: 348 us (clusters: 377, one sweep: 547).
+// 51 us (warp-level tensor cores: 221); 64 x 16384 x 128, M = 512: 348 us (clusters: 377, one sweep: 547).
 //
 // Warp roles (640 threads): 0 issues TMA loads, 1 issues MMAs and owns tensor memory, 2 merges and publishes row
 // statistics, 3 draws items and fetches the denominators of S2 items, 4-19 epilogue: four groups of four warps (one per
@@ -71,6 +71,7 @@ struct TwParams {
     int N, M, mt, units, tiles;   // tiles: 128-key tiles of a unit
     int nt, J, jobs;              // tiles per job, jobs per unit, jobs in all
     int ksteps, dblk;             // 16-channel steps and 64-channel blocks of a row
+    int qrows;                    // rows of a query tile in shared memory and columns of an S2 product: 64 if M <= 64, else 128
     int qslots, kslots;
     int new_tile0;            // tiles from this one on are read through the second key map; INT_MAX if all keys are in the pot
     float scale_log2e;
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(kTwThreads, 1)
 cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                     const __grid_constant__ CUtensorMap mapKnew, const __grid_constant__ TwParams prm)
 {
-    constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);   // 128 x 128, bf16 -> fp32
+    constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);   // 128 rows, bf16 -> fp32; columns: << 17, in eights
     extern __shared__ __align__(1024) uint8_t tw_smem[];
     const uint32_t base = smem_u32(tw_smem);
     if ((int)blockIdx.x >= prm.ctas) {
@@ -239,7 +240,9 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
     pdl_release();
     const TsWait wait{&abort_flag, prm.status, prm.wait_ns, warp == 0 || warp == 3 ? 20u : 0u};
     const uint32_t tile_bytes = (uint32_t)prm.dblk * kTwBlkBytes;
-    const uint32_t q_base = base + kTwOffTiles, k_base = q_base + (uint32_t)prm.qslots * tile_bytes;
+    // M <= 64: an S1 product still has 128 rows, of which the lower half multiplies whatever lies behind the tile and is never read
+    const uint32_t q_blk = (uint32_t)prm.qrows * 128u, q_bytes = (uint32_t)prm.dblk * q_blk;
+    const uint32_t q_base = base + kTwOffTiles, k_base = q_base + (uint32_t)prm.qslots * q_bytes;
 
     // the item list as a consumer warp sees it: item n of this CTA, negative at the end
     auto take_item = [&](uint32_t n, bool &ok) {
@@ -291,9 +294,9 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                     ok = wait(bar(kTwQEmpty + s), (use & 1) ^ 1);
                     if (!ok) return;
                     ++qn;
-                    mbar_expect_tx(bar(kTwQFull + s), tile_bytes);
+                    mbar_expect_tx(bar(kTwQFull + s), q_bytes);
                     for (int blk = 0; blk < prm.dblk; ++blk)
-                        tma_load_3d(q_base + s * tile_bytes + blk * kTwBlkBytes, &mapQ, 64 * blk, b * kTwTile, it.unit, bar(kTwQFull + s));
+                        tma_load_3d(q_base + s * q_bytes + blk * q_blk, &mapQ, 64 * blk, b * kTwTile, it.unit, bar(kTwQFull + s));
                 };
                 // with two query slots the query tile first (its slot is free); with one it waits for the previous item's
                 // last MMA, and the key slots that are free by then are filled meanwhile
@@ -319,7 +322,7 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         uint32_t qs = 0, qph = 0, ks = 0, kph = 0, buf = 0, bph = 1;
         bool ok = true, any = false;
         const uint64_t q_desc = smem_desc_sw128(q_base), k_desc = smem_desc_sw128(k_base);
-        const uint32_t tile16 = tile_bytes >> 4;
+        const uint32_t tile16 = tile_bytes >> 4, q_tile16 = q_bytes >> 4;
         for (uint32_t n = 0; ok; ++n) {
             int pos = take_item(n, ok);
             ok = __all_sync(0xffffffffu, ok);
@@ -343,15 +346,17 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                         if (leader) mbar_arrive(bar(kTwSFull + buf));
                     } else {
                         tc_fence_after();
-                        const uint64_t dq = q_desc + qs * tile16, dk = k_desc + ks1 * tile16;
+                        const uint64_t dq = q_desc + qs * q_tile16, dk = k_desc + ks1 * tile16;
                         uint64_t da = it.sweep ? dk : dq, db = it.sweep ? dq : dk;
+                        const uint32_t step_a = it.sweep ? kTwBlkBytes >> 4 : q_blk >> 4, step_b = it.sweep ? q_blk >> 4 : kTwBlkBytes >> 4;
+                        const uint32_t idesc = kIdesc | (it.sweep ? (uint32_t)prm.qrows : 128u) >> 3 << 17;
                         const uint32_t d = tmem + buf * 128;
                         if (leader) {
-                            for (int k = 0; k < prm.ksteps; k += 4, da += kTwBlkBytes >> 4, db += kTwBlkBytes >> 4) {
-                                tc_mma_bf16(d, da, db, kIdesc, k ? 1u : 0u);
+                            for (int k = 0; k < prm.ksteps; k += 4, da += step_a, db += step_b) {
+                                tc_mma_bf16(d, da, db, idesc, k ? 1u : 0u);
 #pragma unroll
                                 for (int i = 1; i < 4; ++i)
-                                    if (k + i < prm.ksteps) tc_mma_bf16(d, da + 2 * i, db + 2 * i, kIdesc, 1u);
+                                    if (k + i < prm.ksteps) tc_mma_bf16(d, da + 2 * i, db + 2 * i, idesc, 1u);
                             }
                             tc_commit(bar(kTwSFull + buf));
                             if (b == mt - 1) tc_commit(bar(kTwKEmpty + ks1));   // the slot may be refilled once these MMAs have read it
@@ -554,7 +559,7 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                     for (int t = first; t < it.w; t += kTwGroups) {
                         ok = wwait(bar(kTwSFull + g), ((task0 + (uint32_t)t) >> 2) & 1);
                         if (!ok) break;
-                        if (t >= it.n) {
+                        if (t >= it.n || q * 32 >= prm.qrows) {   // (an empty task; rows that no query has)
                             release();
                             continue;
                         }
@@ -618,6 +623,7 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             } else {
                 const uint32_t par = ns & 1;
                 ok = wwait(bar(kTwLFull + par), (ns >> 1) & 1);
+                const int cols = prm.qrows;
                 float u = 0.f;   // with several row blocks a group has at most one tile of an item, and u adds over them
                 for (int b = 0; b < mt && ok; ++b, task0 += (uint32_t)it.w) {
                     const float *nl = ltab + (par * kTwMaxBlocks + b) * kTwTile;
@@ -635,7 +641,7 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                         tmem_ld16(tb, r0);
                         tmem_wait_ld16(r0);
 #pragma unroll 1
-                        for (int i = 0; i < 6; i += 2) {
+                        for (int i = 0; i < cols / 16 - 2; i += 2) {
                             tmem_ld16(tb + 16 * (i + 1), r1);
                             sweep2_acc<kTwPoly, 16>(r0, c, nl + 16 * i, sa, pa);
                             tmem_wait_ld16(r1);
@@ -643,11 +649,11 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                             sweep2_acc<kTwPoly, 16>(r1, c, nl + 16 * i + 16, sa, pa);
                             tmem_wait_ld16(r0);
                         }
-                        tmem_ld16(tb + 112, r1);
+                        tmem_ld16(tb + cols - 16, r1);
                         tmem_wait_ld16(r1);
                         release();
-                        sweep2_acc<kTwPoly, 16>(r0, c, nl + 96, sa, pa);
-                        sweep2_acc<kTwPoly, 16>(r1, c, nl + 112, sa, pa);
+                        sweep2_acc<kTwPoly, 16>(r0, c, nl + cols - 32, sa, pa);
+                        sweep2_acc<kTwPoly, 16>(r1, c, nl + cols - 16, sa, pa);
                         const float2 p2 = fadd2_ftz(pa[0], pa[1]);
                         float sum = ((sa[0] + sa[1]) + (sa[2] + sa[3])) + (p2.x + p2.y);
                         if (mt > 1) sum = u += sum;
@@ -721,7 +727,8 @@ inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const 
 {
     if (!tw_applicable(plan, N, M) || (Knew && (new_first % kTwTile != 0 || new_first >= N))) return IPOT_E_INVALID;
     CUtensorMap mapQ, mapK, mapKnew;
-    if (tc_encode_rows(enc, &mapQ, Q, cfg.d, M, units, (size_t)M, kTwTile) != IPOT_OK) return IPOT_E_CUDA;
+    const int qrows = M <= kTwTile / 2 ? kTwTile / 2 : kTwTile;
+    if (tc_encode_rows(enc, &mapQ, Q, cfg.d, M, units, (size_t)M, qrows) != IPOT_OK) return IPOT_E_CUDA;
     if (Knew && new_first == 0) {  // every key is in the chunk
         if (tc_encode_rows(enc, &mapK, Knew, cfg.d, N, units, (size_t)N, kTwTile) != IPOT_OK) return IPOT_E_CUDA;
         Knew = nullptr;
@@ -736,9 +743,14 @@ inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const 
     prm.dblk = (cfg.d + 63) / 64;
     prm.ksteps = (cfg.d + 15) / 16;
     const uint32_t tile_bytes = (uint32_t)prm.dblk * kTwBlkBytes;
-    const int slots = (int)((kTwSmemMax - kTwOffTiles) / tile_bytes);
-    prm.qslots = slots >= 5 ? 2 : 1;
-    prm.kslots = slots - prm.qslots < kTwMaxK ? slots - prm.qslots : kTwMaxK;
+    prm.qrows = qrows;
+    const uint32_t q_bytes = tile_bytes * (uint32_t)qrows / kTwTile, room = kTwSmemMax - kTwOffTiles;
+    // Up to 64 query rows take half a tile: rows of 256 channels then have room for a second one, so that an item's queries no
+    // longer wait for the item before it, and half of the exponentials are not computed (64 units x 4096 keys x 256 channels,
+    // M = 64: 55.3 -> 51.4 us; 256 x 2048 x 96, M = 64: 48.3 -> 45.9).
+    prm.qslots = (room - 2 * q_bytes) / tile_bytes >= (qrows < kTwTile ? 2 : 3) ? 2 : 1;
+    const int slots = (int)((room - (uint32_t)prm.qslots * q_bytes) / tile_bytes);
+    prm.kslots = slots < kTwMaxK ? slots : kTwMaxK;
     const int ctas = plan.sm_count - spare_sms > 0 ? plan.sm_count - spare_sms : 1;   // spare_sms: left to the ranking, as in tc_launch
     // Tiles per job: few, so that the items spread evenly over the CTAs, but not so few that the start of an item (query
     // tile, hand-over of the statistics: about half a tile's time) weighs.  With several row blocks a job's key tiles stay
@@ -767,7 +779,7 @@ inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const 
     prm.ctas = 2 * prm.jobs < ctas ? 2 * prm.jobs : ctas;
     if (nuc.batch > 0) nuc.ctas = nuc.batch < plan.sm_count - prm.ctas ? nuc.batch : plan.sm_count - prm.ctas;
     prm.nuc = nuc;
-    const size_t smem = kTwOffTiles + (size_t)(prm.qslots + prm.kslots) * tile_bytes;
+    const size_t smem = kTwOffTiles + (size_t)prm.qslots * q_bytes + (size_t)prm.kslots * tile_bytes;
     return launch_pdl(cap_score_tw_kernel, dim3(prm.ctas + nuc.ctas), dim3(kTwThreads), smem, stream, mapQ, mapK, mapKnew, prm) == cudaSuccess ? IPOT_OK : IPOT_E_CUDA;
 }
 

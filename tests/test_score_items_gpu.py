@@ -72,3 +72,15 @@ def test_items_wait_that_runs_out_ends_the_launch_and_the_pot_recovers():
         assert (ipot.device_array(sp, (cfg.units, nb), "f32").cpu().numpy() == want).all()
     finally:
         ipot.ipot_destroy(h)
+
+
+@pytest.mark.parametrize("d", [72, 256])
+@pytest.mark.parametrize("M", [63, 64, 65])
+def test_items_query_tile_heights(M, d):
+    """Up to 64 query rows are fetched as half a tile and multiplied as 64 columns, more as whole ones; the CaP's own keys join
+    the denominators of the rows there are."""
+    cfg = inputs.small_config(cfg_id=940 + M - 63, pot_size=1300, keep=500, nuc_slots=100, cap_rows=M, Hq=4, Hkv=4, d=d, dtype="bf16", layers=5, batch=2)
+    t = inputs.make_cycle(cfg)
+    t["K_cap"] = inputs.make_kcap(cfg, 0)
+    same, cnt = compare_cycle(cfg, t, gpu_cycle(cfg, t, ITEMS, n=1290), n=1290)
+    assert same >= cnt - 1
