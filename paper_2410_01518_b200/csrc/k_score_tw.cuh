@@ -63,10 +63,10 @@ constexpr uint32_t kTwSmemMax = 227 * 1024;
 struct TwParams {
     float *scores;            // [units][N]
     const float2 *cap_stats;  // NULL, or [units][M] (max, sum) over the CaP's own keys that join every row's denominator
-    float2 *part;             // [units][J][mt * 128]: the jobs' (ref, sum) pairs
+    float *sums, *refs;       // [units][J][mt * 128]: the jobs' (ref, sum) pairs
     float *nl;                // [units][mt * 128]: -log2 of the denominators
     int *sync;                // next S1 job, next S2 job, CTAs that have left, then [units] row blocks whose denominators are known,
-                              // [units * mt] jobs that have reported; zero between launches
+                              // [units * mt] jobs that have reported (65536 added for one with a reference other than 0); zero between launches
     int *status;
     int N, M, mt, units, tiles;   // tiles: 128-key tiles of a unit
     int nt, J, jobs;              // tiles per job, jobs per unit, jobs in all
@@ -400,101 +400,118 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 const uint32_t par = nb & 1;
                 ok = __all_sync(0xffffffffu, wait(bar(kTwRFull + par), (nb >> 1) & 1));
                 if (!ok) break;
-                float m[4], l[4];
+                // A lane has rows 4 * lane ... + 3.  As long as every reference is 0 the sums add up as they are: this warp gets
+                // few issue slots beside the epilogue, and a unit whose denominators are late holds up everybody's S2 items.
+                const float4 *in = reinterpret_cast<const float4 *>(rows + par * kTwGroups * kTwTile) + 2 * lane;
+                float m[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
+                bool plain = true;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    m[i] = 0.f;
-                    l[i] = 0.f;
-#pragma unroll
-                    for (int g = 0; g < kTwGroups; ++g) {
-                        const float2 s = rows[(par * kTwGroups + g) * kTwTile + 32 * i + lane];
-                        tw_merge(m[i], l[i], s.x, s.y);
-                    }
-                    tw_normalise(m[i], l[i]);
+                for (int g = 0; g < kTwGroups; ++g) {
+                    const float4 x = in[g * (kTwTile / 2)], y = in[g * (kTwTile / 2) + 1];
+                    plain = plain && x.x == 0.f && x.z == 0.f && y.x == 0.f && y.z == 0.f;
+                    l[0] += x.y;
+                    l[1] += x.w;
+                    l[2] += y.y;
+                    l[3] += y.w;
                 }
-                __syncwarp();
+                if (!__all_sync(0xffffffffu, plain)) {
+#pragma unroll 1
+                    for (int g = 0; g < kTwGroups; ++g) {
+                        const float4 x = in[g * (kTwTile / 2)], y = in[g * (kTwTile / 2) + 1];
+                        if (g == 0) l[0] = l[1] = l[2] = l[3] = 0.f;
+                        tw_merge(m[0], l[0], x.x, x.y);
+                        tw_merge(m[1], l[1], x.z, x.w);
+                        tw_merge(m[2], l[2], y.x, y.y);
+                        tw_merge(m[3], l[3], y.z, y.w);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) tw_normalise(m[i], l[i]);
+                plain = __all_sync(0xffffffffu, m[0] == 0.f && m[1] == 0.f && m[2] == 0.f && m[3] == 0.f);
                 if (lane == 0) mbar_arrive(bar(kTwREmpty + par));
                 if (it.unit * prm.J + it.r == prm.withhold_job) continue;
                 if (prm.J > 1) {
-                    float2 *dst = prm.part + ((size_t)it.unit * prm.J + it.r) * R + b * kTwTile;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) __stcg(&dst[32 * i + lane], make_float2(m[i], l[i]));
+                    const size_t first = (size_t)it.unit * prm.J * R + b * kTwTile + 4 * lane, mine = first + (size_t)it.r * R;
+                    __stcg(reinterpret_cast<float4 *>(prm.sums + mine), make_float4(l[0], l[1], l[2], l[3]));
+                    __stcg(reinterpret_cast<float4 *>(prm.refs + mine), make_float4(m[0], m[1], m[2], m[3]));
                     __syncwarp();
                     int done = 0;
-                    if (lane == 0) done = atom_add_acq_rel_gpu(prm.sync + kTwSyncHead + prm.units + it.unit * mt + b, 1);
+                    if (lane == 0) done = atom_add_acq_rel_gpu(prm.sync + kTwSyncHead + prm.units + it.unit * mt + b, plain ? 1 : 65537);
                     done = __shfl_sync(0xffffffffu, done, 0);
-                    if (done != prm.J - 1) continue;   // another CTA completes the row block
-                    const float2 *src = prm.part + (size_t)it.unit * prm.J * R + b * kTwTile + lane;
+                    if ((done & 65535) != prm.J - 1) continue;   // another CTA completes the row block
+                    // in job order, so that the result does not depend on who folds
 #pragma unroll
                     for (int i = 0; i < 4; ++i) m[i] = l[i] = 0.f;
+                    if (plain && done == prm.J - 1) {
 #pragma unroll 1
-                    for (int e0 = 0; e0 < prm.J; e0 += 4) {   // 16 loads in flight; in job order, so that the result does not depend on who folds
-                        float2 s[4][4];
+                        for (int e0 = 0; e0 < prm.J; e0 += 8) {   // eight loads in flight
+                            const float *src = prm.sums + first + (size_t)e0 * R;
+                            float4 v[8];
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
+                            for (int e = 0; e < 8; ++e, src += R) v[e] = e0 + e < prm.J ? __ldcg(reinterpret_cast<const float4 *>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                            for (int i = 0; i < 4; ++i)
-                                s[e][i] = e0 + e < prm.J ? __ldcg(src + (size_t)(e0 + e) * R + 32 * i) : make_float2(0.f, 0.f);
-                        bool plain = true;   // every reference is 0: the sums add up as they are
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) plain = plain && s[e][i].x == 0.f && m[i] == 0.f;
-                        if (__all_sync(0xffffffffu, plain)) {
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) l[i] += s[e][i].y;
-                        } else {
-#pragma unroll 1
-                            for (int e = 0; e < 4 && e0 + e < prm.J; ++e) {   // rare: read again one by one
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) {
-                                    const float2 v = __ldcg(src + (size_t)(e0 + e) * R + 32 * i);
-                                    tw_merge(m[i], l[i], v.x, v.y);
-                                }
+                            for (int e = 0; e < 8; ++e) {
+                                l[0] += v[e].x;
+                                l[1] += v[e].y;
+                                l[2] += v[e].z;
+                                l[3] += v[e].w;
                             }
+                        }
+                    } else {
+#pragma unroll 1
+                        for (int e = 0; e < prm.J; ++e) {
+                            const float4 a = __ldcg(reinterpret_cast<const float4 *>(prm.refs + first + (size_t)e * R));
+                            const float4 v = __ldcg(reinterpret_cast<const float4 *>(prm.sums + first + (size_t)e * R));
+                            tw_merge(m[0], l[0], a.x, v.x);
+                            tw_merge(m[1], l[1], a.y, v.y);
+                            tw_merge(m[2], l[2], a.z, v.z);
+                            tw_merge(m[3], l[3], a.w, v.w);
                         }
                     }
                 }
+                float nl[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const int row = b * kTwTile + 32 * i + lane;
-                    float nl = -INFINITY;   // rows beyond M: probability 0
+                    const int row = b * kTwTile + 4 * lane + i;
+                    nl[i] = -INFINITY;   // rows beyond M: probability 0
                     if (row < prm.M) {
                         if (prm.cap_stats) {   // the CaP keys' share of this row's denominator (Appendix B listing)
                             const float2 own = __ldg(&prm.cap_stats[(size_t)it.unit * prm.M + row]);
                             tw_merge(m[i], l[i], own.x, own.y);
                         }
-                        nl = -(m[i] + lg2(l[i]));
+                        nl[i] = -(m[i] + lg2(l[i]));
                     }
-                    __stcg(&prm.nl[(size_t)it.unit * R + row], nl);
                 }
+                __stcg(reinterpret_cast<float4 *>(prm.nl + (size_t)it.unit * R + b * kTwTile + 4 * lane), make_float4(nl[0], nl[1], nl[2], nl[3]));
                 __syncwarp();
                 if (lane == 0) atom_add_acq_rel_gpu(prm.sync + kTwSyncHead + it.unit, 1);
             }
         }
     } else if (warp == 3) {
         // ---------------------------------------------------------------- draws items, fetches the denominators of S2 items
-        // Every look at a counter is a trip to L2, so one job of either kind is always held in advance, and whether the S2 job
-        // is ready is asked while the ring is full.
+        // Every look at a counter is a trip to L2, so one S2 job is always held in advance, and whether it is ready is asked while
+        // the ring is full.  An S1 job is drawn when it is handed out: one held back behind S2 items (which go first) kept its
+        // unit's denominators, and at the end every CTA, waiting.
         if (lane == 0) {
             uint32_t ns = 0;
             bool ok = true;
             int known = -1;   // the last unit found ready
-            int s1 = atomicAdd(prm.sync, 1), s2 = atomicAdd(prm.sync + 1, 1);
+            bool first_left = true;   // S1 jobs may be left
+            int s2 = atomicAdd(prm.sync + 1, 1);
             for (uint32_t n = 0; ok; ++n) {
-                if (s1 < prm.jobs && s2 < prm.jobs && s2 / prm.J != known && ld_acquire_gpu(prm.sync + kTwSyncHead + s2 / prm.J) == mt)
+                if (first_left && s2 < prm.jobs && s2 / prm.J != known && ld_acquire_gpu(prm.sync + kTwSyncHead + s2 / prm.J) == mt)
                     known = s2 / prm.J;
                 ok = wait(bar(kTwPace + n % kTwAhead), ((n / kTwAhead) & 1) ^ 1) && wait(bar(kTwIEmpty + (n & (kTwRing - 1))), ((n / kTwRing) & 1) ^ 1);
                 if (!ok) break;
                 int pos = -1;
-                if (s2 < prm.jobs && (s1 >= prm.jobs || s2 / prm.J == known)) {
+                if (first_left && !(s2 < prm.jobs && s2 / prm.J == known)) {
+                    const int s1 = atomicAdd(prm.sync, 1);
+                    first_left = s1 < prm.jobs;
+                    if (first_left) pos = s1;
+                }
+                if (pos < 0 && s2 < prm.jobs) {
                     pos = s2 | kTwSecond;
                     s2 = atomicAdd(prm.sync + 1, 1);
-                } else if (s1 < prm.jobs) {
-                    pos = s1;
-                    s1 = atomicAdd(prm.sync, 1);
                 }
                 items[n & (kTwRing - 1)] = pos;
                 mbar_arrive(bar(kTwIFull + (n & (kTwRing - 1))));
@@ -692,7 +709,7 @@ constexpr int kTwMaxJobs = 128;   // jobs a unit is cut into at most (the fold r
 struct TwPlan {
     bool usable = false;
     int sm_count = 0, max_mt = 0, max_jobs = 0;
-    float2 *part = nullptr;
+    float *part = nullptr;
     float *nl = nullptr;
     int *sync = nullptr;
 };
@@ -711,7 +728,7 @@ inline void tw_plan_init(TwPlan &plan, const TcPlan &enc, const ipot_config_t &c
     const int tiles = (cfg.pot_size + kTwTile - 1) / kTwTile;
     plan.max_jobs = tiles < kTwMaxJobs ? tiles : kTwMaxJobs;
     const size_t rows = (size_t)units * plan.max_mt * kTwTile, sync_ints = kTwSyncHead + (size_t)units * (1 + plan.max_mt);
-    mem.add((void **)&plan.part, rows * plan.max_jobs * sizeof(float2));
+    mem.add((void **)&plan.part, 2 * rows * plan.max_jobs * sizeof(float));
     mem.add((void **)&plan.nl, rows * sizeof(float));
     mem.add((void **)&plan.sync, sync_ints * sizeof(int), true);
     plan.usable = true;
@@ -738,7 +755,7 @@ inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const 
     if (!Knew) mapKnew = mapK;
     else if (tc_encode_rows(enc, &mapKnew, Knew, cfg.d, N - new_first, units, (size_t)(N - new_first), kTwTile) != IPOT_OK) return IPOT_E_CUDA;
     TwParams prm;
-    prm.scores = scores; prm.cap_stats = cap_stats; prm.part = plan.part; prm.nl = plan.nl; prm.sync = plan.sync; prm.status = status;
+    prm.scores = scores; prm.cap_stats = cap_stats; prm.nl = plan.nl; prm.sync = plan.sync; prm.status = status;
     prm.N = N; prm.M = M; prm.mt = (M + kTwTile - 1) / kTwTile; prm.units = units; prm.tiles = (N + kTwTile - 1) / kTwTile;
     prm.dblk = (cfg.d + 63) / 64;
     prm.ksteps = (cfg.d + 15) / 16;
@@ -772,6 +789,8 @@ inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const 
     if (!prm.nt) return IPOT_E_INVALID;
     prm.J = (prm.tiles + prm.nt - 1) / prm.nt;
     prm.jobs = prm.J * units;
+    prm.sums = plan.part;
+    prm.refs = plan.part + (size_t)prm.jobs * prm.mt * kTwTile;
     prm.new_tile0 = Knew ? new_first / kTwTile : 0x7fffffff;
     prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d));
     prm.wait_ns = wait_ns;
