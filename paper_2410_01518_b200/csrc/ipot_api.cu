@@ -255,21 +255,19 @@ int launch_warp_mma(ipot *p, const void *Q, const float2 *cap_stats, int M, int 
     return IPOT_OK;
 }
 
-// The fastest scorer the shape allows.  d = 64 and 128, measured on 8 to 128 units of 2048 to 32768 keys, M = 128 to 512 (us:
-// one sweep / clusters / items): the one-sweep kernel wins up to about 48 slabs of 256 keys (64 x 8192, M = 256:
-// 100 / 104 / 108; 8 x 16384, M = 512: 75 / 109 / 99), unless there are several row blocks for every one of many units,
-// which the two-sweep kernels fetch the keys for once (128 x 8192, M = 512: 396 / 388 / 336).  Longer items wait for too
-// many other blocks' statistics (128 x 16384, M = 128: 320 / 221 / 214; 16 x 32768: 117 / 104 / 65); then the item kernel for
-// one row block and for many units of several, else the cluster kernel, whose last units are waited for less
-// (32 x 16384, M = 384: 206 / 152 / 188; 64 x 16384, M = 512: 547 / 377 / 348).
+// The fastest scorer the shape allows.  d = 64 and 128, measured on 8 to 256 units of 2048 to 16384 keys, M = 16 to 512 (us:
+// one sweep / clusters / items): the one-sweep kernel computes every exponential once and wins on short items (256 x 4096,
+// M = 128: 84 / 113 / 100; M = 256: 163 / - / 174; M = 512: 314 / 403 / 328), but from about 24 slabs of 256 keys on an item waits
+// for too many other blocks' statistics (64 x 6144, M = 128: 55 / 51 / 46; 128 x 6144, M = 256: 149 / 150 / 135; 128 x 8192, M = 256:
+// 199 / - / 175; 64 x 16384, M = 512: 541 / 378 / 313), if there are items enough to deal (32 x 8192, M = 64: 34 / 37 / 33;
+// 16 x 8192, M = 256: 35 / - / 35; 8 x 8192, M = 512: 35 / - / 46).  The cluster kernel is left for what the item kernel does not take.
 // Other head dimensions have the item kernel or warp-level tensor cores, and the former wins everywhere
-// (d = 256, 64 x 4096, M = 64: 59 us against 221; d = 96, 8 x 640, M = 16: 12.5 against 18.5).
+// (d = 256, 64 x 4096, M = 64: 51 us against 221; d = 96, 8 x 640, M = 16: 12.5 against 18.5).
 int auto_scorer(int units, int N, int M, bool tc_ok, bool ts_ok, bool items_ok, bool mma_ok)
 {
-    const bool long_items = N > 12288 && (long long)units * N >= 32 * 8192;
-    const bool many = M > 2 * kTcRows && N >= 8192 && (long long)units * N >= 128 * 8192;
-    if (items_ok && ((!tc_ok && !ts_ok) || many || (long_items && (M <= kTcRows || !ts_ok)))) return IPOT_SCORER_TENSOR_ITEMS;
-    if (ts_ok && (!tc_ok || (long_items && M > kTcRows))) return IPOT_SCORER_TENSOR_SWEEPS;
+    const bool long_items = N >= 6144 && (long long)units * N >= 32 * 8192;
+    if (items_ok && ((!tc_ok && !ts_ok) || long_items)) return IPOT_SCORER_TENSOR_ITEMS;
+    if (ts_ok && (!tc_ok || (long_items && N > 12288 && M > kTcRows))) return IPOT_SCORER_TENSOR_SWEEPS;
     if (tc_ok) return IPOT_SCORER_TENSOR;
     return mma_ok ? IPOT_SCORER_WARP_MMA : IPOT_SCORER_SIMT;
 }

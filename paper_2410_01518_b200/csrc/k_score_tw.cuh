@@ -22,7 +22,7 @@
 // Four warps per scheduler work on four different buffers, each at its own place of the load - exponential - sum
 // sequence, so that the two pipes stay busy (16 warps that share a buffer idle together at its ends).  A unit's keys
 // are fetched once per sweep for all of its row blocks.  Measured alone: 64 units x 4096 keys x 256 channels, M = 64:
-// 51 us (warp-level tensor cores: 221); 64 x 16384 x 128, M = 512: 348 us (clusters: 377, one sweep: 547).
+// 51 us (warp-level tensor cores: 221); 64 x 16384 x 128, M = 512: 313 us (clusters: 377, one sweep: 541).
 //
 // Warp roles (640 threads): 0 issues TMA loads, 1 issues MMAs and owns tensor memory, 2 merges and publishes row
 // statistics, 3 draws items and fetches the denominators of S2 items, 4-19 epilogue: four groups of four warps (one per
@@ -108,7 +108,7 @@ constexpr float kTwSumMin = 8.0779357e-28f;   // 2^-90
 constexpr float kTwReach = 100.f;             // the polynomial's exponent field is safe up to 2^127: stay well inside
 
 // General path of S1 for the 128 logits of a thread's row: the tile's maximum becomes the reference (first nvalid
-// columns only).  Taken for ragged tiles and when the reference did not fit.
+// columns only).  Taken when the reference did not fit.
 __device__ __noinline__ float2 tw_row_slow(uint32_t taddr, int nvalid, float c, float ref, float l)
 {
     float mx = -INFINITY;
@@ -136,6 +136,25 @@ __device__ __noinline__ float2 tw_row_slow(uint32_t taddr, int nvalid, float c, 
     }
     const float mn = l > 0.f ? fmaxf(ref, m) : m;
     return make_float2(mn, (l > 0.f ? l * ex2(ref - mn) : 0.f) + s * ex2(m - mn));
+}
+
+// A tile of which only the first nvalid columns hold keys: their sum against the reference there is (the caller looks at whether
+// it fits; taking the tile's maximum instead would give the job a reference of its own and its unit the general fold).
+__device__ __noinline__ float tw_row_ragged(uint32_t taddr, int nvalid, float c, float ref)
+{
+    float s = 0.f;
+#pragma unroll 1
+    for (int i = 0; 16 * i < nvalid; ++i) {
+        uint32_t v[16];
+        tmem_ld16(taddr + 16 * i, v);
+        tmem_wait_ld16(v);
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+            if (16 * i + e < nvalid) a[e & 3] += ex2(fmaf(__uint_as_float(v[e]), c, -ref));
+        s += (a[0] + a[1]) + (a[2] + a[3]);
+    }
+    return s;
 }
 
 // (ref, sum) pairs of disjoint key sets -> one pair; a sum of 0 is an empty set whatever its reference is
@@ -458,14 +477,40 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                             }
                         }
                     } else {
+                        // the largest reference, then the sums moved to it (an empty pair's reference does not count)
+                        auto pairs = [&](int e0, float4 (&a)[4], float4 (&v)[4]) {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const size_t at = first + (size_t)min(e0 + e, prm.J - 1) * R;
+                                a[e] = __ldcg(reinterpret_cast<const float4 *>(prm.refs + at));
+                                v[e] = __ldcg(reinterpret_cast<const float4 *>(prm.sums + at));
+                                if (e0 + e >= prm.J) v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            }
+                        };
+                        float4 a[4], v[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) m[i] = -INFINITY;
 #pragma unroll 1
-                        for (int e = 0; e < prm.J; ++e) {
-                            const float4 a = __ldcg(reinterpret_cast<const float4 *>(prm.refs + first + (size_t)e * R));
-                            const float4 v = __ldcg(reinterpret_cast<const float4 *>(prm.sums + first + (size_t)e * R));
-                            tw_merge(m[0], l[0], a.x, v.x);
-                            tw_merge(m[1], l[1], a.y, v.y);
-                            tw_merge(m[2], l[2], a.z, v.z);
-                            tw_merge(m[3], l[3], a.w, v.w);
+                        for (int e0 = 0; e0 < prm.J; e0 += 4) {
+                            pairs(e0, a, v);
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                m[0] = fmaxf(m[0], v[e].x > 0.f ? a[e].x : -INFINITY);
+                                m[1] = fmaxf(m[1], v[e].y > 0.f ? a[e].y : -INFINITY);
+                                m[2] = fmaxf(m[2], v[e].z > 0.f ? a[e].z : -INFINITY);
+                                m[3] = fmaxf(m[3], v[e].w > 0.f ? a[e].w : -INFINITY);
+                            }
+                        }
+#pragma unroll 1
+                        for (int e0 = 0; e0 < prm.J; e0 += 4) {
+                            pairs(e0, a, v);
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                l[0] += v[e].x > 0.f ? v[e].x * ex2(a[e].x - m[0]) : 0.f;
+                                l[1] += v[e].y > 0.f ? v[e].y * ex2(a[e].y - m[1]) : 0.f;
+                                l[2] += v[e].z > 0.f ? v[e].z * ex2(a[e].z - m[2]) : 0.f;
+                                l[3] += v[e].w > 0.f ? v[e].w * ex2(a[e].w - m[3]) : 0.f;
+                            }
                         }
                     }
                 }
@@ -620,6 +665,14 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                                     sweep1_slow<16>(r0, 0, 16, c, ref, l);
                                     sweep1_slow<16>(r1, 0, 16, c, ref, l);
                                 }
+                            }
+                        }
+                        if (nvalid < kTwTile) {
+                            const float sum = l + tw_row_ragged(tb, nvalid, c, ref);
+                            redo = !__all_sync(0xffffffffu, sum <= kTwSumMax && sum >= kTwSumMin);
+                            if (!redo) {
+                                l = sum;
+                                release();
                             }
                         }
                         if (redo) {

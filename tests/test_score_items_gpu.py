@@ -84,3 +84,17 @@ def test_items_query_tile_heights(M, d):
     t["K_cap"] = inputs.make_kcap(cfg, 0)
     same, cnt = compare_cycle(cfg, t, gpu_cycle(cfg, t, ITEMS, n=1290), n=1290)
     assert same >= cnt - 1
+
+
+@pytest.mark.parametrize("n", [1025, 1100, 4096 + 127])
+def test_items_ragged_last_tile_beside_references(n):
+    """The last tile's keys are summed against the reference there is, or, where the sum is out of range, against their own:
+    with keys small everywhere, large everywhere but in the last tile, and large only in it."""
+    cfg = inputs.small_config(cfg_id=950, pot_size=n, keep=300, nuc_slots=0, cap_rows=48, Hq=4, Hkv=1, d=128, dtype="bf16", layers=3)
+    t = inputs.make_cycle(cfg)
+    K = inputs.widen(t["K"], "bf16").astype(np.float32)
+    last = (n - 1) // 128 * 128
+    K[1, :, :, :last] *= 50.0
+    K[2, :, :, last:] *= 50.0
+    t["K"] = inputs.store(K, "bf16")
+    compare_cycle(cfg, t, gpu_cycle(cfg, t, ITEMS))
