@@ -657,8 +657,12 @@ def main():
     units, e, d, M = cfg.units, cfg.elem_bytes, cfg.d, cfg.G * cfg.cap_rows
     score_bytes = units * (N * d * e + M * d * e + 4 * N)      # K once + Q + scores out
     score_flops = 2.0 * units * M * N * d                      # one pass (a second sweep is overhead, not algorithm)
-    # K and V, read + write, all kept rows; in rotary mode the rotated copy of K is written as well
-    compact_bytes = units * (5 if args.rope else 4) * cfg.keep * d * e
+    # K and V, read + write; in rotary mode the rotated copy of K is written as well.  Rows that have to move: all but the
+    # leading ones that keep their slots in the pot, counted in the last step's index lists
+    slots = torch.arange(cfg.keep, dtype=torch.int32)
+    in_place = (idx_host == slots) & ((slots < N - n_new) | (args.append != "deferred"))
+    moved_rows = units * cfg.keep - int(in_place.to(torch.int32).cumprod(1).sum())
+    compact_bytes = (5 if args.rope else 4) * moved_rows * d * e
     names = ["nuc_rank", "cap_score", "select", "compact"]
     # the dominant kernel; scoring and compaction are close, scoring is named unless compaction is clearly longer
     dom = 3 if kms[3] > 1.05 * kms[1] else 1
@@ -693,6 +697,7 @@ def main():
     roof["cap_score_tflops"] = score_tflops
     roof["cap_score_frac_of_hbm_peak"] = score_gbs / pk["hbm_gbs"]
     roof["cap_score_frac_of_bf16_sustained"] = score_tflops / pk["bf16_tflops"]
+    roof["compact_rows_moved"] = moved_rows / (units * cfg.keep)
     roof["compact_gbs"] = compact_bytes / (kms[3] * 1e-3) / 1e9
     roof["compact_frac_of_hbm_peak"] = roof["compact_gbs"] / pk["hbm_gbs"]
     # the whole step against the copy rate: algorithmic bytes of scoring + compaction (+ the append's copy when it is
