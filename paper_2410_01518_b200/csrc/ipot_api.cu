@@ -570,6 +570,14 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
         delete p;
         return IPOT_E_CUDA;
     }
+    if (cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        free_all(p);
+        delete p;
+        return IPOT_E_CUDA;
+    }
     const size_t pot_bytes = (size_t)p->units * cfg->pot_size * p->row_bytes;
     const int maxM = p->G * cfg->max_cap_rows;
     p->max_parts = (maxM + 127) / 128;
@@ -598,7 +606,7 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
     tc_plan_init(p->tc, p->cfg, p->sm_count, mem);
     tw_plan_init(p->tw, p->tc, p->cfg, p->sm_count, mem);
     if (cfg->dtype == IPOT_F32) f32_plan_init(p->f32, p->units, maxM, cfg->pot_size, mem);
-    bool ok = mem.allocate(&p->arena);
+    bool ok = mem.allocate(&p->arena, p->side);
     if (!ok) {
         cudaGetLastError();
         free_all(p);
@@ -614,14 +622,6 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
          cudaFuncSetAttribute(cap_row_stats_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma_scorer_smem_bytes(256)) == cudaSuccess &&
          cudaFuncSetAttribute(cap_column_sums_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma_scorer_smem_bytes(256)) == cudaSuccess;
     if (!ok) {
-        cudaGetLastError();
-        free_all(p);
-        delete p;
-        return IPOT_E_CUDA;
-    }
-    if (cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         free_all(p);
         delete p;
