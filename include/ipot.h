@@ -132,13 +132,18 @@ int ipot_set_scorer(ipot_t *pot, int scorer);
  *                                 (IPOT_SCORER_TENSOR_SWEEPS) or of the grid (IPOT_SCORER_TENSOR), or job `value` of
  *                                 IPOT_SCORER_TENSOR_ITEMS, never reports its statistics, so every wait for them runs into
  *                                 the limit; -1 = off (default)
+ *   IPOT_TUNE_TEST_WITHHOLD_CHUNK for tests of the give-up path only: chunk `value` (0-7) of every tensor never reports to
+ *                                 the compaction's other chunks that it has been read; -1 = off (default)
+ * The compaction's waits have a limit of their own, 200 ms, which cannot be set: after one that ran out (IPOT_E_TIMEOUT, too)
+ * some rows have been moved and others have not, so the pot has to be emptied (ipot_reset) and filled again.
  * Errors: INVALID (unknown `what`, value out of range).  Takes effect at the next launch.
  */
 enum {
     IPOT_TUNE_SWEEPS_CLUSTER = 1,
     IPOT_TUNE_SWEEPS_FMA_EIGHTHS = 2,
     IPOT_TUNE_WAIT_LIMIT_NS = 3,
-    IPOT_TUNE_TEST_WITHHOLD_RANK = 4
+    IPOT_TUNE_TEST_WITHHOLD_RANK = 4,
+    IPOT_TUNE_TEST_WITHHOLD_CHUNK = 5
 };
 int ipot_set_tuning(ipot_t *pot, int what, long long value);
 

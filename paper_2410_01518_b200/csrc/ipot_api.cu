@@ -59,6 +59,7 @@ struct ipot {
     uint8_t *nuc_mask;   // [batch][mask_stride(N)]
     int32_t *idx;        // [units][keep]
     GatherPlan gather;   // what the selection leaves for the gather
+    int withhold_chunk;  // IPOT_TUNE_TEST_WITHHOLD_CHUNK
     int *status;         // sticky device status word
     void *stage_q;       // device staging for the *_host calls
     void *stage_kc;
@@ -430,7 +431,7 @@ int run_cycle(ipot *p, const void *Q, const void *Kc, int cap_rows, const float 
     const bool outside = pend.K && pend.V && pend.first == 0;
     const int group = outside ? 1 : (int)std::min<long long>(p->units, (1LL << 30) / p->gather.chunks);
     const GatherParams g{(uint4 *)p->K, (uint4 *)p->V, p->idx, p->gather, p->status, keep, N, row_vecs, p->units, group,
-                         (size_t)p->cfg.pot_size * row_vecs, pend, p->ts.wait_ns, one_wave(p, dim3(p->gather.chunks, 2, p->units))};
+                         (size_t)p->cfg.pot_size * row_vecs, pend, p->withhold_chunk, one_wave(p, dim3(p->gather.chunks, 2, p->units))};
     if (!p->rope) IPOT_CUDA(launch_gather(p, compact_kernel, g));
     else IPOT_CUDA(p->cfg.dtype == IPOT_F32 ? launch_gather_rope<float>(p, g) : launch_gather_rope<__nv_bfloat16>(p, g));
     p->launches += 1;
@@ -564,6 +565,7 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
     p->row_bytes = cfg->d * p->elem_bytes;
     p->stream = (cudaStream_t)cfg->stream;
     p->scorer = IPOT_SCORER_AUTO;
+    p->withhold_chunk = -1;
     if (cudaGetDevice(&p->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
         cudaGetLastError();
@@ -682,6 +684,10 @@ int ipot_set_tuning(ipot_t *p, int what, long long value)
     case IPOT_TUNE_TEST_WITHHOLD_RANK:
         if (value < -1 || value > 7) return IPOT_E_INVALID;
         p->ts.withhold_rank = (int)value;
+        return IPOT_OK;
+    case IPOT_TUNE_TEST_WITHHOLD_CHUNK:
+        if (value < -1 || value > 7) return IPOT_E_INVALID;
+        p->withhold_chunk = (int)value;
         return IPOT_OK;
     default:
         return IPOT_E_INVALID;

@@ -70,6 +70,9 @@ struct PendingRows {
 // survivors in place: 52 us, with every chunk copied 92).
 constexpr int kGatherThreads = 128;
 constexpr int kGatherBytes = 16384;
+// Time limit of a wait for another chunk.  Its own, and not to be set: a chunk that gives up leaves the pot half moved, where a
+// scorer that gives up only loses scores.
+constexpr unsigned long long kGatherWaitNs = 200ull * 1000 * 1000;
 
 inline int gather_rows(int row_vecs) { return kGatherBytes / 16 / row_vecs; }
 inline int gather_chunks(int keep, int row_vecs) { return (keep + gather_rows(row_vecs) - 1) / gather_rows(row_vecs); }
@@ -95,7 +98,7 @@ struct GatherParams {
     int units, group;        // units in all, and in a group that is walked chunk by chunk
     size_t unit_vecs;
     PendingRows pend;
-    unsigned long long wait_ns;
+    int withhold_chunk;      // -1; test hook: this chunk of every tensor is never reported as read
     bool release;            // one wave of blocks: the next kernel may be set up
 };
 
@@ -157,7 +160,7 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
     __syncthreads();
     // the survivors up to here have not moved (src ascends and is no less than its row): so are the bytes, in the rotated copy too
     if (src_sm[n - 1] == r0 + n - 1 && r0 + n <= alt_first) {
-        if (threadIdx.x == 0) asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(sync + 2 + chunk), "r"(launch) : "memory");
+        if (threadIdx.x == 0 && chunk != p.withhold_chunk) asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(sync + 2 + chunk), "r"(launch) : "memory");
         return;
     }
     {
@@ -186,7 +189,7 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
                 int seen;
                 asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(sync + 2 + c) : "memory");
                 up = seen == launch;
-                if (!up && (tries & 255u) == 0 && global_timer_ns() - t0 > p.wait_ns) {
+                if (!up && (tries & 255u) == 0 && global_timer_ns() - t0 > kGatherWaitNs) {
                     set_status(p.status, kStatusTimeout);
                     gave_up = 1;
                     up = true;
@@ -198,14 +201,14 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk copy below reads what the threads have brought in
     __syncthreads();
     if (threadIdx.x == 0) {
-        asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(sync + 2 + chunk), "r"(launch) : "memory");
+        if (chunk != p.withhold_chunk) asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(sync + 2 + chunk), "r"(launch) : "memory");
         if (!gave_up) {   // (a wait that ran out: the rows stay as they are)
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
                          ::"l"(base + (size_t)r0 * p.row_vecs), "r"(sbuf), "r"((uint32_t)nvec * 16u) : "memory");
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
     }
-    if (tensor == 0) rotate(buf, unit, r0, n, p.row_vecs);
+    if (tensor == 0 && !gave_up) rotate(buf, unit, r0, n, p.row_vecs);   // (nor does the rotated copy change)
     if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the block's memory is free again
 }
 

@@ -20,7 +20,7 @@ IPOT_OK, IPOT_E_INVALID, IPOT_E_STATE, IPOT_E_NOMEM, IPOT_E_CUDA, IPOT_E_TIMEOUT
 IPOT_NOALLOC_MAX_ROWS = 65536
 IPOT_BF16, IPOT_F32 = 0, 1
 IPOT_SCORER_AUTO, IPOT_SCORER_SIMT, IPOT_SCORER_TENSOR, IPOT_SCORER_WARP_MMA, IPOT_SCORER_TENSOR_SWEEPS, IPOT_SCORER_TENSOR_ITEMS = 0, 1, 2, 3, 4, 5
-IPOT_TUNE_SWEEPS_CLUSTER, IPOT_TUNE_SWEEPS_FMA_EIGHTHS, IPOT_TUNE_WAIT_LIMIT_NS, IPOT_TUNE_TEST_WITHHOLD_RANK = 1, 2, 3, 4
+IPOT_TUNE_SWEEPS_CLUSTER, IPOT_TUNE_SWEEPS_FMA_EIGHTHS, IPOT_TUNE_WAIT_LIMIT_NS, IPOT_TUNE_TEST_WITHHOLD_RANK, IPOT_TUNE_TEST_WITHHOLD_CHUNK = 1, 2, 3, 4, 5
 IPOT_ROPE_HALF, IPOT_ROPE_INTERLEAVED = 1, 2
 
 # every symbol include/ipot.h declares

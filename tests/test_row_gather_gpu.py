@@ -1,9 +1,11 @@
 """GPU parity of the in-place gather of the survivors (Appendix B "KV-cache compression") at the edges of its chunks of
 about 16 KiB of whole rows, against the CPU checker: rows are moved, so every byte must match."""
+import numpy as np
 import pytest
+import torch
 
 from paper_2410_01518_b200 import inputs, ipot
-from parity import compare_cycle, gpu_cycle
+from parity import check_rotated, compare_cycle, from_dev_bits, gpu_cycle, make_pot, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -48,3 +50,42 @@ def test_gather_rows_in_place(in_place, first, rope):
     gpu = gpu_cycle(cfg, t, ipot.IPOT_SCORER_AUTO, n=n, deferred_from=first)
     same, cnt = compare_cycle(cfg, t, gpu, n=n)
     assert same == cnt == cfg.units
+
+
+def test_gather_wait_that_runs_out_leaves_rows_and_rotated_copy_together():
+    """Chunk 0 of every tensor never reports that it has been read (a test hook): the chunk behind it cannot be overwritten, the
+    launch ends by itself with IPOT_E_TIMEOUT, the rows it did not move still have their own rotated rows beside them, and
+    after ipot_reset the same pot runs a correct cycle.  The scorers' limit does not apply to the gather: with it as short as
+    it may be set, a cycle of a pot whose scorer has no waits ends without a status."""
+    n, keep, d = 600, 500, 128
+    cfg = inputs.small_config(cfg_id=890, pot_size=n, keep=keep, nuc_slots=0, cap_rows=4, Hq=3, Hkv=3, d=d, dtype="bf16")
+    t = inputs.make_cycle(cfg)
+    t["rope"] = (*inputs.make_rope_table(n, d, "bf16"), False)
+    want = gpu_cycle(cfg, t, ipot.IPOT_SCORER_SIMT)
+    Kd, Vd, Qd, cos, sin = (to_dev(x, "bf16") for x in (t["K"], t["V"], t["Q"], *t["rope"][:2]))
+    h = make_pot(cfg)
+    try:
+        ipot.ipot_set_scorer(h, ipot.IPOT_SCORER_SIMT)
+        ipot.ipot_enable_rope(h, cos, sin, ipot.IPOT_ROPE_HALF)
+        ipot.ipot_set_tuning(h, ipot.IPOT_TUNE_WAIT_LIMIT_NS, 1000)
+        for withheld in (-1, 0, -1):
+            ipot.ipot_set_tuning(h, ipot.IPOT_TUNE_TEST_WITHHOLD_CHUNK, withheld)
+            ipot.ipot_reset(h)
+            ipot.ipot_append_chunk(h, Kd, Vd, n)
+            if withheld < 0:
+                ipot.ipot_score_and_compress(h, Qd, cfg.cap_rows, None)
+                torch.cuda.synchronize()
+                K = from_dev_bits(ipot.device_array(ipot.ipot_view(h)[0], (cfg.units, n, d), "bf16")[:, :keep], "bf16")
+                rot = from_dev_bits(ipot.device_array(ipot.ipot_view_rope(h), (cfg.units, n, d), "bf16")[:, :keep], "bf16")
+                assert (K == want[2]).all() and (rot == want[4]).all()
+            else:
+                assert ipot.ipot_sync_status(h) == 0   # (nothing before ran out)
+                ipot.ipot_score_and_compress(h, Qd, cfg.cap_rows, None)
+                assert ipot.ipot_sync_status(h) == ipot.IPOT_E_TIMEOUT
+                K = from_dev_bits(ipot.device_array(ipot.ipot_view(h)[0], (cfg.units, n, d), "bf16")[:, :keep], "bf16")
+                rot = from_dev_bits(ipot.device_array(ipot.ipot_view_rope(h), (cfg.units, n, d), "bf16")[:, :keep], "bf16")
+                assert (K != want[2]).any()            # some chunk did give up
+                for unit in range(cfg.units):
+                    check_rotated(rot[unit], K[unit], np.arange(keep), t["rope"], "bf16")
+    finally:
+        ipot.ipot_destroy(h)
