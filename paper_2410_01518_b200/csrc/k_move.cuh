@@ -57,8 +57,9 @@ struct PendingRows {
 // then writes it back as one bulk copy.  idx is ascending, so idx[r] >= r, and a slot of the chunk's own destination
 // range can only be the source of a row r' <= r: before a block overwrites slots [r0, r1) it waits until the chunks
 // holding those r' (at most two, as at most r1 - r0 survivors come from r1 - r0 slots) have been read.  Chunks are handed out
-// by a ticket per tensor in ascending order and a block reads its chunk before it waits for anything, so every wait
-// is for a block that is already running and does not itself wait first.  The flags are relaxed accesses: when one is
+// by a ticket per tensor in ascending order and a block reads its chunk and raises its flag before it waits for anything, so
+// every wait is for a block that is already running and does not itself wait first.  (With the flag raised behind the wait a
+// pot that keeps nearly everything, where every chunk waits for the one before, was a chain of flag round trips.)  The flags are relaxed accesses: when one is
 // raised the chunk's bytes ARE in shared memory (the copies have been waited for), so there is no access left that a
 // fence would have to order, and a release / acquire pair per block costs more than the copy of a chunk
 // (256 units x 4096 -> 2048 rows of 256 bytes, all in the pot: 138 us with the pair, 91 without any flag).
@@ -109,6 +110,7 @@ __device__ __forceinline__ void gather_cp_async16(uint32_t dst, const void *src)
 
 // What a rotary pot does with a gathered key chunk in shared memory besides moving it (k_rope.cuh); nothing here.
 struct GatherNoRotate {
+    static constexpr bool kOn = false;
     __device__ __forceinline__ void operator()(const uint4 *, int, int, int, int) const {}
 };
 
@@ -178,38 +180,46 @@ __device__ __forceinline__ void gather_block(const GatherParams &p, const Rotate
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    if (threadIdx.x == kGatherThreads - 32 && r0 < alt_first && chunk > 0) {
-        // while the rows are on their way: the chunks whose sources lie in this chunk's slots (no source in slots whose rows
-        // are outside the pot) have been read
-        const int c1 = q1 > q0 ? min(chunk - 1, (q1 - 1) / rows) : -1;
-        const unsigned long long t0 = global_timer_ns();
-        for (int c = max(0, q0 / rows); c <= c1; ++c) {
-            bool up = false;
-            for (uint32_t tries = 1; !up; ++tries) {
-                int seen;
-                asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(sync + 2 + c) : "memory");
-                up = seen == launch;
-                if (!up && (tries & 255u) == 0 && global_timer_ns() - t0 > kGatherWaitNs) {
-                    set_status(p.status, kStatusTimeout);
-                    gave_up = 1;
-                    up = true;
-                }
-            }
-        }
+    // The lane that has the flags.  Which chunks' sources lie in this chunk's slots (none in slots whose rows are outside the pot),
+    // and a first look at their flags while the rows are on their way.
+    const bool lead = threadIdx.x == kGatherThreads - 32;
+    int wait_c = 0, wait_end = -1;
+    auto read_up = [&]() {
+        int seen;
+        asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(sync + 2 + wait_c) : "memory");
+        return seen == launch;
+    };
+    if (lead && r0 < alt_first && q1 > q0) {
+        wait_c = q0 / rows;
+        wait_end = min(chunk - 1, (q1 - 1) / rows);
+        while (wait_c <= wait_end && read_up()) ++wait_c;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk copy below reads what the threads have brought in
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (lead) {
         if (chunk != p.withhold_chunk) asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(sync + 2 + chunk), "r"(launch) : "memory");
+        const unsigned long long t0 = wait_c <= wait_end ? global_timer_ns() : 0;
+        for (uint32_t tries = 1; wait_c <= wait_end; ++tries) {
+            if (read_up()) {
+                ++wait_c;
+            } else if ((tries & 255u) == 0 && global_timer_ns() - t0 > kGatherWaitNs) {
+                set_status(p.status, kStatusTimeout);
+                gave_up = 1;
+                break;
+            }
+        }
         if (!gave_up) {   // (a wait that ran out: the rows stay as they are)
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
                          ::"l"(base + (size_t)r0 * p.row_vecs), "r"(sbuf), "r"((uint32_t)nvec * 16u) : "memory");
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
     }
-    if (tensor == 0 && !gave_up) rotate(buf, unit, r0, n, p.row_vecs);   // (nor does the rotated copy change)
-    if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the block's memory is free again
+    if (Rotate::kOn && tensor == 0) {
+        if (r0 < alt_first) __syncthreads();   // (else nothing was waited for)
+        if (!gave_up) rotate(buf, unit, r0, n, p.row_vecs);   // (nor does the rotated copy change)
+    }
+    if (lead) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the block's memory is free again
 }
 
 __global__ void __launch_bounds__(kGatherThreads) compact_kernel(const __grid_constant__ GatherParams p)

@@ -195,6 +195,7 @@ append_rope_kernel(const uint4 *__restrict__ src, size_t src_unit_vecs, uint4 *p
 // nothing; keys and values share the launch.  Bound: HBM, 5 * keep rows per unit.  (A walk over the rows with the
 // row pair's halves in registers across a barrier took 170 us for 256 units x 4096 -> 2048 rows, this one 106.)
 template <typename T, bool kInterleaved> struct GatherRotate {
+    static constexpr bool kOn = true;
     uint4 *Krot;
     const T *cos_t, *sin_t;
     size_t unit_vecs;
