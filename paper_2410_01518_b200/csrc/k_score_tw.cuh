@@ -458,6 +458,7 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                     if (lane == 0) done = atom_add_acq_rel_gpu(prm.sync + kTwSyncHead + prm.units + it.unit * mt + b, plain ? 1 : 65537);
                     done = __shfl_sync(0xffffffffu, done, 0);
                     if ((done & 65535) != prm.J - 1) continue;   // another CTA completes the row block
+                    __syncwarp();   // what lane 0 has acquired is ordered before the other lanes' reads too (a shuffle alone orders no memory)
                     // in job order, so that the result does not depend on who folds
 #pragma unroll
                     for (int i = 0; i < 4; ++i) m[i] = l[i] = 0.f;
