@@ -148,8 +148,8 @@ enum {
 int ipot_set_tuning(ipot_t *pot, int what, long long value);
 
 /* Forget the contents: len = 0.  Nothing is launched.  Also the way back to a defined state after
- * ipot_sync_status() reported IPOT_E_TIMEOUT: the scorer's exchange buffers are cleared before their next use
- * (the sticky status itself stays). */
+ * ipot_sync_status() reported IPOT_E_TIMEOUT (the sticky status itself stays; that call has arranged for the scorer's
+ * exchange buffers to be cleared before their next use). */
 int ipot_reset(ipot_t *pot);
 
 /*

@@ -805,9 +805,12 @@ struct TcPlan {
     int max_items = 0, max_slabs = 0;
     float2 *stats = nullptr;          // [max_items][max_slabs][128]
     // "fresh" marking of the statistics: every launch writes all entries of its (items x slabs) layout
-    // with the sign opposite to the previous launch's; a layout change, or a launch that gave up, clears the array first
+    // with the sign opposite to the previous launch's; a layout change, or a launch that gave up or failed, clears the array first.
+    // A captured launch runs again and again with the one sign it was captured with, between launches that nobody counts: it
+    // clears the array itself, and so does every launch after it.
     float sign = 1.f;
     int last_items = 0, last_slabs = 0;
+    bool captured = false;
 };
 
 inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, int sm_count, DeviceArena &mem)
@@ -903,7 +906,15 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
     prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d));
     prm.wait_ns = wait_ns;
     prm.withhold_cta = withhold_cta;
-    if (items != plan.last_items || prm.slabs != plan.last_slabs) {
+    if (!plan.captured) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) {
+            cudaGetLastError();
+            return IPOT_E_CUDA;
+        }
+        plan.captured = capture != cudaStreamCaptureStatusNone;
+    }
+    if (plan.captured || items != plan.last_items || prm.slabs != plan.last_slabs) {
         if (cudaMemsetAsync(plan.stats, 0, (size_t)items * prm.slabs * kTcRows * sizeof(float2), stream) != cudaSuccess) {
             cudaGetLastError();
             return IPOT_E_CUDA;
@@ -930,6 +941,7 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
     lc.attrs = at; lc.numAttrs = 1;
     if (cudaLaunchKernelEx(&lc, nuc.ctas > 0 ? cap_score_tc_kernel<true> : cap_score_tc_kernel<false>, mapQ, mapK, mapKnew, prm) != cudaSuccess) {
         cudaGetLastError();
+        plan.last_items = 0;   // the array still holds what the last launch that ran has left
         return IPOT_E_CUDA;
     }
     *parts = mtiles;

@@ -48,3 +48,74 @@ def test_pot_on_its_own_stream_while_the_default_stream_is_busy(d, dtype):
     assert (u.cpu().numpy() == want[0]).all() and (idx.cpu().numpy() == want[1]).all()
     got = K.cpu().numpy() if dtype == "f32" else K.view(torch.int16).cpu().numpy().view(np.uint16)
     assert (got == want[2]).all()
+
+
+@pytest.mark.parametrize("d,dtype,layers,n,rope", [(128, "bf16", 2, 1500, False), (128, "bf16", 32, 4096, False), (96, "bf16", 2, 1500, False),
+                                                   (128, "bf16", 2, 1500, True), (64, "f32", 2, 1500, False)])
+def test_captured_pass_replays_on_other_inputs(d, dtype, layers, n, rope):
+    """A whole pass (reset, append, cycle, a generated token) captured into a CUDA graph: every replay is a pass over what the
+    input buffers hold by then, also between and after passes that are not captured.  (The one-sweep scorer tells its own
+    statistics from an earlier launch's by a sign; its replays all have the same one.)  The larger pot is ranked on the
+    side stream, the others inside the scorer's grid or on the pot's own stream."""
+    cfg = inputs.small_config(cfg_id=965, pot_size=n, keep=n // 3, nuc_slots=n // 6, cap_rows=8, Hq=16, Hkv=8, d=d, dtype=dtype, layers=layers)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    shapes = {"K": (layers, 1, cfg.Hkv, n, d), "V": (layers, 1, cfg.Hkv, n, d), "Q": (layers, 1, cfg.Hq, cfg.cap_rows, d), "q": (layers, 1, cfg.Hq, d)}
+    data = [{k: torch.randn(s, generator=g, device="cuda", dtype=dt) for k, s in shapes.items()} | {"aux": torch.rand((1, n), generator=g, device="cuda")}
+            for _ in range(2)]
+    buf = {k: v.clone() for k, v in data[0].items()}
+    out = torch.zeros(shapes["q"], device="cuda")
+    if rope:
+        cos, sin = (to_dev(x, dtype) for x in inputs.make_rope_table(n, d, dtype))
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def new_pot():
+        h = ipot.ipot_create_ex(n, cfg.keep, layers, cfg.Hq, cfg.Hkv, d, dtype=ipot.IPOT_F32 if dtype == "f32" else ipot.IPOT_BF16,
+                                nuc_slots=cfg.nuc_slots, max_cap_rows=cfg.cap_rows, stream=s.cuda_stream)
+        if rope:
+            ipot.ipot_enable_rope(h, cos, sin, ipot.IPOT_ROPE_HALF)
+        return h
+
+    def one_pass(h):
+        ipot.ipot_reset(h)
+        ipot.ipot_append_chunk(h, buf["K"], buf["V"], n)
+        ipot.ipot_score_and_compress(h, buf["Q"], cfg.cap_rows, buf["aux"])
+        if d != 96:
+            ipot.ipot_decode_attention(h, buf["q"], out)
+
+    def results(h):
+        s.synchronize()
+        assert ipot.ipot_sync_status(h) == 0
+        K = ipot.device_array(ipot.ipot_view(h)[0], (cfg.units, n, d), dtype)[:, :cfg.keep]
+        return [x.clone() for x in (ipot.device_array(ipot.ipot_last_scores(h)[0], (cfg.units, n), "f32"),
+                                    ipot.device_array(ipot.ipot_last_indices(h), (cfg.units, cfg.keep), "i32"), K, out)]
+
+    def load(i):
+        s.synchronize()
+        for k in buf:
+            buf[k].copy_(data[i][k])
+        torch.cuda.synchronize()
+
+    h, want, graph = new_pot(), [], torch.cuda.CUDAGraph()
+    try:
+        for i in range(2):
+            load(i)
+            h1 = new_pot()
+            one_pass(h1)
+            want.append(results(h1))
+            ipot.ipot_destroy(h1)
+        load(0)
+        one_pass(h)
+        results(h)
+        with torch.cuda.graph(graph, stream=s):
+            one_pass(h)
+        for i, replay in ((1, True), (0, True), (1, True), (0, False), (1, False), (0, True), (1, True), (0, False)):
+            load(i)
+            with torch.cuda.stream(s):
+                graph.replay() if replay else one_pass(h)
+            assert all(torch.equal(a, b) for a, b in zip(results(h), want[i])), (i, replay)
+    finally:
+        torch.cuda.synchronize()
+        del graph
+        ipot.ipot_destroy(h)
