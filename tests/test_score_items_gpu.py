@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2410_01518_b200 import inputs, ipot
 from parity import compare_cycle, gpu_cycle, make_pot, to_dev
 
@@ -98,3 +99,21 @@ def test_items_ragged_last_tile_beside_references(n):
     K[2, :, :, last:] *= 50.0
     t["K"] = inputs.store(K, "bf16")
     compare_cycle(cfg, t, gpu_cycle(cfg, t, ITEMS))
+
+
+@pytest.mark.parametrize("d,other", [(40, ipot.IPOT_SCORER_SIMT), (72, ipot.IPOT_SCORER_SIMT), (96, ipot.IPOT_SCORER_WARP_MMA),
+                                     (192, ipot.IPOT_SCORER_WARP_MMA), (256, ipot.IPOT_SCORER_WARP_MMA), (128, ipot.IPOT_SCORER_TENSOR)])
+def test_items_are_as_exact_as_the_kernels_they_stand_in_for(d, other):
+    """Error against 64 bits, 2-norm and largest, beside that of the scorer such a pot would have otherwise.  Both sum 32-bit
+    exponentials of 32-bit logits, so the two differ by the luck of their rounding: a factor of 2 is allowed, where a
+    polynomial of degree 4 and denominators as one rounded logarithm made it 3 to 5."""
+    cfg = inputs.small_config(cfg_id=970, pot_size=4000, keep=1000, nuc_slots=0, cap_rows=32, Hq=8, Hkv=4, d=d, dtype="bf16", layers=2)
+    t = inputs.make_cycle(cfg)
+    Q = inputs.widen(t["Q"], "bf16").astype(np.float32)
+    t["Q"] = inputs.store(Q + 2.5 * Q[:, :, :, :1], "bf16")    # a query head's rows share a direction
+    ref = oracle.cycle(t["Q"], t["K"], t["V"], t["aux"], cfg.keep, 0)["u"]
+    err = []
+    for scorer in (ITEMS, other):
+        u = gpu_cycle(cfg, t, scorer)[0].astype(np.float64)
+        err.append((np.linalg.norm(u - ref) / np.linalg.norm(ref), np.abs(u / ref - 1).max()))
+    assert err[0][0] <= 2 * err[1][0] and err[0][1] <= 2 * err[1][1], err
