@@ -22,11 +22,11 @@ __device__ __forceinline__ unsigned long long global_timer_ns()
     return t;
 }
 
-// Monotone map float -> uint32: a < b  <=>  key(a) < key(b) (for non-NaN values).
+// Monotone map float -> uint32: a < b  <=>  key(a) < key(b) (for non-NaN values; a NaN lies beyond the infinity of its sign).
 __device__ __forceinline__ uint32_t order_key(float f)
 {
-    uint32_t b = __float_as_uint(f);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+    const uint32_t b = __float_as_uint(f);
+    return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
 }
 
 // One 16-byte vector of storage elements -> floats.

@@ -36,6 +36,9 @@ struct SelShared {
     int remaining;
 };
 
+// The key of a slot that exists: never 0, which the NaN with all bits set would have.
+__device__ __forceinline__ uint32_t slot_key(float f) { return max(order_key(f), 1u); }
+
 // Exclusive prefix sum of v over the block in thread order; `total` = block sum.  One barrier; consecutive
 // calls alternate `parity` so that a warp that runs ahead does not overwrite totals still being read.
 template <int kThreads>
@@ -91,9 +94,9 @@ __device__ __forceinline__ void block_radix_select(const uint32_t (&key)[kKpt], 
     mx = __reduce_max_sync(0xffffffffu, lane < kWarps ? sh.wmax[lane] : 0u);
     res = __reduce_add_sync(0xffffffffu, lane < kWarps ? sh.wres[lane] : 0u);
     int remaining = k - (int)res;
-    if (remaining <= 0) {   // only reserved slots
-        tau = 0xFFFFFFFEu;
-        need_eq = 0;
+    if (remaining <= 0) {   // only reserved slots, the lowest ones where there are more (a NaN of all ones has their key, too)
+        tau = 0xFFFFFFFFu;
+        need_eq = k;
         return;
     }
     uint32_t lo = mn, span = mx - mn;   // the boundary lies in [lo, lo + span]
@@ -242,7 +245,7 @@ __device__ __forceinline__ void nuc_rank_streams(const float *__restrict__ aux, 
             float s[kKpt];
             load_row<kKpt>(aux + (size_t)b * N, slot0, N, s);
 #pragma unroll
-            for (int i = 0; i < kKpt; ++i) key[i] = slot0 + i < N ? order_key(s[i]) : 0u;
+            for (int i = 0; i < kKpt; ++i) key[i] = slot0 + i < N ? slot_key(s[i]) : 0u;
         }
         __syncthreads();
         uint32_t tau;
@@ -339,7 +342,7 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
         }
 #pragma unroll
         for (int i = 0; i < kPiece; ++i)
-            key[h + i] = first + i >= N ? 0u : (r[i >> 2] >> (8 * (i & 3))) & 0xFFu ? 0xFFFFFFFFu : order_key(s[i]);
+            key[h + i] = first + i >= N ? 0u : (r[i >> 2] >> (8 * (i & 3))) & 0xFFu ? 0xFFFFFFFFu : slot_key(s[i]);
     }
     __syncthreads();
     uint32_t tau;

@@ -230,6 +230,24 @@ def test_exact_ties_resolve_to_lower_slots():
     assert same == n
 
 
+@pytest.mark.parametrize("pattern", [0x7FFFFFFF, 0x7FC00000, 0x7F800001, 0xFFFFFFFF])
+@pytest.mark.parametrize("n,count", [(1000, 400), (1000, 900), (200, 150)])   # more NaNs than reserved slots, and than slots kept; no ranking in the scorer's grid
+def test_ranking_of_nan_novelty(pattern, n, count):
+    """Novelty has to be finite; a NaN in it still takes one slot each and no more: exactly `keep` survivors, among them the
+    lowest slots of the NaNs that rank above every number, or the numbers before the NaN that ranks below."""
+    keep, T = n // 2, n // 4
+    cfg = inputs.small_config(cfg_id=985, pot_size=n, keep=keep, nuc_slots=T, cap_rows=4, Hq=4, Hkv=2, d=64, dtype="bf16", batch=2)
+    t = inputs.make_cycle(cfg)
+    where = np.sort(np.random.default_rng(count).permutation(n)[:count])
+    t["aux"].view(np.uint32)[:, where] = pattern
+    _, idx, K, _ = gpu_cycle(cfg, t)   # (asserts the status)
+    others = np.setdiff1d(np.arange(n), where)
+    reserved = where[:T] if pattern < 0x80000000 else np.concatenate([others, where])[:T] if len(others) <= T else []
+    for unit in range(cfg.units):
+        assert len(set(idx[unit].tolist())) == keep and (np.diff(idx[unit]) > 0).all() and set(reserved) <= set(idx[unit].tolist())
+        assert (K[unit] == t["K"].reshape(cfg.units, n, cfg.d)[unit][idx[unit]]).all()
+
+
 @pytest.mark.parametrize("pot,keep,T", [(4096, 2048, 1024), (9000, 5001, 100), (16400, 5000, 0), (20000, 12288, 4096)])
 def test_exact_ties_in_large_pots(pot, keep, T):
     """Every score equal and every novelty equal: the survivors are the first `keep` slots whatever the pot size.
