@@ -119,10 +119,11 @@ f32_tile_kernel(const __grid_constant__ F32Params p)
         }
 #pragma unroll
         for (int off = 8; off >= 1; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        const float from = m == -INFINITY ? 0.f : m;   // (a tile whose logits all lie below fp32's range: zeros, not NaNs)
 #pragma unroll
         for (int b = 0; b < KB; ++b) {
             const int key = j0 + tx + 16 * b;
-            const float e = exp2f(x[b] - m);
+            const float e = exp2f(x[b] - from);
             if (key < p.N) {
                 l += e;
                 if (row < p.M) p.e[((size_t)g * p.M + row) * p.e_stride + key] = e;

@@ -121,6 +121,7 @@ __device__ __noinline__ float2 tw_row_slow(uint32_t taddr, int nvalid, float c, 
         for (int e = 0; e < 16; ++e)
             if (16 * i + e < nvalid) mx = fmaxf(mx, __uint_as_float(v[e]));
     }
+    if (mx == -INFINITY) return make_float2(ref, l);   // no key, or logits beyond fp32's range: nothing to add
     const float m = mx * c;
     float s = 0.f;
 #pragma unroll 1

@@ -27,3 +27,18 @@ def test_f32_scorer_shapes(case):
     units = None if cfg.units <= 16 else np.linspace(0, cfg.units - 1, 16).astype(np.int32)
     same, cnt = compare_cycle(cfg, t, gpu_cycle(cfg, t, ipot.IPOT_SCORER_AUTO, n=n), n=n, units=units)
     assert same >= cnt - 1
+
+
+@pytest.mark.parametrize("d,dtype,P", [(64, "f32", 16), (128, "f32", 64), (96, "bf16", 16)])
+def test_logits_below_the_range_of_fp32(d, dtype, P):
+    """Finite inputs whose logits overflow to -inf for whole tiles of keys: those keys score 0 and the others as if they
+    were not there."""
+    cfg = inputs.small_config(cfg_id=960, pot_size=1300, keep=400, nuc_slots=100, cap_rows=P, Hq=8, Hkv=2, d=d, dtype=dtype, layers=2)
+    t = inputs.make_cycle(cfg)
+    Q, K = (inputs.widen(t[k], dtype).astype(np.float32) for k in ("Q", "K"))
+    Q[..., 0], K[..., 0] = 1e10, 0
+    K[..., 128:700, 0] = -1e30
+    t["Q"], t["K"] = inputs.store(Q, dtype), inputs.store(K, dtype)
+    gpu = gpu_cycle(cfg, t)
+    same, cnt = compare_cycle(cfg, t, gpu)
+    assert same >= cnt - 1 and (gpu[0][:, 128:700] == 0).all()
