@@ -5,8 +5,8 @@
 // novelty_kernel, grid (segments, tokens): a block of 128 threads reads one segment of at most 8192 logits of one row
 // with 16-byte loads (eight per thread in flight) and reduces it to (reference, sum 2^(z log2e - reference)), the
 // reference being the segment's largest logit in log2 units.  Rows are cut into segments so that the grid is
-// fine-grained (a whole 32k-256k row per block would leave a long tail on 148 SMs), and evenly, so that no segment is a
-// small remainder.  A row that does not start on a 16-byte boundary (every vocabulary that is not a multiple of eight)
+// fine-grained (a whole 32k-256k row per block would leave a long tail on 148 SMs): whole segments and a remainder where
+// every row starts on a 16-byte boundary, even ones otherwise.  A row that does not start on a 16-byte boundary (every vocabulary that is not a multiple of eight)
 // is read the same way from its first boundary on: with element loads for such rows, 777 rows of 50257 bf16 logits took
 // 41 us.  The block that finishes a row last (a counter per row, no waiting) merges the row's segments, fetches the label's
 // logit and writes log-sum-exp minus it to the token's slot of the novelty array.
@@ -28,6 +28,9 @@ constexpr int kNovSegElems = 8192;
 constexpr int kNovMaxRows = 65535;   // tokens per call (grid y limit); the row counters are sized for it
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
+// The reference before any logit: finite, so that masked logits (-inf, or the type's lowest value, whose product with log2e is
+// -inf) add 0 to a thread that has seen nothing else yet; as -inf it made the thread's sum NaN for good.
+constexpr float kNovLowest = -3.402823466e38f;
 
 __device__ __forceinline__ float nov_ex2(float x)
 {
@@ -51,7 +54,7 @@ struct NovStat {
     __device__ __forceinline__ void raise(float lm)
     {
         const float nref = fmaxf(ref, lm * kLog2e);
-        const float f = nov_ex2(ref - nref);  // first time: ref = -inf, f = 0, s is 0 anyway
+        const float f = nov_ex2(ref - nref);  // (first time: s is 0 anyway)
         s = __fmul2_rn(s, make_float2(f, f));
         ref = nref;
     }
@@ -71,8 +74,7 @@ struct NovStat {
 __device__ __forceinline__ void nov_merge(float &ref, float &sum, float ref2, float sum2)
 {
     const float rn = fmaxf(ref, ref2);
-    const float a = (ref == -INFINITY) ? 0.f : sum * nov_ex2(ref - rn);
-    const float b = (ref2 == -INFINITY) ? 0.f : sum2 * nov_ex2(ref2 - rn);
+    const float a = sum * nov_ex2(ref - rn), b = sum2 * nov_ex2(ref2 - rn);   // (both references are finite)
     ref = rn;
     sum = a + b;
 }
@@ -129,7 +131,7 @@ novelty_kernel(const T *__restrict__ logits, size_t row_stride, int V, int segs,
     const size_t row = blockIdx.y;
     const int v0 = seg * seg_elems, v1 = min(V, v0 + seg_elems);
     const T *z = logits + row * row_stride;
-    NovStat st{-INFINITY, make_float2(0.f, 0.f)};
+    NovStat st{kNovLowest, make_float2(0.f, 0.f)};
     // The row may start anywhere (an odd vocabulary): the elements before its first 16-byte boundary and behind its last
     // one, fewer than VE each, are read one by one by different warps, everything between them in 16-byte loads.
     const T *p = z + v0;
@@ -164,7 +166,7 @@ novelty_kernel(const T *__restrict__ logits, size_t row_stride, int V, int segs,
     ref = wred[0][0];
 #pragma unroll
     for (int w = 1; w < kNovThreads / 32; ++w) ref = fmaxf(ref, wred[0][w]);
-    float sum = (st.ref == -INFINITY) ? 0.f : (st.s.x + st.s.y) * nov_ex2(st.ref - ref);
+    float sum = (st.s.x + st.s.y) * nov_ex2(st.ref - ref);
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
     if (lane == 0) wred[1][warp] = sum;
@@ -179,7 +181,7 @@ novelty_kernel(const T *__restrict__ logits, size_t row_stride, int V, int segs,
         if (atomicAdd(&counters[row], 1) != segs - 1) return;  // another block finishes the row
         __threadfence();
         counters[row] = 0;  // ready for the next call
-        ref = -INFINITY;
+        ref = kNovLowest;
         sum = 0.f;
         for (int s = 0; s < segs; ++s) {
             const float2 p = __ldcg(&partial[row * segs + s]);

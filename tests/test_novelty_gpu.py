@@ -117,3 +117,22 @@ def test_produced_novelty_drives_a_cycle():
     assert close(t["aux"], oracle.token_novelty(inputs.widen(z, "bf16"), lab).reshape(cfg.batch, 512)).all()
     same, n = compare_cycle(cfg, t, gpu)
     assert n == cfg.units and same >= n - 1
+
+
+@pytest.mark.parametrize("mask", [-np.inf, -3.38e38])   # what masked vocabulary entries are set to (the second nearly bf16's lowest value)
+@pytest.mark.parametrize("V,dtype,first,last", [(16384, "f32", 4096, 16384), (50257, "bf16", 9000, 50257), (8200, "bf16", 8192, 8200), (32000, "f32", 30000, 31999)])
+def test_masked_logits_count_as_nothing(V, dtype, first, last, mask):
+    """Logits [0, first) and [last, V) are masked: threads, segments and row ends that see masked logits first, or nothing else."""
+    n = 6
+    cfg = inputs.small_config(cfg_id=601, batch=1, pot_size=64, keep=8, nuc_slots=4)
+    z, _ = inputs.make_logits(0x77 + V, n, V, dtype)
+    z[:, :first] = z[:, last:] = inputs.store(np.full(1, mask, dtype=np.float32), dtype)[0]
+    lab = np.linspace(first, last - 1, n).astype(np.int32)
+    aux = torch.full((1, n), -7.0, device="cuda")
+    h = make_pot(cfg)
+    try:
+        ipot.ipot_nuc_scores(h, to_dev(z, dtype), ipot.IPOT_F32 if dtype == "f32" else ipot.IPOT_BF16, V, torch.from_numpy(lab).cuda(), n, V, aux, n, 0)
+        assert ipot.ipot_sync_status(h) == 0
+    finally:
+        ipot.ipot_destroy(h)
+    assert close(aux.cpu().numpy()[0], oracle.token_novelty(inputs.widen(z, dtype), lab)).all()
