@@ -75,12 +75,12 @@ enum {
                                 pots the tcgen05 kernels do not; IPOT_E_INVALID if the shape does not allow it */
     IPOT_SCORER_TENSOR_SWEEPS = 4, /* tcgen05 kernel that goes over the keys twice (row log-sum-exps, then probabilities
                                 and their column sums) inside thread-block clusters, so that no block waits for a block
-                                it is not co-scheduled with (bf16, d = 64 or 128, at most 512 folded query rows):
-                                IPOT_E_INVALID if the shape does not allow it */
+                                it is not co-scheduled with (bf16, d = 64 or 128, at most 512 folded query rows); on request
+                                only: IPOT_E_INVALID if the shape does not allow it */
     IPOT_SCORER_TENSOR_ITEMS = 5 /* tcgen05 kernel in two sweeps whose pieces are dealt to the SMs one by one (bf16, any
                                 d, at most 1024 folded query rows): what AUTO takes for head dimensions other than
-                                64 and 128, and for many query rows over many long units; IPOT_E_INVALID if the shape
-                                does not allow it */
+                                64 and 128, and for long units if there are many; IPOT_E_INVALID if the
+                                shape does not allow it */
 };
 
 typedef struct {

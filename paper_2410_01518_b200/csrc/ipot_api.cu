@@ -256,19 +256,25 @@ int launch_warp_mma(ipot *p, const void *Q, const float2 *cap_stats, int M, int 
     return IPOT_OK;
 }
 
-// The fastest scorer the shape allows.  d = 64 and 128, measured on 8 to 256 units of 2048 to 16384 keys, M = 16 to 512 (us:
-// one sweep / clusters / items): the one-sweep kernel computes every exponential once and wins on short items (256 x 4096,
-// M = 128: 84 / 113 / 100; M = 256: 163 / - / 174; M = 512: 314 / 403 / 328), but from about 24 slabs of 256 keys on an item waits
-// for too many other blocks' statistics (64 x 6144, M = 128: 55 / 51 / 46; 128 x 6144, M = 256: 149 / 150 / 135; 128 x 8192, M = 256:
-// 199 / - / 175; 64 x 16384, M = 512: 541 / 378 / 313), if there are items enough to deal (32 x 8192, M = 64: 34 / 37 / 33;
-// 16 x 8192, M = 256: 35 / - / 35; 8 x 8192, M = 512: 35 / - / 46).  The cluster kernel is left for what the item kernel does not take.
+// The fastest scorer the shape allows.  d = 64 and 128: the one-sweep kernel computes every exponential once, but beyond 32 slabs
+// of 256 keys an item's blocks wait too long for each other's statistics, and the two-sweep kernel whose work is dealt item by item
+// is faster if there are items enough to deal.  Rows of 64 channels cost the one-sweep kernel as much as wider ones: there it
+// is from 6144 keys on.  Measured as steps of a stream with deferred appends (us, one sweep / items), d = 128:
+//   128 units x 8192 keys, M = 64, 128, 256:  145 / 151, 146 / 168, 233 / 239;  64 x 8192, M = 512, 768, 1024: 219 / 219, 310 / 299, 400 / 387
+//   128 x 9216:                               188 / 169, 188 / 185, 304 / 277;  64 x 9216, M = 512: 289 / 243
+//    64 x 12288:                              138 / 119, 138 / 127, 217 / 191;  64 x 16384:         582 / 406
+//    32 x 9216:                               66 / 67, 66 / 68, 98 / 90;        16 x 16384: 71 / 67, 71 / 68, 105 / 90
+//    24 x 12288, M = 128: 67 / 67 (as whole passes 67 / 71);  32 x 10240: 71 / 66, 71 / 70, 107 / 96
+// and d = 64, M = 64, 128, 256:  64 x 4096: 43 / 49, 44 / 51, 64 / 68;  64 x 6144: 59 / 57, 60 / 60, 95 / 90;  128 x 8192: 129 / 112, 129 / 120,
+// 219 / 184;  32 x 8192, M = 128: 49 / 53.
 // Other head dimensions have the item kernel or warp-level tensor cores, and the former wins everywhere
 // (d = 256, 64 x 4096, M = 64: 51 us against 221; d = 96, 8 x 640, M = 16: 12.5 against 18.5).
-int auto_scorer(int units, int N, int M, bool tc_ok, bool ts_ok, bool items_ok, bool mma_ok)
+int auto_scorer(int units, int N, int M, int d, bool tc_ok, bool items_ok, bool mma_ok)
 {
-    const bool long_items = N >= 6144 && (long long)units * N >= 32 * 8192;
-    if (items_ok && ((!tc_ok && !ts_ok) || long_items)) return IPOT_SCORER_TENSOR_ITEMS;
-    if (ts_ok && (!tc_ok || (long_items && N > 12288 && M > kTcRows))) return IPOT_SCORER_TENSOR_SWEEPS;
+    const long long keys = (long long)units * N;
+    const bool many = d == 64 && N >= 6144 && keys >= 64 * 6144;
+    const bool long_items = (N > 8192 || (N == 8192 && M > 512)) && keys >= 32 * 8192 && (M > kTcRows || N >= 16384 || keys >= 32 * 10240);
+    if (items_ok && (!tc_ok || many || long_items)) return IPOT_SCORER_TENSOR_ITEMS;
     if (tc_ok) return IPOT_SCORER_TENSOR;
     return mma_ok ? IPOT_SCORER_WARP_MMA : IPOT_SCORER_SIMT;
 }
@@ -287,7 +293,7 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
     if (scorer == IPOT_SCORER_WARP_MMA && !mma_ok) return IPOT_E_INVALID;
     const bool items_ok = tw_applicable(p->tw, N, M);
     if (scorer == IPOT_SCORER_TENSOR_ITEMS && !items_ok) return IPOT_E_INVALID;
-    if (scorer == IPOT_SCORER_AUTO) scorer = auto_scorer(p->units, N, M, tc_ok, ts_ok, items_ok, mma_ok);
+    if (scorer == IPOT_SCORER_AUTO) scorer = auto_scorer(p->units, N, M, p->cfg.d, tc_ok, items_ok, mma_ok);
     // keys of a deferred append: the tensor-core scorers read whole slabs of them where they are, anything else
     // wants them in the pot
     const int slab_keys = scorer == IPOT_SCORER_TENSOR         ? kTcSlab

@@ -117,3 +117,28 @@ def test_items_are_as_exact_as_the_kernels_they_stand_in_for(d, other):
         u = gpu_cycle(cfg, t, scorer)[0].astype(np.float64)
         err.append((np.linalg.norm(u - ref) / np.linalg.norm(ref), np.abs(u / ref - 1).max()))
     assert err[0][0] <= 2 * err[1][0] and err[0][1] <= 2 * err[1][1], err
+
+
+@pytest.mark.parametrize("units,n,P,Hq_per_kv,d,want", [
+    (64, 8192, 16, 4, 128, ipot.IPOT_SCORER_TENSOR), (64, 8193, 16, 4, 128, ITEMS), (40, 8192, 129, 4, 128, ITEMS), (35, 9216, 32, 4, 128, ipot.IPOT_SCORER_TENSOR),
+    (35, 9216, 33, 4, 128, ITEMS), (32, 10240, 16, 1, 64, ITEMS), (64, 6143, 16, 1, 64, ipot.IPOT_SCORER_TENSOR), (64, 6144, 16, 1, 64, ITEMS),
+    (16, 12288, 33, 4, 128, ipot.IPOT_SCORER_TENSOR), (2, 300, 16, 1, 96, ITEMS)])
+def test_automatic_choice(units, n, P, Hq_per_kv, d, want):
+    """Both sides of every line of the automatic choice; the scores agree with those of the kernel that was not chosen."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    K = torch.randn((units, 1, 1, n, d), generator=g, device="cuda").bfloat16()
+    Q = torch.randn((units, 1, Hq_per_kv, P, d), generator=g, device="cuda").bfloat16()
+    u = []
+    for scorer in (ipot.IPOT_SCORER_AUTO, ipot.IPOT_SCORER_WARP_MMA):
+        h = ipot.ipot_create_ex(n, n // 4, units, Hq_per_kv, 1, d, nuc_slots=0, max_cap_rows=P)
+        try:
+            ipot.ipot_set_scorer(h, scorer)
+            ipot.ipot_set_profiling(h, True)
+            ipot.ipot_append_chunk(h, K, K, n)
+            ipot.ipot_score_and_compress(h, Q, P, None)
+            assert ipot.ipot_sync_status(h) == 0
+            assert ipot.ipot_kernel_ms(h)[2] == (want if scorer == ipot.IPOT_SCORER_AUTO else scorer)
+            u.append(ipot.device_array(ipot.ipot_last_scores(h)[0], (units, n), "f32").clone())
+        finally:
+            ipot.ipot_destroy(h)
+    assert ((u[0] - u[1]).norm() / u[1].norm()).item() < 2e-6   # (two kernels within 1e-6 of the exact scores each)
