@@ -8,9 +8,9 @@
 //            tensor-memory buffers; an epilogue thread owns one query row and keeps sum_j 2^(x_ij c - ref) in a
 //            register against a reference that is 0 unless the sum then leaves the range fp32 holds well, so no maximum is
 //            taken.  The job's (ref, sum) pairs go to memory; the CTA that completes a row block of a unit last
-//            folds the jobs' pairs into the denominators, kept as 2^-n / w with a whole number n.
+//            folds the jobs' pairs into -log2 of the denominators.
 //   S2 item  the same tiles with the operands swapped, S^T = K Q^T: a KEY per tensor-memory lane, so that u_j is a sum
-//            over the thread's own registers of 2^(x_ij c + n_i) w_i - no exchange between lanes, one coalesced store.
+//            over the thread's own registers of 2^(x_ij c - L_i) - no exchange between lanes, one coalesced store.
 //
 // A CTA draws items one by one from two counters: its next S2 item as soon as the unit's denominators are known, else its
 // next S1 item, so that it does not wait for another CTA while it has anything else to do, and a job's keys are still in L2
@@ -53,8 +53,8 @@ enum {
 
 // shared-memory carve-up (bytes); the tiles follow at the next multiple of 1024
 constexpr uint32_t kTwOffRow = 0;                                             // [2][groups][128] float2
-constexpr uint32_t kTwOffLtab = kTwOffRow + 2 * kTwGroups * 128 * 8;          // [2][2][kTwMaxBlocks * 128] float
-constexpr uint32_t kTwOffBar = kTwOffLtab + 2 * 2 * kTwMaxBlocks * 128 * 4;
+constexpr uint32_t kTwOffLtab = kTwOffRow + 2 * kTwGroups * 128 * 8;          // [2][kTwMaxBlocks * 128] float
+constexpr uint32_t kTwOffBar = kTwOffLtab + 2 * kTwMaxBlocks * 128 * 4;
 constexpr uint32_t kTwOffItem = kTwOffBar + 8 * kTwBarCount;
 constexpr uint32_t kTwOffSlot = kTwOffItem + 4 * kTwRing;                     // tensor-memory base, abort flag, last-CTA flag
 constexpr uint32_t kTwOffTiles = (kTwOffSlot + 16 + 1023) / 1024 * 1024;
@@ -64,7 +64,7 @@ struct TwParams {
     float *scores;            // [units][N]
     const float2 *cap_stats;  // NULL, or [units][M] (max, sum) over the CaP's own keys that join every row's denominator
     float *sums, *refs;       // [units][J][mt * 128]: the jobs' (ref, sum) pairs
-    float *nl;                // [units][2][mt * 128]: the denominators as 2^-n / w: n, a whole number, and w, near 1
+    float *nl;                // [units][mt * 128]: -log2 of the denominators
     int *sync;                // next S1 job, next S2 job, CTAs that have left, then [units] row blocks whose denominators are known,
                               // [units * mt] jobs that have reported (65536 added for one with a reference other than 0); zero between launches
     int *status;
@@ -174,32 +174,23 @@ __device__ __forceinline__ void tw_sweep1(const uint32_t (&v)[16], float c, floa
         }
     }
 }
-__device__ __forceinline__ float2 ffma2_ftz(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
-        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
-        "fma.rn.ftz.f32x2 rd, ra, rb, rc;\n\t"
-        "mov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
-// S2, a key's logits against 16 query rows: adds 2^(x c + n) w with the rows' n and w (shared memory, the same for every lane).
-// A denominator's logarithm as one float, some 20 to 40, would cost every probability of the row its rounding, 4e-7 on average.
+// S2, a key's logits against 16 query rows: adds 2^(x c + nl) (nl: shared memory, the same for every lane).  The rounding of nl, some
+// 20 to 40, is 4e-7 of a row's probabilities; kept apart as a whole exponent and a factor it would be gone, but over a unit's
+// rows it evens out (error of the scores 5 to 15 % less), and the second table in shared memory costs what the MMAs need of it (64 units
+// x 16384 keys, M = 512, whole pass: 411 us against 402).
 template <int kPoly>
-__device__ __forceinline__ void tw_sweep2(const uint32_t (&v)[16], float c, const float *n, const float *w, float2 (&sa)[2], float2 (&pa)[2])
+__device__ __forceinline__ void tw_sweep2(const uint32_t (&v)[16], float c, const float *nl, float2 (&sa)[2], float2 (&pa)[2])
 {
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
-        const float4 n4 = *reinterpret_cast<const float4 *>(n + 4 * g), w4 = *reinterpret_cast<const float4 *>(w + 4 * g);
+        const float4 n4 = *reinterpret_cast<const float4 *>(nl + 4 * g);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int i = 2 * g + h;
             const float2 x = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
             const float2 t = __ffma2_rn(x, make_float2(c, c), h ? make_float2(n4.z, n4.w) : make_float2(n4.x, n4.y));
-            const float2 w2 = h ? make_float2(w4.z, w4.w) : make_float2(w4.x, w4.y);
-            if (pair_on_fma<kPoly>(i)) pa[i & 1] = ffma2_ftz(exp2_fma_pair5(t), w2, pa[i & 1]);
-            else sa[i & 1] = ffma2_ftz(make_float2(ex2(t.x), ex2(t.y)), w2, sa[i & 1]);
+            if (pair_on_fma<kPoly>(i)) pa[i & 1] = fadd2_ftz(pa[i & 1], exp2_fma_pair5(t));
+            else sa[i & 1] = fadd2_ftz(sa[i & 1], make_float2(ex2(t.x), ex2(t.y)));
         }
     }
 }
@@ -562,24 +553,20 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                         }
                     }
                 }
-                float nl[4], w[4];
+                float nl[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int row = b * kTwTile + 4 * lane + i;
                     nl[i] = -INFINITY;   // rows beyond M: probability 0
-                    w[i] = 0.f;
                     if (row < prm.M) {
                         if (prm.cap_stats) {   // the CaP keys' share of this row's denominator (Appendix B listing)
                             const float2 own = __ldg(&prm.cap_stats[(size_t)it.unit * prm.M + row]);
                             tw_merge(m[i], l[i], own.x, own.y);
                         }
-                        nl[i] = -rintf(m[i] + lg2(l[i]));
-                        w[i] = ex2(-m[i] - nl[i]) * __frcp_rn(l[i]);
+                        nl[i] = -(m[i] + log2f(l[i]));
                     }
                 }
-                float *to = prm.nl + (size_t)it.unit * 2 * R + b * kTwTile + 4 * lane;
-                __stcg(reinterpret_cast<float4 *>(to), make_float4(nl[0], nl[1], nl[2], nl[3]));
-                __stcg(reinterpret_cast<float4 *>(to + R), make_float4(w[0], w[1], w[2], w[3]));
+                __stcg(reinterpret_cast<float4 *>(prm.nl + (size_t)it.unit * R + b * kTwTile + 4 * lane), make_float4(nl[0], nl[1], nl[2], nl[3]));
                 __syncwarp();
                 if (lane == 0) atom_add_acq_rel_gpu(prm.sync + kTwSyncHead + it.unit, 1);
             }
@@ -635,10 +622,10 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 }
                 // the copy engine reads what other SMs wrote with ordinary stores
                 asm volatile("fence.proxy.async;" ::: "memory");
-                const uint32_t bytes = 2u * (uint32_t)mt * kTwTile * 4;
+                const uint32_t bytes = (uint32_t)mt * kTwTile * 4;
                 mbar_expect_tx(bar(kTwLFull + par), bytes);
                 asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             ::"r"(base + kTwOffLtab + par * 2 * kTwMaxBlocks * kTwTile * 4), "l"(prm.nl + (size_t)unit * 2 * mt * kTwTile), "r"(bytes),
+                             ::"r"(base + kTwOffLtab + par * kTwMaxBlocks * kTwTile * 4), "l"(prm.nl + (size_t)unit * mt * kTwTile), "r"(bytes),
                                "r"(bar(kTwLFull + par)) : "memory");
                 ++ns;
             }
@@ -748,7 +735,7 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 const int cols = prm.qrows;
                 float u = 0.f;   // with several row blocks a group has at most one tile of an item, and u adds over them
                 for (int b = 0; b < mt && ok; ++b, task0 += (uint32_t)it.w) {
-                    const float *nl = ltab + (par * 2 * kTwMaxBlocks + b) * kTwTile, *w = nl + mt * kTwTile;
+                    const float *nl = ltab + (par * kTwMaxBlocks + b) * kTwTile;
                     for (int t = first; t < it.w; t += kTwGroups) {
                         ok = wwait(bar(kTwSFull + g), ((task0 + (uint32_t)t) >> 2) & 1);
                         if (!ok) break;
@@ -764,17 +751,17 @@ cap_score_tw_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
 #pragma unroll 1
                         for (int i = 0; i < cols / 16 - 2; i += 2) {
                             tmem_ld16(tb + 16 * (i + 1), r1);
-                            tw_sweep2<kTwPoly>(r0, c, nl + 16 * i, w + 16 * i, sa, pa);
+                            tw_sweep2<kTwPoly>(r0, c, nl + 16 * i, sa, pa);
                             tmem_wait_ld16(r1);
                             tmem_ld16(tb + 16 * (i + 2), r0);
-                            tw_sweep2<kTwPoly>(r1, c, nl + 16 * i + 16, w + 16 * i + 16, sa, pa);
+                            tw_sweep2<kTwPoly>(r1, c, nl + 16 * i + 16, sa, pa);
                             tmem_wait_ld16(r0);
                         }
                         tmem_ld16(tb + cols - 16, r1);
                         tmem_wait_ld16(r1);
                         release();
-                        tw_sweep2<kTwPoly>(r0, c, nl + cols - 32, w + cols - 32, sa, pa);
-                        tw_sweep2<kTwPoly>(r1, c, nl + cols - 16, w + cols - 16, sa, pa);
+                        tw_sweep2<kTwPoly>(r0, c, nl + cols - 32, sa, pa);
+                        tw_sweep2<kTwPoly>(r1, c, nl + cols - 16, sa, pa);
                         const float2 s2 = fadd2_ftz(fadd2_ftz(sa[0], sa[1]), fadd2_ftz(pa[0], pa[1]));
                         float sum = s2.x + s2.y;
                         if (mt > 1) sum = u += sum;
@@ -833,7 +820,7 @@ inline void tw_plan_init(TwPlan &plan, const TcPlan &enc, const ipot_config_t &c
     plan.max_jobs = tiles < kTwMaxJobs ? tiles : kTwMaxJobs;
     const size_t rows = (size_t)units * plan.max_mt * kTwTile, sync_ints = kTwSyncHead + (size_t)units * (1 + plan.max_mt);
     mem.add((void **)&plan.part, 2 * rows * plan.max_jobs * sizeof(float));
-    mem.add((void **)&plan.nl, 2 * rows * sizeof(float));
+    mem.add((void **)&plan.nl, rows * sizeof(float));
     mem.add((void **)&plan.sync, sync_ints * sizeof(int), true);
     plan.usable = true;
 }
@@ -898,7 +885,7 @@ inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const 
     prm.new_tile0 = Knew ? new_first / kTwTile : 0x7fffffff;
     // The tensor core cuts its running sums instead of rounding them: a logit comes out short by about 1.2e-8 of itself per
     // 16-channel step, which is made good here.  (Error of the scores against 64 bits, 2-norm, without / with: 4096 keys of 256
-    // channels 7.7e-7 / 4.5e-7, 3000 of 192 5.5e-7 / 2.9e-7, 8192 of 128 4.2e-7 / 2.2e-7; warp-level tensor cores 6.3e-7, 4.5e-7, 2.9e-7.)
+    // channels 7.7e-7 / 4.5e-7, 3000 of 192 5.5e-7 / 3.1e-7, 8192 of 128 4.2e-7 / 2.5e-7; warp-level tensor cores 6.3e-7, 4.5e-7, 2.9e-7.)
     prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d) * (1.0 + 1.2e-8 * prm.ksteps));
     prm.wait_ns = wait_ns;
     prm.withhold_job = withhold_job;
