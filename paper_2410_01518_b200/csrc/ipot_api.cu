@@ -88,6 +88,7 @@ struct ipot {
     // the novelty ranking does not depend on the scores: it runs beside the scorer on a stream of its own
     cudaStream_t side;
     cudaEvent_t ev_fork, ev_join;
+    cudaEvent_t ev_zero;   // the counters are zero (queued on the side stream by ipot_create)
 };
 
 namespace {
@@ -128,12 +129,31 @@ void free_all(ipot *p)
     cudaFree(p->arena); cudaFree(p->Krot); cudaFree(p->nov_scratch);
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
     if (p->ev_join) cudaEventDestroy(p->ev_join);
+    if (p->ev_zero) cudaEventDestroy(p->ev_zero);
     if (p->side) cudaStreamDestroy(p->side);
     if (p->ev) {
         for (int i = 0; i < kProfSlots; ++i)
             for (auto &e : p->ev[i]) if (e) cudaEventDestroy(e);
         delete[] p->ev;
     }
+}
+
+// Nothing on stream s runs before the counters are zero.  A stream whose work is being captured cannot wait for what is outside its
+// graph; there the host waits.
+int wait_for_zeros(ipot *p, cudaStream_t s)
+{
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone) {
+        IPOT_CUDA(cudaStreamWaitEvent(s, p->ev_zero, 0));
+        return IPOT_OK;
+    }
+    cudaGetLastError();
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    IPOT_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t waited = cudaEventSynchronize(p->ev_zero);
+    IPOT_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    IPOT_CUDA(waited);
+    return IPOT_OK;
 }
 
 // Blocks that fit the device at once (the row movers keep eight per SM).
@@ -580,7 +600,8 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
     }
     if (cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&p->ev_zero, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         free_all(p);
         delete p;
@@ -635,6 +656,12 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
         delete p;
         return IPOT_E_CUDA;
     }
+    if (cudaEventRecord(p->ev_zero, p->side) != cudaSuccess || wait_for_zeros(p, p->stream) != IPOT_OK) {
+        cudaGetLastError();
+        free_all(p);
+        delete p;
+        return IPOT_E_CUDA;
+    }
     *out = p;
     return IPOT_OK;
 }
@@ -652,6 +679,7 @@ int ipot_set_stream(ipot_t *p, void *s)
 {
     if (!p) return IPOT_E_INVALID;
     int rc = materialise(p, true, true);  // queued on the stream that is being left
+    if (rc == IPOT_OK) rc = wait_for_zeros(p, (cudaStream_t)s);
     if (rc != IPOT_OK) return rc;
     p->stream = (cudaStream_t)s;
     return IPOT_OK;

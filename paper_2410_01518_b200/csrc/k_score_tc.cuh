@@ -763,8 +763,8 @@ struct DeviceArena {
         if (n < kMost) wants[n] = {ptr, (bytes + 255) / 256 * 256 + (bytes ? 0 : 256), zero};
         ++n;
     }
-    // false: out of memory.  The zeros are written through `stream` and have been written when this returns: the pot's own stream
-    // may be one that does not wait for the null stream, and kernels rely on their counters from the first launch on.
+    // false: out of memory.  The zeros are queued on `stream`: kernels rely on their counters from the first launch on, so every stream
+    // of the pot waits for them.
     bool allocate(void **base, cudaStream_t stream)
     {
         if (n > kMost) return false;
@@ -774,7 +774,7 @@ struct DeviceArena {
             if (wants[i].zero) zeros += wants[i].bytes;
         }
         if (cudaMalloc(base, total) != cudaSuccess) return false;
-        if (cudaMemsetAsync(*base, 0, zeros, stream) != cudaSuccess || cudaStreamSynchronize(stream) != cudaSuccess) return false;
+        if (cudaMemsetAsync(*base, 0, zeros, stream) != cudaSuccess) return false;
         char *at = (char *)*base, *at_zero = at;
         at += zeros;
         for (int i = 0; i < n; ++i) {

@@ -10,8 +10,9 @@ from parity import gpu_cycle, to_dev
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("handed_over", [False, True])   # the pot is created on the stream, or on the default stream
 @pytest.mark.parametrize("d,dtype", [(96, "bf16"), (128, "bf16"), (128, "f32")])   # item scorer, one-sweep scorer, f32 scorer
-def test_pot_on_its_own_stream_while_the_default_stream_is_busy(d, dtype):
+def test_pot_on_its_own_stream_while_the_default_stream_is_busy(d, dtype, handed_over):
     """The default stream is held up by a bounded spin, and the memory that the pot is likely to get held other bytes before:
     counters that were cleared behind the spin would not be zero when the pot's own kernels run."""
     cfg = inputs.small_config(cfg_id=960, pot_size=2000, keep=900, nuc_slots=300, cap_rows=16, Hq=8, Hkv=4, d=d, dtype=dtype, layers=2, batch=2)
@@ -29,8 +30,10 @@ def test_pot_on_its_own_stream_while_the_default_stream_is_busy(d, dtype):
     held.record()
     h = ipot.ipot_create_ex(cfg.pot_size, cfg.keep, cfg.layers, cfg.Hq, cfg.Hkv, d, batch=cfg.batch,
                             dtype=ipot.IPOT_F32 if dtype == "f32" else ipot.IPOT_BF16, nuc_slots=cfg.nuc_slots, max_cap_rows=cfg.cap_rows,
-                            stream=s.cuda_stream)
+                            stream=None if handed_over else s.cuda_stream)
     try:
+        if handed_over:
+            ipot.ipot_set_stream(h, s.cuda_stream)
         with torch.cuda.stream(s):
             for _ in range(2):
                 ipot.ipot_reset(h)
@@ -109,6 +112,7 @@ def test_captured_pass_replays_on_other_inputs(d, dtype, layers, n, rope):
         one_pass(h)
         results(h)
         with torch.cuda.graph(graph, stream=s):
+            ipot.ipot_set_stream(h, s.cuda_stream)
             one_pass(h)
         for i, replay in ((1, True), (0, True), (1, True), (0, False), (1, False), (0, True), (1, True), (0, False)):
             load(i)
