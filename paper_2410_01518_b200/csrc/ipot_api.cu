@@ -239,7 +239,8 @@ int launch_simt(ipot *p, const void *Q, const float2 *cap_stats, int M, int N)
     return IPOT_OK;
 }
 
-// f32 pots: every logit computed once, unless one unit's logits exceed the scratch (M * N above 16 million)
+// f32 pots: every logit computed once, unless one unit's logits exceed the scratch (M * N above 14.9 million: 4.5 bytes each) or it
+// did not fit into the device's memory
 int launch_f32(ipot *p, const void *Q, const float2 *cap_stats, int M, int N)
 {
     if (!f32_applicable(p->f32, M, N)) return launch_simt<float>(p, Q, cap_stats, M, N);
@@ -632,10 +633,27 @@ int ipot_create_ex(const ipot_config_t *cfg, ipot_t **out)
     alloc(&p->stage_q, (size_t)p->units * maxM * p->row_bytes);
     alloc(&p->stage_kc, (size_t)p->units * cfg->max_cap_rows * p->row_bytes);
     alloc((void **)&p->stage_aux, (size_t)cfg->batch * cfg->pot_size * 4);
+    // The scratch of the faster scorers comes last: where it does not fit any more a pot does without, the item and f32 scorers'
+    // first (6 to 25 % of a bf16 pot of many query rows), then the one-sweep scorer's.
+    const int without_tc = mem.n;
     tc_plan_init(p->tc, p->cfg, p->sm_count, mem);
+    const int without_tw = mem.n;
     tw_plan_init(p->tw, p->tc, p->cfg, p->sm_count, mem);
     if (cfg->dtype == IPOT_F32) f32_plan_init(p->f32, p->units, maxM, cfg->pot_size, mem);
     bool ok = mem.allocate(&p->arena, p->side);
+    if (!ok && !p->arena && mem.n > without_tw) {
+        cudaGetLastError();
+        mem.n = without_tw;
+        p->tw.usable = false;
+        p->f32 = F32Plan();
+        ok = mem.allocate(&p->arena, p->side);
+    }
+    if (!ok && !p->arena && mem.n > without_tc) {
+        cudaGetLastError();
+        mem.n = without_tc;
+        p->tc.usable = false;
+        ok = mem.allocate(&p->arena, p->side);
+    }
     if (!ok) {
         cudaGetLastError();
         free_all(p);
