@@ -79,8 +79,8 @@ enum {
                                 only: IPOT_E_INVALID if the shape does not allow it */
     IPOT_SCORER_TENSOR_ITEMS = 5 /* tcgen05 kernel in two sweeps whose pieces are dealt to the SMs one by one (bf16, any
                                 d, at most 1024 folded query rows): what AUTO takes for head dimensions other than
-                                64 and 128, and for long units if there are many; IPOT_E_INVALID if the
-                                shape does not allow it */
+                                64 and 128, and for long units if there are many; IPOT_E_INVALID if the shape does not
+                                allow it (or its scratch did not fit into the device's memory) */
 };
 
 typedef struct {
@@ -243,8 +243,8 @@ int ipot_score_and_compress_cap_host(ipot_t *pot, const void *Q_cap_host, const 
  * be written straight into the aux_scores array of the next ipot_score_and_compress call.
  *   logits       : device, [batch][n_tokens] rows of `vocab` values, `row_stride` elements apart
  *                  (row_stride >= vocab), of type logits_dtype (IPOT_BF16 or IPOT_F32; need not be the
- *                  pot's type); rows that start on a 16-byte boundary are read with 16-byte loads,
- *                  others element by element.  Caller-owned, read-only.
+ *                  pot's type); read with 16-byte loads wherever a row starts.  Masked entries may be
+ *                  -inf or the type's lowest value.  Caller-owned, read-only.
  *   labels       : device, [batch][n_tokens] int32 token ids; a negative id marks an ignored position
  *                  (novelty 0); an id >= vocab also gives 0 and raises the sticky status IPOT_E_BOUNDS.
  *   aux_out      : device fp32; token t of stream b goes to aux_out[b * aux_stride + slot0 + t], i.e.
