@@ -12,34 +12,33 @@
 //   tcgen05  S = Q K^T (128 x 256 fp32) accumulates in one of two 256-column tensor
 //            memory buffers, one 128-column half at a time: the logits never leave
 //            the SM;
-//   pass 1   (16 epilogue warps; a thread owns one query row x two chunks of 32 columns,
-//            one in each half of the buffer) per chunk: maximum, e = 2^(x - max)
-//            written back over the logits, sum - one tensor-memory read and one
-//            write per logit; a quarter of the exponentials run on the FMA pipe; the chunks move
-//            through two sets of 16 registers, the second chunk's first half being fetched behind the
-//            exponentials of the first chunk's second half;
-//   combine  (4 warps, one thread per query row) merges the eight (max, sum) pairs of
-//            its row into the slab's statistics and publishes them with one 8-byte
-//            store whose sum carries the launch's sign as a "fresh" mark; then reads
-//            the row's statistics of all slabs of the item, re-reading until every
-//            one is fresh, and turns them into the row's global maximum m, its
-//            denominator l (plus, when given, the share of the CaP's own keys) and the
-//            weights 2^(max_chunk - m) / l of the stored e values;
-//   pass 2   (the same 16 warps, one task behind: after pass 1 of task t+1 they
-//            finish task t, whose weights have arrived meanwhile)
-//            u_j = sum_i e_ij 2^(max_i - m_i) / l_i as a weighted column sum: the
-//            16x256b tensor-memory load shape hands every thread four rows of a
-//            column pair, so the sum over a warp's 32 rows is four packed FMAs plus
-//            a three-step exchange between lanes; the four warps that own the same
-//            columns add their row quarters through shared memory (their own
-//            128-thread barrier) and store: 256 floats per task.
-// The two 128-column halves of a buffer are handed over separately (MMA -> pass 1,
-// pass 2 -> MMA), so the tensor core refills one half while the other is still read.
+//   epilogue (16 warps in four groups, a group per 128 columns of tensor memory; groups 0, 1 have the CTA's even
+//            tasks, 2, 3 the odd ones, so that one pair computes while the other waits for the exchange)
+//     pass 1   a thread owns one query row: e = 2^x is written back over the logits and summed, against the reference
+//              0 - no maximum is taken unless a warp's sums then leave the comfortable range; a quarter of the
+//              exponentials run on the FMA pipe.  The warps of a scheduler take pass 1 in turns, pair after pair: both
+//              pairs at once finish later than one of them could, and every reader of their sums waits;
+//     exchange the thread publishes its row's sum over the 128 keys with one 4-byte store that carries the launch's
+//              sign as a "fresh" mark, reads half of the row's sums of the whole item (the other group of the pair reads
+//              the other half), re-reading until every one is fresh, and turns them into the row's denominator
+//              l (plus, when given, the share of the CaP's own keys);
+//     pass 2   u_j = sum_i e_ij / l_i as a weighted column sum: the 16x256b tensor-memory load shape hands every
+//              thread four rows of a column pair, so the sum over a warp's 32 rows is four packed FMAs plus a
+//              three-step exchange between lanes; the four row quarters meet in shared memory and are added and
+//              stored behind the next task's barrier: 256 floats per task.
+// A row block of fewer rows keeps the warps of its empty quarters out of all of this.
+//
+// Bound: a task's way through tensor memory - product 700 cycles, pass 1 3000 to 4000 beside the other pair's
+// work, exchange 3500, pass 2 1700 - and tensor memory holds two tasks.  (Pass 1 and pass 2 alone would take an SM 2500 cycles per
+// task, without the exchange the launch takes 66 us.)  Measured against the form before, in which all 16 warps
+// shared a task, took maxima, and four more warps combined and polled (us, alone): 256 units x 4096 keys, M = 128 90.1 -> 85.2; 128 x
+// 8192, M = 256 197 -> 173; 60 x 2999, M = 57 20.8 -> 18.5; 64 x 16384, M = 512 537 -> 384.  Error of the scores against
+// 64 bits 4.5e-7 -> 1.6e-7 (fewer roundings, a polynomial of degree 5, the tensor core's cut sums made good).
 //
 // Blocks of one grid wait on each other (pass 2 needs the other slabs' statistics),
 // so the grid is launched cooperatively with at most one CTA per SM: all of it is
-// resident.  A CTA publishes pass 1 of task t+1 before it waits for task t, so the
-// waits cannot form a cycle.  Every wait (mbarrier or statistics) is bounded by a time
+// resident.  A pair publishes its task before it waits for others, and takes its tasks in
+// order, so the waits cannot form a cycle.  Every wait (mbarrier or statistics) is bounded by a time
 // limit (a launch parameter); one that runs out records IPOT_E_TIMEOUT in the status
 // word and raises a block-wide flag.  From then on every wait of the block returns at
 // once: the producer and the MMA issuer stop putting work in flight and wait for what
@@ -57,8 +56,13 @@
 
 namespace ipotk {
 
-constexpr int kTcThreads = 704;      // warp 0: TMA, 1: MMA + TMEM owner, 2-17: pass 1 / pass 2, 18-21: combine
+constexpr int kTcThreads = 576;      // warp 0: TMA, 1: MMA + TMEM owner, 2-17: epilogue, four groups of four warps
 constexpr int kTcRows = 128;         // query rows per item (TMEM lanes)
+constexpr int kTcHalf = 128;         // keys per epilogue group and entry of the statistics
+// The first look at a task's statistics comes this much after its own have left: the others' are never there at once, and what is not
+// polled leaves L2 to the keys.  Measured (256 units x 4096 keys, M = 128 / 128 x 8192, M = 256, us): 0 ns 88.6 / 175.1, 300 85.2 / 172.7,
+// 600 85.8 / 180.5; a CTA's first task (all there is in a small launch) does not wait (8 units x 4096: 8.3, 8.4, 10.1).
+constexpr unsigned kTcPollDelayNs = 300;
 constexpr int kTcSlab = 256;         // keys per task (TMEM columns per buffer)
 constexpr int kTcFmaEighths = 2;     // share of pass 1's exponentials evaluated on the FMA pipe
 constexpr int kTcD = 128;            // largest head dimension; 64 uses the first 64-channel half of every tile
@@ -68,27 +72,28 @@ constexpr uint32_t kTcStageBytes = kTcQBytes + kTcKBytes;    // 96 KiB
 
 // shared-memory carve-up (bytes from the 1024-aligned base)
 constexpr uint32_t kTcOffStage = 0;                                        // [2] { Q, K }
-constexpr uint32_t kTcOffColpart = 2 * kTcStageBytes;                      // [2 parities][4 row quarters][256] float
-constexpr uint32_t kTcOffTstat = kTcOffColpart + 2 * 4 * kTcSlab * 4;          // [2 buffers][8 chunks][128] float2
-constexpr uint32_t kTcOffFbuf = kTcOffTstat + 2 * 8 * kTcRows * 8;         // [2 buffers][8 chunks][128] float
-constexpr uint32_t kTcOffBar = kTcOffFbuf + 2 * 8 * kTcRows * 4;
+constexpr uint32_t kTcOffColpart = 2 * kTcStageBytes;                      // [4 groups][2 parities][4 row quarters][128] float
+constexpr uint32_t kTcOffLpart = kTcOffColpart + 4 * 2 * 4 * kTcHalf * 4;      // [2 pairs][2 parities][2 halves][128] float
+constexpr uint32_t kTcOffBar = kTcOffLpart + 2 * 2 * 2 * kTcRows * 4;
 constexpr uint32_t kTcOffTmemSlot = kTcOffBar + 192;                       // the allocated TMEM base address
 constexpr uint32_t kTcOffAbort = kTcOffBar + 196;                          // set once a wait of the CTA has run out; + 4: the block's deadline (8 bytes)
 constexpr uint32_t kTcSmemBytes = kTcOffBar + 256;                         // no static shared memory: the base is 1024-aligned
 
-// barriers: per stage Full, Empty, EReady, FReady; per (buffer, half) SFull, TEmpty at index 2 * buffer + half
-enum { kBarFull = 0, kBarEmpty = 2, kBarEReady = 4, kBarFReady = 6, kBarSFull = 8, kBarTEmpty = 12, kBarDrain = 16, kBarCount = 17 };
+// barriers: per stage Full, Empty; per group (= buffer half 2 * buffer + half) SFull, TEmpty
+enum { kBarFull = 0, kBarEmpty = 2, kBarSFull = 4, kBarTEmpty = 8, kBarDrain = 12, kBarCount = 13 };
 
 struct TcParams {
     float *scores;        // partial array p (query rows 128p ...) at scores + p * part_stride, unit stride N
     size_t part_stride;
-    float2 *stats;        // [items][slabs][128] (max in log2 units, sum * sign); all of the other sign or 0 at launch
+    float *stats;         // [items][entries][128] a row's sum over 128 keys, times the launch's sign (infinite: its reference is not 0, see
+                          // refs); all of the other sign or 0 at launch
+    float2 *refs;         // [items][entries][128] (reference, sum) of those
     const float2 *cap_stats;  // NULL, or [units][M] (max, sum) over the CaP's own keys that join every row's denominator
     float sign;           // +1 or -1: this launch's "fresh" mark
     unsigned long long wait_ns;  // limit of every wait
     int withhold_cta;     // -1; test hook: this CTA never publishes its slab statistics
     int *status;
-    int N, M, mtiles, slabs, tasks;
+    int N, M, mtiles, slabs, entries, tasks;
     int dhalves;          // d / 64: 64-channel halves of a tile (1 or 2)
     int new_slab0;        // slabs from this one on are read through the second key map (the chunk of a deferred
                           // append, row 0 = key 256 * new_slab0); INT_MAX if all keys are in the pot
@@ -259,28 +264,35 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Named barrier of the four epilogue warps (one per TMEM lane quarter) that own the same columns.
-// (Barrier numbers are immediates so that the kernel claims five of the SM's barriers, not all sixteen.)
-__device__ __forceinline__ void column_group_sync(int cq)
+// Named barriers: of the four warps of an epilogue group, and of the two groups that share a buffer.
+// (Barrier numbers are immediates so that the kernel claims seven of the SM's barriers, not all sixteen.)
+__device__ __forceinline__ void group_sync(int g)
 {
-    switch (cq) {
+    switch (g) {
     case 0: asm volatile("bar.sync 1, 128;" ::: "memory"); break;
     case 1: asm volatile("bar.sync 2, 128;" ::: "memory"); break;
     case 2: asm volatile("bar.sync 3, 128;" ::: "memory"); break;
     default: asm volatile("bar.sync 4, 128;" ::: "memory"); break;
     }
 }
-// The slab statistics are exchanged between CTAs with single 8-byte relaxed accesses at gpu scope:
-// one store publishes (max, marked sum) together, and a reader sees either the old or the new pair.
-__device__ __forceinline__ float2 ld_gpu_f32x2(const float2 *p)
+__device__ __forceinline__ void pair_sync(int pair)
 {
-    float2 v;
-    asm volatile("ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+    if (pair == 0) asm volatile("bar.sync 5, 256;" ::: "memory");
+    else asm volatile("bar.sync 6, 256;" ::: "memory");
+}
+// Turns: the warps of a TMEM lane quarter (= scheduler) of one pair take pass 1 after those of the other pair have done theirs.
+__device__ __forceinline__ void turn_wait(int pair, int q) { asm volatile("bar.sync %0, 128;" ::"r"(7 + pair * 4 + q) : "memory"); }
+__device__ __forceinline__ void turn_pass(int pair, int q) { asm volatile("bar.arrive %0, 128;" ::"r"(11 - pair * 4 + q) : "memory"); }
+// The statistics are exchanged between CTAs with relaxed accesses at gpu scope: a reader sees the old or the new value of each entry.
+__device__ __forceinline__ float ld_gpu_f32(const float *p)
+{
+    float v;
+    asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ void st_gpu_f32x2(float2 *p, float a, float b)
+__device__ __forceinline__ void st_gpu_f32(float *p, float v)
 {
-    asm volatile("st.relaxed.gpu.global.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
+    asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
 }
 __device__ __forceinline__ float ex2(float x)
 {
@@ -295,88 +307,152 @@ __device__ __forceinline__ float max3(float a, float b, float c)
     return y;
 }
 
-// Maximum of 32 logits folded into four independent running maxima (no long dependency chain).
-template <bool kFull>
-__device__ __forceinline__ void chunk_max(const uint32_t (&v)[32], int col0, int nvalid, float (&mx)[4])
-{
-    if (kFull) {
-#pragma unroll
-        for (int i = 0; i < 32; i += 8) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) mx[j] = max3(mx[j], __uint_as_float(v[i + 2 * j]), __uint_as_float(v[i + 2 * j + 1]));
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-            if (col0 + i < nvalid) mx[i & 3] = fmaxf(mx[i & 3], __uint_as_float(v[i]));
+// 16 columns against the reference 0: v <- 2^(v c), added into two packed running sums; pm: the largest logit among those that went
+// to the FMA pipe, whose exponent arithmetic wraps around where the special-function unit returns +inf.
+struct PieceSum {
+    float2 s[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    float pm = -INFINITY;
+    __device__ __forceinline__ float total() const
+    {
+        const float2 t = __fadd2_rn(s[0], s[1]);
+        return t.x + t.y;
     }
-}
-
-// v <- 2^(v c - mxc) (0 beyond nvalid); the new values are also added into four packed running sums.
-// kTcFmaEighths of every eight pairs are evaluated on the FMA pipe (relative error 2.7e-6, values below 2^-126
-// come out as subnormal bit patterns that pass 2 multiplies like any other number): measured on the
-// 256-unit 4096-key launch, 2 eighths 86.2 us, none 87.7, 3 eighths 86.8, 4 eighths 89.9.
-template <bool kFull>
-__device__ __forceinline__ void chunk_exp(uint32_t (&v)[32], int col0, int nvalid, float c, float mxc, float2 (&sum)[4])
+};
+__device__ __forceinline__ void piece_exp(uint32_t (&v)[16], float c, PieceSum &p)
 {
-    const float2 c2 = make_float2(c, c), nm2 = make_float2(-mxc, -mxc);
-#pragma unroll
-    for (int i = 0; i < 32; i += 2) {
-        const float2 x = __ffma2_rn(make_float2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), c2, nm2);
-        float2 e2 = pair_on_fma<kTcFmaEighths>(i >> 1) ? exp2_fma_pair(x) : make_float2(ex2(x.x), ex2(x.y));
-        if (!kFull) {
-            if (col0 + i >= nvalid) e2.x = 0.f;
-            if (col0 + i + 1 >= nvalid) e2.y = 0.f;
-        }
-        sum[(i >> 1) & 3] = __fadd2_rn(sum[(i >> 1) & 3], e2);
-        v[i] = __float_as_uint(e2.x);
-        v[i + 1] = __float_as_uint(e2.y);
-    }
-}
-
-// Pass 1 for one query row over one chunk of 32 columns (slab columns from col0): returns the chunk's
-// maximum (log2 units) and the sum of e = 2^(x - max), and leaves e in tensor memory.  With no valid column
-// the maximum is -inf, the sum 0 and zeros are stored.
-template <bool kFull>
-__device__ __forceinline__ float2 pass1_chunk(uint32_t taddr, int col0, int nvalid, float c)
-{
-    uint32_t v[32];
-    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-    tmem_ld32(taddr, v);
-    tmem_wait_ld(v);
-    chunk_max<kFull>(v, col0, nvalid, mx);
-    const float mxr = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-    const float mxc = (mxr == -INFINITY) ? 0.f : mxr * c;
-    float2 sum[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    chunk_exp<kFull>(v, col0, nvalid, c, mxc, sum);
-    tmem_st32(taddr, v);
-    const float2 s01 = __fadd2_rn(sum[0], sum[1]), s23 = __fadd2_rn(sum[2], sum[3]);
-    return make_float2((mxr == -INFINITY) ? -INFINITY : mxc, (s01.x + s01.y) + (s23.x + s23.y));
-}
-
-// The same over 16 columns of a full chunk: maximum into four running maxima / exponentials into four packed sums.
-// `first_pair`: index of the piece's first column pair within its chunk (it fixes which pairs take the FMA pipe).
-__device__ __forceinline__ void piece_max(const uint32_t (&v)[16], float (&mx)[4])
-{
-#pragma unroll
-    for (int i = 0; i < 16; i += 8) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) mx[j] = max3(mx[j], __uint_as_float(v[i + 2 * j]), __uint_as_float(v[i + 2 * j + 1]));
-    }
-}
-template <int kFirstPair>
-__device__ __forceinline__ void piece_exp(uint32_t (&v)[16], float c, float mxc, float2 (&sum)[4])
-{
-    const float2 c2 = make_float2(c, c), nm2 = make_float2(-mxc, -mxc);
+    const float2 c2 = make_float2(c, c);
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
-        const float2 x = __ffma2_rn(make_float2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), c2, nm2);
-        const float2 e2 = pair_on_fma<kTcFmaEighths>(kFirstPair + (i >> 1)) ? exp2_fma_pair(x) : make_float2(ex2(x.x), ex2(x.y));
-        sum[(i >> 1) & 3] = __fadd2_rn(sum[(i >> 1) & 3], e2);
+        const float2 x = make_float2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), t = __fmul2_rn(x, c2);
+        float2 e2;
+        if (pair_on_fma<kTcFmaEighths>(i >> 1)) {
+            p.pm = max3(p.pm, x.x, x.y);
+            e2 = exp2_fma_pair5(t);
+        } else {
+            e2 = make_float2(ex2(t.x), ex2(t.y));
+        }
+        p.s[(i >> 1) & 1] = __fadd2_rn(p.s[(i >> 1) & 1], e2);
         v[i] = __float_as_uint(e2.x);
         v[i + 1] = __float_as_uint(e2.y);
     }
 }
+constexpr float kTcSumMax = 1.2676506e30f;    // 2^100
+constexpr float kTcSumMin = 9.0949470e-13f;   // 2^-40: nothing above 2^-86 of the sum is lost to flushing
+constexpr float kTcReach = 100.f;
+constexpr float kTcTiny = 1.1754944e-38f;     // an entry that adds nothing is still not 0
+
+// Pass 1 for a warp some of whose rows left the comfortable range: the first `done` pieces of 16 columns have been stored as 2^(x c);
+// everything is brought to the reference that the rest needs.  (reference, sum)
+__device__ __noinline__ float2 pass1_slow(uint32_t taddr, int done, int nvalid, float c)
+{
+    float mx = -INFINITY;
+    tmem_wait_st();
+#pragma unroll 1
+    for (int i = done; 16 * i < nvalid; ++i) {
+        uint32_t v[16];
+        tmem_ld16(taddr + 16 * i, v);
+        tmem_wait_ld16(v);
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+            if (16 * i + e < nvalid) mx = fmaxf(mx, __uint_as_float(v[e]));
+    }
+    float m = mx * c;
+    if (done) m = fmaxf(m, 0.f);
+    if (m == -INFINITY) m = 0.f;   // every logit beyond fp32's range
+    const float down = ex2(-m);
+    float s = 0.f;
+#pragma unroll 1
+    for (int i = 0; 16 * i < nvalid; ++i) {
+        uint32_t v[16];
+        tmem_ld16(taddr + 16 * i, v);
+        tmem_wait_ld16(v);
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const float x = __uint_as_float(v[e]);
+            const float y = i < done ? x * down : 16 * i + e < nvalid ? ex2(fmaf(x, c, -m)) : 0.f;
+            a[e & 3] += y;
+            v[e] = __float_as_uint(y);
+        }
+        s += (a[0] + a[1]) + (a[2] + a[3]);
+        tmem_st16(taddr + 16 * i, v);
+    }
+    return make_float2(m, s);
+}
+// Pass 1 where only the first nvalid (1 .. 127) of the 128 columns hold keys
+__device__ __noinline__ float2 pass1_ragged(uint32_t taddr, int nvalid, float c)
+{
+    float s = 0.f;
+#pragma unroll 1
+    for (int i = 0; 16 * i < nvalid; ++i) {
+        uint32_t v[16];
+        tmem_ld16(taddr + 16 * i, v);
+        tmem_wait_ld16(v);
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const float y = 16 * i + e < nvalid ? ex2(__uint_as_float(v[e]) * c) : 0.f;
+            a[e & 3] += y;
+            v[e] = __float_as_uint(y);
+        }
+        s += (a[0] + a[1]) + (a[2] + a[3]);
+        if (!__all_sync(0xffffffffu, s >= kTcSumMin && s <= kTcSumMax)) return pass1_slow(taddr, i, nvalid, c);
+        tmem_st16(taddr + 16 * i, v);
+    }
+    return make_float2(0.f, s);
+}
+// Sum of n (up to 16) of a row's entries, re-read until each carries the launch's mark.  Only what is still stale is read again: the polls
+// of all CTAs together are a large part of what L2 delivers (all of it again, in 16-byte loads of a transposed array: 109 us against 90).
+__device__ __forceinline__ float poll_entries(const float *st, int n, float sgn, volatile int *ab, int *status)
+{
+    float v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = e < n ? 0.f : kTcTiny * sgn;
+    for (uint32_t tries = 1;; ++tries) {
+        bool fresh = true;
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+            if (!(v[e] * sgn > 0.f)) v[e] = ld_gpu_f32(st + (size_t)e * kTcRows);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) fresh = fresh && v[e] * sgn > 0.f;
+        if (fresh) break;
+        if ((tries & 63u) == 0 && (*ab || global_timer_ns() > *reinterpret_cast<volatile unsigned long long *>(ab + 1))) {
+            if (!*ab) {
+                *ab = 1;
+                set_status(status, kStatusTimeout);
+            }
+            break;
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = fabsf(v[e]);
+#pragma unroll
+    for (int step = 1; step < 16; step <<= 1) {
+#pragma unroll
+        for (int e = 0; e < 16; e += 2 * step) v[e] += v[e + step];
+    }
+    return v[0];
+}
+// A row's denominator when some entry's reference is not 0: all entries in order, relative to the largest reference
+__device__ __noinline__ float2 merge_entries(const float *st, const float2 *refs, int entries)
+{
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    float m = -INFINITY, l = 0.f;
+#pragma unroll 1
+    for (int e = 0; e < entries; ++e) {
+        const float v = fabsf(ld_gpu_f32(st + (size_t)e * kTcRows));
+        float2 t = make_float2(0.f, v);
+        if (v == INFINITY) {
+            const float *r = reinterpret_cast<const float *>(refs + (size_t)e * kTcRows);
+            t = make_float2(ld_gpu_f32(r), ld_gpu_f32(r + 1));
+        } else if (v <= kTcTiny) continue;   // an empty entry's reference does not count
+        const float mn = fmaxf(m, t.x);
+        l = (m == -INFINITY ? 0.f : l * ex2(m - mn)) + t.y * ex2(t.x - mn);
+        m = mn;
+    }
+    return m == -INFINITY ? make_float2(0.f, kTcTiny) : make_float2(m, l);
+}
+
 // Pass 2 for one warp over 32 rows x 32 columns: a[] and b[] are the 16x256b loads of the warp's TMEM lanes
 // 0..15 and 16..31, fr2[i] the weight of row lane/4 + 8i duplicated into both halves.  On exit
 // x[2j + h] = sum over this thread's four rows of f_r e[r][8j + 2(lane%4) + h].
@@ -446,7 +522,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
     int &abort_flag = *reinterpret_cast<int *>(gbase + kTcOffAbort);
     const uint32_t bar0 = base + kTcOffBar;
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (uniform: what follows from it lives in uniform registers)
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -454,12 +530,10 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar(kBarFull + b), 1);
             mbar_init(bar(kBarEmpty + b), 1);
-            mbar_init(bar(kBarEReady + b), 512);
-            mbar_init(bar(kBarFReady + b), 128);
-            for (int h = 0; h < 2; ++h) {
-                mbar_init(bar(kBarSFull + 2 * b + h), 1);
-                mbar_init(bar(kBarTEmpty + 2 * b + h), 512);
-            }
+        }
+        for (int g = 0; g < 4; ++g) {
+            mbar_init(bar(kBarSFull + g), 1);
+            mbar_init(bar(kBarTEmpty + g), 4);
         }
         mbar_init(bar(kBarDrain), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -510,6 +584,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         const bool leader = elect_one();
         const uint64_t q_desc = smem_desc_sw128(base + kTcOffStage), k_desc = smem_desc_sw128(base + kTcOffStage + kTcQBytes);
         uint32_t k = 0;
+        bool any = false;
         for (int task = blockIdx.x; task < prm.tasks; task += prm.ctas, ++k) {
             const uint32_t b = k & 1, ph = (k >> 1) & 1;
             if (!__all_sync(0xffffffffu, mbar_wait(bar(kBarFull + b), ph, ab, prm.status))) break;
@@ -517,6 +592,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             for (uint32_t h = 0; h < 2; ++h) {
                 ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarTEmpty + 2 * b + h), ph ^ 1, ab, prm.status));
                 if (!ok) break;
+                any = true;
                 tc_fence_after();
                 const uint64_t da = q_desc + b * (kTcStageBytes >> 4), db = k_desc + b * (kTcStageBytes >> 4) + h * (128 * 128 >> 4);
                 const uint32_t d = tmem + b * kTcSlab + h * 128;
@@ -535,220 +611,186 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             }
             if (!ok) break;
         }
-        if (k) {  // every MMA has finished (and read its operands) before tensor memory is released
+        if (any) {  // every MMA has finished (and read its operands) before tensor memory is released
             if (leader) tc_commit(bar(kBarDrain));
             mbar_wait(bar(kBarDrain), 0, ab, prm.status, false);
         }
         __syncwarp();
-    } else if (warp < 18) {
-        // ---------------------------------------------------------------- pass 1 / pass 2 (512 threads)
+    } else {
+        // ---------------------------------------------------------------- epilogue: groups 0, 1 have the even tasks, 2, 3 the odd ones
         const int q = warp & 3;                 // TMEM lane quarter this warp may touch
-        const int w = warp - 2;                 // 0..15
-        const int cq = w >> 2;                  // this warp's columns: [32 cq, 32 cq + 32) of each buffer half
+        const int g = (warp - 2) >> 2;          // group: buffer g >> 1, columns 128 (g & 1) ... of it
+        const int pair = g >> 1, half = g & 1;
         const int row = q * 32 + lane;
-        float2 *tstat = reinterpret_cast<float2 *>(gbase + kTcOffTstat);
-        const float *fbuf = reinterpret_cast<const float *>(gbase + kTcOffFbuf);
-        float *colpart = reinterpret_cast<float *>(gbase + kTcOffColpart);
-        const float c = prm.scale_log2e;
-        const int n_local = (prm.tasks - (int)blockIdx.x + prm.ctas - 1) / prm.ctas;
-        for (int k = 0; k <= n_local; ++k) {
-            if (k < n_local) {
-                // ---- pass 1 of local task k
-                const int task = blockIdx.x + k * prm.ctas;
-                const int slab = task % tasks_per_item;
-                const int nvalid = min(kTcSlab, prm.N - slab * kTcSlab);
-                const uint32_t b = k & 1, ph = (k >> 1) & 1;
-                const uint32_t t0 = tmem + ((uint32_t)(q * 32) << 16) + b * kTcSlab + cq * 32;
-                if (nvalid == kTcSlab) {
-                    // two chunks of 32 columns (one per buffer half) in four pieces of 16 through two register sets:
-                    // the second half's first piece is fetched while the first half's second piece is still being
-                    // exponentiated, so that its tensor-memory latency is not waited for
-                    uint32_t X[16], Y[16];
-                    mbar_wait(bar(kBarSFull + 2 * b), ph, ab, prm.status);
-                    tc_fence_after();
-                    tmem_ld16(t0, X);
-                    tmem_ld16(t0 + 16, Y);
-                    tmem_wait_ld16(X);
-                    tmem_wait_ld16(Y);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                        piece_max(X, mx);
-                        piece_max(Y, mx);
-                        const float mxc = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c;
-                        float2 sum[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-                        piece_exp<0>(X, c, mxc, sum);
-                        tmem_st16(t0 + h * 128, X);
-                        // the second half's logits: fetched behind the next piece's exponentials if the tensor core has
-                        // delivered them by now (lane 0's answer for the whole warp: a phase that is complete stays complete)
-                        const bool early = h == 0 && __shfl_sync(0xffffffffu, mbar_test_wait(bar(kBarSFull + 2 * b + 1), ph) ? 1 : 0, 0);
-                        if (early) {
-                            tc_fence_after();
-                            tmem_ld16(t0 + 128, X);
-                        }
-                        piece_exp<8>(Y, c, mxc, sum);
-                        tmem_st16(t0 + h * 128 + 16, Y);
-                        if (h == 0) {
-                            if (!early) {
-                                mbar_wait(bar(kBarSFull + 2 * b + 1), ph, ab, prm.status);
-                                tc_fence_after();
-                                tmem_ld16(t0 + 128, X);
-                            }
-                            tmem_ld16(t0 + 128 + 16, Y);
-                        }
-                        const float2 s01 = __fadd2_rn(sum[0], sum[1]), s23 = __fadd2_rn(sum[2], sum[3]);
-                        tstat[(b * 8 + h * 4 + cq) * kTcRows + row] = make_float2(mxc, (s01.x + s01.y) + (s23.x + s23.y));
-                        if (h == 0) {
-                            tmem_wait_ld16(X);
-                            tmem_wait_ld16(Y);
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        mbar_wait(bar(kBarSFull + 2 * b + h), ph, ab, prm.status);
-                        tc_fence_after();
-                        tstat[(b * 8 + h * 4 + cq) * kTcRows + row] = pass1_chunk<false>(t0 + h * 128, h * 128 + cq * 32, nvalid, c);
-                    }
-                }
-                tmem_wait_st();
-                tc_fence_before();  // pass 2 reads these TMEM words from other lanes of the warp
-                mbar_arrive(bar(kBarEReady + b));
-            }
-            if (k >= 1) {
-                // ---- pass 2 of local task k - 1
-                const int kk = k - 1;
-                const int task = blockIdx.x + kk * prm.ctas;
-                const int item = task / tasks_per_item, slab = task - item * tasks_per_item;
-                const int unit = item / prm.mtiles, mt = item - unit * prm.mtiles;
-                const int nvalid = min(kTcSlab, prm.N - slab * kTcSlab);
-                const uint32_t b = kk & 1, ph = (kk >> 1) & 1;
-                const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + b * kTcSlab + cq * 32;
-                mbar_wait(bar(kBarFReady + b), ph, ab, prm.status);
+        const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + g * kTcHalf;
+        float *lpart = reinterpret_cast<float *>(gbase + kTcOffLpart) + pair * (4 * kTcRows);
+        float *colpart = reinterpret_cast<float *>(gbase + kTcOffColpart) + g * (8 * kTcHalf);
+        const float c = prm.scale_log2e, sgn = prm.sign;
+        const int E = prm.entries, mid = (E + 1) >> 1;
+        // task -> (unit, row block, slab) is counted on from task to task: three divisions at the head of each were 250 ns of a pair's cycle
+        const int step = 2 * prm.ctas, dslab = step % tasks_per_item, ditem = step / tasks_per_item, dmt = ditem % prm.mtiles, dunit = ditem / prm.mtiles;
+        const int task0 = blockIdx.x + pair * prm.ctas;
+        int slab = task0 % tasks_per_item, item = task0 / tasks_per_item, mt = item % prm.mtiles, unit = item / prm.mtiles;
+        float *out = nullptr;                   // where this thread's score of the task before goes
+        int out_rows = 0;
+        auto store = [&](uint32_t par) {        // adds the row quarters
+            if (!out) return;
+            const float *cp = colpart + par * 4 * kTcHalf + row;
+            *out = out_rows > 96 ? (cp[0] + cp[kTcHalf]) + (cp[2 * kTcHalf] + cp[3 * kTcHalf])
+                   : out_rows > 64 ? (cp[0] + cp[kTcHalf]) + cp[2 * kTcHalf]
+                   : out_rows > 32 ? cp[0] + cp[kTcHalf] : cp[0];
+        };
+        uint32_t j = 0;                         // tasks of this pair so far
+        for (int task = task0; task < prm.tasks; task += step, ++j) {
+            const int rows = min(kTcRows, prm.M - mt * kTcRows), nvalid = min(kTcHalf, prm.N - slab * kTcSlab - half * kTcHalf);
+            const bool works = q * 32 < rows && nvalid > 0;   // (uniform over the warp)
+            const uint32_t par = j & 1;
+            float2 own = make_float2(-INFINITY, 0.f);  // the CaP keys' share of this row's denominator (Appendix B listing)
+            if (prm.cap_stats && row < rows) own = __ldg(&prm.cap_stats[(size_t)unit * prm.M + mt * kTcRows + row]);
+            float *st = prm.stats + (size_t)item * E * kTcRows + row;
+            const int e = 2 * slab + half;      // this group's entry
+            float2 s = make_float2(0.f, 1.f);
+            mbar_wait(bar(kBarSFull + g), par, ab, prm.status);
+            if (pair | j) turn_wait(pair, q);
+            // ---- pass 1: exponentials against the reference 0, written back over the logits, and their sum
+            if (works) {
                 tc_fence_after();
-                float *cpart = colpart + (kk & 1) * (4 * kTcSlab);
+                if (nvalid == kTcHalf) {
+                    // Pieces of 16 columns in two register sets.  A piece is looked at and stored behind the exponentials of the next one: with
+                    // the look straight after its own, every piece waited out its own chain of sums.
+                    uint32_t A[16], B[16];
+                    PieceSum pa, pb;
+                    auto fits = [&](const PieceSum &p) {   // (false for NaN; what the second set adds need not be large)
+                        const float t = p.total();
+                        return __all_sync(0xffffffffu, t <= kTcSumMax && (&p == &pb || t >= kTcSumMin) && p.pm * c <= kTcReach) != 0;
+                    };
+                    int done = 0;
+                    tmem_ld16(tb, A);
+                    tmem_wait_ld16(A);
+                    tmem_ld16(tb + 16, B);
+                    piece_exp(A, c, pa);
+#pragma unroll 1
+                    for (;;) {
+                        tmem_wait_ld16(B);
+                        piece_exp(B, c, pb);
+                        if (!fits(pa)) break;
+                        tmem_st16(tb + 16 * done, A);
+                        if (++done < 7) {
+                            tmem_ld16(tb + 16 * done + 16, A);
+                            tmem_wait_ld16(A);
+                            piece_exp(A, c, pa);
+                        }
+                        if (!fits(pb)) break;
+                        tmem_st16(tb + 16 * done, B);
+                        if (++done == 8) break;
+                        tmem_ld16(tb + 16 * done + 16, B);
+                    }
+                    if (done == 8) s.y = pa.total() + pb.total();
+                    else s = pass1_slow(tb, done, kTcHalf, c);
+                } else {
+                    s = pass1_ragged(tb, nvalid, c);
+                }
+            }
+            if (task + prm.ctas < prm.tasks) turn_pass(pair, q);
+            if (nvalid > 0 && (int)blockIdx.x != prm.withhold_cta) {
+                float *to = st + (size_t)e * kTcRows;
+                if (s.x == 0.f) {
+                    st_gpu_f32(to, s.y == 0.f ? kTcTiny * sgn : s.y * sgn);
+                } else {
+                    float *r = reinterpret_cast<float *>(prm.refs + ((size_t)item * E + e) * kTcRows + row);
+                    st_gpu_f32(r, s.x);
+                    st_gpu_f32(r + 1, s.y);
+                    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+                    st_gpu_f32(to, INFINITY * sgn);
+                }
+            }
+            // ---- the row's entries of the whole item, each half of the pair one half of them
+            float l = 0.f;
+            if (row < rows) {
+                if (j) __nanosleep(kTcPollDelayNs);
+                const int end = half ? E : mid;
+                for (int i = half ? mid : 0; i < end; i += 16) l += poll_entries(st + (size_t)i * kTcRows, end - i, sgn, ab, prm.status);
+            }
+            lpart[(par * 2 + half) * kTcRows + row] = l;
+            if (works) {
+                tmem_wait_st();
+                tc_fence_before();
+            }
+            pair_sync(pair);
+            // ---- the row's weight
+            float weight = 0.f;
+            if (row < rows) {
+                float m = 0.f;
+                l = lpart[(par * 2) * kTcRows + row] + lpart[(par * 2 + 1) * kTcRows + row];
+                if (l == INFINITY) {
+                    const float2 t = merge_entries(st, prm.refs + (size_t)item * E * kTcRows + row, E);
+                    m = t.x;
+                    l = t.y;
+                }
+                if (own.x > -INFINITY) {
+                    const float mb = fmaxf(m, own.x);
+                    l = fmaf(own.y, ex2(own.x - mb), l * ex2(m - mb));
+                    m = mb;
+                }
+                float inv_l;
+                asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv_l) : "f"(l));
+                weight = s.x == m ? inv_l : ex2(s.x - m) * inv_l;
+            }
+            // ---- pass 2: weighted column sums
+            if (works) {
+                tc_fence_after();
+                float2 fr2[4];  // the weights of rows lane/4 + 8i, duplicated for the packed FMAs
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {  // this warp's 32 columns of buffer half h
-                    float2 fr2[4];  // the weights of rows lane/4 + 8i for this chunk, duplicated for the packed FMAs
-                    {
-                        const float *f = fbuf + (b * 8 + h * 4 + cq) * kTcRows + q * 32 + (lane >> 2);
+                for (int i = 0; i < 4; ++i) {
+                    const float f = __shfl_sync(0xffffffffu, weight, (lane >> 2) + 8 * i);
+                    fr2[i] = make_float2(f, f);
+                }
+                const int at = 8 * (lane >> 3) + 2 * (lane & 3) + ((lane >> 2) & 1);
+                float *cp = colpart + (par * 4 + q) * kTcHalf + at;
+                uint32_t va[2][16], vb[2][16];
+                tmem_ld_16x256b_x4(tb, va[0]);
+                tmem_ld_16x256b_x4(tb + (16u << 16), vb[0]);
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) fr2[i] = make_float2(f[8 * i], f[8 * i]);
+                for (int i = 0; i < 4; ++i) {
+                    tmem_wait_ld16(va[i & 1]);
+                    tmem_wait_ld16(vb[i & 1]);
+                    if (i < 3) {
+                        tmem_ld_16x256b_x4(tb + 32 * i + 32, va[(i + 1) & 1]);
+                        tmem_ld_16x256b_x4(tb + 32 * i + 32 + (16u << 16), vb[(i + 1) & 1]);
+                    } else {   // the buffer half may be overwritten by the next task of this group
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar(kBarTEmpty + g));
                     }
                     float x[8];
-                    uint32_t va[16], vb[16];
-                    tmem_ld_16x256b_x4(trow + h * 128, va);
-                    tmem_ld_16x256b_x4(trow + h * 128 + (16u << 16), vb);
-                    tmem_wait_ld16(va);
-                    tmem_wait_ld16(vb);
-                    tc_fence_before();
-                    mbar_arrive(bar(kBarTEmpty + 2 * b + h));   // this half may be overwritten by the task after next
-                    pass2_rows(va, vb, fr2, x);
-                    const float u = pass2_reduce(x, lane);
-                    const int g = lane >> 2, pp = lane & 3;
-                    cpart[q * kTcSlab + h * 128 + cq * 32 + 8 * (g >> 1) + 2 * pp + (g & 1)] = u;
+                    pass2_rows(va[i & 1], vb[i & 1], fr2, x);
+                    cp[32 * i] = pass2_reduce(x, lane);
                 }
-                // ---- add the four row quarters of this column group, store its 64 scores
-                column_group_sync(cq);
-                if (q < 2) {  // warp q = 0 stores the group's columns of half 0, warp q = 1 those of half 1
-                    const int col = q * 128 + cq * 32 + lane;
-                    if (col < nvalid) {
-                        float *out = prm.scores + (size_t)mt * prm.part_stride + (size_t)unit * prm.N + slab * kTcSlab;
-                        out[col] = (cpart[col] + cpart[kTcSlab + col]) + (cpart[2 * kTcSlab + col] + cpart[3 * kTcSlab + col]);
-                    }
-                }
-                // no second barrier: the next task writes the other parity of colpart, and the one after
-                // that is separated from these reads by the next task's barrier
+            } else if (lane == 0) {
+                mbar_arrive(bar(kBarTEmpty + g));
+            }
+            store(par ^ 1);   // the task before: its column sums have been complete since the barrier
+            out = nullptr;
+            if (row < nvalid) {   // (here a key)
+                out = prm.scores + (size_t)mt * prm.part_stride + (size_t)unit * prm.N + slab * kTcSlab + half * kTcHalf + row;
+                out_rows = rows;
+            }
+            slab += dslab;
+            int carry = 0;
+            if (slab >= tasks_per_item) {
+                slab -= tasks_per_item;
+                carry = 1;
+            }
+            item += ditem + carry;
+            mt += dmt + carry;
+            unit += dunit;
+            if (mt >= prm.mtiles) {
+                mt -= prm.mtiles;
+                ++unit;
             }
         }
-    } else {
-        // ---------------------------------------------------------------- combine (128 threads, one per query row)
-        const int row = threadIdx.x - 576;
-        const float2 *tstat = reinterpret_cast<const float2 *>(gbase + kTcOffTstat);
-        float *fbuf = reinterpret_cast<float *>(gbase + kTcOffFbuf);
-        const float sgn = prm.sign;
-        uint32_t k = 0;
-        for (int task = blockIdx.x; task < prm.tasks; task += prm.ctas, ++k) {
-            const int item = task / tasks_per_item, slab = task - item * tasks_per_item;
-            const int mt = item % prm.mtiles;
-            const uint32_t b = k & 1, ph = (k >> 1) & 1;
-            const bool row_valid = mt * kTcRows + row < prm.M;
-            float2 own = make_float2(-INFINITY, 0.f);  // the CaP keys' share of this row's denominator (Appendix B listing)
-            if (prm.cap_stats && row_valid) own = __ldg(&prm.cap_stats[(size_t)(item / prm.mtiles) * prm.M + mt * kTcRows + row]);
-            mbar_wait(bar(kBarEReady + b), ph, ab, prm.status);
-            // ---- merge the eight chunks of the row, publish the slab's statistics
-            // (this warp shares its scheduler with four busy epilogue warps and every task waits for this code: the
-            // loads are issued together and maxima and sums are folded as trees, not as chains)
-            float cm[8], ce[8];
-            {
-                float2 t[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) t[i] = tstat[(b * 8 + i) * kTcRows + row];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) cm[i] = t[i].x;
-                const float ms0 = max3(max3(cm[0], cm[1], cm[2]), max3(cm[3], cm[4], cm[5]), fmaxf(cm[6], cm[7]));  // chunk 0 always holds a valid key
-#pragma unroll
-                for (int i = 0; i < 8; ++i) ce[i] = (cm[i] == -INFINITY) ? 0.f : t[i].y * ex2(cm[i] - ms0);
-            }
-            const float ms = max3(max3(cm[0], cm[1], cm[2]), max3(cm[3], cm[4], cm[5]), fmaxf(cm[6], cm[7]));
-            const float ls = ((ce[0] + ce[1]) + (ce[2] + ce[3])) + ((ce[4] + ce[5]) + (ce[6] + ce[7]));
-            if (tasks_per_item > 1 && (int)blockIdx.x != prm.withhold_cta) st_gpu_f32x2(&prm.stats[((size_t)item * tasks_per_item + slab) * kTcRows + row], ms, ls * sgn);
-
-            // ---- this row's statistics of every slab of the item; re-read until all carry this launch's mark
-            const float2 *st = prm.stats + (size_t)item * tasks_per_item * kTcRows + row;
-            float m = -INFINITY, l = 0.f;
-            if (tasks_per_item == 1) {  // the item is this slab: nothing to exchange
-                m = ms;
-                l = ls;
-            }
-            for (int s0 = 0; s0 < (tasks_per_item > 1 ? tasks_per_item : 0); s0 += 16) {
-                float2 sv[16];
-                uint32_t tries = 0;
-                bool fresh;
-#pragma unroll
-                for (int s = 0; s < 16; ++s)  // beyond the item: neutral and fresh; this CTA's own slab: known; others: stale
-                    sv[s] = (s0 + s >= tasks_per_item) ? make_float2(-INFINITY, sgn) : (s0 + s == slab) ? make_float2(ms, ls * sgn) : make_float2(0.f, 0.f);
-                do {  // only the entries that are still stale are read again
-                    fresh = true;
-#pragma unroll
-                    for (int s = 0; s < 16; ++s) {
-                        if (!(sv[s].y * sgn > 0.f)) sv[s] = ld_gpu_f32x2(&st[(size_t)(s0 + s) * kTcRows]);
-                        fresh = fresh && (sv[s].y * sgn > 0.f);
-                    }
-                    if (!fresh && (*ab || ((++tries & 1023u) == 0 && global_timer_ns() > *reinterpret_cast<volatile unsigned long long *>(ab + 1)))) {
-                        if (!*ab) {
-                            *ab = 1;
-                            set_status(prm.status, kStatusTimeout);
-                        }
-                        break;
-                    }
-                } while (!fresh);
-                const float mb = max3(max3(max3(sv[0].x, sv[1].x, sv[2].x), max3(sv[3].x, sv[4].x, sv[5].x), max3(sv[6].x, sv[7].x, sv[8].x)),
-                                      max3(max3(sv[9].x, sv[10].x, sv[11].x), max3(sv[12].x, sv[13].x, sv[14].x), fmaxf(sv[15].x, m)), -INFINITY);
-                float w[16];
-#pragma unroll
-                for (int s = 0; s < 16; ++s) w[s] = fabsf(sv[s].y) * ex2(sv[s].x - mb);
-#pragma unroll
-                for (int step = 1; step < 16; step <<= 1) {
-#pragma unroll
-                    for (int s = 0; s < 16; s += 2 * step) w[s] += w[s + step];
-                }
-                l = ((m == -INFINITY) ? 0.f : l * ex2(m - mb)) + w[0];
-                m = mb;
-            }
-            if (own.x > -INFINITY) {
-                const float mb = fmaxf(m, own.x);
-                l = fmaf(own.y, ex2(own.x - mb), l * ex2(m - mb));
-                m = mb;
-            }
-            float inv_l;
-            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv_l) : "f"(l));
-            if (!row_valid) inv_l = 0.f;
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                fbuf[(b * 8 + i) * kTcRows + row] = (cm[i] == -INFINITY) ? 0.f : ex2(cm[i] - m) * inv_l;
-            mbar_arrive(bar(kBarFReady + b));
-        }
+        group_sync(g);
+        store((j & 1) ^ 1);
     }
 
     // ---------------------------------------------------------------- teardown
@@ -816,14 +858,15 @@ struct TcPlan {
     bool usable = false;
     TcEncodeFn encode = nullptr;
     int sm_count = 0;
-    int max_items = 0, max_slabs = 0;
-    float2 *stats = nullptr;          // [max_items][max_slabs][128]
-    // "fresh" marking of the statistics: every launch writes all entries of its (items x slabs) layout
+    int max_items = 0, max_entries = 0;
+    float *stats = nullptr;           // [max_items][max_entries][128]
+    float2 *refs = nullptr;           // the same
+    // "fresh" marking of the statistics: every launch writes all entries of its (items x entries) layout
     // with the sign opposite to the previous launch's; a layout change, or a launch that gave up or failed, clears the array first.
     // A captured launch runs again and again with the one sign it was captured with, between launches that nobody counts: it
     // clears the array itself, and so does every launch after it.
     float sign = 1.f;
-    int last_items = 0, last_slabs = 0;
+    int last_items = 0, last_entries = 0;
     bool captured = false;
 };
 
@@ -854,8 +897,9 @@ inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, int sm_count, D
     const int G = cfg.Hq / cfg.Hkv;
     const int units = cfg.layers * cfg.batch * cfg.Hkv;
     plan.max_items = units * ((G * cfg.max_cap_rows + kTcRows - 1) / kTcRows);
-    plan.max_slabs = (cfg.pot_size + kTcSlab - 1) / kTcSlab;
-    mem.add((void **)&plan.stats, (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float2));
+    plan.max_entries = (cfg.pot_size + kTcHalf - 1) / kTcHalf;
+    mem.add((void **)&plan.stats, (size_t)plan.max_items * plan.max_entries * kTcRows * sizeof(float));
+    mem.add((void **)&plan.refs, (size_t)plan.max_items * plan.max_entries * kTcRows * sizeof(float2));
     plan.usable = true;
 }
 
@@ -863,7 +907,7 @@ inline bool tc_applicable(TcPlan &plan, const ipot_config_t &cfg, int N, int M)
 {
     if (!plan.usable || cfg.dtype != IPOT_BF16 || (cfg.d != 128 && cfg.d != 64) || N < 1 || M < 1) return false;
     const int units = cfg.layers * cfg.batch * cfg.Hkv;
-    return units * ((M + kTcRows - 1) / kTcRows) <= plan.max_items && (N + kTcSlab - 1) / kTcSlab <= plan.max_slabs;
+    return units * ((M + kTcRows - 1) / kTcRows) <= plan.max_items && (N + kTcHalf - 1) / kTcHalf <= plan.max_entries;
 }
 
 // [units][unit_rows][d] bf16, of which `rows` per unit are addressable; box = 64 x box_rows x 1, 128-byte swizzle.
@@ -911,13 +955,14 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
     if (!Knew) mapKnew = mapK;
     else if (tc_encode_rows(plan, &mapKnew, Knew, cfg.d, N - new_first, units, (size_t)(N - new_first), kTcSlab) != IPOT_OK) return IPOT_E_CUDA;
     TcParams prm;
-    prm.scores = scores; prm.part_stride = part_stride; prm.stats = plan.stats; prm.cap_stats = cap_stats; prm.status = status;
+    prm.scores = scores; prm.part_stride = part_stride; prm.stats = plan.stats; prm.refs = plan.refs; prm.cap_stats = cap_stats; prm.status = status;
     prm.N = N; prm.M = M; prm.mtiles = mtiles; prm.slabs = (N + kTcSlab - 1) / kTcSlab;
+    prm.entries = (N + kTcHalf - 1) / kTcHalf;
     const int items = units * mtiles;
     prm.tasks = items * prm.slabs;
     prm.dhalves = cfg.d / 64;
     prm.new_slab0 = Knew ? new_first / kTcSlab : 0x7fffffff;
-    prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d));
+    prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d) * (1.0 + 1.2e-8 * (cfg.d / 16)));
     prm.wait_ns = wait_ns;
     prm.withhold_cta = withhold_cta;
     if (!plan.captured) {
@@ -928,13 +973,13 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
         }
         plan.captured = capture != cudaStreamCaptureStatusNone;
     }
-    if (plan.captured || items != plan.last_items || prm.slabs != plan.last_slabs) {
-        if (cudaMemsetAsync(plan.stats, 0, (size_t)items * prm.slabs * kTcRows * sizeof(float2), stream) != cudaSuccess) {
+    if (plan.captured || items != plan.last_items || prm.entries != plan.last_entries) {
+        if (cudaMemsetAsync(plan.stats, 0, (size_t)items * prm.entries * kTcRows * sizeof(float), stream) != cudaSuccess) {
             cudaGetLastError();
             return IPOT_E_CUDA;
         }
         plan.last_items = items;
-        plan.last_slabs = prm.slabs;
+        plan.last_entries = prm.entries;
     }
     plan.sign = -plan.sign;
     prm.sign = plan.sign;

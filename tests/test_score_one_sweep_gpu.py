@@ -1,0 +1,87 @@
+"""GPU parity of the one-sweep tensor-core scorer (IPOT_SCORER_TENSOR) at the edges of its tiles and statistics, against the CPU
+checker, through the C ABI, under the tolerances of tests/parity.py.  Eq. 2, Sec. 3.3.1."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2410_01518_b200 import inputs, ipot
+from parity import compare_cycle, gpu_cycle, make_pot, to_dev
+
+pytestmark = pytest.mark.gpu
+TC = ipot.IPOT_SCORER_TENSOR
+
+SHAPES = [
+    # (rows used, cap_rows, Hq, Hkv, d, layers, batch): a part of one half slab, its end and the key behind it, a last slab of one half,
+    # more statistics than one look takes (16 per half of the item), 1 to 128 rows in a block at the ends of the 32-row
+    # quarters, a second block of one row
+    (2, 1, 1, 1, 64, 1, 1), (100, 32, 1, 1, 128, 1, 1), (128, 33, 1, 1, 128, 1, 1), (129, 64, 2, 2, 128, 1, 2), (256, 13, 5, 1, 64, 1, 1),
+    (257, 24, 4, 1, 128, 2, 1), (385, 97, 1, 1, 128, 1, 1), (2047, 32, 8, 2, 128, 3, 1), (2999, 19, 12, 4, 128, 5, 3), (4097, 43, 3, 1, 128, 1, 1),
+    (4353, 25, 5, 1, 128, 2, 1), (8193, 50, 6, 1, 64, 1, 1), (4096, 32, 32, 8, 128, 21, 1),
+]
+
+
+@pytest.mark.parametrize("case", range(len(SHAPES)))
+def test_one_sweep_edges(case):
+    n, P, Hq, Hkv, d, L, B = SHAPES[case]
+    cfg = inputs.small_config(cfg_id=960 + case, pot_size=n + 3, keep=max(1, n // 2), nuc_slots=n // 4, cap_rows=P, Hq=Hq, Hkv=Hkv, d=d,
+                              dtype="bf16", layers=L, batch=B)
+    t = inputs.make_cycle(cfg)
+    units = None if cfg.units <= 24 else np.linspace(0, cfg.units - 1, 24).astype(np.int32)
+    same, cnt = compare_cycle(cfg, t, gpu_cycle(cfg, t, TC, n=n), n=n, units=units)
+    assert same >= cnt - 1
+
+
+@pytest.mark.parametrize("cap_keys", [False, True])
+@pytest.mark.parametrize("n", [1024, 999])
+@pytest.mark.parametrize("big", [None, 3, 20, 40, 70, 100, 127, 200, 400])
+def test_one_sweep_logits_outside_the_default_range(big, n, cap_keys):
+    """Exponentials are summed against the reference 0 until a warp's sums leave the comfortable range; a key of enormous logits
+    in each piece of a tile, with tiny keys in front of it, makes every way of leaving it happen.  None: every logit
+    of a row lies hundreds of exponent steps below 0."""
+    cfg = inputs.small_config(cfg_id=990, pot_size=1024, keep=400, nuc_slots=0, cap_rows=20, Hq=4, Hkv=1, d=128, dtype="bf16", layers=2)
+    t = inputs.make_cycle(cfg)
+    K, Q = (inputs.widen(t[x], "bf16").astype(np.float32) for x in "KQ")
+    if big is None:
+        axis = np.zeros(cfg.d, np.float32)
+        axis[5] = 60.0
+        Q, K = Q + axis, K - axis
+    else:
+        K[:, :, :, big] *= 60.0
+        K[1, :, :, :16] *= 0.01
+    t["K"], t["Q"] = inputs.store(K, "bf16"), inputs.store(Q, "bf16")
+    if cap_keys:
+        t["K_cap"] = inputs.make_kcap(cfg)
+    compare_cycle(cfg, t, gpu_cycle(cfg, t, TC, n=n), n=n)
+
+
+def test_one_sweep_calls_of_different_row_counts_share_one_pot():
+    """The statistics of a launch are told from those of the launches before by their sign; calls with fewer rows in between must
+    leave no row with a sign that a later call takes for its own."""
+    cfg = inputs.small_config(cfg_id=991, pot_size=3000, keep=400, nuc_slots=0, cap_rows=32, Hq=8, Hkv=2, d=128, dtype="bf16", layers=4)
+    t = inputs.make_cycle(cfg)
+    Q = inputs.widen(t["Q"], "bf16").astype(np.float32)
+    h = make_pot(cfg)
+
+    class Scores:
+        pass
+
+    def score(P, scale):
+        q = to_dev(inputs.store(np.ascontiguousarray(Q[..., :P, :] * scale), "bf16"), "bf16")
+        ipot.ipot_score_only(h, q, P)
+        ipot.ipot_sync_status(h)
+        addr, n = ipot.ipot_last_scores(h)
+        s = Scores()
+        s.__cuda_array_interface__ = {"shape": (cfg.units, n), "typestr": "<f4", "data": (addr, False), "version": 2}
+        return torch.as_tensor(s, device="cuda").clone()
+    try:
+        ipot.ipot_set_scorer(h, TC)
+        K, V = to_dev(t["K"], "bf16"), to_dev(t["V"], "bf16")
+        ipot.ipot_append_chunk(h, K, V, cfg.pot_size)
+        want = {P: score(P, 1.0) for P in (32, 1, 9, 17)}
+        for P in (32, 1, 32, 9, 9, 17, 1, 1, 32, 17, 32):
+            score(P if P == 32 else 1, 0.5)      # other numbers in between
+            assert torch.equal(score(P, 1.0), want[P])
+        for P, got in want.items():              # each row's probabilities sum to 1
+            assert torch.allclose(got.sum(1), torch.full((cfg.units,), float(P * cfg.Hq // cfg.Hkv), device="cuda"), rtol=1e-4)
+    finally:
+        ipot.ipot_destroy(h)
