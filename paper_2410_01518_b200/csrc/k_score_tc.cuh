@@ -18,21 +18,22 @@
 //              0 - no maximum is taken unless a warp's sums then leave the comfortable range; a quarter of the
 //              exponentials run on the FMA pipe.  The warps of a scheduler take pass 1 in turns, pair after pair: both
 //              pairs at once finish later than one of them could, and every reader of their sums waits;
-//     exchange the thread publishes its row's sum over the 128 keys with one 4-byte store that carries the launch's
-//              sign as a "fresh" mark, reads half of the row's sums of the whole item (the other group of the pair reads
-//              the other half), re-reading until every one is fresh, and turns them into the row's denominator
-//              l (plus, when given, the share of the CaP's own keys);
+//     exchange the two groups of a pair add their row sums through shared memory and publish them with one 4-byte store
+//              that carries the launch's sign as a "fresh" mark; a thread reads half of its row's sums of the whole item
+//              (the other group of the pair the other half), re-reading until every one is fresh, and the pair turns
+//              them into the row's denominator l (plus, when given, the share of the CaP's own keys);
 //     pass 2   u_j = sum_i e_ij / l_i as a weighted column sum: the 16x256b tensor-memory load shape hands every
 //              thread four rows of a column pair, so the sum over a warp's 32 rows is four packed FMAs plus a
 //              three-step exchange between lanes; the four row quarters meet in shared memory and are added and
 //              stored behind the next task's barrier: 256 floats per task.
 // A row block of fewer rows keeps the warps of its empty quarters out of all of this.
 //
-// Bound: a task's way through tensor memory - product 700 cycles, pass 1 3000 to 4000 beside the other pair's
-// work, exchange 3500, pass 2 1700 - and tensor memory holds two tasks.  (Pass 1 and pass 2 alone would take an SM 2500 cycles per
-// task, without the exchange the launch takes 66 us.)  Measured against the form before, in which all 16 warps
-// shared a task, took maxima, and four more warps combined and polled (us, alone): 256 units x 4096 keys, M = 128 90.1 -> 85.2; 128 x
-// 8192, M = 256 197 -> 173; 60 x 2999, M = 57 20.8 -> 18.5; 64 x 16384, M = 512 537 -> 384.  Error of the scores against
+// Bound: a task's way through tensor memory, and tensor memory holds two tasks: product 700 cycles, pass 1 4100 beside the other
+// pair's work, exchange 2000, pass 2 1800, hand-overs 500.  (Pass 1 and pass 2 alone would take an SM 2500 cycles per task, without the
+// exchange a launch of 256 units takes 66 us.)  The polls are what the exchange costs: with an entry per 128 keys instead of one per
+// 256 the last of these figures were 85.2, 173, 18.5 and 384.  Measured against the form in which all 16 warps
+// shared a task, took maxima, and four more warps combined and polled (us, alone): 256 units x 4096 keys, M = 128 90.1 -> 82; 128 x
+// 8192, M = 256 197 -> 157; 60 x 2999, M = 57 20.8 -> 18.5; 64 x 16384, M = 512 537 -> 333.  Error of the scores against
 // 64 bits 4.5e-7 -> 1.6e-7 (fewer roundings, a polynomial of degree 5, the tensor core's cut sums made good).
 //
 // Blocks of one grid wait on each other (pass 2 needs the other slabs' statistics),
@@ -61,7 +62,7 @@ constexpr int kTcRows = 128;         // query rows per item (TMEM lanes)
 constexpr int kTcHalf = 128;         // keys per epilogue group and entry of the statistics
 // The first look at a task's statistics comes this much after its own have left: the others' are never there at once, and what is not
 // polled leaves L2 to the keys.  Measured (256 units x 4096 keys, M = 128 / 128 x 8192, M = 256, us): 0 ns 88.6 / 175.1, 300 85.2 / 172.7,
-// 600 85.8 / 180.5; a CTA's first task (all there is in a small launch) does not wait (8 units x 4096: 8.3, 8.4, 10.1).
+// 600 85.8 / 180.5 (before the pair's sums were joined; since then 0 to 300 are equal); a CTA's first task (all there is in a small launch) does not wait (8 units x 4096: 8.3, 8.4, 10.1).
 constexpr unsigned kTcPollDelayNs = 300;
 constexpr int kTcSlab = 256;         // keys per task (TMEM columns per buffer)
 constexpr int kTcFmaEighths = 2;     // share of pass 1's exponentials evaluated on the FMA pipe
@@ -74,7 +75,8 @@ constexpr uint32_t kTcStageBytes = kTcQBytes + kTcKBytes;    // 96 KiB
 constexpr uint32_t kTcOffStage = 0;                                        // [2] { Q, K }
 constexpr uint32_t kTcOffColpart = 2 * kTcStageBytes;                      // [4 groups][2 parities][4 row quarters][128] float
 constexpr uint32_t kTcOffLpart = kTcOffColpart + 4 * 2 * 4 * kTcHalf * 4;      // [2 pairs][2 parities][2 halves][128] float
-constexpr uint32_t kTcOffBar = kTcOffLpart + 2 * 2 * 2 * kTcRows * 4;
+constexpr uint32_t kTcOffSpart = kTcOffLpart + 2 * 2 * 2 * kTcRows * 4;        // [2 pairs][2 parities][128] float2
+constexpr uint32_t kTcOffBar = kTcOffSpart + 2 * 2 * kTcRows * 8;
 constexpr uint32_t kTcOffTmemSlot = kTcOffBar + 192;                       // the allocated TMEM base address
 constexpr uint32_t kTcOffAbort = kTcOffBar + 196;                          // set once a wait of the CTA has run out; + 4: the block's deadline (8 bytes)
 constexpr uint32_t kTcSmemBytes = kTcOffBar + 256;                         // no static shared memory: the base is 1024-aligned
@@ -85,15 +87,15 @@ enum { kBarFull = 0, kBarEmpty = 2, kBarSFull = 4, kBarTEmpty = 8, kBarDrain = 1
 struct TcParams {
     float *scores;        // partial array p (query rows 128p ...) at scores + p * part_stride, unit stride N
     size_t part_stride;
-    float *stats;         // [items][entries][128] a row's sum over 128 keys, times the launch's sign (infinite: its reference is not 0, see
+    float *stats;         // [items][slabs][128] a row's sum over a slab's keys, times the launch's sign (infinite: its reference is not 0, see
                           // refs); all of the other sign or 0 at launch
-    float2 *refs;         // [items][entries][128] (reference, sum) of those
+    float2 *refs;         // [items][slabs][128] (reference, sum) of those
     const float2 *cap_stats;  // NULL, or [units][M] (max, sum) over the CaP's own keys that join every row's denominator
     float sign;           // +1 or -1: this launch's "fresh" mark
     unsigned long long wait_ns;  // limit of every wait
     int withhold_cta;     // -1; test hook: this CTA never publishes its slab statistics
     int *status;
-    int N, M, mtiles, slabs, entries, tasks;
+    int N, M, mtiles, slabs, tasks;
     int dhalves;          // d / 64: 64-channel halves of a tile (1 or 2)
     int new_slab0;        // slabs from this one on are read through the second key map (the chunk of a deferred
                           // append, row 0 = key 256 * new_slab0); INT_MAX if all keys are in the pot
@@ -401,20 +403,21 @@ __device__ __noinline__ float2 pass1_ragged(uint32_t taddr, int nvalid, float c)
     }
     return make_float2(0.f, s);
 }
-// Sum of n (up to 16) of a row's entries, re-read until each carries the launch's mark.  Only what is still stale is read again: the polls
+// Sum of n (up to kMost) of a row's entries, re-read until each carries the launch's mark.  Only what is still stale is read again: the polls
 // of all CTAs together are a large part of what L2 delivers (all of it again, in 16-byte loads of a transposed array: 109 us against 90).
+template <int kMost>
 __device__ __forceinline__ float poll_entries(const float *st, int n, float sgn, volatile int *ab, int *status)
 {
-    float v[16];
+    float v[kMost];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) v[e] = e < n ? 0.f : kTcTiny * sgn;
+    for (int e = 0; e < kMost; ++e) v[e] = e < n ? 0.f : kTcTiny * sgn;
     for (uint32_t tries = 1;; ++tries) {
         bool fresh = true;
 #pragma unroll
-        for (int e = 0; e < 16; ++e)
+        for (int e = 0; e < kMost; ++e)
             if (!(v[e] * sgn > 0.f)) v[e] = ld_gpu_f32(st + (size_t)e * kTcRows);
 #pragma unroll
-        for (int e = 0; e < 16; ++e) fresh = fresh && v[e] * sgn > 0.f;
+        for (int e = 0; e < kMost; ++e) fresh = fresh && v[e] * sgn > 0.f;
         if (fresh) break;
         if ((tries & 63u) == 0 && (*ab || global_timer_ns() > *reinterpret_cast<volatile unsigned long long *>(ab + 1))) {
             if (!*ab) {
@@ -425,11 +428,11 @@ __device__ __forceinline__ float poll_entries(const float *st, int n, float sgn,
         }
     }
 #pragma unroll
-    for (int e = 0; e < 16; ++e) v[e] = fabsf(v[e]);
+    for (int e = 0; e < kMost; ++e) v[e] = fabsf(v[e]);
 #pragma unroll
-    for (int step = 1; step < 16; step <<= 1) {
+    for (int step = 1; step < kMost; step <<= 1) {
 #pragma unroll
-        for (int e = 0; e < 16; e += 2 * step) v[e] += v[e + step];
+        for (int e = 0; e < kMost; e += 2 * step) v[e] += v[e + step];
     }
     return v[0];
 }
@@ -624,9 +627,10 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         const int row = q * 32 + lane;
         const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + g * kTcHalf;
         float *lpart = reinterpret_cast<float *>(gbase + kTcOffLpart) + pair * (4 * kTcRows);
+        float2 *spart = reinterpret_cast<float2 *>(gbase + kTcOffSpart) + pair * (2 * kTcRows);
         float *colpart = reinterpret_cast<float *>(gbase + kTcOffColpart) + g * (8 * kTcHalf);
         const float c = prm.scale_log2e, sgn = prm.sign;
-        const int E = prm.entries, mid = (E + 1) >> 1;
+        const int S = prm.slabs, mid = (S + 1) >> 1;
         // task -> (unit, row block, slab) is counted on from task to task: three divisions at the head of each were 250 ns of a pair's cycle
         const int step = 2 * prm.ctas, dslab = step % tasks_per_item, ditem = step / tasks_per_item, dmt = ditem % prm.mtiles, dunit = ditem / prm.mtiles;
         const int task0 = blockIdx.x + pair * prm.ctas;
@@ -647,9 +651,8 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             const uint32_t par = j & 1;
             float2 own = make_float2(-INFINITY, 0.f);  // the CaP keys' share of this row's denominator (Appendix B listing)
             if (prm.cap_stats && row < rows) own = __ldg(&prm.cap_stats[(size_t)unit * prm.M + mt * kTcRows + row]);
-            float *st = prm.stats + (size_t)item * E * kTcRows + row;
-            const int e = 2 * slab + half;      // this group's entry
-            float2 s = make_float2(0.f, 1.f);
+            float *st = prm.stats + (size_t)item * S * kTcRows + row;
+            float2 s = make_float2(0.f, nvalid > 0 ? 1.f : 0.f);
             mbar_wait(bar(kBarSFull + g), par, ab, prm.status);
             if (pair | j) turn_wait(pair, q);
             // ---- pass 1: exponentials against the reference 0, written back over the logits, and their sum
@@ -692,14 +695,20 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 }
             }
             if (task + prm.ctas < prm.tasks) turn_pass(pair, q);
-            if (nvalid > 0 && (int)blockIdx.x != prm.withhold_cta) {
-                float *to = st + (size_t)e * kTcRows;
-                if (s.x == 0.f) {
-                    st_gpu_f32(to, s.y == 0.f ? kTcTiny * sgn : s.y * sgn);
+            // ---- the pair's two sums together are the slab's entry
+            if (half) spart[par * kTcRows + row] = s;
+            pair_sync(pair);
+            if (!half && (int)blockIdx.x != prm.withhold_cta) {
+                const float2 o = spart[par * kTcRows + row];
+                float *to = st + (size_t)slab * kTcRows;
+                const float sum = s.y + o.y;
+                if (s.x == 0.f && o.x == 0.f && sum == sum) {   // (a NaN takes the other way, or it would never count as fresh)
+                    st_gpu_f32(to, sum == 0.f ? kTcTiny * sgn : sum * sgn);
                 } else {
-                    float *r = reinterpret_cast<float *>(prm.refs + ((size_t)item * E + e) * kTcRows + row);
-                    st_gpu_f32(r, s.x);
-                    st_gpu_f32(r + 1, s.y);
+                    const float m = fmaxf(s.y == 0.f ? -INFINITY : s.x, o.y == 0.f ? -INFINITY : o.x);   // (one of them is not empty)
+                    float *r = reinterpret_cast<float *>(prm.refs + ((size_t)item * S + slab) * kTcRows + row);
+                    st_gpu_f32(r, m);
+                    st_gpu_f32(r + 1, (s.y == 0.f ? 0.f : s.y * ex2(s.x - m)) + (o.y == 0.f ? 0.f : o.y * ex2(o.x - m)));
                     asm volatile("fence.acq_rel.gpu;" ::: "memory");
                     st_gpu_f32(to, INFINITY * sgn);
                 }
@@ -708,8 +717,10 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             float l = 0.f;
             if (row < rows) {
                 if (j) __nanosleep(kTcPollDelayNs);
-                const int end = half ? E : mid;
-                for (int i = half ? mid : 0; i < end; i += 16) l += poll_entries(st + (size_t)i * kTcRows, end - i, sgn, ab, prm.status);
+                const int end = half ? S : mid;
+                int i = half ? mid : 0;
+                for (; i + 8 < end; i += 16) l += poll_entries<16>(st + (size_t)i * kTcRows, end - i, sgn, ab, prm.status);
+                if (i < end) l += poll_entries<8>(st + (size_t)i * kTcRows, end - i, sgn, ab, prm.status);
             }
             lpart[(par * 2 + half) * kTcRows + row] = l;
             if (works) {
@@ -723,7 +734,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 float m = 0.f;
                 l = lpart[(par * 2) * kTcRows + row] + lpart[(par * 2 + 1) * kTcRows + row];
                 if (l == INFINITY) {
-                    const float2 t = merge_entries(st, prm.refs + (size_t)item * E * kTcRows + row, E);
+                    const float2 t = merge_entries(st, prm.refs + (size_t)item * S * kTcRows + row, S);
                     m = t.x;
                     l = t.y;
                 }
@@ -858,15 +869,15 @@ struct TcPlan {
     bool usable = false;
     TcEncodeFn encode = nullptr;
     int sm_count = 0;
-    int max_items = 0, max_entries = 0;
-    float *stats = nullptr;           // [max_items][max_entries][128]
+    int max_items = 0, max_slabs = 0;
+    float *stats = nullptr;           // [max_items][max_slabs][128]
     float2 *refs = nullptr;           // the same
-    // "fresh" marking of the statistics: every launch writes all entries of its (items x entries) layout
+    // "fresh" marking of the statistics: every launch writes all entries of its (items x slabs) layout
     // with the sign opposite to the previous launch's; a layout change, or a launch that gave up or failed, clears the array first.
     // A captured launch runs again and again with the one sign it was captured with, between launches that nobody counts: it
     // clears the array itself, and so does every launch after it.
     float sign = 1.f;
-    int last_items = 0, last_entries = 0;
+    int last_items = 0, last_slabs = 0;
     bool captured = false;
 };
 
@@ -897,9 +908,9 @@ inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, int sm_count, D
     const int G = cfg.Hq / cfg.Hkv;
     const int units = cfg.layers * cfg.batch * cfg.Hkv;
     plan.max_items = units * ((G * cfg.max_cap_rows + kTcRows - 1) / kTcRows);
-    plan.max_entries = (cfg.pot_size + kTcHalf - 1) / kTcHalf;
-    mem.add((void **)&plan.stats, (size_t)plan.max_items * plan.max_entries * kTcRows * sizeof(float));
-    mem.add((void **)&plan.refs, (size_t)plan.max_items * plan.max_entries * kTcRows * sizeof(float2));
+    plan.max_slabs = (cfg.pot_size + kTcSlab - 1) / kTcSlab;
+    mem.add((void **)&plan.stats, (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float));
+    mem.add((void **)&plan.refs, (size_t)plan.max_items * plan.max_slabs * kTcRows * sizeof(float2));
     plan.usable = true;
 }
 
@@ -907,7 +918,7 @@ inline bool tc_applicable(TcPlan &plan, const ipot_config_t &cfg, int N, int M)
 {
     if (!plan.usable || cfg.dtype != IPOT_BF16 || (cfg.d != 128 && cfg.d != 64) || N < 1 || M < 1) return false;
     const int units = cfg.layers * cfg.batch * cfg.Hkv;
-    return units * ((M + kTcRows - 1) / kTcRows) <= plan.max_items && (N + kTcHalf - 1) / kTcHalf <= plan.max_entries;
+    return units * ((M + kTcRows - 1) / kTcRows) <= plan.max_items && (N + kTcSlab - 1) / kTcSlab <= plan.max_slabs;
 }
 
 // [units][unit_rows][d] bf16, of which `rows` per unit are addressable; box = 64 x box_rows x 1, 128-byte swizzle.
@@ -957,7 +968,6 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
     TcParams prm;
     prm.scores = scores; prm.part_stride = part_stride; prm.stats = plan.stats; prm.refs = plan.refs; prm.cap_stats = cap_stats; prm.status = status;
     prm.N = N; prm.M = M; prm.mtiles = mtiles; prm.slabs = (N + kTcSlab - 1) / kTcSlab;
-    prm.entries = (N + kTcHalf - 1) / kTcHalf;
     const int items = units * mtiles;
     prm.tasks = items * prm.slabs;
     prm.dhalves = cfg.d / 64;
@@ -973,13 +983,13 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
         }
         plan.captured = capture != cudaStreamCaptureStatusNone;
     }
-    if (plan.captured || items != plan.last_items || prm.entries != plan.last_entries) {
-        if (cudaMemsetAsync(plan.stats, 0, (size_t)items * prm.entries * kTcRows * sizeof(float), stream) != cudaSuccess) {
+    if (plan.captured || items != plan.last_items || prm.slabs != plan.last_slabs) {
+        if (cudaMemsetAsync(plan.stats, 0, (size_t)items * prm.slabs * kTcRows * sizeof(float), stream) != cudaSuccess) {
             cudaGetLastError();
             return IPOT_E_CUDA;
         }
         plan.last_items = items;
-        plan.last_entries = prm.entries;
+        plan.last_slabs = prm.slabs;
     }
     plan.sign = -plan.sign;
     prm.sign = plan.sign;
