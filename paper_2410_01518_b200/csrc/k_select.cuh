@@ -13,7 +13,7 @@
 // digit's keys are taken as a whole: two passes nearly always, where digits of 8
 // bits from the top took four (one stream's ranking of 4096 slots: 5.7 -> 4.4 us).
 //
-// One block per problem.  A thread keeps 16 (pot sizes above 16384: 32) consecutive
+// One block per problem.  A thread keeps 16 (pot sizes above 16384: 32; 4 or 8 where every unit has an SM) consecutive
 // slots' keys in registers from the first load to the last store, and the block has
 // only as many threads as that takes (256 for a pot of 4096): the per-thread work of
 // a pass (histogram scan, barriers) is then shared by 16 keys, which is what the
@@ -311,7 +311,7 @@ select_kernel(const float *__restrict__ scores, int parts, size_t part_stride,
     pdl_release();
     uint32_t key[kKpt];
     // a reserved slot outranks every score: finite scores map below 0xFF800000
-    constexpr int kPiece = kKpt > 16 ? 8 : 16;   // slots loaded at a time (what 64 registers a thread allow)
+    constexpr int kPiece = kKpt > 16 ? 8 : kKpt;   // slots loaded at a time (what 64 registers a thread allow)
 #pragma unroll
     for (int h = 0; h < kKpt; h += kPiece) {
         const int first = slot0 + h;
@@ -390,11 +390,18 @@ inline void launch_nuc_mask(int blocks, cudaStream_t st, const float *aux, uint8
     kern<<<blocks, threads, 0, st>>>(aux, mask, N, T, batch);
 }
 inline cudaError_t launch_select(int blocks, cudaStream_t st, const float *scores, int parts, size_t part_stride, const uint8_t *mask,
-                                 int32_t *idx, float *summed, int N, int keep, int Hkv, int batch, int *status, const GatherPlan &plan)
+                                 int32_t *idx, float *summed, int N, int keep, int Hkv, int batch, int *status, const GatherPlan &plan, int sm_count)
 {
     auto kern = N <= 4096 ? select_kernel<256, 16> : N <= 8192 ? select_kernel<512, 16> : N <= 16384 ? select_kernel<1024, 16> : select_kernel<1024, 32>;
-    return launch_pdl(kern, dim3(blocks), dim3(N <= 4096 ? 256 : N <= 8192 ? 512 : 1024), 0, st, scores, parts, part_stride, mask, idx, summed, N, keep, Hkv, batch,
-                      status, plan);
+    int threads = N <= 4096 ? 256 : N <= 8192 ? 512 : 1024;
+    // A unit per SM: what counts is one block's chain, not the number of instructions, and a thread of 4 (8) keys is through
+    // its histogram and its scans earlier (whole passes, us: 8 units x 4096 28.9 -> 26.8, x 2000 25.5 -> 23.0, x 1000 23.4 -> 20.9, x 8192 36.5 -> 36.1;
+    // 8 keys below 4096 slots as well: 27.4, 24.6, 21.7).
+    if (N <= 8192 && blocks <= sm_count) {
+        kern = N <= 512 ? select_kernel<128, 4> : N <= 1024 ? select_kernel<256, 4> : N <= 2048 ? select_kernel<512, 4> : N <= 4096 ? select_kernel<1024, 4> : select_kernel<1024, 8>;
+        threads = N <= 512 ? 128 : N <= 1024 ? 256 : N <= 2048 ? 512 : 1024;
+    }
+    return launch_pdl(kern, dim3(blocks), dim3(threads), 0, st, scores, parts, part_stride, mask, idx, summed, N, keep, Hkv, batch, status, plan);
 }
 
 // summed[i] = parts[0][i] + parts[1][i] + ... in index order (the order select_kernel uses).

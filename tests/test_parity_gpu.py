@@ -477,3 +477,25 @@ def test_seeded_random_large_pots(seed):
     gpu = gpu_cycle(cfg, t, ipot.IPOT_SCORER_AUTO, n=n, deferred_from=deferred)
     same, cnt = compare_cycle(cfg, t, gpu, n=n)
     assert cnt == cfg.units and same >= cnt - 1, seed
+
+
+@pytest.mark.parametrize("n", [2, 31, 511, 512, 513, 1024, 1025, 2047, 2048, 2049, 4095, 4096, 4097, 8191, 8192])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_selection_of_few_units_at_the_edges_of_its_block_shapes(n, dtype):
+    """Pots of fewer units than SMs use blocks of other shapes (4 or 8 slots a thread), f32 pots of up to 2048 slots rank the novelty in
+    the scorer's launch.  Against a sort of the scores that the same cycle reports: every third key is the same, so that whole runs
+    of scores tie, and novelty has few values.  The survivors are whole numbers: no tolerance."""
+    cfg = inputs.small_config(cfg_id=840, pot_size=n + 1, keep=max(1, n // 2 - 1), nuc_slots=n // 5, cap_rows=2, Hq=2, Hkv=2, d=64, dtype=dtype, layers=2)
+    t = inputs.make_cycle(cfg)
+    t["K"][:, :, :, ::3] = t["K"][:, :, :, :1]
+    t["K"][1, :, :, :] = t["K"][1, :, :, :1]
+    t["aux"] = np.round(t["aux"] * 16).astype(np.float32) / 16
+    gpu = gpu_cycle(cfg, t, n=n)
+    compare_cycle(cfg, t, gpu, n=n)
+    slots = np.arange(n)
+    novel = np.lexsort((slots, -t["aux"][0, :n]))[:cfg.nuc_slots]      # the last key is the first to sort by; ties: lower slot
+    for u in range(cfg.units):
+        reserved = np.zeros(n, bool)
+        reserved[novel] = True
+        order = np.lexsort((slots, -gpu[0][u], ~reserved))
+        assert np.array_equal(gpu[1][u], np.sort(order[:cfg.keep])), (n, dtype, u)
