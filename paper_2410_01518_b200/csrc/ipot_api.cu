@@ -241,13 +241,13 @@ int launch_simt(ipot *p, const void *Q, const float2 *cap_stats, int M, int N)
 
 // f32 pots: every logit computed once, unless one unit's logits exceed the scratch (M * N above 14.9 million: 4.5 bytes each) or it
 // did not fit into the device's memory
-int launch_f32(ipot *p, const void *Q, const float2 *cap_stats, int M, int N)
+int launch_f32(ipot *p, const void *Q, const float2 *cap_stats, int M, int N, NucJob nuc)
 {
     if (!f32_applicable(p->f32, M, N)) return launch_simt<float>(p, Q, cap_stats, M, N);
     const int d = p->cfg.d;
     int n = 0;
     IPOT_CUDA(f32_launch(p->f32, (const float *)Q, (const float *)score_keys(p), cap_stats, p->row_stats, p->scores, p->units, M, N, d,
-                         (size_t)p->cfg.pot_size * d, (float)(1.4426950408889634 / std::sqrt((double)d)), p->sm_count, p->stream, &n));
+                         (size_t)p->cfg.pot_size * d, (float)(1.4426950408889634 / std::sqrt((double)d)), p->sm_count, p->stream, &n, nuc));
     p->launches += n;
     return IPOT_OK;
 }
@@ -336,7 +336,8 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
     // a stream against 3 us per round of (128 rows x 256 keys).
     const long long rounds = ((long long)p->units * ((M + kTcRows - 1) / kTcRows) * ((N + kTcSlab - 1) / kTcSlab) + p->sm_count - 1) / p->sm_count;
     // ... or rides along in the scorer's own launch: the fork and join by events cost a small cycle 5 us
-    const bool in_scorer = T > 0 && aux && N > kTcSlab && N <= kNucMaxSlots && rounds <= 12 && p->sm_count > 1 && (scorer == IPOT_SCORER_TENSOR || scorer == IPOT_SCORER_TENSOR_ITEMS);
+    const bool in_scorer = T > 0 && aux && (p->cfg.dtype == IPOT_F32 ? f32_ranks(p->f32, p->units, M, N, p->sm_count)
+                                            : N > kTcSlab && N <= kNucMaxSlots && rounds <= 12 && p->sm_count > 1 && (scorer == IPOT_SCORER_TENSOR || scorer == IPOT_SCORER_TENSOR_ITEMS));
     const bool side_nuc = T > 0 && aux && p->side && !in_scorer;
     const int nuc_blocks = slab_keys ? (int)std::min<long long>(std::min(p->cfg.batch, std::max(1, p->sm_count / 4)), 1 + (8LL * p->cfg.batch - 1) / (3 * rounds)) : p->cfg.batch;
     NucJob nuc{};
@@ -377,7 +378,7 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
     } else if (scorer == IPOT_SCORER_WARP_MMA) {
         rc = launch_warp_mma(p, Q, cap_stats, M, N);
     } else {
-        rc = p->cfg.dtype == IPOT_F32 ? launch_f32(p, Q, cap_stats, M, N) : launch_simt<__nv_bfloat16>(p, Q, cap_stats, M, N);
+        rc = p->cfg.dtype == IPOT_F32 ? launch_f32(p, Q, cap_stats, M, N, nuc) : launch_simt<__nv_bfloat16>(p, Q, cap_stats, M, N);
     }
     if (ev && rc == IPOT_OK) IPOT_CUDA(cudaEventRecord(ev[2], p->stream));   // the scorer's end, before the join below
     if (side_nuc) IPOT_CUDA(cudaStreamWaitEvent(p->stream, p->ev_join, 0));   // (also when the scorer refused: nothing is left behind on the side stream)
@@ -445,7 +446,7 @@ int run_cycle(ipot *p, const void *Q, const void *Kc, int cap_rows, const float 
     if (rc != IPOT_OK) return rc;
     const size_t part_stride = (size_t)p->units * p->cfg.pot_size;
     IPOT_CUDA(launch_select(p->units, p->stream, p->scores, parts, part_stride, T > 0 ? p->nuc_mask : nullptr, p->idx,
-                  parts > 1 ? p->summed : nullptr, N, keep, p->cfg.Hkv, p->cfg.batch, p->status, p->gather));
+                  parts > 1 ? p->summed : nullptr, N, keep, p->cfg.Hkv, p->cfg.batch, p->status, p->gather, p->sm_count));
     p->launches += 1;
     IPOT_CUDA(cudaGetLastError());
     if (ev) IPOT_CUDA(cudaEventRecord(ev[3], p->stream));

@@ -16,6 +16,7 @@
 // registers (324 us), scalar FMAs instead of packed pairs cost 12 %.
 #pragma once
 #include "common.cuh"
+#include "k_select.cuh"  // NucJob
 #include "k_score_simt.cuh"  // merge_stats
 
 namespace ipotk {
@@ -39,10 +40,21 @@ struct F32Params {
 };
 
 // RT x KT tile; thread (tx, ty) = (t % 16, t / 16) owns rows ty + 8 a and keys tx + 16 b.
-template <int RT, int KT>
+// kRank: the blocks of the grid's last layer rank the streams' novelty (up to kF32RankSlots slots): on a stream of its own beside
+// a launch of one wave the ranking cost a cycle two events, two waits and a launch, 5 us of 23 (2 units x 512 slots x 64 channels).
+constexpr int kF32RankSlots = 16 * kF32Threads;
+template <int RT, int KT, bool kRank>
 __global__ void __launch_bounds__(kF32Threads, 4)
-f32_tile_kernel(const __grid_constant__ F32Params p)
+f32_tile_kernel(const __grid_constant__ F32Params p, const __grid_constant__ NucJob nuc)
 {
+    if (kRank && blockIdx.z == gridDim.z - 1) {
+        __shared__ SelShared sel;
+        pdl_wait();
+        pdl_release();
+        const int b = blockIdx.y * gridDim.x + blockIdx.x;
+        if (b < nuc.ctas) nuc_rank_streams<kF32Threads, 16>(nuc.aux, nuc.mask, p.N, nuc.T, nuc.batch, b, nuc.ctas, sel);
+        return;
+    }
     constexpr int RA = RT / 8, KB = KT / 16;
     __shared__ __align__(16) float qs[2][RT * kF32Stride];
     __shared__ __align__(16) float ks[2][KT * kF32Stride];
@@ -266,12 +278,26 @@ inline void f32_plan_init(F32Plan &plan, int units, int max_M, int pot_size, Dev
 
 inline bool f32_applicable(const F32Plan &plan, int M, int N) { return plan.scratch && f32_unit_bytes(M, N) <= plan.bytes; }
 
-inline cudaError_t f32_launch(const F32Plan &plan, const float *Q, const float *K, const float2 *extra, float2 *row_stats, float *scores, int units,
-                              int M, int N, int d, size_t k_unit_stride, float scale_log2e, int sm_count, cudaStream_t stream, int *launches)
+// the largest tile that still gives every SM a block
+inline int f32_tile(int units, int M, int N, int sm_count)
 {
-    // the largest tile that still gives every SM a block
     int t = 64;
     while (t > 16 && (long long)units * ((M + t - 1) / t) * ((N + t - 1) / t) < sm_count) t /= 2;
+    return t;
+}
+// The ranking rides along where the tiles are one wave (four blocks per SM) of one launch: behind more, it runs beside them unnoticed.
+inline bool f32_ranks(const F32Plan &plan, int units, int M, int N, int sm_count)
+{
+    const int t = f32_tile(units, M, N, sm_count);
+    return f32_applicable(plan, M, N) && N <= kF32RankSlots && (long long)units * ((M + t - 1) / t) * ((N + t - 1) / t) <= 4LL * sm_count &&
+           (size_t)units * f32_unit_bytes(M, N) <= plan.bytes && units < 65535;
+}
+
+// nuc.batch > 0: the first launch ranks the streams as well (only where f32_ranks() says so)
+inline cudaError_t f32_launch(const F32Plan &plan, const float *Q, const float *K, const float2 *extra, float2 *row_stats, float *scores, int units,
+                              int M, int N, int d, size_t k_unit_stride, float scale_log2e, int sm_count, cudaStream_t stream, int *launches, NucJob nuc)
+{
+    const int t = f32_tile(units, M, N, sm_count);
     F32Params p;
     p.Q = Q; p.K = K; p.extra = extra; p.row = row_stats; p.scores = scores; p.counters = plan.counters;
     p.M = M; p.N = N; p.d = d; p.k_unit_stride = k_unit_stride; p.scale_log2e = scale_log2e;
@@ -285,9 +311,13 @@ inline cudaError_t f32_launch(const F32Plan &plan, const float *Q, const float *
         const int n = units - u0 < per ? units - u0 : per;
         p.unit0 = u0;
         p.part = (float2 *)(plan.scratch + (size_t)n * M * p.e_stride * 4);
-        const dim3 grid(p.key_tiles, (M + t - 1) / t, n);
-        auto tile = t == 64 ? f32_tile_kernel<64, 64> : t == 32 ? f32_tile_kernel<32, 32> : f32_tile_kernel<16, 16>;
-        cudaError_t err = launch_pdl(tile, grid, dim3(kF32Threads), 0, stream, p);
+        const bool rank = nuc.batch > 0 && u0 == 0;
+        const dim3 grid(p.key_tiles, (M + t - 1) / t, n + rank);
+        if (rank) nuc.ctas = std::min(nuc.batch, (int)(grid.x * grid.y));
+        auto tile = t == 64   ? (rank ? f32_tile_kernel<64, 64, true> : f32_tile_kernel<64, 64, false>)
+                    : t == 32 ? (rank ? f32_tile_kernel<32, 32, true> : f32_tile_kernel<32, 32, false>)
+                              : (rank ? f32_tile_kernel<16, 16, true> : f32_tile_kernel<16, 16, false>);
+        cudaError_t err = launch_pdl(tile, grid, dim3(kF32Threads), 0, stream, p, nuc);
         if (!p.fold_here && err == cudaSuccess) {
             err = launch_pdl(f32_fold_kernel, dim3((M + 3) / 4, n), dim3(kF32Threads), 0, stream, p);
             *launches += 1;
