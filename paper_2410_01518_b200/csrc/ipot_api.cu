@@ -277,24 +277,24 @@ int launch_warp_mma(ipot *p, const void *Q, const float2 *cap_stats, int M, int 
     return IPOT_OK;
 }
 
-// The fastest scorer the shape allows.  d = 64 and 128: the one-sweep kernel computes every exponential once, but beyond 32 slabs
-// of 256 keys an item's blocks wait too long for each other's statistics, and the two-sweep kernel whose work is dealt item by item
-// is faster if there are items enough to deal.  Rows of 64 channels cost the one-sweep kernel as much as wider ones: there it
-// is from 6144 keys on.  Measured as steps of a stream with deferred appends (us, one sweep / items), d = 128:
-//   128 units x 8192 keys, M = 64, 128, 256:  145 / 151, 146 / 168, 233 / 239;  64 x 8192, M = 512, 768, 1024: 219 / 219, 310 / 299, 400 / 387
-//   128 x 9216:                               188 / 169, 188 / 185, 304 / 277;  64 x 9216, M = 512: 289 / 243
-//    64 x 12288:                              138 / 119, 138 / 127, 217 / 191;  64 x 16384:         582 / 406
-//    32 x 9216:                               66 / 67, 66 / 68, 98 / 90;        16 x 16384: 71 / 67, 71 / 68, 105 / 90
-//    24 x 12288, M = 128: 67 / 67 (as whole passes 67 / 71);  32 x 10240: 71 / 66, 71 / 70, 107 / 96
-// and d = 64, M = 64, 128, 256:  64 x 4096: 43 / 49, 44 / 51, 64 / 68;  64 x 6144: 59 / 57, 60 / 60, 95 / 90;  128 x 8192: 129 / 112, 129 / 120,
-// 219 / 184;  32 x 8192, M = 128: 49 / 53.
+// The fastest scorer the shape allows.  d = 64 and 128: the one-sweep kernel computes every exponential once; only where an item is
+// spread over most of the blocks (beyond 64 slabs of 256 keys) do they wait for each other's statistics long enough for the two-sweep
+// kernel, whose work is dealt item by item, to be faster - if there are several row blocks and items enough to deal.  Rows of 64
+// channels cost the one-sweep kernel as much as wider ones: there it is from 64 slabs on.  Measured as steps of a stream with
+// deferred appends (us, one sweep / items), d = 128:
+//   64 units x 8192 keys, M = 768, 1024: 249 / 289, 320 / 379;  64 x 12288, M = 512: 272 / 308;  64 x 16384, M = 256, 512, 1024: 217 / 248, 376 / 404, 694 / 712
+//   32 x 16384, M = 512: 203 / 208;  16 x 16384, M = 128, 512: 55 / 66, 120 / 126
+//   64 x 20480, M = 512: 534 / 475;  32 x 20480, M = 256: 174 / 168;  32 x 24576, M = 256: 195 / 193;  16 x 24576, M = 64, 512: 84 / 88, 190 / 222
+//   32 x 32768, M = 256: 282 / 263;  16 x 32768, M = 64: 109 / 112;  8 x 32768, M = 512: 170 / 158
+// and d = 64, M = 64, 128, 256, 512:  64 x 6144: 50 / 54, -, 78 / 87, -;  128 x 8192: 99 / 110, 101 / 118, 165 / 178, -;
+// 64 x 12288: -, 88 / 90, 141 / 148, 245 / 244;  64 x 16384: 113 / 110, -, 190 / 186, 340 / 309;  16 x 16384: 50 / 56, -, 72 / 77, -.
 // Other head dimensions have the item kernel or warp-level tensor cores, and the former wins everywhere
 // (d = 256, 64 x 4096, M = 64: 51 us against 221; d = 96, 8 x 640, M = 16: 12.5 against 18.5).
 int auto_scorer(int units, int N, int M, int d, bool tc_ok, bool items_ok, bool mma_ok)
 {
     const long long keys = (long long)units * N;
-    const bool many = d == 64 && N >= 6144 && keys >= 64 * 6144;
-    const bool long_items = (N > 8192 || (N == 8192 && M > 512)) && keys >= 32 * 8192 && (M > kTcRows || N >= 16384 || keys >= 32 * 10240);
+    const bool many = d == 64 && N >= 16384 && keys >= 64 * 16384;
+    const bool long_items = M > kTcRows && keys >= 32 * 8192 && (N > 24576 || (N > 16384 && units >= 32));
     if (items_ok && (!tc_ok || many || long_items)) return IPOT_SCORER_TENSOR_ITEMS;
     if (tc_ok) return IPOT_SCORER_TENSOR;
     return mma_ok ? IPOT_SCORER_WARP_MMA : IPOT_SCORER_SIMT;
