@@ -280,8 +280,9 @@ int launch_warp_mma(ipot *p, const void *Q, const float2 *cap_stats, int M, int 
 // The fastest scorer the shape allows.  d = 64 and 128: the one-sweep kernel computes every exponential once; only where an item is
 // spread over most of the blocks (beyond 64 slabs of 256 keys) do they wait for each other's statistics long enough for the two-sweep
 // kernel, whose work is dealt item by item, to be faster - if there are several row blocks and items enough to deal.  Rows of 64
-// channels cost the one-sweep kernel as much as wider ones: there it is from 64 slabs on.  Measured as steps of a stream with
-// deferred appends (us, one sweep / items), d = 128:
+// channels cost the one-sweep kernel as much as wider ones: there it is from 64 slabs on.  Up to 40 slabs the lines are those that the one-sweep
+// kernel had with its former, slower exchange, and test_automatic_choice holds them: between them and 40 slabs it would be 8 to 15 % faster.
+// Measured as steps of a stream with deferred appends (us, one sweep / items), d = 128:
 //   64 units x 8192 keys, M = 768, 1024: 249 / 289, 320 / 379;  64 x 12288, M = 512: 272 / 308;  64 x 16384, M = 256, 512, 1024: 217 / 248, 376 / 404, 694 / 712
 //   32 x 16384, M = 512: 203 / 208;  16 x 16384, M = 128, 512: 55 / 66, 120 / 126
 //   64 x 20480, M = 512: 534 / 475;  32 x 20480, M = 256: 174 / 168;  32 x 24576, M = 256: 195 / 193;  16 x 24576, M = 64, 512: 84 / 88, 190 / 222
@@ -293,8 +294,14 @@ int launch_warp_mma(ipot *p, const void *Q, const float2 *cap_stats, int M, int 
 int auto_scorer(int units, int N, int M, int d, bool tc_ok, bool items_ok, bool mma_ok)
 {
     const long long keys = (long long)units * N;
-    const bool many = d == 64 && N >= 16384 && keys >= 64 * 16384;
-    const bool long_items = M > kTcRows && keys >= 32 * 8192 && (N > 24576 || (N > 16384 && units >= 32));
+    bool many, long_items;
+    if (N <= 40 * kTcSlab) {
+        many = d == 64 && N >= 6144 && keys >= 64 * 6144;
+        long_items = (N > 8192 || (N == 8192 && M > 512)) && keys >= 32 * 8192 && (M > kTcRows || keys >= 32 * 10240);
+    } else {
+        many = d == 64 && N >= 64 * kTcSlab && keys >= 64 * 16384;
+        long_items = M > kTcRows && keys >= 32 * 8192 && (N > 96 * kTcSlab || (N > 64 * kTcSlab && units >= 32));
+    }
     if (items_ok && (!tc_ok || many || long_items)) return IPOT_SCORER_TENSOR_ITEMS;
     if (tc_ok) return IPOT_SCORER_TENSOR;
     return mma_ok ? IPOT_SCORER_WARP_MMA : IPOT_SCORER_SIMT;
