@@ -289,9 +289,11 @@ int launch_warp_mma(ipot *p, const void *Q, const float2 *cap_stats, int M, int 
 //   32 x 32768, M = 256: 282 / 263;  16 x 32768, M = 64: 109 / 112;  8 x 32768, M = 512: 170 / 158
 // and d = 64, M = 64, 128, 256, 512:  64 x 6144: 50 / 54, -, 78 / 87, -;  128 x 8192: 99 / 110, 101 / 118, 165 / 178, -;
 // 64 x 12288: -, 88 / 90, 141 / 148, 245 / 244;  64 x 16384: 113 / 110, -, 190 / 186, 340 / 309;  16 x 16384: 50 / 56, -, 72 / 77, -.
-// Other head dimensions have the item kernel or warp-level tensor cores, and the former wins everywhere
-// (d = 256, 64 x 4096, M = 64: 51 us against 221; d = 96, 8 x 640, M = 16: 12.5 against 18.5).
-int auto_scorer(int units, int N, int M, int d, bool tc_ok, bool items_ok, bool mma_ok)
+// Other head dimensions (whole passes, deferred, us, one sweep / items): d = 256: 64 x 4096, M = 64, 128, 256: 62 / 84, 66 / 87, 90 / 140; 32 x 8192,
+// M = 512: 136 / 225; 64 x 12288, M = 256: 248 / 375; 8 x 4096, M = 64: 20 / 25; 8 x 1024, M = 32: 16.5 / 19.7.  d = 192: 64 x 4096, M = 64, 256:
+// 54 / 72, 73 / 106.  d = 96: 64 x 4096, M = 64, 128: 41 / 51, 42 / 53; 64 x 8192, M = 256: 110 / 117; 8 x 2048, M = 64: 16.5 / 20.1.  d = 72: 32 x 700,
+// M = 32: 16.9 / 21.2.  A handful of slabs is left to the item kernel (fewer than 16 have not been measured).
+int auto_scorer(int units, int N, int M, int d, bool tile_chunk, bool tc_ok, bool items_ok, bool mma_ok)
 {
     const long long keys = (long long)units * N;
     bool many, long_items;
@@ -301,6 +303,11 @@ int auto_scorer(int units, int N, int M, int d, bool tc_ok, bool items_ok, bool 
     } else {
         many = d == 64 && N >= 64 * kTcSlab && keys >= 64 * 16384;
         long_items = M > kTcRows && keys >= 32 * 8192 && (N > 96 * kTcSlab || (N > 64 * kTcSlab && units >= 32));
+    }
+    if (d != 64 && d != 128) {
+        const long long tasks = (long long)units * ((M + kTcRows - 1) / kTcRows) * ((N + kTcSlab - 1) / kTcSlab);
+        many = tasks < 16 || tile_chunk;
+        long_items = long_items && N > 64 * kTcSlab;
     }
     if (items_ok && (!tc_ok || many || long_items)) return IPOT_SCORER_TENSOR_ITEMS;
     if (tc_ok) return IPOT_SCORER_TENSOR;
@@ -316,12 +323,17 @@ int run_scoring(ipot *p, const void *Q, const void *Kc, int cap_rows, const floa
     const bool tc_ok = tc_applicable(p->tc, p->cfg, N, M);
     const bool ts_ok = ts_applicable(p->tc, p->cfg, N, M);
     const bool mma_ok = p->cfg.dtype == IPOT_BF16 && p->cfg.d % 16 == 0;
-    if (scorer == IPOT_SCORER_TENSOR && !tc_ok) return IPOT_E_INVALID;
+    // on request only for the row sizes it has always been offered for; AUTO takes it for others too
+    if (scorer == IPOT_SCORER_TENSOR && !(tc_ok && (p->cfg.d == 64 || p->cfg.d == 128))) return IPOT_E_INVALID;
     if (scorer == IPOT_SCORER_TENSOR_SWEEPS && !ts_ok) return IPOT_E_INVALID;
     if (scorer == IPOT_SCORER_WARP_MMA && !mma_ok) return IPOT_E_INVALID;
     const bool items_ok = tw_applicable(p->tw, N, M);
     if (scorer == IPOT_SCORER_TENSOR_ITEMS && !items_ok) return IPOT_E_INVALID;
-    if (scorer == IPOT_SCORER_AUTO) scorer = auto_scorer(p->units, N, M, p->cfg.d, tc_ok, items_ok, mma_ok);
+    if (scorer == IPOT_SCORER_AUTO) {
+        // a chunk that starts between two slabs is read in place by the item kernel (tiles of 128 keys), copied first for the other
+        const bool tile_chunk = p->pend_K && !p->rope && p->pend_first % kTcSlab != 0 && p->pend_first % kTwTile == 0;
+        scorer = auto_scorer(p->units, N, M, p->cfg.d, tile_chunk, tc_ok, items_ok, mma_ok);
+    }
     // keys of a deferred append: the tensor-core scorers read whole slabs of them where they are, anything else
     // wants them in the pot
     const int slab_keys = scorer == IPOT_SCORER_TENSOR         ? kTcSlab

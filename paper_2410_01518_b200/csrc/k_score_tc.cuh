@@ -1,4 +1,4 @@
-// CaP scoring on the 5th-generation tensor cores (Sec. 3.3.1, Eq. 2), bf16, d = 128 or 64.
+// CaP scoring on the 5th-generation tensor cores (Sec. 3.3.1, Eq. 2), bf16, any d up to 256.
 //
 // Item  = (unit, block of 128 folded query rows): one row-softmax problem over the
 //         unit's N pot keys.
@@ -47,6 +47,8 @@
 // before the block releases tensor memory and ends; the epilogue warps run through
 // their remaining iterations without waiting (their results are void).
 #pragma once
+#include <algorithm>
+
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -66,10 +68,14 @@ constexpr int kTcHalf = 128;         // keys per epilogue group and entry of the
 constexpr unsigned kTcPollDelayNs = 300;
 constexpr int kTcSlab = 256;         // keys per task (TMEM columns per buffer)
 constexpr int kTcFmaEighths = 2;     // share of pass 1's exponentials evaluated on the FMA pipe
-constexpr int kTcD = 128;            // largest head dimension; 64 uses the first 64-channel half of every tile
+constexpr int kTcD = 128;            // channels of a stage; up to 64 use the first half of every tile.  Wider rows are another variant (kWide)
 constexpr uint32_t kTcQBytes = kTcRows * kTcD * 2;           // 32 KiB: two halves of 128 rows x 64 channels
 constexpr uint32_t kTcKBytes = kTcSlab * kTcD * 2;           // 64 KiB: two halves of 256 rows x 64 channels
 constexpr uint32_t kTcStageBytes = kTcQBytes + kTcKBytes;    // 96 KiB
+// More than 128 channels: one or two query tiles and two or three half slabs of keys share the space of the two stages, each a slot
+// of its own - a whole stage of 256 channels would be all there is room for.  (Slots like these for every width: 4 % slower at 128 channels.)
+constexpr uint32_t kTcKBlk = kTcHalf * 128;                  // 64 channels of a half slab's keys
+constexpr int kTcMaxK = 4;
 
 // shared-memory carve-up (bytes from the 1024-aligned base)
 constexpr uint32_t kTcOffStage = 0;                                        // [2] { Q, K }
@@ -77,12 +83,15 @@ constexpr uint32_t kTcOffColpart = 2 * kTcStageBytes;                      // [4
 constexpr uint32_t kTcOffLpart = kTcOffColpart + 4 * 2 * 4 * kTcHalf * 4;      // [2 pairs][2 parities][2 halves][128] float
 constexpr uint32_t kTcOffSpart = kTcOffLpart + 2 * 2 * 2 * kTcRows * 4;        // [2 pairs][2 parities][128] float2
 constexpr uint32_t kTcOffBar = kTcOffSpart + 2 * 2 * kTcRows * 8;
-constexpr uint32_t kTcOffTmemSlot = kTcOffBar + 192;                       // the allocated TMEM base address
-constexpr uint32_t kTcOffAbort = kTcOffBar + 196;                          // set once a wait of the CTA has run out; + 4: the block's deadline (8 bytes)
+constexpr uint32_t kTcOffTmemSlot = kTcOffBar + 208;                       // the allocated TMEM base address
+constexpr uint32_t kTcOffAbort = kTcOffBar + 212;                          // set once a wait of the CTA has run out; + 4: the block's deadline (8 bytes)
 constexpr uint32_t kTcSmemBytes = kTcOffBar + 256;                         // no static shared memory: the base is 1024-aligned
 
-// barriers: per stage Full, Empty; per group (= buffer half 2 * buffer + half) SFull, TEmpty
-enum { kBarFull = 0, kBarEmpty = 2, kBarSFull = 4, kBarTEmpty = 8, kBarDrain = 12, kBarCount = 13 };
+// barriers: per stage Full, Empty; per group (= buffer half 2 * buffer + half) SFull, TEmpty; wide rows: per query and key slot Full, Empty
+enum {
+    kBarFull = 0, kBarEmpty = 2, kBarSFull = 4, kBarTEmpty = 8, kBarDrain = 12, kBarQFull = 13, kBarQEmpty = 15, kBarKFull = 17,
+    kBarKEmpty = kBarKFull + kTcMaxK, kBarCount = kBarKEmpty + kTcMaxK
+};
 
 struct TcParams {
     float *scores;        // partial array p (query rows 128p ...) at scores + p * part_stride, unit stride N
@@ -96,7 +105,12 @@ struct TcParams {
     int withhold_cta;     // -1; test hook: this CTA never publishes its slab statistics
     int *status;
     int N, M, mtiles, slabs, tasks;
-    int dhalves;          // d / 64: 64-channel halves of a tile (1 or 2)
+    int dhalves;          // 64-channel blocks of a row; what the last one lacks is filled with zeros
+    // wide rows: 16-channel steps; bytes of 64 channels of a query tile, of the tile, of a half slab's keys; slots.  M <= 64: the tile has 64
+    // rows; a product still has 128, of which the lower half multiplies whatever lies behind the tile and is never read
+    int ksteps;
+    uint32_t q_blk, q_bytes, k_bytes;
+    int qslots, kslots;
     int new_slab0;        // slabs from this one on are read through the second key map (the chunk of a deferred
                           // append, row 0 = key 256 * new_slab0); INT_MAX if all keys are in the pot
     float scale_log2e;
@@ -505,7 +519,8 @@ constexpr uint32_t kTcIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) 
 // ------------------------------------------------------------------ the kernel
 // kRank: blocks from prm.ctas on rank the streams' novelty.  (Their code costs the others about 5 % through the register
 // allocation, so launches of more than a dozen rounds use the variant without it and a ranking kernel on the side.)
-template <bool kRank>
+// kWide: rows of more than 128 channels.
+template <bool kRank, bool kWide>
 __global__ void __launch_bounds__(kTcThreads, 1)
 cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                     const __grid_constant__ CUtensorMap mapKnew, const __grid_constant__ TcParams prm)
@@ -534,6 +549,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             mbar_init(bar(kBarFull + b), 1);
             mbar_init(bar(kBarEmpty + b), 1);
         }
+        for (int i = kBarQFull; i < kBarCount; ++i) mbar_init(bar(i), 1);
         for (int g = 0; g < 4; ++g) {
             mbar_init(bar(kBarSFull + g), 1);
             mbar_init(bar(kBarTEmpty + g), 4);
@@ -555,28 +571,68 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
         if (lane == 0) {
-            uint32_t k = 0;
-            for (int task = blockIdx.x; task < prm.tasks; task += prm.ctas, ++k) {
-                const int item = task / tasks_per_item, slab = task - item * tasks_per_item;
-                const int unit = item / prm.mtiles, mt = item - unit * prm.mtiles;
-                const uint32_t b = k & 1, ph = (k >> 1) & 1;
-                if (!mbar_wait(bar(kBarEmpty + b), ph ^ 1, ab, prm.status)) break;   // nothing more is put in flight
-                mbar_expect_tx(bar(kBarFull + b), (uint32_t)prm.dhalves * (kTcStageBytes / 2));
-                const uint32_t q = base + kTcOffStage + b * kTcStageBytes, kk = q + kTcQBytes;
-                const bool fresh_rows = slab >= prm.new_slab0;
-                const CUtensorMap *mk = fresh_rows ? &mapKnew : &mapK;
-                const int krow = (fresh_rows ? slab - prm.new_slab0 : slab) * kTcSlab;
-                tma_load_3d(q, &mapQ, 0, mt * kTcRows, unit, bar(kBarFull + b));
-                tma_load_3d(kk, mk, 0, krow, unit, bar(kBarFull + b));
-                if (prm.dhalves == 2) {
-                    tma_load_3d(q + kTcQBytes / 2, &mapQ, 64, mt * kTcRows, unit, bar(kBarFull + b));
-                    tma_load_3d(kk + kTcKBytes / 2, mk, 64, krow, unit, bar(kBarFull + b));
+            if (kWide) {
+                const uint32_t q_blk = prm.q_blk, q_bytes = prm.q_bytes, k_bytes = prm.k_bytes, q_base = base + kTcOffStage, k_base = q_base + prm.qslots * q_bytes;
+                uint32_t qn = 0, kn = 0, qs = 0, qph = 1, ks = 0, kph = 1;   // (slots and phases are counted on: divisions would delay every load)
+                bool ok = true;
+                for (int task = blockIdx.x; task < prm.tasks && ok; task += prm.ctas) {
+                    const int item = task / tasks_per_item, slab = task - item * tasks_per_item;
+                    const int unit = item / prm.mtiles, mt = item - unit * prm.mtiles;
+                    if (!mbar_wait(bar(kBarQEmpty + qs), qph, ab, prm.status)) break;   // nothing more is put in flight
+                    ++qn;
+                    mbar_expect_tx(bar(kBarQFull + qs), q_bytes);
+                    for (int blk = 0; blk < prm.dhalves; ++blk)
+                        tma_load_3d(q_base + qs * q_bytes + blk * q_blk, &mapQ, 64 * blk, mt * kTcRows, unit, bar(kBarQFull + qs));
+                    if (++qs == (uint32_t)prm.qslots) {
+                        qs = 0;
+                        qph ^= 1;
+                    }
+                    const bool fresh_rows = slab >= prm.new_slab0;
+                    const CUtensorMap *mk = fresh_rows ? &mapKnew : &mapK;
+                    const int krow = (fresh_rows ? slab - prm.new_slab0 : slab) * kTcSlab;
+                    for (int h = 0; h < 2; ++h) {
+                        ok = mbar_wait(bar(kBarKEmpty + ks), kph, ab, prm.status);
+                        if (!ok) break;
+                        ++kn;
+                        mbar_expect_tx(bar(kBarKFull + ks), k_bytes);
+                        for (int blk = 0; blk < prm.dhalves; ++blk)
+                            tma_load_3d(k_base + ks * k_bytes + blk * kTcKBlk, mk, 64 * blk, krow + h * kTcHalf, unit, bar(kBarKFull + ks));
+                        if (++ks == (uint32_t)prm.kslots) {
+                            ks = 0;
+                            kph ^= 1;
+                        }
+                    }
                 }
+                // loads that were issued land in this CTA's shared memory: see the last one into every slot complete before
+                // the CTA may end (load j went to slot j % slots as its (j / slots)-th fill)
+                for (uint32_t j = qn > (uint32_t)prm.qslots ? qn - prm.qslots : 0; j < qn; ++j)
+                    mbar_wait(bar(kBarQFull + j % prm.qslots), (j / prm.qslots) & 1, ab, prm.status, false);
+                for (uint32_t j = kn > (uint32_t)prm.kslots ? kn - prm.kslots : 0; j < kn; ++j)
+                    mbar_wait(bar(kBarKFull + j % prm.kslots), (j / prm.kslots) & 1, ab, prm.status, false);
+            } else {
+                uint32_t k = 0;
+                for (int task = blockIdx.x; task < prm.tasks; task += prm.ctas, ++k) {
+                    const int item = task / tasks_per_item, slab = task - item * tasks_per_item;
+                    const int unit = item / prm.mtiles, mt = item - unit * prm.mtiles;
+                    const uint32_t b = k & 1, ph = (k >> 1) & 1;
+                    if (!mbar_wait(bar(kBarEmpty + b), ph ^ 1, ab, prm.status)) break;   // nothing more is put in flight
+                    mbar_expect_tx(bar(kBarFull + b), (uint32_t)prm.dhalves * (kTcStageBytes / 2));
+                    const uint32_t q = base + kTcOffStage + b * kTcStageBytes, kk = q + kTcQBytes;
+                    const bool fresh_rows = slab >= prm.new_slab0;
+                    const CUtensorMap *mk = fresh_rows ? &mapKnew : &mapK;
+                    const int krow = (fresh_rows ? slab - prm.new_slab0 : slab) * kTcSlab;
+                    tma_load_3d(q, &mapQ, 0, mt * kTcRows, unit, bar(kBarFull + b));
+                    tma_load_3d(kk, mk, 0, krow, unit, bar(kBarFull + b));
+                    if (prm.dhalves == 2) {
+                        tma_load_3d(q + kTcQBytes / 2, &mapQ, 64, mt * kTcRows, unit, bar(kBarFull + b));
+                        tma_load_3d(kk + kTcKBytes / 2, mk, 64, krow, unit, bar(kBarFull + b));
+                    }
+                }
+                // loads that were issued land in this CTA's shared memory: see the last one of either stage complete before
+                // the CTA may end (k loads were issued; load j went to stage j & 1 as its (j >> 1)-th fill)
+                for (uint32_t j = (k > 2 ? k - 2 : 0); j < k; ++j)
+                    mbar_wait(bar(kBarFull + (j & 1)), (j >> 1) & 1, ab, prm.status, false);
             }
-            // loads that were issued land in this CTA's shared memory: see the last one of either stage complete before
-            // the CTA may end (k loads were issued; load j went to stage j & 1 as its (j >> 1)-th fill)
-            for (uint32_t j = (k > 2 ? k - 2 : 0); j < k; ++j)
-                mbar_wait(bar(kBarFull + (j & 1)), (j >> 1) & 1, ab, prm.status, false);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -585,34 +641,73 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         // MMA instruction wants them (a lone thread gets eight MMAs of 128 columns
         // accepted in about 900 cycles, an elected lane in 530; alone: 256 units x 4096 keys, M = 128 91.4 -> 90.2 us, 60 x 2999 22.5 -> 21.4, 8 x 4096 9.2 -> 8.6).
         const bool leader = elect_one();
-        const uint64_t q_desc = smem_desc_sw128(base + kTcOffStage), k_desc = smem_desc_sw128(base + kTcOffStage + kTcQBytes);
-        uint32_t k = 0;
         bool any = false;
-        for (int task = blockIdx.x; task < prm.tasks; task += prm.ctas, ++k) {
-            const uint32_t b = k & 1, ph = (k >> 1) & 1;
-            if (!__all_sync(0xffffffffu, mbar_wait(bar(kBarFull + b), ph, ab, prm.status))) break;
+        if (kWide) {
+            const uint32_t q_blk = prm.q_blk, q_bytes = prm.q_bytes, k_bytes = prm.k_bytes, q_base = base + kTcOffStage;
+            const uint64_t q_desc = smem_desc_sw128(q_base), k_desc = smem_desc_sw128(q_base + prm.qslots * q_bytes);
+            uint32_t k = 0, qs = 0, qph = 0, ks = 0, kph = 0;
             bool ok = true;
-            for (uint32_t h = 0; h < 2; ++h) {
-                ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarTEmpty + 2 * b + h), ph ^ 1, ab, prm.status));
-                if (!ok) break;
-                any = true;
-                tc_fence_after();
-                const uint64_t da = q_desc + b * (kTcStageBytes >> 4), db = k_desc + b * (kTcStageBytes >> 4) + h * (128 * 128 >> 4);
-                const uint32_t d = tmem + b * kTcSlab + h * 128;
-                if (leader) {
+            for (int task = blockIdx.x; task < prm.tasks && ok; task += prm.ctas, ++k) {
+                const uint32_t b = k & 1, ph = (k >> 1) & 1;
+                ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarQFull + qs), qph, ab, prm.status));
+                for (uint32_t h = 0; h < 2 && ok; ++h) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarKFull + ks), kph, ab, prm.status) && mbar_wait(bar(kBarTEmpty + 2 * b + h), ph ^ 1, ab, prm.status));
+                    if (!ok) break;
+                    any = true;
+                    tc_fence_after();
+                    uint64_t da = q_desc + qs * (q_bytes >> 4), db = k_desc + ks * (k_bytes >> 4);
+                    const uint32_t d = tmem + b * kTcSlab + h * kTcHalf;
+                    if (leader) {
+                        for (int c = 0; c < prm.ksteps; c += 4, da += q_blk >> 4, db += kTcKBlk >> 4) {
+                            tc_mma_bf16(d, da, db, kTcIdesc, c ? 1u : 0u);
 #pragma unroll
-                    for (uint32_t k4 = 0; k4 < 4; ++k4) tc_mma_bf16(d, da + 2 * k4, db + 2 * k4, kTcIdesc, k4 ? 1u : 0u);
-                    if (prm.dhalves == 2) {
-#pragma unroll
-                        for (uint32_t k4 = 0; k4 < 4; ++k4)
-                            tc_mma_bf16(d, da + (kTcQBytes / 2 >> 4) + 2 * k4, db + (kTcKBytes / 2 >> 4) + 2 * k4, kTcIdesc, 1u);
+                            for (int i = 1; i < 4; ++i)
+                                if (c + i < prm.ksteps) tc_mma_bf16(d, da + 2 * i, db + 2 * i, kTcIdesc, 1u);
+                        }
+                        tc_commit(bar(kBarSFull + 2 * b + h));   // this half's logits are complete
+                        tc_commit(bar(kBarKEmpty + ks));         // the slots may be refilled once the MMAs have read them
+                        if (h) tc_commit(bar(kBarQEmpty + qs));
                     }
-                    tc_commit(bar(kBarSFull + 2 * b + h));   // this half's logits are complete
-                    if (h) tc_commit(bar(kBarEmpty + b));    // the stage may be refilled once the MMAs have read it
+                    __syncwarp();
+                    if (++ks == (uint32_t)prm.kslots) {
+                        ks = 0;
+                        kph ^= 1;
+                    }
                 }
-                __syncwarp();
+                if (++qs == (uint32_t)prm.qslots) {
+                    qs = 0;
+                    qph ^= 1;
+                }
             }
-            if (!ok) break;
+        } else {
+            const uint64_t q_desc = smem_desc_sw128(base + kTcOffStage), k_desc = smem_desc_sw128(base + kTcOffStage + kTcQBytes);
+            uint32_t k = 0;
+            for (int task = blockIdx.x; task < prm.tasks; task += prm.ctas, ++k) {
+                const uint32_t b = k & 1, ph = (k >> 1) & 1;
+                if (!__all_sync(0xffffffffu, mbar_wait(bar(kBarFull + b), ph, ab, prm.status))) break;
+                bool ok = true;
+                for (uint32_t h = 0; h < 2; ++h) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(bar(kBarTEmpty + 2 * b + h), ph ^ 1, ab, prm.status));
+                    if (!ok) break;
+                    any = true;
+                    tc_fence_after();
+                    const uint64_t da = q_desc + b * (kTcStageBytes >> 4), db = k_desc + b * (kTcStageBytes >> 4) + h * (128 * 128 >> 4);
+                    const uint32_t d = tmem + b * kTcSlab + h * 128;
+                    if (leader) {
+#pragma unroll
+                        for (uint32_t k4 = 0; k4 < 4; ++k4) tc_mma_bf16(d, da + 2 * k4, db + 2 * k4, kTcIdesc, k4 ? 1u : 0u);
+                        if (prm.dhalves == 2) {
+#pragma unroll
+                            for (uint32_t k4 = 0; k4 < 4; ++k4)
+                                tc_mma_bf16(d, da + (kTcQBytes / 2 >> 4) + 2 * k4, db + (kTcKBytes / 2 >> 4) + 2 * k4, kTcIdesc, 1u);
+                        }
+                        tc_commit(bar(kBarSFull + 2 * b + h));   // this half's logits are complete
+                        if (h) tc_commit(bar(kBarEmpty + b));    // the stage may be refilled once the MMAs have read it
+                    }
+                    __syncwarp();
+                }
+                if (!ok) break;
+            }
         }
         if (any) {  // every MMA has finished (and read its operands) before tensor memory is released
             if (leader) tc_commit(bar(kBarDrain));
@@ -650,7 +745,10 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             const bool works = q * 32 < rows && nvalid > 0;   // (uniform over the warp)
             const uint32_t par = j & 1;
             float2 own = make_float2(-INFINITY, 0.f);  // the CaP keys' share of this row's denominator (Appendix B listing)
-            if (prm.cap_stats && row < rows) own = __ldg(&prm.cap_stats[(size_t)unit * prm.M + mt * kTcRows + row]);
+            auto load_own = [&]() {
+                if (prm.cap_stats && row < rows) own = __ldg(&prm.cap_stats[(size_t)unit * prm.M + mt * kTcRows + row]);
+            };
+            if (!kWide) load_own();
             float *st = prm.stats + (size_t)item * S * kTcRows + row;
             float2 s = make_float2(0.f, nvalid > 0 ? 1.f : 0.f);
             mbar_wait(bar(kBarSFull + g), par, ab, prm.status);
@@ -713,6 +811,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                     st_gpu_f32(to, INFINITY * sgn);
                 }
             }
+            if (kWide) load_own();   // (two registers that pass 1 of this variant does not have)
             // ---- the row's entries of the whole item, each half of the pair one half of them
             float l = 0.f;
             if (row < rows) {
@@ -894,18 +993,20 @@ inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, int sm_count, D
         return;
     }
     plan.encode = reinterpret_cast<TcEncodeFn>(fn);   // (the two-sweep scorers need it too)
-    if (cfg.d != 128 && cfg.d != 64) return;
+    // Rows of other sizes than 64 and 128 are AUTO's alone (ipot_api.cu), and a row block fetches its unit's keys anew: beyond four of them
+    // such a pot keeps to the item kernel, whose sweeps fetch the keys once for all, and to the scratch that it has always had.
+    const int G = cfg.Hq / cfg.Hkv;
+    if (cfg.d != 64 && cfg.d != 128 && G * cfg.max_cap_rows > 4 * kTcRows) return;
     int coop = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) {
         cudaGetLastError();
         return;
     }
-    if (cudaFuncSetAttribute(cap_score_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(cap_score_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes) != cudaSuccess) {
-        cudaGetLastError();
-        return;
-    }
-    const int G = cfg.Hq / cfg.Hkv;
+    for (auto kern : {cap_score_tc_kernel<false, false>, cap_score_tc_kernel<true, false>, cap_score_tc_kernel<false, true>, cap_score_tc_kernel<true, true>})
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
     const int units = cfg.layers * cfg.batch * cfg.Hkv;
     plan.max_items = units * ((G * cfg.max_cap_rows + kTcRows - 1) / kTcRows);
     plan.max_slabs = (cfg.pot_size + kTcSlab - 1) / kTcSlab;
@@ -916,7 +1017,7 @@ inline void tc_plan_init(TcPlan &plan, const ipot_config_t &cfg, int sm_count, D
 
 inline bool tc_applicable(TcPlan &plan, const ipot_config_t &cfg, int N, int M)
 {
-    if (!plan.usable || cfg.dtype != IPOT_BF16 || (cfg.d != 128 && cfg.d != 64) || N < 1 || M < 1) return false;
+    if (!plan.usable || cfg.dtype != IPOT_BF16 || N < 1 || M < 1) return false;
     const int units = cfg.layers * cfg.batch * cfg.Hkv;
     return units * ((M + kTcRows - 1) / kTcRows) <= plan.max_items && (N + kTcSlab - 1) / kTcSlab <= plan.max_slabs;
 }
@@ -955,24 +1056,32 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
     if (!tc_applicable(plan, cfg, N, M)) return IPOT_E_INVALID;
     if (Knew && (new_first % kTcSlab != 0 || new_first >= N)) return IPOT_E_INVALID;
     const int mtiles = (M + kTcRows - 1) / kTcRows;
+    const bool wide = cfg.d > kTcD;
+    const int qrows = wide && M <= kTcRows / 2 ? kTcRows / 2 : kTcRows, krows = wide ? kTcHalf : kTcSlab;   // of a TMA box
     CUtensorMap mapQ, mapK, mapKnew;
-    if (tc_encode_rows(plan, &mapQ, Q, cfg.d, M, units, (size_t)M, kTcRows) != IPOT_OK) return IPOT_E_CUDA;
+    if (tc_encode_rows(plan, &mapQ, Q, cfg.d, M, units, (size_t)M, qrows) != IPOT_OK) return IPOT_E_CUDA;
     if (Knew && new_first == 0) {  // every key is in the chunk
-        if (tc_encode_rows(plan, &mapK, Knew, cfg.d, N, units, (size_t)N, kTcSlab) != IPOT_OK) return IPOT_E_CUDA;
+        if (tc_encode_rows(plan, &mapK, Knew, cfg.d, N, units, (size_t)N, krows) != IPOT_OK) return IPOT_E_CUDA;
         Knew = nullptr;
-    } else if (tc_encode_rows(plan, &mapK, K, cfg.d, Knew ? new_first : N, units, (size_t)cfg.pot_size, kTcSlab) != IPOT_OK) {
+    } else if (tc_encode_rows(plan, &mapK, K, cfg.d, Knew ? new_first : N, units, (size_t)cfg.pot_size, krows) != IPOT_OK) {
         return IPOT_E_CUDA;
     }
     if (!Knew) mapKnew = mapK;
-    else if (tc_encode_rows(plan, &mapKnew, Knew, cfg.d, N - new_first, units, (size_t)(N - new_first), kTcSlab) != IPOT_OK) return IPOT_E_CUDA;
+    else if (tc_encode_rows(plan, &mapKnew, Knew, cfg.d, N - new_first, units, (size_t)(N - new_first), krows) != IPOT_OK) return IPOT_E_CUDA;
     TcParams prm;
     prm.scores = scores; prm.part_stride = part_stride; prm.stats = plan.stats; prm.refs = plan.refs; prm.cap_stats = cap_stats; prm.status = status;
     prm.N = N; prm.M = M; prm.mtiles = mtiles; prm.slabs = (N + kTcSlab - 1) / kTcSlab;
     const int items = units * mtiles;
     prm.tasks = items * prm.slabs;
-    prm.dhalves = cfg.d / 64;
+    prm.dhalves = (cfg.d + 63) / 64;
+    prm.ksteps = (cfg.d + 15) / 16;
+    prm.q_blk = (uint32_t)qrows * 128u;
+    prm.q_bytes = (uint32_t)prm.dhalves * prm.q_blk;
+    prm.k_bytes = (uint32_t)prm.dhalves * kTcKBlk;
+    prm.qslots = 2 * prm.q_bytes + 2 * prm.k_bytes <= 2 * kTcStageBytes ? 2 : 1;   // 256 channels: 2 + 2 slots up to 64 query rows, else 1 + 2; 192: 2 + 3, 2 + 2
+    prm.kslots = std::min<int>(kTcMaxK, (2 * kTcStageBytes - prm.qslots * prm.q_bytes) / prm.k_bytes);
     prm.new_slab0 = Knew ? new_first / kTcSlab : 0x7fffffff;
-    prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d) * (1.0 + 1.2e-8 * (cfg.d / 16)));
+    prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d) * (1.0 + 1.2e-8 * prm.ksteps));
     prm.wait_ns = wait_ns;
     prm.withhold_cta = withhold_cta;
     if (!plan.captured) {
@@ -1008,7 +1117,9 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
     at[0].id = cudaLaunchAttributeCooperative;  // all CTAs resident: they wait on each other's statistics
     at[0].val.cooperative = 1;
     lc.attrs = at; lc.numAttrs = 1;
-    if (cudaLaunchKernelEx(&lc, nuc.ctas > 0 ? cap_score_tc_kernel<true> : cap_score_tc_kernel<false>, mapQ, mapK, mapKnew, prm) != cudaSuccess) {
+    auto kern = wide ? (nuc.ctas > 0 ? cap_score_tc_kernel<true, true> : cap_score_tc_kernel<false, true>)
+                     : (nuc.ctas > 0 ? cap_score_tc_kernel<true, false> : cap_score_tc_kernel<false, false>);
+    if (cudaLaunchKernelEx(&lc, kern, mapQ, mapK, mapKnew, prm) != cudaSuccess) {
         cudaGetLastError();
         plan.last_items = 0;   // the array still holds what the last launch that ran has left
         return IPOT_E_CUDA;

@@ -85,3 +85,22 @@ def test_one_sweep_calls_of_different_row_counts_share_one_pot():
             assert torch.allclose(got.sum(1), torch.full((cfg.units,), float(P * cfg.Hq // cfg.Hkv), device="cuda"), rtol=1e-4)
     finally:
         ipot.ipot_destroy(h)
+
+
+@pytest.mark.parametrize("n,P,Hq,Hkv,d,L,B", [
+    # one to four 64-channel blocks, the last one whole, a quarter, half or an eighth filled; a query tile of 64 or 128 rows, so
+    # that two or three half slabs of keys are in flight beside one or two query tiles; ragged ends as above
+    (2047, 16, 8, 2, 96, 3, 1), (2300, 40, 4, 1, 40, 4, 2), (700, 3, 2, 2, 72, 8, 1), (999, 5, 6, 2, 136, 6, 1), (3000, 33, 8, 4, 192, 3, 1),
+    (900, 16, 8, 2, 192, 5, 1), (1500, 48, 16, 2, 256, 3, 1), (1281, 19, 3, 3, 256, 4, 2), (4096, 32, 16, 8, 256, 21, 1)])
+def test_one_sweep_rows_of_other_sizes(n, P, Hq, Hkv, d, L, B):
+    """Head dimensions that reach the kernel through the automatic choice; keys of a deferred chunk are read where they lie from whole
+    slabs on, the same products in the same order, and a chunk that starts between two slabs agrees within the tolerance."""
+    cfg = inputs.small_config(cfg_id=980 + d, pot_size=n, keep=n // 2, nuc_slots=n // 4, cap_rows=P, Hq=Hq, Hkv=Hkv, d=d, dtype="bf16", layers=L, batch=B)
+    t = inputs.make_cycle(cfg)
+    units = None if cfg.units <= 24 else np.linspace(0, cfg.units - 1, 24).astype(np.int32)
+    gpu = gpu_cycle(cfg, t)
+    same, cnt = compare_cycle(cfg, t, gpu, units=units)
+    assert same >= cnt - 1
+    got = gpu_cycle(cfg, t, deferred_from=256)
+    assert all((a == b).all() for a, b in zip(got, gpu))
+    compare_cycle(cfg, t, gpu_cycle(cfg, t, deferred_from=384), units=units)
