@@ -352,9 +352,12 @@ __device__ __forceinline__ void piece_exp(uint32_t (&v)[16], float c, PieceSum &
         v[i + 1] = __float_as_uint(e2.y);
     }
 }
-constexpr float kTcSumMax = 1.2676506e30f;    // 2^100
+// A row's sums against the reference 0 stay below 2^60: its weights then do not fall below fp32's range while what they multiply still
+// counts (a probability is lost only below 2^-66, and only beside a logit that is 2^126 above the reference).
+constexpr float kTcSumMax = 1.1529215e18f;    // 2^60
 constexpr float kTcSumMin = 9.0949470e-13f;   // 2^-40: nothing above 2^-86 of the sum is lost to flushing
-constexpr float kTcReach = 100.f;
+constexpr float kTcReach = 60.f;
+constexpr float kTcRefLow = -40.f, kTcRefHigh = 110.f;   // sums against such references are published as they are, times 2^reference
 constexpr float kTcTiny = 1.1754944e-38f;     // an entry that adds nothing is still not 0
 
 // Pass 1 for a warp some of whose rows left the comfortable range: the first `done` pieces of 16 columns have been stored as 2^(x c);
@@ -372,7 +375,7 @@ __device__ __noinline__ float2 pass1_slow(uint32_t taddr, int done, int nvalid, 
         for (int e = 0; e < 16; ++e)
             if (16 * i + e < nvalid) mx = fmaxf(mx, __uint_as_float(v[e]));
     }
-    float m = mx * c;
+    float m = ceilf(mx * c);   // a whole number: moving a sum to another reference is exact
     if (done) m = fmaxf(m, 0.f);
     if (m == -INFINITY) m = 0.f;   // every logit beyond fp32's range
     const float down = ex2(-m);
@@ -450,22 +453,35 @@ __device__ __forceinline__ float poll_entries(const float *st, int n, float sgn,
     }
     return v[0];
 }
-// A row's denominator when some entry's reference is not 0: all entries in order, relative to the largest reference
+// A row's denominator when some entry is given as (reference, sum): sixteen entries at a time with all loads in flight, relative to the
+// largest reference.  (Every block that has a slab of the item comes here for one far logit in one of them; entry by entry a step of
+// 8 streams of heavy-tailed keys, 64 units x 16384, took 1243 us.)
 __device__ __noinline__ float2 merge_entries(const float *st, const float2 *refs, int entries)
 {
     asm volatile("fence.acq_rel.gpu;" ::: "memory");
     float m = -INFINITY, l = 0.f;
 #pragma unroll 1
-    for (int e = 0; e < entries; ++e) {
-        const float v = fabsf(ld_gpu_f32(st + (size_t)e * kTcRows));
-        float2 t = make_float2(0.f, v);
-        if (v == INFINITY) {
-            const float *r = reinterpret_cast<const float *>(refs + (size_t)e * kTcRows);
-            t = make_float2(ld_gpu_f32(r), ld_gpu_f32(r + 1));
-        } else if (v <= kTcTiny) continue;   // an empty entry's reference does not count
-        const float mn = fmaxf(m, t.x);
-        l = (m == -INFINITY ? 0.f : l * ex2(m - mn)) + t.y * ex2(t.x - mn);
-        m = mn;
+    for (int e0 = 0; e0 < entries; e0 += 16) {
+        float x[16], s[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) s[e] = e0 + e < entries ? fabsf(ld_gpu_f32(st + (size_t)(e0 + e) * kTcRows)) : 0.f;
+        float mb = m;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            x[e] = s[e] <= kTcTiny ? -INFINITY : 0.f;   // an empty entry's reference does not count
+            if (s[e] == INFINITY) {
+                const float *r = reinterpret_cast<const float *>(refs + (size_t)(e0 + e) * kTcRows);
+                x[e] = ld_gpu_f32(r);
+                s[e] = ld_gpu_f32(r + 1);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) mb = fmaxf(mb, x[e]);
+        if (mb == -INFINITY) continue;
+        l *= m == -INFINITY ? 0.f : ex2(m - mb);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) l = fmaf(s[e], ex2(x[e] - mb), l);
+        m = mb;
     }
     return m == -INFINITY ? make_float2(0.f, kTcTiny) : make_float2(m, l);
 }
@@ -749,7 +765,6 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 if (prm.cap_stats && row < rows) own = __ldg(&prm.cap_stats[(size_t)unit * prm.M + mt * kTcRows + row]);
             };
             if (!kWide) load_own();
-            float *st = prm.stats + (size_t)item * S * kTcRows + row;
             float2 s = make_float2(0.f, nvalid > 0 ? 1.f : 0.f);
             mbar_wait(bar(kBarSFull + g), par, ab, prm.status);
             if (pair | j) turn_wait(pair, q);
@@ -798,22 +813,24 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             pair_sync(pair);
             if (!half && (int)blockIdx.x != prm.withhold_cta) {
                 const float2 o = spart[par * kTcRows + row];
-                float *to = st + (size_t)slab * kTcRows;
-                const float sum = s.y + o.y;
-                if (s.x == 0.f && o.x == 0.f && sum == sum) {   // (a NaN takes the other way, or it would never count as fresh)
+                float *to = prm.stats + ((size_t)item * S + slab) * kTcRows + row;
+                const float m = s.x == o.x ? s.x : fmaxf(s.y == 0.f ? -INFINITY : s.x, o.y == 0.f ? -INFINITY : o.x);   // (one of them is not empty)
+                float sum = s.y + o.y;
+                if (s.x != o.x) sum = (s.y == 0.f ? 0.f : s.y * ex2(s.x - m)) + (o.y == 0.f ? 0.f : o.y * ex2(o.x - m));
+                if (m >= kTcRefLow && m <= kTcRefHigh && sum == sum) {   // (a NaN takes the other way, or it would never count as fresh)
+                    if (m != 0.f) sum *= ex2(m);
                     st_gpu_f32(to, sum == 0.f ? kTcTiny * sgn : sum * sgn);
                 } else {
-                    const float m = fmaxf(s.y == 0.f ? -INFINITY : s.x, o.y == 0.f ? -INFINITY : o.x);   // (one of them is not empty)
                     float *r = reinterpret_cast<float *>(prm.refs + ((size_t)item * S + slab) * kTcRows + row);
                     st_gpu_f32(r, m);
-                    st_gpu_f32(r + 1, (s.y == 0.f ? 0.f : s.y * ex2(s.x - m)) + (o.y == 0.f ? 0.f : o.y * ex2(o.x - m)));
+                    st_gpu_f32(r + 1, sum);
                     asm volatile("fence.acq_rel.gpu;" ::: "memory");
                     st_gpu_f32(to, INFINITY * sgn);
                 }
             }
-            if (kWide) load_own();   // (two registers that pass 1 of this variant does not have)
             // ---- the row's entries of the whole item, each half of the pair one half of them
             float l = 0.f;
+            const float *st = prm.stats + (size_t)item * S * kTcRows + row;
             if (row < rows) {
                 if (j) __nanosleep(kTcPollDelayNs);
                 const int end = half ? S : mid;
