@@ -70,7 +70,8 @@ enum {
 enum {
     IPOT_SCORER_AUTO = 0,   /* the fastest kernel the shape allows: tcgen05, else warp-level tensor cores, else fp32 FMAs */
     IPOT_SCORER_SIMT = 1,   /* fp32 FMA kernel: any supported shape, f32 or bf16 */
-    IPOT_SCORER_TENSOR = 2, /* tcgen05 kernel (bf16, d = 64 or 128): IPOT_E_INVALID if the shape does not allow it */
+    IPOT_SCORER_TENSOR = 2, /* tcgen05 kernel in one sweep (on request bf16, d = 64 or 128: IPOT_E_INVALID if the shape does not
+                                allow it; AUTO takes it for other d too) */
     IPOT_SCORER_WARP_MMA = 3, /* warp-level tensor-core kernels (bf16, d a multiple of 16): what AUTO takes for bf16
                                 pots the tcgen05 kernels do not; IPOT_E_INVALID if the shape does not allow it */
     IPOT_SCORER_TENSOR_SWEEPS = 4, /* tcgen05 kernel that goes over the keys twice (row log-sum-exps, then probabilities
@@ -78,8 +79,8 @@ enum {
                                 it is not co-scheduled with (bf16, d = 64 or 128, at most 512 folded query rows); on request
                                 only: IPOT_E_INVALID if the shape does not allow it */
     IPOT_SCORER_TENSOR_ITEMS = 5 /* tcgen05 kernel in two sweeps whose pieces are dealt to the SMs one by one (bf16, any
-                                d, at most 1024 folded query rows): what AUTO takes for head dimensions other than
-                                64 and 128, and for long units if there are many; IPOT_E_INVALID if the shape does not
+                                d, at most 1024 folded query rows): what AUTO takes for long units, for pots of
+                                other d than 64 and 128 with many query rows and for very small calls; IPOT_E_INVALID if the shape does not
                                 allow it (or its scratch did not fit into the device's memory) */
 };
 

@@ -33,7 +33,7 @@
 // exchange a launch of 256 units takes 66 us.)  The polls are what the exchange costs: with an entry per 128 keys instead of one per
 // 256 the last of these figures were 85.2, 173, 18.5 and 384.  Measured against the form in which all 16 warps
 // shared a task, took maxima, and four more warps combined and polled (us, alone): 256 units x 4096 keys, M = 128 90.1 -> 82; 128 x
-// 8192, M = 256 197 -> 157; 60 x 2999, M = 57 20.8 -> 18.5; 64 x 16384, M = 512 537 -> 333.  Error of the scores against
+// 8192, M = 256 197 -> 157; 60 x 2999, M = 57 20.8 -> 18.5; 64 x 16384, M = 512 537 -> 333; items -> this: 64 x 4096 x 256 channels, M = 64 51 -> 27.  Error of the scores against
 // 64 bits 4.5e-7 -> 1.6e-7 (fewer roundings, a polynomial of degree 5, the tensor core's cut sums made good).
 //
 // Blocks of one grid wait on each other (pass 2 needs the other slabs' statistics),
@@ -653,9 +653,9 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         __syncwarp();
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
-        // The whole warp walks the schedule and one lane issues: descriptors and counters then live in uniform registers, where the
-        // MMA instruction wants them (a lone thread gets eight MMAs of 128 columns
-        // accepted in about 900 cycles, an elected lane in 530; alone: 256 units x 4096 keys, M = 128 91.4 -> 90.2 us, 60 x 2999 22.5 -> 21.4, 8 x 4096 9.2 -> 8.6).
+        // The whole warp walks the schedule and one lane issues: descriptors and counters then live in uniform registers, where the MMA
+        // instruction wants them (a lone thread gets eight MMAs of 128 columns accepted in about 900 cycles, an elected lane in 530;
+        // alone: 256 units x 4096 keys, M = 128 91.4 -> 90.2 us, 60 x 2999 22.5 -> 21.4, 8 x 4096 9.2 -> 8.6).
         const bool leader = elect_one();
         bool any = false;
         if (kWide) {
