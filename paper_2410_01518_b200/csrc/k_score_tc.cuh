@@ -808,6 +808,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 }
             }
             if (task + prm.ctas < prm.tasks) turn_pass(pair, q);
+            if (kWide) load_own();   // (two registers that pass 1 of this variant does not have)
             // ---- the pair's two sums together are the slab's entry
             if (half) spart[par * kTcRows + row] = s;
             pair_sync(pair);

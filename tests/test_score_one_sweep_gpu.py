@@ -104,3 +104,34 @@ def test_one_sweep_rows_of_other_sizes(n, P, Hq, Hkv, d, L, B):
     got = gpu_cycle(cfg, t, deferred_from=256)
     assert all((a == b).all() for a, b in zip(got, gpu))
     compare_cycle(cfg, t, gpu_cycle(cfg, t, deferred_from=384), units=units)
+
+
+@pytest.mark.parametrize("d", [40, 72, 96, 136, 192, 256])
+@pytest.mark.parametrize("P", [15, 17, 33, 50])   # times four query heads: both sides of 64 and 128 rows, two row blocks
+def test_one_sweep_cap_keys_join_the_softmax_of_every_row_size(d, P):
+    """Both CaP-inclusive calls on head dimensions that reach the kernel through the automatic choice.  The CaP keys take a share of
+    every denominator, so that the scores add up to less than the number of rows."""
+    cfg = inputs.small_config(cfg_id=1000 + d + P, pot_size=1100, keep=500, nuc_slots=100, cap_rows=P, Hq=16, Hkv=4, d=d, dtype="bf16", layers=2)
+    t = inputs.make_cycle(cfg)
+    t["K_cap"] = inputs.make_kcap(cfg)
+    gpu = gpu_cycle(cfg, t)
+    same, cnt = compare_cycle(cfg, t, gpu)
+    assert same >= cnt - 1
+    M = P * cfg.G
+    assert (gpu[0].sum(1) < M * (1 - 1e-3)).all()
+    h = make_pot(cfg)
+    try:
+        ipot.ipot_set_profiling(h, True)
+        K, V, Q, Kc = (to_dev(t[x], "bf16") for x in ("K", "V", "Q", "K_cap"))
+        ipot.ipot_append_chunk(h, K, V, cfg.pot_size)
+        ipot.ipot_score_only_cap(h, Q, Kc, P)
+        assert ipot.ipot_sync_status(h) == 0
+        u = ipot.device_array(ipot.ipot_last_scores(h)[0], (cfg.units, cfg.pot_size), "f32").cpu().numpy()
+        assert (u == gpu[0]).all()
+        ipot.ipot_reset(h)
+        ipot.ipot_append_chunk(h, K, V, cfg.pot_size)
+        ipot.ipot_score_and_compress_cap(h, Q, Kc, P, torch.from_numpy(t["aux"]).cuda())
+        assert ipot.ipot_sync_status(h) == 0
+        assert ipot.ipot_kernel_ms(h)[2] == TC
+    finally:
+        ipot.ipot_destroy(h)
