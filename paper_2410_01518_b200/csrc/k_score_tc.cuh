@@ -15,8 +15,8 @@
 //   epilogue (16 warps in four groups, a group per 128 columns of tensor memory; groups 0, 1 have the CTA's even
 //            tasks, 2, 3 the odd ones, so that one pair computes while the other waits for the exchange)
 //     pass 1   a thread owns one query row: e = 2^x is written back over the logits and summed, against the reference
-//              0 - no maximum is taken unless a warp's sums then leave the comfortable range; a quarter of the
-//              exponentials run on the FMA pipe.  The warps of a scheduler take pass 1 in turns, pair after pair: both
+//              0 - no maximum is taken as long as a row's first logits add up to 1 and none is 2^100 above the reference; other rows get one of
+//              their own (+3 %) -; a quarter of the exponentials run on the FMA pipe.  The warps of a scheduler take pass 1 in turns, pair after pair: both
 //              pairs at once finish later than one of them could, and every reader of their sums waits;
 //     exchange the two groups of a pair add their row sums through shared memory and publish them with one 4-byte store
 //              that carries the launch's sign as a "fresh" mark; a thread reads half of its row's sums of the whole item
@@ -323,7 +323,25 @@ __device__ __forceinline__ float max3(float a, float b, float c)
     return y;
 }
 
-// 16 columns against the reference 0: v <- 2^(v c), added into two packed running sums; pm: the largest logit among those that went
+// The reference of a row over a half slab: 0 if the largest of its first logits lies between 0 and 2^kTcNear, else that logit, in binary
+// orders and rounded down to a whole number (moving a sum to another reference is then exact, and no exponential is below its
+// probability).  Where no logit is within fp32's range it is 0 and pass1_slow looks at the others.
+constexpr float kTcNear = 32.f;
+__device__ __forceinline__ float row_reference(float mx, float c)
+{
+    const float r = floorf(mx * c);
+    return (r >= 0.f && r <= kTcNear) || !(fabsf(r) < INFINITY) ? 0.f : r;
+}
+__device__ __forceinline__ float piece_reference(const uint32_t (&v)[16], float c)
+{
+    float mx[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mx[j] = fmaxf(__uint_as_float(v[j]), __uint_as_float(v[j + 4]));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mx[j] = max3(mx[j], __uint_as_float(v[j + 8]), __uint_as_float(v[j + 12]));
+    return row_reference(fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]), c);
+}
+// 16 columns against the reference r: v <- 2^(v c - r), added into two packed running sums; pm: the largest logit among those that went
 // to the FMA pipe, whose exponent arithmetic wraps around where the special-function unit returns +inf.
 struct PieceSum {
     float2 s[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -334,12 +352,12 @@ struct PieceSum {
         return t.x + t.y;
     }
 };
-__device__ __forceinline__ void piece_exp(uint32_t (&v)[16], float c, PieceSum &p)
+__device__ __forceinline__ void piece_exp(uint32_t (&v)[16], float c, float r, PieceSum &p)
 {
-    const float2 c2 = make_float2(c, c);
+    const float2 c2 = make_float2(c, c), nr2 = make_float2(-r, -r);
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
-        const float2 x = make_float2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), t = __fmul2_rn(x, c2);
+        const float2 x = make_float2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), t = __ffma2_rn(x, c2, nr2);
         float2 e2;
         if (pair_on_fma<kTcFmaEighths>(i >> 1)) {
             p.pm = max3(p.pm, x.x, x.y);
@@ -352,17 +370,38 @@ __device__ __forceinline__ void piece_exp(uint32_t (&v)[16], float c, PieceSum &
         v[i + 1] = __float_as_uint(e2.y);
     }
 }
-// A row's sums against the reference 0 stay below 2^60: its weights then do not fall below fp32's range while what they multiply still
-// counts (a probability is lost only below 2^-66, and only beside a logit that is 2^126 above the reference).
-constexpr float kTcSumMax = 1.1529215e18f;    // 2^60
-constexpr float kTcSumMin = 9.0949470e-13f;   // 2^-40: nothing above 2^-86 of the sum is lost to flushing
-constexpr float kTcReach = 60.f;
-constexpr float kTcRefLow = -40.f, kTcRefHigh = 110.f;   // sums against such references are published as they are, times 2^reference
+// A row's exponentials are taken against its reference and kept where they are up to 2^100 above it; what is 2^126 below it is lost, and its
+// probability is smaller than that.  A weight then is as small as 2^-226 before nothing of its row counts: see kTcLift.
+constexpr float kTcSumMax = 1.2676506e30f;    // 2^100
+constexpr float kTcSumMin = 0.99f;            // of a row's first logits; with a reference its own term is 1 (less: they are all beyond fp32's range)
+constexpr float kTcReach = 100.f;
+constexpr float kTcRefLow = -90.f, kTcPlainMax = 3.3230700e35f;   // a sum is published as it is, times 2^reference, up to 2^118 (128 of them are still finite)
 constexpr float kTcTiny = 1.1754944e-38f;     // an entry that adds nothing is still not 0
+// Where a row's weight is below 2^-100 its warp's weights are multiplied by 2^110 and the column sums divided by it: 2^-226 times
+// exponentials of up to 2^100 is a probability that fp32 holds.
+constexpr float kTcLift = 110.f, kTcLifted = 1.2980742e33f, kTcUnlift = 7.7037198e-34f;
 
-// Pass 1 for a warp some of whose rows left the comfortable range: the first `done` pieces of 16 columns have been stored as 2^(x c);
+// (reference, sum) with the sum in [1, 2): sums that are far apart can then be brought to one reference without a factor that underflows
+// while what it multiplies still counts.  An empty sum has no reference.
+__device__ __forceinline__ float2 normalised(float2 a)
+{
+    const int b = __float_as_int(a.y);
+    if (!(a.y < INFINITY)) return a;
+    if (b < 0x00800000) return make_float2(-INFINITY, 0.f);
+    return make_float2(a.x + (float)((b >> 23) - 127), __int_as_float((b & 0x007FFFFF) | 0x3F800000));
+}
+__device__ __noinline__ float2 add_sums(float2 a, float2 b)
+{
+    a = normalised(a);
+    b = normalised(b);
+    const float m = fmaxf(a.x, b.x);
+    if (m == -INFINITY) return make_float2(0.f, kTcTiny);
+    return make_float2(m, fmaf(a.y, ex2(a.x - m), b.y * ex2(b.x - m)));
+}
+
+// Pass 1 for a warp some of whose rows left the range: the first `done` pieces of 16 columns have been stored against the reference r;
 // everything is brought to the reference that the rest needs.  (reference, sum)
-__device__ __noinline__ float2 pass1_slow(uint32_t taddr, int done, int nvalid, float c)
+__device__ __noinline__ float2 pass1_slow(uint32_t taddr, int done, int nvalid, float c, float r)
 {
     float mx = -INFINITY;
     tmem_wait_st();
@@ -375,10 +414,10 @@ __device__ __noinline__ float2 pass1_slow(uint32_t taddr, int done, int nvalid, 
         for (int e = 0; e < 16; ++e)
             if (16 * i + e < nvalid) mx = fmaxf(mx, __uint_as_float(v[e]));
     }
-    float m = ceilf(mx * c);   // a whole number: moving a sum to another reference is exact
-    if (done) m = fmaxf(m, 0.f);
+    float m = floorf(mx * c);
+    if (done) m = fmaxf(m, r);
     if (m == -INFINITY) m = 0.f;   // every logit beyond fp32's range
-    const float down = ex2(-m);
+    const float d = m - r, d1 = fminf(d, 113.f), down1 = ex2(-d1), down2 = ex2(d1 - d);   // (one factor would underflow beside 2^100)
     float s = 0.f;
 #pragma unroll 1
     for (int i = 0; 16 * i < nvalid; ++i) {
@@ -389,7 +428,7 @@ __device__ __noinline__ float2 pass1_slow(uint32_t taddr, int done, int nvalid, 
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
             const float x = __uint_as_float(v[e]);
-            const float y = i < done ? x * down : 16 * i + e < nvalid ? ex2(fmaf(x, c, -m)) : 0.f;
+            const float y = i < done ? x * down1 * down2 : 16 * i + e < nvalid ? ex2(fmaf(x, c, -m)) : 0.f;
             a[e & 3] += y;
             v[e] = __float_as_uint(y);
         }
@@ -398,27 +437,81 @@ __device__ __noinline__ float2 pass1_slow(uint32_t taddr, int done, int nvalid, 
     }
     return make_float2(m, s);
 }
+// Pass 1 for 128 keys: (reference, sum).  kSeek: with references, else against 0; false if that does not do for the first logits.
+// Pieces of 16 columns in two register sets.  A piece is looked at and stored behind the exponentials of the next one: with the look straight
+// after its own, every piece waited out its own chain of sums.
+template <bool kSeek>
+__device__ __forceinline__ bool pass1_full(uint32_t tb, float c, float2 &s)
+{
+    uint32_t A[16], B[16];
+    PieceSum pa, pb;
+    float r = 0.f;
+    auto fits = [&](const PieceSum &p) {   // (false for NaN; what the second set adds need not be large)
+        const float t = p.total();
+        return __all_sync(0xffffffffu, t <= kTcSumMax && (&p == &pb || t >= kTcSumMin) && fmaf(p.pm, c, -r) <= kTcReach) != 0;
+    };
+    int done = 0;
+    tmem_ld16(tb, A);
+    tmem_wait_ld16(A);
+    if (kSeek) r = piece_reference(A, c);
+    tmem_ld16(tb + 16, B);
+    piece_exp(A, c, r, pa);
+#pragma unroll 1
+    for (;;) {
+        tmem_wait_ld16(B);
+        piece_exp(B, c, r, pb);
+        if (!fits(pa)) {
+            if (!kSeek && !done) return false;
+            break;
+        }
+        tmem_st16(tb + 16 * done, A);
+        if (++done < 7) {
+            tmem_ld16(tb + 16 * done + 16, A);
+            tmem_wait_ld16(A);
+            piece_exp(A, c, r, pa);
+        }
+        if (!fits(pb)) break;
+        tmem_st16(tb + 16 * done, B);
+        if (++done == 8) break;
+        tmem_ld16(tb + 16 * done + 16, B);
+    }
+    if (done == 8) s = make_float2(r, pa.total() + pb.total());
+    else s = pass1_slow(tb, done, kTcHalf, c, r);
+    return true;
+}
+__device__ __noinline__ float2 pass1_seek(uint32_t tb, float c)
+{
+    float2 s;
+    pass1_full<true>(tb, c, s);
+    return s;
+}
 // Pass 1 where only the first nvalid (1 .. 127) of the 128 columns hold keys
 __device__ __noinline__ float2 pass1_ragged(uint32_t taddr, int nvalid, float c)
 {
-    float s = 0.f;
+    float s = 0.f, r = 0.f;
 #pragma unroll 1
     for (int i = 0; 16 * i < nvalid; ++i) {
         uint32_t v[16];
         tmem_ld16(taddr + 16 * i, v);
         tmem_wait_ld16(v);
+        if (i == 0) {
+            float mx = -INFINITY;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) mx = fmaxf(mx, e < nvalid ? __uint_as_float(v[e]) : -INFINITY);
+            r = row_reference(mx, c);
+        }
         float a[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
-            const float y = 16 * i + e < nvalid ? ex2(__uint_as_float(v[e]) * c) : 0.f;
+            const float y = 16 * i + e < nvalid ? ex2(fmaf(__uint_as_float(v[e]), c, -r)) : 0.f;
             a[e & 3] += y;
             v[e] = __float_as_uint(y);
         }
         s += (a[0] + a[1]) + (a[2] + a[3]);
-        if (!__all_sync(0xffffffffu, s >= kTcSumMin && s <= kTcSumMax)) return pass1_slow(taddr, i, nvalid, c);
+        if (!__all_sync(0xffffffffu, s >= kTcSumMin && s <= kTcSumMax)) return pass1_slow(taddr, i, nvalid, c, r);
         tmem_st16(taddr + 16 * i, v);
     }
-    return make_float2(0.f, s);
+    return make_float2(r, s);
 }
 // Sum of n (up to kMost) of a row's entries, re-read until each carries the launch's mark.  Only what is still stale is read again: the polls
 // of all CTAs together are a large part of what L2 delivers (all of it again, in 16-byte loads of a transposed array: 109 us against 90).
@@ -454,7 +547,7 @@ __device__ __forceinline__ float poll_entries(const float *st, int n, float sgn,
     return v[0];
 }
 // A row's denominator when some entry is given as (reference, sum): sixteen entries at a time with all loads in flight, relative to the
-// largest reference.  (Every block that has a slab of the item comes here for one far logit in one of them; entry by entry a step of
+// largest of them.  (Every block that has a slab of the item comes here for one far logit in one of them; entry by entry a step of
 // 8 streams of heavy-tailed keys, 64 units x 16384, took 1243 us.)
 __device__ __noinline__ float2 merge_entries(const float *st, const float2 *refs, int entries)
 {
@@ -468,12 +561,18 @@ __device__ __noinline__ float2 merge_entries(const float *st, const float2 *refs
         float mb = m;
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
-            x[e] = s[e] <= kTcTiny ? -INFINITY : 0.f;   // an empty entry's reference does not count
+            x[e] = 0.f;
             if (s[e] == INFINITY) {
                 const float *r = reinterpret_cast<const float *>(refs + (size_t)(e0 + e) * kTcRows);
                 x[e] = ld_gpu_f32(r);
                 s[e] = ld_gpu_f32(r + 1);
             }
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const float2 t = s[e] <= kTcTiny ? make_float2(-INFINITY, 0.f) : normalised(make_float2(x[e], s[e]));   // (an empty entry's reference does not count)
+            x[e] = t.x;
+            s[e] = t.y;
         }
 #pragma unroll
         for (int e = 0; e < 16; ++e) mb = fmaxf(mb, x[e]);
@@ -756,6 +855,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                    : out_rows > 32 ? cp[0] + cp[kTcHalf] : cp[0];
         };
         uint32_t j = 0;                         // tasks of this pair so far
+        bool seek = false;                      // this warp's rows have needed references
         for (int task = task0; task < prm.tasks; task += step, ++j) {
             const int rows = min(kTcRows, prm.M - mt * kTcRows), nvalid = min(kTcHalf, prm.N - slab * kTcSlab - half * kTcHalf);
             const bool works = q * 32 < rows && nvalid > 0;   // (uniform over the warp)
@@ -768,41 +868,16 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             float2 s = make_float2(0.f, nvalid > 0 ? 1.f : 0.f);
             mbar_wait(bar(kBarSFull + g), par, ab, prm.status);
             if (pair | j) turn_wait(pair, q);
-            // ---- pass 1: exponentials against the reference 0, written back over the logits, and their sum
+            // ---- pass 1: exponentials against the row's reference, written back over the logits, and their sum
             if (works) {
                 tc_fence_after();
                 if (nvalid == kTcHalf) {
-                    // Pieces of 16 columns in two register sets.  A piece is looked at and stored behind the exponentials of the next one: with
-                    // the look straight after its own, every piece waited out its own chain of sums.
-                    uint32_t A[16], B[16];
-                    PieceSum pa, pb;
-                    auto fits = [&](const PieceSum &p) {   // (false for NaN; what the second set adds need not be large)
-                        const float t = p.total();
-                        return __all_sync(0xffffffffu, t <= kTcSumMax && (&p == &pb || t >= kTcSumMin) && p.pm * c <= kTcReach) != 0;
-                    };
-                    int done = 0;
-                    tmem_ld16(tb, A);
-                    tmem_wait_ld16(A);
-                    tmem_ld16(tb + 16, B);
-                    piece_exp(A, c, pa);
-#pragma unroll 1
-                    for (;;) {
-                        tmem_wait_ld16(B);
-                        piece_exp(B, c, pb);
-                        if (!fits(pa)) break;
-                        tmem_st16(tb + 16 * done, A);
-                        if (++done < 7) {
-                            tmem_ld16(tb + 16 * done + 16, A);
-                            tmem_wait_ld16(A);
-                            piece_exp(A, c, pa);
-                        }
-                        if (!fits(pb)) break;
-                        tmem_st16(tb + 16 * done, B);
-                        if (++done == 8) break;
-                        tmem_ld16(tb + 16 * done + 16, B);
+                    // Rows whose first logits are all below 0 need references: looking for them costs 3 %, and most warps never do.  The first time
+                    // a warp does it starts again, from then on it looks first.
+                    if (seek || !pass1_full<false>(tb, c, s)) {
+                        s = pass1_seek(tb, c);
+                        seek = true;
                     }
-                    if (done == 8) s.y = pa.total() + pb.total();
-                    else s = pass1_slow(tb, done, kTcHalf, c);
                 } else {
                     s = pass1_ragged(tb, nvalid, c);
                 }
@@ -815,12 +890,14 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             if (!half && (int)blockIdx.x != prm.withhold_cta) {
                 const float2 o = spart[par * kTcRows + row];
                 float *to = prm.stats + ((size_t)item * S + slab) * kTcRows + row;
-                const float m = s.x == o.x ? s.x : fmaxf(s.y == 0.f ? -INFINITY : s.x, o.y == 0.f ? -INFINITY : o.x);   // (one of them is not empty)
-                float sum = s.y + o.y;
-                if (s.x != o.x) sum = (s.y == 0.f ? 0.f : s.y * ex2(s.x - m)) + (o.y == 0.f ? 0.f : o.y * ex2(o.x - m));
-                if (m >= kTcRefLow && m <= kTcRefHigh && sum == sum) {   // (a NaN takes the other way, or it would never count as fresh)
-                    if (m != 0.f) sum *= ex2(m);
-                    st_gpu_f32(to, sum == 0.f ? kTcTiny * sgn : sum * sgn);
+                float m = 0.f, sum = s.y + o.y, plain = sum;
+                if (s.x != 0.f || o.x != 0.f) {
+                    m = fmaxf(s.y == 0.f ? -INFINITY : s.x, o.y == 0.f ? -INFINITY : o.x);   // (one of them is not empty)
+                    sum = (s.y == 0.f ? 0.f : s.y * ex2(s.x - m)) + (o.y == 0.f ? 0.f : o.y * ex2(o.x - m));
+                    plain = m >= kTcRefLow && m <= 118.f ? sum * ex2(m) : INFINITY;
+                }
+                if (plain <= kTcPlainMax) {   // (a NaN takes the other way, or it would never count as fresh)
+                    st_gpu_f32(to, plain == 0.f ? kTcTiny * sgn : plain * sgn);
                 } else {
                     float *r = reinterpret_cast<float *>(prm.refs + ((size_t)item * S + slab) * kTcRows + row);
                     st_gpu_f32(r, m);
@@ -847,23 +924,22 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             pair_sync(pair);
             // ---- the row's weight
             float weight = 0.f;
+            bool far = false;
             if (row < rows) {
-                float m = 0.f;
-                l = lpart[(par * 2) * kTcRows + row] + lpart[(par * 2 + 1) * kTcRows + row];
-                if (l == INFINITY) {
-                    const float2 t = merge_entries(st, prm.refs + (size_t)item * S * kTcRows + row, S);
-                    m = t.x;
-                    l = t.y;
+                float2 t = make_float2(0.f, lpart[(par * 2) * kTcRows + row] + lpart[(par * 2 + 1) * kTcRows + row]);
+                const bool near = s.x == 0.f && t.y < INFINITY && own.x == -INFINITY;
+                if (!near) {
+                    if (t.y == INFINITY) t = merge_entries(st, prm.refs + (size_t)item * S * kTcRows + row, S);
+                    if (own.x > -INFINITY) t = add_sums(t, own);
+                    t = normalised(t);
+                    t.x = fminf(s.x - t.x, 8.f);   // (above 2 only where there is nothing to weigh)
+                    far = t.x < -kTcReach;
                 }
-                if (own.x > -INFINITY) {
-                    const float mb = fmaxf(m, own.x);
-                    l = fmaf(own.y, ex2(own.x - mb), l * ex2(m - mb));
-                    m = mb;
-                }
-                float inv_l;
-                asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv_l) : "f"(l));
-                weight = s.x == m ? inv_l : ex2(s.x - m) * inv_l;
+                asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(weight) : "f"(t.y));
+                if (!near) weight *= ex2(far ? t.x + kTcLift : t.x);
             }
+            const bool lift = __any_sync(0xffffffffu, far);
+            if (lift && !far) weight *= kTcLifted;
             // ---- pass 2: weighted column sums
             if (works) {
                 tc_fence_after();
@@ -892,7 +968,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                     }
                     float x[8];
                     pass2_rows(va[i & 1], vb[i & 1], fr2, x);
-                    cp[32 * i] = pass2_reduce(x, lane);
+                    cp[32 * i] = pass2_reduce(x, lane) * (lift ? kTcUnlift : 1.f);
                 }
             } else if (lane == 0) {
                 mbar_arrive(bar(kBarTEmpty + g));

@@ -135,3 +135,55 @@ def test_one_sweep_cap_keys_join_the_softmax_of_every_row_size(d, P):
         assert ipot.ipot_kernel_ms(h)[2] == TC
     finally:
         ipot.ipot_destroy(h)
+
+
+def _axis_cycle(cfg, rows, base, far, where, far_cap):
+    """Logits along one axis: keys of `base` binary orders (drawn), one of `far` at slot where[layer] (None: among the CaP keys);
+    rows: the factors of the query rows."""
+    t = inputs.make_cycle(cfg)
+    r = np.random.default_rng(7)
+    to_key = np.log(2.0) * np.sqrt(cfg.d) / 8.0
+    K = 0.01 * inputs.widen(t["K"], "bf16").astype(np.float32)
+    K[..., 3] = r.uniform(*base, size=K.shape[:-1]) * to_key
+    Kc = 0.01 * inputs.widen(inputs.make_kcap(cfg), "bf16").astype(np.float32)
+    Kc[..., 3] = r.uniform(*base, size=Kc.shape[:-1]) * to_key
+    for layer, slot in enumerate(where):
+        if slot is None:
+            Kc[layer, :, :, -1, 3] = far * to_key
+        else:
+            K[layer, :, :, slot, 3] = far * to_key
+    Q = np.zeros_like(inputs.widen(t["Q"], "bf16"), dtype=np.float32)
+    Q[..., 3] = 8.0 * np.asarray(rows)
+    t["K"], t["Q"] = inputs.store(K, "bf16"), inputs.store(Q, "bf16")
+    if far_cap:
+        t["K_cap"] = inputs.store(Kc, "bf16")
+    return t
+
+
+@pytest.mark.parametrize("d", [64, 128, 96, 256])
+@pytest.mark.parametrize("far", [30, 61, 99, 103, 117, 119, 126, 131, 150, 180, 226])
+@pytest.mark.parametrize("rows", ["one", "equal", "mixed"])
+def test_one_sweep_keeps_probabilities_beside_a_far_key(rows, far, d):
+    """Keys of 20 to 45 binary orders and one far above them, in the first, a middle and the last piece of a half slab, in other slabs
+    and halves, in the ragged end and among the CaP keys: every probability that fp32 holds has to come out, and the survivors
+    beside the far key are chosen by it."""
+    factors = {"one": [1.0], "equal": [1.0] * 16, "mixed": [1.0] + [0.1, -0.1, 0.02] * 5}[rows]
+    where = [0, 5, 60, 127, 130, 255, 300, 690, None]
+    cfg = inputs.small_config(cfg_id=1200 + d, pot_size=700, keep=128, nuc_slots=0, cap_rows=len(factors), Hq=1, Hkv=1, d=d, dtype="bf16",
+                              layers=len(where))
+    scorer = TC if d in (64, 128) else ipot.IPOT_SCORER_AUTO
+    for cap in (False, True):
+        t = _axis_cycle(cfg, factors, (20, 45), far, where, cap)
+        compare_cycle(cfg, t, gpu_cycle(cfg, t, scorer))
+
+
+@pytest.mark.parametrize("d", [64, 128, 96, 256])
+@pytest.mark.parametrize("top", [-5, -20, -39, -60, -89, -95, -130, -300])
+def test_one_sweep_keeps_probabilities_below_a_low_maximum(top, d):
+    """Every logit of the rows far below 0: what is less than 2^126 below the largest counts."""
+    where = [0, 5, 127, 130, 300, 690, None]
+    cfg = inputs.small_config(cfg_id=1300 + d, pot_size=700, keep=400, nuc_slots=0, cap_rows=3, Hq=1, Hkv=1, d=d, dtype="bf16", layers=len(where))
+    scorer = TC if d in (64, 128) else ipot.IPOT_SCORER_AUTO
+    for cap in (False, True):
+        t = _axis_cycle(cfg, [1.0, 0.9, 1.0], (top - 125, top - 5), top, where, cap)
+        compare_cycle(cfg, t, gpu_cycle(cfg, t, scorer))
