@@ -81,7 +81,8 @@ constexpr int kTcMaxK = 4;
 constexpr uint32_t kTcOffStage = 0;                                        // [2] { Q, K }
 constexpr uint32_t kTcOffColpart = 2 * kTcStageBytes;                      // [4 groups][2 parities][4 row quarters][128] float
 constexpr uint32_t kTcOffLpart = kTcOffColpart + 4 * 2 * 4 * kTcHalf * 4;      // [2 pairs][2 parities][2 halves][128] float
-constexpr uint32_t kTcOffSpart = kTcOffLpart + 2 * 2 * 2 * kTcRows * 4;        // [2 pairs][2 parities][128] float2
+constexpr uint32_t kTcOffLfar = kTcOffLpart + 2 * 2 * 2 * kTcRows * 4;         // [2 pairs][2 parities][2 halves][128] float2: (reference, sum) of those that are infinite
+constexpr uint32_t kTcOffSpart = kTcOffLfar + 2 * 2 * 2 * kTcRows * 8;        // [2 pairs][2 parities][128] float2
 constexpr uint32_t kTcOffBar = kTcOffSpart + 2 * 2 * kTcRows * 8;
 constexpr uint32_t kTcOffTmemSlot = kTcOffBar + 208;                       // the allocated TMEM base address
 constexpr uint32_t kTcOffAbort = kTcOffBar + 212;                          // set once a wait of the CTA has run out; + 4: the block's deadline (8 bytes)
@@ -546,43 +547,43 @@ __device__ __forceinline__ float poll_entries(const float *st, int n, float sgn,
     }
     return v[0];
 }
-// A row's denominator when some entry is given as (reference, sum): sixteen entries at a time with all loads in flight, relative to the
-// largest of them.  (Every block that has a slab of the item comes here for one far logit in one of them; entry by entry a step of
-// 8 streams of heavy-tailed keys, 64 units x 16384, took 1243 us.)
-__device__ __noinline__ float2 merge_entries(const float *st, const float2 *refs, int entries)
+// Sum of n of a row's entries of which some are given as (reference, sum), by the thread that has seen their marks: all loads
+// in flight, relative to the largest.  (Every block that has a slab of the item comes here for one far logit in one of them.)
+__device__ __noinline__ void fold_entries(const TcParams &prm, int item, int row, int half, float2 *to)
 {
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");   // what was written before the marks that this thread has read
+    const int mid = (prm.slabs + 1) >> 1, n = half ? prm.slabs - mid : mid;
+    const size_t first = ((size_t)item * prm.slabs + (half ? mid : 0)) * kTcRows + row;
+    const float *st = prm.stats + first;
+    const float2 *refs = prm.refs + first;
     float m = -INFINITY, l = 0.f;
 #pragma unroll 1
-    for (int e0 = 0; e0 < entries; e0 += 16) {
-        float x[16], s[16];
+    for (int e0 = 0; e0 < n; e0 += 8) {
+        float s[8], x[8], y[8];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) s[e] = e0 + e < entries ? fabsf(ld_gpu_f32(st + (size_t)(e0 + e) * kTcRows)) : 0.f;
+        for (int e = 0; e < 8; ++e) {
+            const size_t at = (size_t)(e0 + e < n ? e0 + e : n - 1) * kTcRows;
+            s[e] = fabsf(ld_gpu_f32(st + at));
+            const float *r = reinterpret_cast<const float *>(refs + at);
+            x[e] = ld_gpu_f32(r);
+            y[e] = ld_gpu_f32(r + 1);
+        }
         float mb = m;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            x[e] = 0.f;
-            if (s[e] == INFINITY) {
-                const float *r = reinterpret_cast<const float *>(refs + (size_t)(e0 + e) * kTcRows);
-                x[e] = ld_gpu_f32(r);
-                s[e] = ld_gpu_f32(r + 1);
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const float2 t = s[e] <= kTcTiny ? make_float2(-INFINITY, 0.f) : normalised(make_float2(x[e], s[e]));   // (an empty entry's reference does not count)
+        for (int e = 0; e < 8; ++e) {
+            float2 t = s[e] == INFINITY ? make_float2(x[e], y[e]) : make_float2(0.f, s[e]);
+            t = e0 + e >= n || t.y <= kTcTiny ? make_float2(-INFINITY, 0.f) : normalised(t);   // (an empty entry has no reference)
             x[e] = t.x;
             s[e] = t.y;
+            mb = fmaxf(mb, t.x);
         }
-#pragma unroll
-        for (int e = 0; e < 16; ++e) mb = fmaxf(mb, x[e]);
         if (mb == -INFINITY) continue;
         l *= m == -INFINITY ? 0.f : ex2(m - mb);
 #pragma unroll
-        for (int e = 0; e < 16; ++e) l = fmaf(s[e], ex2(x[e] - mb), l);
+        for (int e = 0; e < 8; ++e) l = fmaf(s[e], ex2(x[e] - mb), l);
         m = mb;
     }
-    return m == -INFINITY ? make_float2(0.f, kTcTiny) : make_float2(m, l);
+    *to = m == -INFINITY ? make_float2(0.f, kTcTiny) : make_float2(m, l);
 }
 
 // Pass 2 for one warp over 32 rows x 32 columns: a[] and b[] are the 16x256b loads of the warp's TMEM lanes
@@ -837,6 +838,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
         const int row = q * 32 + lane;
         const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + g * kTcHalf;
         float *lpart = reinterpret_cast<float *>(gbase + kTcOffLpart) + pair * (4 * kTcRows);
+        float2 *lfar = reinterpret_cast<float2 *>(gbase + kTcOffLfar) + pair * (4 * kTcRows);
         float2 *spart = reinterpret_cast<float2 *>(gbase + kTcOffSpart) + pair * (2 * kTcRows);
         float *colpart = reinterpret_cast<float *>(gbase + kTcOffColpart) + g * (8 * kTcHalf);
         const float c = prm.scale_log2e, sgn = prm.sign;
@@ -917,6 +919,7 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
                 if (i < end) l += poll_entries<8>(st + (size_t)i * kTcRows, end - i, sgn, ab, prm.status);
             }
             lpart[(par * 2 + half) * kTcRows + row] = l;
+            if (l == INFINITY) fold_entries(prm, item, row, half, lfar + (par * 2 + half) * kTcRows + row);
             if (works) {
                 tmem_wait_st();
                 tc_fence_before();
@@ -926,10 +929,13 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             float weight = 0.f;
             bool far = false;
             if (row < rows) {
-                float2 t = make_float2(0.f, lpart[(par * 2) * kTcRows + row] + lpart[(par * 2 + 1) * kTcRows + row]);
+                const float l0 = lpart[(par * 2) * kTcRows + row], l1 = lpart[(par * 2 + 1) * kTcRows + row];
+                float2 t = make_float2(0.f, l0 + l1);
                 const bool near = s.x == 0.f && t.y < INFINITY && own.x == -INFINITY;
                 if (!near) {
-                    if (t.y == INFINITY) t = merge_entries(st, prm.refs + (size_t)item * S * kTcRows + row, S);
+                    if (t.y == INFINITY)
+                        t = add_sums(l0 == INFINITY ? lfar[(par * 2) * kTcRows + row] : make_float2(0.f, l0),
+                                     l1 == INFINITY ? lfar[(par * 2 + 1) * kTcRows + row] : make_float2(0.f, l1));
                     if (own.x > -INFINITY) t = add_sums(t, own);
                     t = normalised(t);
                     t.x = fminf(s.x - t.x, 8.f);   // (above 2 only where there is nothing to weigh)

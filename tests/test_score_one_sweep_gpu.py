@@ -187,3 +187,21 @@ def test_one_sweep_keeps_probabilities_below_a_low_maximum(top, d):
     for cap in (False, True):
         t = _axis_cycle(cfg, [1.0, 0.9, 1.0], (top - 125, top - 5), top, where, cap)
         compare_cycle(cfg, t, gpu_cycle(cfg, t, scorer))
+
+
+@pytest.mark.parametrize("n", [4100, 9000])
+@pytest.mark.parametrize("d", [64, 128, 256])
+def test_one_sweep_sums_of_many_slabs_far_apart(d, n):
+    """Sums that are published as they are and as (reference, sum) in every mixture: each half of the item's slabs, more than one look's
+    worth of them, and neighbours on both sides of 2^118 whose shares of the denominator differ by little."""
+    far = [{}, {70: 126}, {70: 117.9, 300: 118.1, 2000: 119}, {n - 1: 127, 600: 118}, {9: 117, 2500: 128, n - 300: 128}, {5: 200, n - 2: 199},
+           {k: 100 + k % 60 for k in range(3, n, 251)}, {k: -100 for k in range(n)}, {k: -89 - k // 400 for k in range(n)}]
+    cfg = inputs.small_config(cfg_id=1400 + d, pot_size=n, keep=200, nuc_slots=0, cap_rows=40, Hq=1, Hkv=1, d=d, dtype="bf16", layers=len(far))
+    factors = [1.0, 0.97] + [0.1, -0.1] * 19
+    t = _axis_cycle(cfg, factors, (20, 45), 0, [], False)
+    K = inputs.widen(t["K"], "bf16").astype(np.float32)
+    for layer, at in enumerate(far):
+        for slot, logit in at.items():
+            K[layer, :, :, slot, 3] = logit * np.log(2.0) * np.sqrt(d) / 8.0
+    t["K"] = inputs.store(K, "bf16")
+    compare_cycle(cfg, t, gpu_cycle(cfg, t, TC if d < 256 else ipot.IPOT_SCORER_AUTO))
