@@ -333,15 +333,6 @@ __device__ __forceinline__ float row_reference(float mx, float c)
     const float r = floorf(mx * c);
     return (r >= 0.f && r <= kTcNear) || !(fabsf(r) < INFINITY) ? 0.f : r;
 }
-__device__ __forceinline__ float piece_reference(const uint32_t (&v)[16], float c)
-{
-    float mx[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) mx[j] = fmaxf(__uint_as_float(v[j]), __uint_as_float(v[j + 4]));
-#pragma unroll
-    for (int j = 0; j < 4; ++j) mx[j] = max3(mx[j], __uint_as_float(v[j + 8]), __uint_as_float(v[j + 12]));
-    return row_reference(fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]), c);
-}
 // 16 columns against the reference r: v <- 2^(v c - r), added into two packed running sums; pm: the largest logit among those that went
 // to the FMA pipe, whose exponent arithmetic wraps around where the special-function unit returns +inf.
 struct PieceSum {
@@ -353,6 +344,7 @@ struct PieceSum {
         return t.x + t.y;
     }
 };
+template <int kFma = kTcFmaEighths>
 __device__ __forceinline__ void piece_exp(uint32_t (&v)[16], float c, float r, PieceSum &p)
 {
     const float2 c2 = make_float2(c, c), nr2 = make_float2(-r, -r);
@@ -360,7 +352,7 @@ __device__ __forceinline__ void piece_exp(uint32_t (&v)[16], float c, float r, P
     for (int i = 0; i < 16; i += 2) {
         const float2 x = make_float2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), t = __ffma2_rn(x, c2, nr2);
         float2 e2;
-        if (pair_on_fma<kTcFmaEighths>(i >> 1)) {
+        if (pair_on_fma<kFma>(i >> 1)) {
             p.pm = max3(p.pm, x.x, x.y);
             e2 = exp2_fma_pair5(t);
         } else {
@@ -400,43 +392,67 @@ __device__ __noinline__ float2 add_sums(float2 a, float2 b)
     return make_float2(m, fmaf(a.y, ex2(a.x - m), b.y * ex2(b.x - m)));
 }
 
+__device__ __forceinline__ float piece_max(const uint32_t (&v)[16])
+{
+    float mx[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mx[j] = fmaxf(__uint_as_float(v[j]), __uint_as_float(v[j + 4]));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mx[j] = max3(mx[j], __uint_as_float(v[j + 8]), __uint_as_float(v[j + 12]));
+    return fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]);
+}
 // Pass 1 for a warp some of whose rows left the range: the first `done` pieces of 16 columns have been stored against the reference r;
 // everything is brought to the reference that the rest needs.  (reference, sum)
+// (The other CTAs of the item wait for this: summed column by column it took twice as long, 256 units x 4096 keys with one far key each 120 us
+// against 99.  A second register set would make it shorter still, but the kernel's own values then no longer survive the call in registers, 85 us
+// against 79 without any far key.)
 __device__ __noinline__ float2 pass1_slow(uint32_t taddr, int done, int nvalid, float c, float r)
 {
+    const int n = (nvalid + 15) >> 4;
+    uint32_t A[16];
+    auto keys_only = [&](uint32_t (&v)[16], int i) {
+        if (16 * i + 16 <= nvalid) return;
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+            if (16 * i + e >= nvalid) v[e] = __float_as_uint(-INFINITY);
+    };
     float mx = -INFINITY;
     tmem_wait_st();
 #pragma unroll 1
-    for (int i = done; 16 * i < nvalid; ++i) {
-        uint32_t v[16];
-        tmem_ld16(taddr + 16 * i, v);
-        tmem_wait_ld16(v);
-#pragma unroll
-        for (int e = 0; e < 16; ++e)
-            if (16 * i + e < nvalid) mx = fmaxf(mx, __uint_as_float(v[e]));
+    for (int i = done; i < n; ++i) {
+        tmem_ld16(taddr + 16 * i, A);
+        tmem_wait_ld16(A);
+        keys_only(A, i);
+        mx = fmaxf(mx, piece_max(A));
     }
     float m = floorf(mx * c);
     if (done) m = fmaxf(m, r);
     if (m == -INFINITY) m = 0.f;   // every logit beyond fp32's range
     const float d = m - r, d1 = fminf(d, 113.f), down1 = ex2(-d1), down2 = ex2(d1 - d);   // (one factor would underflow beside 2^100)
-    float s = 0.f;
+    PieceSum p;
 #pragma unroll 1
-    for (int i = 0; 16 * i < nvalid; ++i) {
-        uint32_t v[16];
-        tmem_ld16(taddr + 16 * i, v);
-        tmem_wait_ld16(v);
-        float a[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const float x = __uint_as_float(v[e]);
-            const float y = i < done ? x * down1 * down2 : 16 * i + e < nvalid ? ex2(fmaf(x, c, -m)) : 0.f;
-            a[e & 3] += y;
-            v[e] = __float_as_uint(y);
-        }
-        s += (a[0] + a[1]) + (a[2] + a[3]);
-        tmem_st16(taddr + 16 * i, v);
+    for (int i = done; i < n; ++i) {
+        tmem_ld16(taddr + 16 * i, A);
+        tmem_wait_ld16(A);
+        keys_only(A, i);
+        piece_exp<0>(A, c, m, p);   // (the FMA pipe has no 0 for a logit beyond fp32's range)
+        tmem_st16(taddr + 16 * i, A);
     }
-    return make_float2(m, s);
+#pragma unroll 1
+    for (int i = 0; i < done; ++i) {
+        tmem_ld16(taddr + 16 * i, A);
+        tmem_wait_ld16(A);
+#pragma unroll
+        for (int e = 0; e < 16; e += 2) {
+            float2 y = __fmul2_rn(make_float2(__uint_as_float(A[e]), __uint_as_float(A[e + 1])), make_float2(down1, down1));
+            y = __fmul2_rn(y, make_float2(down2, down2));
+            p.s[(e >> 1) & 1] = __fadd2_rn(p.s[(e >> 1) & 1], y);
+            A[e] = __float_as_uint(y.x);
+            A[e + 1] = __float_as_uint(y.y);
+        }
+        tmem_st16(taddr + 16 * i, A);
+    }
+    return make_float2(m, p.total());
 }
 // Pass 1 for 128 keys: (reference, sum).  kSeek: with references, else against 0; false if that does not do for the first logits.
 // Pieces of 16 columns in two register sets.  A piece is looked at and stored behind the exponentials of the next one: with the look straight
@@ -454,7 +470,7 @@ __device__ __forceinline__ bool pass1_full(uint32_t tb, float c, float2 &s)
     int done = 0;
     tmem_ld16(tb, A);
     tmem_wait_ld16(A);
-    if (kSeek) r = piece_reference(A, c);
+    if (kSeek) r = row_reference(piece_max(A), c);
     tmem_ld16(tb + 16, B);
     piece_exp(A, c, r, pa);
 #pragma unroll 1
