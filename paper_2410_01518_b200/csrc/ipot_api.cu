@@ -282,6 +282,8 @@ int launch_warp_mma(ipot *p, const void *Q, const float2 *cap_stats, int M, int 
 // kernel, whose work is dealt item by item, to be faster - if there are several row blocks and items enough to deal.  Rows of 64
 // channels cost the one-sweep kernel as much as wider ones: there it is from 64 slabs on.  Up to 40 slabs the lines are those that the one-sweep
 // kernel had with its former, slower exchange, and test_automatic_choice holds them: between them and 40 slabs it would be 8 to 15 % faster.
+// A chunk that starts between two slabs is read in place by the item kernel (tiles of 128 keys) and copied first for the other: there the lines
+// are the former ones for every length (64 units x 12800, M = 256: 182 us against 228; 16 x 16896, M = 128 82 / 95; d = 64: 64 x 10752, M = 128 96 / 108).
 // Measured as steps of a stream with deferred appends (us, one sweep / items), d = 128:
 //   64 units x 8192 keys, M = 768, 1024: 249 / 289, 320 / 379;  64 x 12288, M = 512: 272 / 308;  64 x 16384, M = 256, 512, 1024: 217 / 248, 376 / 404, 694 / 712
 //   32 x 16384, M = 512: 203 / 208;  16 x 16384, M = 128, 512: 55 / 66, 120 / 126
@@ -297,9 +299,9 @@ int auto_scorer(int units, int N, int M, int d, bool tile_chunk, bool tc_ok, boo
 {
     const long long keys = (long long)units * N;
     bool many, long_items;
-    if (N <= 40 * kTcSlab) {
+    if (N <= 40 * kTcSlab || (tile_chunk && (d == 64 || d == 128))) {
         many = d == 64 && N >= 6144 && keys >= 64 * 6144;
-        long_items = (N > 8192 || (N == 8192 && M > 512)) && keys >= 32 * 8192 && (M > kTcRows || keys >= 32 * 10240);
+        long_items = (N > 8192 || (N == 8192 && M > 512)) && keys >= 32 * 8192 && (M > kTcRows || N >= 16384 || keys >= 32 * 10240);
     } else {
         many = d == 64 && N >= 64 * kTcSlab && keys >= 64 * 16384;
         long_items = M > kTcRows && keys >= 32 * 8192 && (N > 96 * kTcSlab || (N > 64 * kTcSlab && units >= 32));

@@ -205,3 +205,35 @@ def test_one_sweep_sums_of_many_slabs_far_apart(d, n):
             K[layer, :, :, slot, 3] = logit * np.log(2.0) * np.sqrt(d) / 8.0
     t["K"] = inputs.store(K, "bf16")
     compare_cycle(cfg, t, gpu_cycle(cfg, t, TC if d < 256 else ipot.IPOT_SCORER_AUTO))
+
+
+ITEMS = ipot.IPOT_SCORER_TENSOR_ITEMS
+
+
+@pytest.mark.parametrize("units,n,P,G,d,first,want", [
+    # 15 and 16 slabs of another head dimension; chunks that start on a slab, between two, and off every tile
+    (3, 1280, 8, 1, 96, None, ITEMS), (4, 1024, 8, 1, 96, None, TC), (8, 1024, 8, 1, 96, 256, TC), (8, 1024, 8, 1, 96, 384, ITEMS), (8, 1024, 8, 1, 96, 300, TC),
+    (33, 10752, 8, 4, 128, 256, TC), (33, 10752, 8, 4, 128, 384, ITEMS), (33, 10752, 8, 4, 128, 300, TC), (16, 16384, 8, 4, 128, 384, ITEMS),
+    (8, 10752, 8, 4, 128, 384, TC), (40, 10752, 8, 1, 64, 384, ITEMS), (40, 10752, 8, 1, 64, 512, TC)])
+def test_automatic_choice_beyond_40_slabs_and_of_other_rows(units, n, P, G, d, first, want):
+    """Both sides of each line; the scores agree with those of a kernel that was not chosen."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    K = torch.randn((units, 1, 1, n, d), generator=g, device="cuda").bfloat16()
+    Q = torch.randn((units, 1, G, P, d), generator=g, device="cuda").bfloat16()
+    u = []
+    for scorer in (ipot.IPOT_SCORER_AUTO, ipot.IPOT_SCORER_WARP_MMA):
+        h = ipot.ipot_create_ex(n, n // 4, units, G, 1, d, nuc_slots=0, max_cap_rows=P)
+        try:
+            ipot.ipot_set_scorer(h, scorer)
+            ipot.ipot_set_profiling(h, True)
+            parts = [K] if first is None else [K[:, :, :, :first].contiguous(), K[:, :, :, first:].contiguous()]
+            for i, part in enumerate(parts):
+                ipot.ipot_set_deferred_append(h, i == 1)
+                ipot.ipot_append_chunk(h, part, part, part.shape[3])
+            ipot.ipot_score_and_compress(h, Q, P, None)
+            assert ipot.ipot_sync_status(h) == 0
+            assert ipot.ipot_kernel_ms(h)[2] == (want if scorer == ipot.IPOT_SCORER_AUTO else scorer)
+            u.append(ipot.device_array(ipot.ipot_last_scores(h)[0], (units, n), "f32").clone())
+        finally:
+            ipot.ipot_destroy(h)
+    assert ((u[0] - u[1]).norm() / u[1].norm()).item() < 2e-6   # (two kernels within 1e-6 of the exact scores each)
