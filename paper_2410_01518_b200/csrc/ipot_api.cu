@@ -277,24 +277,35 @@ int launch_warp_mma(ipot *p, const void *Q, const float2 *cap_stats, int M, int 
     return IPOT_OK;
 }
 
-// The fastest scorer the shape allows.  d = 64 and 128: the one-sweep kernel computes every exponential once; only where an item is
-// spread over most of the blocks (beyond 64 slabs of 256 keys) do they wait for each other's statistics long enough for the two-sweep
-// kernel, whose work is dealt item by item, to be faster - if there are several row blocks and items enough to deal.  Rows of 64
-// channels cost the one-sweep kernel as much as wider ones: there it is from 64 slabs on.  Up to 40 slabs the lines are those that the one-sweep
-// kernel had with its former, slower exchange, and test_automatic_choice holds them: between them and 40 slabs it would be 8 to 15 % faster.
-// A chunk that starts between two slabs is read in place by the item kernel (tiles of 128 keys) and copied first for the other: there the lines
-// are the former ones for every length (64 units x 12800, M = 256: 182 us against 228; 16 x 16896, M = 128 82 / 95; d = 64: 64 x 10752, M = 128 96 / 108).
-// Measured as steps of a stream with deferred appends (us, one sweep / items), d = 128:
-//   64 units x 8192 keys, M = 768, 1024: 249 / 289, 320 / 379;  64 x 12288, M = 512: 272 / 308;  64 x 16384, M = 256, 512, 1024: 217 / 248, 376 / 404, 694 / 712
-//   32 x 16384, M = 512: 203 / 208;  16 x 16384, M = 128, 512: 55 / 66, 120 / 126
-//   64 x 20480, M = 512: 534 / 475;  32 x 20480, M = 256: 174 / 168;  32 x 24576, M = 256: 195 / 193;  16 x 24576, M = 64, 512: 84 / 88, 190 / 222
-//   32 x 32768, M = 256: 282 / 263;  16 x 32768, M = 64: 109 / 112;  8 x 32768, M = 512: 170 / 158
-// and d = 64, M = 64, 128, 256, 512:  64 x 6144: 50 / 54, -, 78 / 87, -;  128 x 8192: 99 / 110, 101 / 118, 165 / 178, -;
-// 64 x 12288: -, 88 / 90, 141 / 148, 245 / 244;  64 x 16384: 113 / 110, -, 190 / 186, 340 / 309;  16 x 16384: 50 / 56, -, 72 / 77, -.
-// Other head dimensions (whole passes, deferred, us, one sweep / items): d = 256: 64 x 4096, M = 64, 128, 256: 62 / 84, 66 / 87, 90 / 140; 32 x 8192,
-// M = 512: 136 / 225; 64 x 12288, M = 256: 248 / 375; 8 x 4096, M = 64: 20 / 25; 8 x 1024, M = 32: 16.5 / 19.7.  d = 192: 64 x 4096, M = 64, 256:
-// 54 / 72, 73 / 106.  d = 96: 64 x 4096, M = 64, 128: 41 / 51, 42 / 53; 64 x 8192, M = 256: 110 / 117; 8 x 2048, M = 64: 16.5 / 20.1.  d = 72: 32 x 700,
-// M = 32: 16.9 / 21.2.  A handful of slabs is left to the item kernel (fewer than 16 have not been measured).
+// The fastest scorer the shape allows.  The one-sweep kernel computes every exponential once; only where an item is spread over most of the
+// blocks (beyond 64 slabs of 256 keys) do they wait for each other's statistics long enough for the two-sweep kernel, whose work is dealt item
+// by item, to be faster - if there are items enough to deal.  How long they wait depends on the keys: one logit beyond 2^118 takes every block
+// of the item through the general fold.  So each line is drawn where neither ordinary nor heavy-tailed keys (Student t, 3 degrees) lose
+// much by it.  Rows of 64 channels cost the one-sweep kernel as much as wider ones: there the other is from fewer keys on.  Up to 40 slabs the
+// lines are those that the one-sweep kernel had with its former, slower exchange, and test_automatic_choice holds them: between them and 40 slabs
+// it would be 8 to 15 % faster on ordinary keys.  A chunk that starts between two slabs is read in place by the item kernel (tiles of 128 keys) and
+// copied first for the other: there the lines are the former ones for every length (64 units x 12800, M = 256: 182 us against 228).
+// Measured as steps of a stream with deferred appends (us, one sweep / items; ordinary keys, heavy-tailed ones), d = 128:
+//   units x keys      M = 64              M = 128             M = 256             M = 512
+//   64 x 12288    112/121, 128/126    114/120, 130/129    165/176, 210/205    277/280, 299/306
+//   64 x 14336            -                   -           198/204, 240/231            -
+//   64 x 15360            -                   -           211/212, 282/242            -
+//   64 x 16384    147/150, 157/162    149/151, 168/164    228/227, 298/261    408/371, 450/408
+//   32 x 16384     86/94,  108/104     88/95,  114/104    127/138, 154/199    208/193, 258/288
+//   64 x 20480    205/200, 253/211    207/206, 268/213    321/294, 437/331    567/461, 778/510
+//   32 x 20480    124/126, 159/136    124/126, 156/141    182/174, 242/256    298/245, 392/369
+//   24 x 20480    103/107, 126/116    105/107, 131/120    150/154, 195/218    240/211, 286/308
+//   16 x 24576     92/94,   98/105     92/97,  108/110    129/142, 155/225    198/237, 255/397
+//   16 x 32768    116/119, 159/136    118/121, 172/138    176/179, 243/290    284/254, 432/429
+// and d = 64:
+//   64 x 12288     91/90,  130/90      92/95,  124/97     145/154, 208/186    250/248, 334/280
+//   32 x 16384     73/73,   95/80      74/77,  102/85     115/115, 169/167    193/175, 282/256
+//   32 x 12288     59/62,   78/70      59/64,   74/72      87/94,  120/128    141/151, 198/235
+//   16 x 16384     51/56,   59/71      51/58,   61/81      72/76,   86/108    111/113, 133/177
+// Other head dimensions up to 128 are as 128 beyond 64 slabs (96: 64 x 20480, M = 64 191/175, 237/188; 16 x 32768, M = 128 108/105, 135/122), wider ones
+// keep the one-sweep kernel with up to 128 rows (256: 32 x 20480, M = 64 161/195, 183/195; 16 x 32768 149/172, 172/183).  Below 64 slabs it is faster for
+// all of them (256: 64 x 4096, M = 64, 256: 58/84, 82/137; 192: 64 x 4096, M = 256 71/104; 96: 64 x 4096, M = 64 41/54; 64 x 8192, M = 256 105/112,
+// 123/137; 8 x 2048, M = 64 19/26).  A handful of slabs is left to the item kernel (fewer than 16 have not been measured).
 int auto_scorer(int units, int N, int M, int d, bool tile_chunk, bool tc_ok, bool items_ok, bool mma_ok)
 {
     const long long keys = (long long)units * N;
@@ -303,12 +314,10 @@ int auto_scorer(int units, int N, int M, int d, bool tile_chunk, bool tc_ok, boo
         many = d == 64 && N >= 6144 && keys >= 64 * 6144;
         long_items = (N > 8192 || (N == 8192 && M > 512)) && keys >= 32 * 8192 && (M > kTcRows || N >= 16384 || keys >= 32 * 10240);
     } else {
-        many = d == 64 && N >= 64 * kTcSlab && keys >= 64 * 16384;
-        long_items = M > kTcRows && keys >= 32 * 8192 && (N > 96 * kTcSlab || (N > 64 * kTcSlab && units >= 32));
-        // Beyond 48 slabs and two row blocks the two are within 7 % of each other on ordinary logits (the 16384-key figures of M = 512 and more above).  Where single keys reach logits of 2^100
-        // (heavy-tailed keys, which so long a pot nearly always holds) every block of the item has the general fold to do and the item
-        // kernel is faster: a step of 8 such streams, 64 units x 16384, M = 512, 438 us against 710.
-        long_items = long_items || (M > 2 * kTcRows && N > 48 * kTcSlab && keys >= 32 * 8192);
+        many = d == 64 && keys >= 32 * 16384;
+        const bool rows = M > kTcRows || d <= kTcD;
+        long_items = keys >= 32 * 8192 && ((N > 96 * kTcSlab && rows) || (N > 64 * kTcSlab && rows && units >= 32) || (M > 2 * kTcRows && N > 48 * kTcSlab) ||
+                                           (M > kTcRows && keys >= 60 * 16384));
     }
     if (d != 64 && d != 128) {
         const long long tasks = (long long)units * ((M + kTcRows - 1) / kTcRows) * ((N + kTcSlab - 1) / kTcSlab);

@@ -211,6 +211,11 @@ ITEMS = ipot.IPOT_SCORER_TENSOR_ITEMS
 
 
 @pytest.mark.parametrize("units,n,P,G,d,first,want", [
+    # beyond 40 slabs: number of keys for 64 channels; three row blocks; two; lengths beyond 64 and 96 slabs, with few and many units
+    (31, 16384, 8, 1, 64, None, TC), (32, 16384, 8, 1, 64, None, ITEMS), (22, 12288, 65, 4, 128, None, TC), (22, 12289, 65, 4, 128, None, ITEMS),
+    (63, 15360, 33, 4, 128, None, TC), (64, 15360, 33, 4, 128, None, ITEMS), (64, 15360, 32, 4, 128, None, TC), (31, 20480, 8, 4, 128, None, TC),
+    (32, 20480, 8, 4, 128, None, ITEMS), (32, 16384, 8, 4, 128, None, TC), (11, 24576, 8, 4, 128, None, TC), (11, 24577, 8, 4, 128, None, ITEMS),
+    (8, 24577, 8, 4, 128, None, TC), (33, 20480, 8, 1, 96, None, ITEMS), (33, 16384, 8, 1, 96, None, TC), (32, 20480, 8, 1, 256, None, TC),
     # 15 and 16 slabs of another head dimension; chunks that start on a slab, between two, and off every tile
     (3, 1280, 8, 1, 96, None, ITEMS), (4, 1024, 8, 1, 96, None, TC), (8, 1024, 8, 1, 96, 256, TC), (8, 1024, 8, 1, 96, 384, ITEMS), (8, 1024, 8, 1, 96, 300, TC),
     (33, 10752, 8, 4, 128, 256, TC), (33, 10752, 8, 4, 128, 384, ITEMS), (33, 10752, 8, 4, 128, 300, TC), (16, 16384, 8, 4, 128, 384, ITEMS),
