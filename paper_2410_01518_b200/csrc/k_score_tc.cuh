@@ -31,9 +31,10 @@
 // Bound: a task's way through tensor memory, and tensor memory holds two tasks: product 700 cycles, pass 1 4100 beside the other
 // pair's work, exchange 2000, pass 2 1800, hand-overs 500.  (Pass 1 and pass 2 alone would take an SM 2500 cycles per task, without the
 // exchange a launch of 256 units takes 66 us.)  The polls are what the exchange costs: with an entry per 128 keys instead of one per
-// 256 the last of these figures were 85.2, 173, 18.5 and 384.  Measured against the form in which all 16 warps
+// 256 the last of these figures were 85.2, 173, 18.5 and 384.  Keys far beyond a row's others cost it more: 256 units x 4096 keys of Student t
+// (3 degrees) 88 us, with one far key in every unit 99.  Measured against the form in which all 16 warps
 // shared a task, took maxima, and four more warps combined and polled (us, alone): 256 units x 4096 keys, M = 128 90.1 -> 82; 128 x
-// 8192, M = 256 197 -> 157; 60 x 2999, M = 57 20.8 -> 18.5; 64 x 16384, M = 512 537 -> 333; items -> this: 64 x 4096 x 256 channels, M = 64 51 -> 27.  Error of the scores against
+// 8192, M = 256 197 -> 157; 60 x 2999, M = 57 20.8 -> 18.5; 64 x 16384, M = 512 537 -> 333; items -> this: 64 x 4096 x 256 channels, M = 64 51 -> 33.  Error of the scores against
 // 64 bits 4.5e-7 -> 1.6e-7 (fewer roundings, a polynomial of degree 5, the tensor core's cut sums made good).
 //
 // Blocks of one grid wait on each other (pass 2 needs the other slabs' statistics),
@@ -144,16 +145,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)   // never blocks
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
 // Bounded wait.  Every block notes a deadline (its start + the launch's wait limit) next to its give-up flag; a
 // wait that is still unsatisfied then records IPOT_E_TIMEOUT and raises the flag.  Once the flag is up, later waits
 // of the block return at once (false) - unless heed_flag is off, which is how a role waits for work it has itself
@@ -248,18 +239,6 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[32])
           "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
         :: "memory");
 }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32])
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
-        ::"r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-          "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
-          "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]),
-          "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]),
-          "r"(taddr) : "memory");
-}
 // 16 consecutive fp32 columns of this thread's TMEM lane (asynchronous: see tmem_wait_ld16).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16])
 {
@@ -282,7 +261,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Named barriers: of the four warps of an epilogue group, and of the two groups that share a buffer.
-// (Barrier numbers are immediates so that the kernel claims seven of the SM's barriers, not all sixteen.)
+// (With those of the turns below, fifteen of the SM's sixteen: one block has the SM to itself.)
 __device__ __forceinline__ void group_sync(int g)
 {
     switch (g) {
@@ -1029,6 +1008,12 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
 }
 
 // ------------------------------------------------------------------ host side
+// log2(e) / sqrt(d) for products of the tensor core, which cuts its running sums instead of rounding them: a logit comes out short by about
+// 1.2e-8 of itself per 16-channel step, which is made good here.  (Right on average: products that happen to be exact become as much too large.
+// Error of the item scorer's scores against 64 bits, 2-norm, without / with: 4096 keys of 256 channels 7.7e-7 / 4.5e-7, 3000 of 192
+// 5.5e-7 / 3.1e-7, 8192 of 128 4.2e-7 / 2.5e-7; warp-level tensor cores 6.3e-7, 4.5e-7, 2.9e-7.)
+inline float tensor_scale_log2e(int d) { return (float)(1.4426950408889634 / sqrt((double)d) * (1.0 + 1.2e-8 * ((d + 15) / 16))); }
+
 typedef CUresult (*TcEncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -1197,7 +1182,7 @@ inline int tc_launch(TcPlan &plan, const ipot_config_t &cfg, const void *Q, cons
     prm.qslots = 2 * prm.q_bytes + 2 * prm.k_bytes <= 2 * kTcStageBytes ? 2 : 1;   // 256 channels: 2 + 2 slots up to 64 query rows, else 1 + 2; 192: 2 + 3, 2 + 2
     prm.kslots = std::min<int>(kTcMaxK, (2 * kTcStageBytes - prm.qslots * prm.q_bytes) / prm.k_bytes);
     prm.new_slab0 = Knew ? new_first / kTcSlab : 0x7fffffff;
-    prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d) * (1.0 + 1.2e-8 * prm.ksteps));
+    prm.scale_log2e = tensor_scale_log2e(cfg.d);
     prm.wait_ns = wait_ns;
     prm.withhold_cta = withhold_cta;
     if (!plan.captured) {

@@ -877,10 +877,7 @@ inline int tw_launch(TwPlan &plan, TcPlan &enc, const ipot_config_t &cfg, const 
     prm.sums = plan.part;
     prm.refs = plan.part + (size_t)prm.jobs * prm.mt * kTwTile;
     prm.new_tile0 = Knew ? new_first / kTwTile : 0x7fffffff;
-    // The tensor core cuts its running sums instead of rounding them: a logit comes out short by about 1.2e-8 of itself per
-    // 16-channel step, which is made good here.  (Error of the scores against 64 bits, 2-norm, without / with: 4096 keys of 256
-    // channels 7.7e-7 / 4.5e-7, 3000 of 192 5.5e-7 / 3.1e-7, 8192 of 128 4.2e-7 / 2.5e-7; warp-level tensor cores 6.3e-7, 4.5e-7, 2.9e-7.)
-    prm.scale_log2e = (float)(1.4426950408889634 / sqrt((double)cfg.d) * (1.0 + 1.2e-8 * prm.ksteps));
+    prm.scale_log2e = tensor_scale_log2e(cfg.d);
     prm.wait_ns = wait_ns;
     prm.withhold_job = withhold_job;
     prm.ctas = 2 * prm.jobs < ctas ? 2 * prm.jobs : ctas;
