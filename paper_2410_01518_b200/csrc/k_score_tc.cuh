@@ -542,6 +542,24 @@ __device__ __forceinline__ float poll_entries(const float *st, int n, float sgn,
     }
     return v[0];
 }
+// A slab's entry of a row whose halves have references, or whose sum is no number.  (This and weight_apart are functions of their own to be out of
+// the way: in line they cost a launch of one round 0.3 us, one layer's cycle 29.4 against 29.0.)
+__device__ __noinline__ void publish_apart(const TcParams &prm, size_t at, float2 s, float2 o)
+{
+    float m = fmaxf(s.y == 0.f ? -INFINITY : s.x, o.y == 0.f ? -INFINITY : o.x);
+    if (m == -INFINITY) m = 0.f;
+    const float sum = (s.y == 0.f ? 0.f : s.y * ex2(s.x - m)) + (o.y == 0.f ? 0.f : o.y * ex2(o.x - m));
+    const float plain = m >= kTcRefLow && m <= 118.f ? sum * ex2(m) : INFINITY;
+    if (plain <= kTcPlainMax) {   // (a NaN takes the other way, or it would never count as fresh)
+        st_gpu_f32(prm.stats + at, plain * prm.sign);
+        return;
+    }
+    float *r = reinterpret_cast<float *>(prm.refs + at);
+    st_gpu_f32(r, m);
+    st_gpu_f32(r + 1, sum);
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    st_gpu_f32(prm.stats + at, INFINITY * prm.sign);
+}
 // Sum of n of a row's entries of which some are given as (reference, sum), by the thread that has seen their marks: all loads
 // in flight, relative to the largest.  (Every block that has a slab of the item comes here for one far logit in one of them.)
 __device__ __noinline__ void fold_entries(const TcParams &prm, int item, int row, int half, float2 *to)
@@ -579,6 +597,20 @@ __device__ __noinline__ void fold_entries(const TcParams &prm, int item, int row
         m = mb;
     }
     *to = m == -INFINITY ? make_float2(0.f, kTcTiny) : make_float2(m, l);
+}
+
+// A row's weight where a sum is not plain or the slab has a reference, and whether it is given 2^kTcLift times as large
+__device__ __noinline__ float2 weight_apart(float l0, float l1, const float2 *lfar, float2 own, float ref)
+{
+    float2 t = make_float2(0.f, l0 + l1);
+    if (t.y == INFINITY) t = add_sums(l0 == INFINITY ? lfar[0] : make_float2(0.f, l0), l1 == INFINITY ? lfar[kTcRows] : make_float2(0.f, l1));
+    if (own.x > -INFINITY) t = add_sums(t, own);
+    t = normalised(t);
+    const float d = fminf(ref - t.x, 8.f);   // (above 2 only where there is nothing to weigh)
+    const bool far = d < -kTcReach;
+    float w;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(t.y));
+    return make_float2(w * ex2(far ? d + kTcLift : d), far ? 1.f : 0.f);
 }
 
 // Pass 2 for one warp over 32 rows x 32 columns: a[] and b[] are the 16x256b loads of the warp's TMEM lanes
@@ -886,22 +918,9 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             pair_sync(pair);
             if (!half && (int)blockIdx.x != prm.withhold_cta) {
                 const float2 o = spart[par * kTcRows + row];
-                float *to = prm.stats + ((size_t)item * S + slab) * kTcRows + row;
-                float m = 0.f, sum = s.y + o.y, plain = sum;
-                if (s.x != 0.f || o.x != 0.f) {
-                    m = fmaxf(s.y == 0.f ? -INFINITY : s.x, o.y == 0.f ? -INFINITY : o.x);   // (one of them is not empty)
-                    sum = (s.y == 0.f ? 0.f : s.y * ex2(s.x - m)) + (o.y == 0.f ? 0.f : o.y * ex2(o.x - m));
-                    plain = m >= kTcRefLow && m <= 118.f ? sum * ex2(m) : INFINITY;
-                }
-                if (plain <= kTcPlainMax) {   // (a NaN takes the other way, or it would never count as fresh)
-                    st_gpu_f32(to, plain == 0.f ? kTcTiny * sgn : plain * sgn);
-                } else {
-                    float *r = reinterpret_cast<float *>(prm.refs + ((size_t)item * S + slab) * kTcRows + row);
-                    st_gpu_f32(r, m);
-                    st_gpu_f32(r + 1, sum);
-                    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-                    st_gpu_f32(to, INFINITY * sgn);
-                }
+                const size_t at = ((size_t)item * S + slab) * kTcRows + row;
+                if (s.x == 0.f && o.x == 0.f && s.y + o.y <= kTcPlainMax) st_gpu_f32(prm.stats + at, s.y + o.y == 0.f ? kTcTiny * sgn : (s.y + o.y) * sgn);
+                else publish_apart(prm, at, s, o);
             }
             // ---- the row's entries of the whole item, each half of the pair one half of them
             float l = 0.f;
@@ -925,27 +944,16 @@ cap_score_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
             bool far = false;
             if (row < rows) {
                 const float l0 = lpart[(par * 2) * kTcRows + row], l1 = lpart[(par * 2 + 1) * kTcRows + row];
-                float2 t = make_float2(0.f, l0 + l1);
-                bool near = t.y < INFINITY;
-                if (!near)
-                    t = add_sums(l0 == INFINITY ? lfar[(par * 2) * kTcRows + row] : make_float2(0.f, l0),
-                                 l1 == INFINITY ? lfar[(par * 2 + 1) * kTcRows + row] : make_float2(0.f, l1));
-                if (own.x > -INFINITY) {
-                    if (near && own.x <= 110.f) {   // (in the general form for every row it cost 32 layers with CaP keys 3 us)
-                        t.y = fmaf(own.y, ex2(own.x), t.y);
-                    } else {
-                        t = add_sums(t, own);
-                        near = false;
-                    }
+                float l = l0 + l1;
+                const bool plain_own = own.x > -INFINITY && own.x <= 110.f;
+                if (plain_own) l = fmaf(own.y, ex2(own.x), l);
+                if (s.x == 0.f && l < INFINITY && (plain_own || own.x == -INFINITY)) {
+                    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(weight) : "f"(l));
+                } else {
+                    const float2 t = weight_apart(l0, l1, lfar + (par * 2) * kTcRows + row, own, s.x);
+                    weight = t.x;
+                    far = t.y != 0.f;
                 }
-                near = near && s.x == 0.f;
-                if (!near) {
-                    t = normalised(t);
-                    t.x = fminf(s.x - t.x, 8.f);   // (above 2 only where there is nothing to weigh)
-                    far = t.x < -kTcReach;
-                }
-                asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(weight) : "f"(t.y));
-                if (!near) weight *= ex2(far ? t.x + kTcLift : t.x);
             }
             const bool lift = __any_sync(0xffffffffu, far);
             if (lift && !far) weight *= kTcLifted;
