@@ -79,9 +79,9 @@ enum {
                                 it is not co-scheduled with (bf16, d = 64 or 128, at most 512 folded query rows); on request
                                 only: IPOT_E_INVALID if the shape does not allow it */
     IPOT_SCORER_TENSOR_ITEMS = 5 /* tcgen05 kernel in two sweeps whose pieces are dealt to the SMs one by one (bf16, any
-                                d, at most 1024 folded query rows): what AUTO takes for long units, for pots of
-                                other d than 64 and 128 with many query rows and for very small calls; IPOT_E_INVALID if the shape does not
-                                allow it (or its scratch did not fit into the device's memory) */
+                                d, at most 1024 folded query rows): what AUTO takes for long units in quantity, for those whose deferred chunk
+                                starts between two slabs of 256 keys, for pots of other d than 64 and 128 with many query rows and for very
+                                small calls; IPOT_E_INVALID if the shape does not allow it (or its scratch did not fit into the device's memory) */
 };
 
 typedef struct {

@@ -32,7 +32,7 @@
 // pair's work, exchange 2000, pass 2 1800, hand-overs 500.  (Pass 1 and pass 2 alone would take an SM 2500 cycles per task, without the
 // exchange a launch of 256 units takes 66 us.)  The polls are what the exchange costs: with an entry per 128 keys instead of one per
 // 256 the last of these figures were 85.2, 173, 18.5 and 384.  Keys far beyond a row's others cost it more: 256 units x 4096 keys of Student t
-// (3 degrees) 88 us, with one far key in every unit 99.  Measured against the form in which all 16 warps
+// (3 degrees) 88 us, with one far key in every unit 101.  Measured against the form in which all 16 warps
 // shared a task, took maxima, and four more warps combined and polled (us, alone): 256 units x 4096 keys, M = 128 90.1 -> 82; 128 x
 // 8192, M = 256 197 -> 157; 60 x 2999, M = 57 20.8 -> 18.5; 64 x 16384, M = 512 537 -> 333; items -> this: 64 x 4096 x 256 channels, M = 64 51 -> 33.  Error of the scores against
 // 64 bits 4.5e-7 -> 1.6e-7 (fewer roundings, a polynomial of degree 5, the tensor core's cut sums made good).
@@ -383,7 +383,7 @@ __device__ __forceinline__ float piece_max(const uint32_t (&v)[16])
 // Pass 1 for a warp some of whose rows left the range: the first `done` pieces of 16 columns have been stored against the reference r;
 // everything is brought to the reference that the rest needs.  (reference, sum)
 // (The other CTAs of the item wait for this: summed column by column it took twice as long, 256 units x 4096 keys with one far key each 120 us
-// against 99.  A second register set would make it shorter still, but the kernel's own values then no longer survive the call in registers, 85 us
+// against 100.  A second register set would make it shorter still, but the kernel's own values then no longer survive the call in registers, 85 us
 // against 79 without any far key.)
 __device__ __noinline__ float2 pass1_slow(uint32_t taddr, int done, int nvalid, float c, float r)
 {
