@@ -98,7 +98,7 @@ enum {
 struct TcParams {
     float *scores;        // partial array p (query rows 128p ...) at scores + p * part_stride, unit stride N
     size_t part_stride;
-    float *stats;         // [items][slabs][128] a row's sum over a slab's keys, times the launch's sign (infinite: its reference is not 0, see
+    float *stats;         // [items][slabs][128] a row's sum over a slab's keys, times the launch's sign (infinite: beyond the plain range, see
                           // refs); all of the other sign or 0 at launch
     float2 *refs;         // [items][slabs][128] (reference, sum) of those
     const float2 *cap_stats;  // NULL, or [units][M] (max, sum) over the CaP's own keys that join every row's denominator
@@ -303,8 +303,8 @@ __device__ __forceinline__ float max3(float a, float b, float c)
     return y;
 }
 
-// The reference of a row over a half slab: 0 if the largest of its first logits lies between 0 and 2^kTcNear, else that logit, in binary
-// orders and rounded down to a whole number (moving a sum to another reference is then exact, and no exponential is below its
+// The reference of a row over a half slab: 0 if the largest of its first logits (in binary orders) lies between 0 and kTcNear, else that logit
+// rounded down to a whole number (moving a sum to another reference is then exact, and no exponential is below its
 // probability).  Where no logit is within fp32's range it is 0 and pass1_slow looks at the others.
 constexpr float kTcNear = 32.f;
 __device__ __forceinline__ float row_reference(float mx, float c)
